@@ -1,0 +1,604 @@
+// Tensor-core linear with the weights as the row operand of tcgen05.mma and the tokens as its N side (cta_group::2).
+//
+// A pair of CTAs computes 256 output columns (128 each) for up to 512 tokens, over a slice of the contraction; the
+// accumulator is the transposed output tile.  Every weight is dequantized once per chunk of tokens, whatever their number,
+// the tensor core does no work for rows past the next multiple of 16, and each CTA loads half of the tokens.
+// Roles: warps 0 and 1 load this CTA's half of the (one or two) token boxes by TMA, warp 2 the packed codes (bulk
+// copies, a ring of their own), warp 3 of the leader issues the MMAs, sixteen warps dequantize.  Four of those share a
+// step of 64 contraction elements (one thread = one row of 64 weights, so a block of 64 or more costs one table), four
+// steps are in work at a time.  A ring stage holds a step's token rows and weight tile.  The slices of the contraction are further
+// pairs of the same cluster: each CTA lays its fp32 accumulators down in its own (idle) shared memory and adds up and stores its share of the
+// tokens (rank order: the same bits on every run).
+// Forward reads the weight tile as a K-major operand, the input gradient the same bytes as an MN-major operand.
+// Every wait is bounded (see linear_tc.cuh).
+//
+// What bounds it: the loop of the issuing warp (a dependent chain of about a hundred clocks per wait and commit, so one
+// full and one empty barrier per step, 32-bit descriptors, no divisions), then dequantization (about 500 clocks per 64
+// weights of a row and warp).
+#pragma once
+
+namespace lq {
+namespace tc {
+
+constexpr int kSwDeqWarps = 16;
+constexpr int kSwFirstDeq = 4;                                  // warps 0..3: token boxes, packed codes, MMA
+constexpr int kSwThreads = (kSwFirstDeq + kSwDeqWarps) * 32;
+constexpr int kSwWBytes = 128 * 128;                            // this CTA's bf16 weight tile of one step
+constexpr int kSwMaxStages = 8;
+constexpr int kSwTail = 512;                                    // barriers, tensor-memory slot, abort flag
+
+struct SwapParams {
+    QView q;
+    __nv_bfloat16* out;
+    int* status;
+    int M;
+    int out_cols;            // N (forward) or K (backward)
+    int steps_q, steps_d;    // contraction steps with dequantized weights / of the rank-r term
+    int c_base;              // first output column of this launch
+    int nbox, box;           // token boxes (1 or 2) and tokens per box (a multiple of 16, at most 256; half of them per CTA)
+    int ss, sp;              // stages of the token + weight ring and of the packed-code ring
+    uint32_t tmem_cols;
+};
+
+// Ring position with a stage count known at run time; advances by up to a few passes.
+struct RingAt {
+    int s; uint32_t ph;
+    __device__ __forceinline__ RingAt(int step, int S) : s(step % S), ph((step / S) & 1) {}
+    __device__ __forceinline__ void advance(int n, int S) { s += n; while (s >= S) { s -= S; ph ^= 1u; } }
+};
+
+// Shared-memory matrix descriptor as two words: the low one (address, leading offset) advances with the operand, the high
+// one (stride offset 1024 bytes, descriptor version, 128-byte swizzle) is constant.
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr, uint32_t lbo_bytes) { return ((saddr & 0x3FFFFu) >> 4) | ((lbo_bytes >> 4) << 16); }
+// Commit to the barrier at the same offset in the CTAs of `mask` (cluster ranks).
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t mask) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(bar), "h"(mask) : "memory");
+}
+__device__ __forceinline__ void tc_mma2_lo(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(kDescHi), "r"(accumulate) : "memory");
+}
+
+// The 64 weights of one row of a step.  words0 / words1: shared-memory addresses of the first word of the two 32-column
+// groups (the others 128 bytes apart); s[h] = scale of the columns 16 h .. 16 h + 15; nsc = distinct scales (1, 2, 4).
+// Chunk o (16 bytes) of the row lives at dst + (16 o ^ xr).
+template <int B>
+__device__ __forceinline__ void dequant_row64(uint32_t words0, uint32_t words1, const float (&s)[4], int nsc, uint32_t dst, uint32_t xr,
+                                              const float* __restrict__ lut8) {
+    BlockTable<B == 8 ? 2 : B> tab;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        uint32_t w[B];
+#pragma unroll
+        for (int i = 0; i < B; ++i) w[i] = lds_u32((g ? words1 : words0) + i * 128);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int h = 2 * g + (c >> 1);
+            const uint32_t x = dst + ((g * 64 + c * 16) ^ xr);
+            if constexpr (B == 8) {
+                uint32_t packed[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t ww = w[2 * c + (e >> 1)] >> (16 * (e & 1));
+                    const float q0 = lut8[(ww & 255u) << 5], q1 = lut8[((ww >> 8) & 255u) << 5];
+                    const __nv_bfloat162 hh = __floats2bfloat162_rn(__fmul_rn(q0, s[h]), __fmul_rn(q1, s[h]));
+                    packed[e] = *reinterpret_cast<const uint32_t*>(&hh);
+                }
+                sts_v4(x, packed[0], packed[1], packed[2], packed[3]);
+            } else {
+                if ((c & 1) == 0 && (h == 0 || nsc == 4 || (nsc == 2 && h == 2))) tab.build(s[h]);
+                const uint32_t sel = chunk_selector<B>(w, c);
+                uint32_t selA = sel, selB = 0u;
+                if constexpr (B == 4) { selA = sel & 0x77777777u; selB = ((sel >> 1) & 0x44444444u) | 0x32103210u; }
+                uint32_t o[4];
+                tab.lookup4(selA, selB, o[0], o[1]);
+                tab.lookup4(selA >> 16, selB >> 16, o[2], o[3]);
+                sts_v4(x, o[0], o[1], o[2], o[3]);
+            }
+        }
+    }
+}
+
+__device__ __forceinline__ float4 ld_dsmem_f32x4(uint32_t local_addr, uint32_t rank) {
+    uint32_t ra;
+    float4 v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(local_addr), "r"(rank));
+    asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(ra) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+template <int B, bool BWD>
+__global__ void __launch_bounds__(kSwThreads, 1)
+tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT,
+                      const __grid_constant__ CUtensorMap tmF, const SwapParams p) {
+    constexpr int P_BYTES = 1024 * B;
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+    const int half_box = p.box >> 1, half_bytes = half_box * 128;
+    const int x_bytes = p.nbox * half_bytes;
+    const int stage_bytes = kSwWBytes + x_bytes;                         // [weight tile][token boxes]
+    uint8_t* p_ring = base + p.ss * stage_bytes;
+    uint8_t* tail = p_ring + p.sp * P_BYTES;
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);     // full[8], empty[8], full_p[8], empty_p[8], fbar[2], acc_full, drain
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 36 * 8);
+    volatile int* abort_s = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    float* lut8 = reinterpret_cast<float*>(tail + kSwTail);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank() & 1u;                           // CTA of the pair; 0 = leader
+    const int c0 = p.c_base + blockIdx.x * 128;                          // first output column of this CTA
+    const int m0 = blockIdx.y * (p.nbox * p.box);                        // first token
+    const int nsplit = gridDim.z, split = blockIdx.z;
+    const int q_lo = static_cast<int>(static_cast<long long>(p.steps_q) * split / nsplit);
+    const int nq = static_cast<int>(static_cast<long long>(p.steps_q) * (split + 1) / nsplit) - q_lo;
+    const int total = nq + (split == 0 ? p.steps_d : 0);                 // the rank-r steps go to the first slice
+    const int have = min(2, max(0, (p.out_cols - c0 + 63) >> 6));        // 64-column tiles of this CTA that exist
+    const Ctl ctl{abort_s, p.status};
+
+    const uint32_t ring = smem_u32(base), bar0 = smem_u32(bars);
+    auto full = [&](int s) { return bar0 + 8 * s; };                     // the step's operands (leader: of both CTAs)
+    auto empty = [&](int s) { return bar0 + 64 + 8 * s; };
+    auto full_p = [&](int s) { return bar0 + 128 + 8 * s; };
+    auto empty_p = [&](int s) { return bar0 + 192 + 8 * s; };
+    auto fbar = [&](int d) { return bar0 + 256 + 8 * d; };
+    const uint32_t acc_full = bar0 + 272, drain = bar0 + 280;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kSwMaxStages; ++s) {
+            // token boxes and four dequantization warps; leader: also the word of the second CTA that its step is complete
+            mbar_init(full(s), p.nbox + 4 + (rank == 0 ? 1 : 0));
+            mbar_init(empty(s), 1);
+            mbar_init(full_p(s), 1);
+            mbar_init(empty_p(s), 4);
+        }
+        mbar_init(fbar(0), 1);
+        mbar_init(fbar(1), 1);
+        mbar_init(acc_full, 1);
+        mbar_init(drain, 1);
+        *abort_s = 0;
+        fence_barrier_init();
+    }
+    if constexpr (B == 8) {
+        for (int i = threadIdx.x; i < 256 * 32; i += kSwThreads) lut8[i] = c_codebook[3][i >> 5];     // one copy per bank
+    }
+    if (warp == 3) { tmem_alloc2(smem_u32(tmem_slot), p.tmem_cols); tmem_relinquish2(); }
+    tc_fence_before();
+    __syncthreads();
+    cluster_barrier();                                    // barriers of both CTAs are initialised before any remote arrive
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    bool acc_ok = false;
+
+    if (warp < p.nbox) {
+        // ------------------------------------------------------------------ this CTA's half of token box `warp`
+        RingAt r(0, p.ss);
+        const int row = m0 + warp * p.box + static_cast<int>(rank) * half_box;
+        uint32_t dst0 = ring + kSwWBytes + warp * half_bytes;
+        int k = q_lo * BK;
+        for (int step = 0; step < total; ++step, r.advance(1, p.ss), k += BK) {
+            if (!wait(empty(r.s), r.ph ^ 1, ctl, 51)) break;
+            if (step == nq) {
+                // the rank-r intermediate comes from the kernel in front (programmatic dependent launch)
+                pdl_wait();
+                fence_proxy_async_all();
+            }
+            __syncwarp();
+            if (elect_one()) {
+                mbar_expect_tx(full(r.s), half_bytes);
+                if (step < nq) tma_load_2d(dst0 + r.s * stage_bytes, &tmX, k, row, full(r.s));
+                else tma_load_2d(dst0 + r.s * stage_bytes, &tmT, (step - nq) * BK, row, full(r.s));
+            }
+            __syncwarp();
+        }
+        if (*abort_s && warp == 0) {
+            for (int s = 0; s < p.ss; ++s) {          // let copies in flight land before the CTA exits (bounded)
+                const long long t0 = clock64();
+                while (!mbar_try_wait(full(s), 0) && !mbar_try_wait(full(s), 1) && clock64() - t0 < 20000000LL) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp == 2) {
+        // ------------------------------------------------------------------ packed codes
+        const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
+        RingAt r(0, p.sp);
+        for (int step = 0; step < nq; ++step, r.advance(1, p.sp)) {
+            if (!wait(empty_p(r.s), r.ph ^ 1, ctl, 52)) break;
+            __syncwarp();
+            if (elect_one()) {
+                const uint32_t dst = smem_u32(p_ring) + r.s * P_BYTES;
+                const int qs = q_lo + step;
+                if (have == 0) {
+                    mbar_arrive(full_p(r.s));             // nothing behind the last column: the scales below are zero
+                } else if (!BWD) {
+                    mbar_expect_tx(full_p(r.s), P_BYTES);
+                    bulk_load(dst, codes + (static_cast<size_t>(c0 >> 7) * p.q.ktiles + qs) * P_BYTES, P_BYTES, full_p(r.s));
+                } else {
+                    // 64 rows (half a tile) of the two 64-column tiles of this CTA
+                    const uint8_t* src = codes + (static_cast<size_t>(qs >> 1) * p.q.ktiles + (c0 >> 6)) * P_BYTES + (qs & 1) * (P_BYTES / 2);
+                    mbar_expect_tx(full_p(r.s), have * (P_BYTES / 2));
+                    for (int t = 0; t < have; ++t) bulk_load(dst + t * (P_BYTES / 2), src + t * P_BYTES, P_BYTES / 2, full_p(r.s));
+                }
+            }
+            __syncwarp();
+        }
+        if (*abort_s) {
+            for (int s = 0; s < p.sp; ++s) {
+                const long long t0 = clock64();
+                while (!mbar_try_wait(full_p(s), 0) && !mbar_try_wait(full_p(s), 1) && clock64() - t0 < 20000000LL) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp == 3) {
+        // ------------------------------------------------------------------ MMA issuer (leader), messenger (second CTA)
+        if (rank == 1) {
+            // tells the leader that this CTA's half of a step is complete
+            RingAt r(0, p.ss);
+            for (int step = 0; step < total; ++step, r.advance(1, p.ss)) {
+                if (!wait(full(r.s), r.ph, ctl, 60)) break;
+                __syncwarp();
+                if (elect_one()) mbar_arrive_cluster(full(r.s), cluster_rank() & ~1u);
+            }
+        } else {
+            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 15) |
+                                   (static_cast<uint32_t>(p.box >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
+            const uint32_t a0 = desc_lo(ring, BWD ? 8192 : 16), b0 = desc_lo(ring + kSwWBytes, 16);
+            const uint32_t stage16 = stage_bytes >> 4, box16 = half_bytes >> 4;
+            constexpr uint32_t ka = (BWD ? 2048 : 32) >> 4;            // 16 contraction elements further: rows down, or columns along
+            const uint16_t pair_mask = static_cast<uint16_t>(3u << (cluster_rank() & ~1u));
+            bool ok = true;
+            uint32_t acc = 0;
+            RingAt r(0, p.ss);
+            for (int step = 0; step < total; ++step, r.advance(1, p.ss)) {
+                ok = mbar_try_wait_acq_cluster(full(r.s), r.ph) || wait_cluster(full(r.s), r.ph, ctl, 53);
+                if (!ok) break;
+                __syncwarp();
+                tc_fence_after();
+                const uint32_t a = a0 + r.s * stage16, b = b0 + r.s * stage16;
+                if (elect_one()) {
+                    tc_mma2_lo(tmem, a, b, idesc, acc);
+                    tc_mma2_lo(tmem, a + ka, b + 2, idesc, 1u);
+                    tc_mma2_lo(tmem, a + 2 * ka, b + 4, idesc, 1u);
+                    tc_mma2_lo(tmem, a + 3 * ka, b + 6, idesc, 1u);
+                    if (p.nbox == 2) {
+                        const uint32_t b2 = b + box16;
+                        tc_mma2_lo(tmem + 256, a, b2, idesc, acc);
+                        tc_mma2_lo(tmem + 256, a + ka, b2 + 2, idesc, 1u);
+                        tc_mma2_lo(tmem + 256, a + 2 * ka, b2 + 4, idesc, 1u);
+                        tc_mma2_lo(tmem + 256, a + 3 * ka, b2 + 6, idesc, 1u);
+                    }
+                    tc_commit_pair(step + 1 < total ? empty(r.s) : acc_full, pair_mask);
+                }
+                acc = 1u;
+                __syncwarp();
+            }
+            if (!ok) {
+                __syncwarp();
+                if (elect_one()) tc_commit_pair(drain, pair_mask);      // wait (bounded) for issued MMAs before tensor memory is freed
+                const long long t0 = clock64();
+                while (!mbar_try_wait(drain, 0) && clock64() - t0 < 20000000LL) {}
+            }
+        }
+        __syncwarp();
+    } else if (warp >= kSwFirstDeq) {
+        // ------------------------------------------------------------------ dequantization: four warps per step
+        const int dw = warp - kSwFirstDeq;
+        const int grp = dw >> 2, wi = dw & 3;
+        const QView& q = p.q;
+        // forward: row c0 + 32 wi + lane of the tile; backward: contraction row 32 (wi & 1) + lane, 64-column tile wi >> 1
+        const int row_local = BWD ? (wi & 1) * 32 + lane : wi * 32 + lane;
+        const int my_col = BWD ? c0 + (wi >> 1) * 64 : 0;
+        const bool live = BWD ? my_col < q.K : c0 + row_local < q.N;
+        const uint32_t dst0 = ring + (BWD ? (wi >> 1) * 8192 : 0) + row_local * 128;
+        const uint32_t xr = (row_local & 7) << 4;
+        const uint32_t wsrc = smem_u32(p_ring) + (BWD ? (wi >> 1) * (128 * B) + (wi & 1) * (64 * B) : wi * (64 * B)) * 4;
+        const int nsc = q.B0 == 16 ? 4 : q.B0 == 32 ? 2 : 1;
+        // scale codes of the row's 64 columns (aligned, at most four, one second-level group: B1 >= 16)
+        auto fetch = [&](int st) {
+            RawScale r{0u, 0.0f};
+            const int row = BWD ? st * BK + row_local : c0 + row_local;
+            if (live && row < q.N) {
+                const uint32_t blk = static_cast<uint32_t>(row) * q.KB + ((BWD ? my_col : st * BK) >> q.logB0);
+                if (nsc == 4) r.sc = __ldg(reinterpret_cast<const uint32_t*>(q.sc + blk));
+                else if (nsc == 2) r.sc = __ldg(reinterpret_cast<const uint16_t*>(q.sc + blk));
+                else r.sc = __ldg(q.sc + blk);
+                r.v = __ldg(q.v + (blk >> q.logB1));
+            }
+            return r;
+        };
+        float v_cached = -1.0f, sigma = 0.0f;
+        RawScale slot[2];
+        slot[0] = (grp < nq) ? fetch(q_lo + grp) : RawScale{0u, 0.0f};
+        slot[1] = (grp + 4 < nq) ? fetch(q_lo + grp + 4) : RawScale{0u, 0.0f};
+        RingAt rw(grp, p.ss), rp(grp, p.sp);
+        bool ok = true;
+        for (int step8 = grp; step8 < total && ok; step8 += 8) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int step = step8 + 4 * u;
+                if (step >= total || !ok) break;
+                const uint32_t stage = rw.s * stage_bytes;
+                if (step < nq) {
+                    const RawScale rs = slot[u];
+                    if (step + 8 < nq) slot[u] = fetch(q_lo + step + 8);
+                    if (rs.v != v_cached) { v_cached = rs.v; sigma = __fdiv_rn(rs.v, q.levels); }
+                    float s[4];
+                    s[0] = __fmul_rn(static_cast<float>(rs.sc & 255u), sigma);
+                    s[1] = s[0]; s[2] = s[0]; s[3] = s[0];
+                    if (nsc == 2) { s[2] = __fmul_rn(static_cast<float>(rs.sc >> 8), sigma); s[3] = s[2]; }
+                    if (nsc == 4) {
+                        s[1] = __fmul_rn(static_cast<float>((rs.sc >> 8) & 255u), sigma);
+                        s[2] = __fmul_rn(static_cast<float>((rs.sc >> 16) & 255u), sigma);
+                        s[3] = __fmul_rn(static_cast<float>(rs.sc >> 24), sigma);
+                    }
+                    const int kt = BWD ? (my_col >> 6) : q_lo + step;
+                    const uint32_t src = wsrc + rp.s * P_BYTES;
+                    ok = wait(empty(rw.s), rw.ph ^ 1, ctl, 55) && wait(full_p(rp.s), rp.ph, ctl, 56);
+                    if (!ok) break;
+                    dequant_row64<B>(src + slab_row_slot(lane, 0, kt) * 4, src + (B * 32 + slab_row_slot(lane, 1, kt)) * 4, s, nsc,
+                                     dst0 + stage, xr, lut8 + lane);
+                    fence_proxy_async();            // make the generic-proxy stores visible to the tensor core
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(empty_p(rp.s));
+                    rp.advance(4, p.sp);
+                } else {
+                    // rank-r step: the weight-side operand ([L1] rows or L2 rows) comes by TMA
+                    ok = wait(empty(rw.s), rw.ph ^ 1, ctl, 57);
+                    if (!ok) break;
+                    if (wi == 0) {
+                        const int d = step - nq;
+                        if (lane == 0) {
+                            if (!BWD) {
+                                mbar_expect_tx(fbar(d), kSwWBytes);
+                                tma_load_2d(ring + stage, &tmF, d * BK, c0, fbar(d));
+                            } else {
+                                mbar_expect_tx(fbar(d), have * 8192);
+                                for (int t = 0; t < have; ++t) tma_load_2d(ring + stage + t * 8192, &tmF, c0 + t * 64, d * BK, fbar(d));
+                            }
+                        }
+                        ok = wait(fbar(d), 0, ctl, 59);
+                        if (!ok) break;
+                    }
+                    __syncwarp();
+                }
+                if (lane == 0) mbar_arrive(full(rw.s));
+                rw.advance(4, p.ss);
+            }
+        }
+        // ------------------------------------------------------------------ epilogue: warp = 32 output columns x every fourth chunk of 32 tokens
+        acc_ok = ok && wait(acc_full, 0, ctl, 58);
+        if (acc_ok) {
+            tc_fence_after();
+            const int quarter = warp & 3, chunks = (p.box + 31) >> 5;
+            float* accbuf = reinterpret_cast<float*>(base);           // [token][128 columns], over the idle rings
+            for (int ch = dw >> 2; ch < p.nbox * chunks; ch += 4) {
+                const int h = ch / chunks, t0 = (ch - h * chunks) * 32;
+                uint32_t v[32];
+                tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + h * 256 + t0, v);
+                tmem_ld_wait();
+                if (nsplit > 1) {
+                    float* dst = accbuf + static_cast<size_t>(h * p.box + t0) * 128 + quarter * 32 + lane;
+#pragma unroll
+                    for (int i = 0; i < 32; ++i)
+                        if (t0 + i < p.box) dst[i * 128] = __uint_as_float(v[i]);
+                } else {
+                    // even lanes store columns (n, n + 1) of the even tokens, odd lanes those of the odd tokens
+                    const int n = c0 + quarter * 32 + (lane & ~1);
+                    const int odd = lane & 1;
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) {
+                        const float a = __uint_as_float(v[2 * i]), b = __uint_as_float(v[2 * i + 1]);
+                        const float other = __shfl_xor_sync(0xffffffffu, odd ? a : b, 1);
+                        const uint32_t w = odd ? pack_bf16(other, b) : pack_bf16(a, other);
+                        const int t = t0 + 2 * i + odd, m = m0 + h * p.box + t;
+                        if (t < p.box && m < p.M && n < p.out_cols)
+                            *reinterpret_cast<uint32_t*>(p.out + static_cast<size_t>(m) * p.out_cols + n) = w;
+                    }
+                }
+            }
+        }
+    }
+    if (nsplit > 1) {
+        // every CTA adds up and stores its share of the tokens from the CTAs with the same columns; the barriers are executed
+        // by all threads of all CTAs, whatever happened before
+        const uint32_t acc_addr = ring;
+        const int tokens = p.nbox * p.box;
+        const int t_lo = tokens * split / nsplit, t_hi = tokens * (split + 1) / nsplit;
+        __syncthreads();
+        cluster_barrier();
+        for (int item = threadIdx.x; item < (t_hi - t_lo) * 32; item += kSwThreads) {
+            const int t = t_lo + (item >> 5), cg = (item & 31) * 4;
+            const int m = m0 + t;
+            if (m >= p.M) break;                                   // tokens rise with the item
+            float4 part[4];
+#pragma unroll
+            for (int z = 0; z < 4; ++z)
+                if (z < nsplit) part[z] = ld_dsmem_f32x4(acc_addr + static_cast<uint32_t>(t * 128 + cg) * 4u, rank + 2 * z);
+            float4 sum = part[0];
+#pragma unroll
+            for (int z = 1; z < 4; ++z)
+                if (z < nsplit) { sum.x += part[z].x; sum.y += part[z].y; sum.z += part[z].z; sum.w += part[z].w; }
+            if (c0 + cg < p.out_cols)
+                *reinterpret_cast<uint2*>(p.out + static_cast<size_t>(m) * p.out_cols + c0 + cg) = make_uint2(pack_bf16(sum.x, sum.y), pack_bf16(sum.z, sum.w));
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_barrier();            // tensor and shared memory are released only when no CTA of the cluster uses them any more
+    if (warp == 3) tmem_dealloc2(tmem, p.tmem_cols);
+}
+
+// ------------------------------------------------------------------------------------ host side
+// Clusters of `n` CTAs (one CTA per SM, all of its shared memory) that can be resident at the same time.  A cluster lives
+// inside one GPC, so fewer fit than SMs / n: 15 clusters of eight on a B200, not 18.  Asked once per cluster size; the
+// figures measured on a B200 stand in when there is no device to ask.
+inline int tc_max_clusters(int n) {
+    static int cached[4] = {-1, -1, -1, -1};       // n = 2, 4, 6, 8
+    const int idx = n / 2 - 1;
+    if (cached[idx] >= 0) return cached[idx];
+    const int fallback[4] = {74, 36, 24, 15};
+    int got = 0;
+    auto kern = tc_swap_linear_kernel<3, false>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2, 1, n / 2);
+    cfg.blockDim = dim3(kSwThreads);
+    cfg.dynamicSmemBytes = kSmemLimit;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = n / 2;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&got, kern, &cfg) != cudaSuccess || got <= 0) {
+        cudaGetLastError();
+        got = fallback[idx];
+    }
+    cached[idx] = got;
+    return got;
+}
+
+struct SwapPlan {
+    int chunks, nbox, box, ks;       // token chunks, boxes and tokens per box, slices of the contraction
+    int ss, sp, smem;
+    uint32_t tmem_cols;
+    long long ctas;
+    double us;                       // estimated time
+};
+
+// Ring depths; false when they do not fit.
+inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
+    const int stage = kSwWBytes + pl.nbox * pl.box * 64, pk = 1024 * b0;
+    const int fixed = 1024 + kSwTail + (b0 == 8 ? 32768 : 0);
+    const int room = kSmemLimit - fixed;
+    pl.ss = (room - 4 * pk) / stage;
+    if (pl.ss > kSwMaxStages) pl.ss = kSwMaxStages;
+    if (pl.ss < 3) return false;
+    pl.sp = (room - pl.ss * stage) / pk;
+    if (pl.sp > kSwMaxStages) pl.sp = kSwMaxStages;
+    const int bytes = pl.ss * stage + pl.sp * pk;
+    if (ks > 1 && pl.nbox * pl.box * 512 > bytes) return false;      // the accumulators are laid over the rings
+    pl.smem = fixed + bytes;
+    return true;
+}
+
+// The split of a call that costs least by a simple model: waves of clusters, each with a fixed cost, its steps (the
+// slower of dequantization and tensor core) and its reduction.
+inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+    SwapPlan best{};
+    best.us = -1.0;
+    const double dq = b0 == 2 ? 0.26 : b0 == 3 ? 0.28 : b0 == 4 ? 0.36 : 0.42;      // us per step of 128 x 64 weights
+    const long long pairs = (out_cols + 255) / 256;
+    const int first = static_cast<int>((M + 511) / 512);
+    for (int ch = first; ch <= first + 7; ++ch) {
+        SwapPlan pl{};
+        const int per = static_cast<int>((M + ch - 1) / ch);
+        if (ch > first && per < 32) break;
+        pl.nbox = per > 256 ? 2 : 1;
+        pl.box = ((per + pl.nbox - 1) / pl.nbox + 15) / 16 * 16;
+        const int tokens = pl.nbox * pl.box;
+        pl.chunks = static_cast<int>((M + tokens - 1) / tokens);
+        pl.tmem_cols = 32;
+        while (static_cast<int>(pl.tmem_cols) < (pl.nbox == 2 ? 512 : pl.box)) pl.tmem_cols *= 2;
+        for (int ks = 1; ks <= 4 && ks <= steps_q; ++ks) {
+            if (!swap_rings(b0, ks, pl)) continue;
+            pl.ks = ks;
+            pl.ctas = 2 * pairs * pl.chunks * ks;
+            const long long at_once = tc_max_clusters(2 * ks);
+            const long long waves = (pairs * pl.chunks + at_once - 1) / at_once;
+            const double step = dq > tokens * 0.00115 ? dq : tokens * 0.00115;
+            const double body = 4.0 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 2.0 + tokens * 0.008 : tokens * 0.006);
+            pl.us = waves * body;
+            if (best.us < 0 || pl.us < best.us) best = pl;
+        }
+    }
+    return best;
+}
+
+// The same, with the plans of the last few shapes kept by the calling thread (pure arithmetic, about 3 us).
+inline const SwapPlan& swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+    struct Entry { int b0 = 0, steps_q = 0, steps_d = 0; int64_t M = 0, out_cols = 0; SwapPlan plan; };
+    constexpr int kEntries = 32;
+    thread_local Entry cache[kEntries];
+    const uint64_t h = (static_cast<uint64_t>(M) * 0x9E3779B97F4A7C15ull) ^ (static_cast<uint64_t>(out_cols) * 0xC2B2AE3D27D4EB4Full) ^
+                       (static_cast<uint64_t>(steps_q * 8 + steps_d * 64 + b0) * 0x165667B19E3779F9ull);
+    Entry& e = cache[(h >> 40) % kEntries];
+    if (e.b0 != b0 || e.M != M || e.out_cols != out_cols || e.steps_q != steps_q || e.steps_d != steps_d) {
+        e.plan = make_swap_plan(b0, M, out_cols, steps_q, steps_d);
+        e.b0 = b0; e.M = M; e.out_cols = out_cols; e.steps_q = steps_q; e.steps_d = steps_d;
+    }
+    return e.plan;
+}
+
+template <int B, bool BWD>
+inline int launch_swap(const CUtensorMap& tX, const CUtensorMap& tT, const CUtensorMap& tF, const SwapParams& p, const SwapPlan& pl,
+                       int pairs, cudaStream_t st, bool after_pre) {
+    auto kern = tc_swap_linear_kernel<B, BWD>;
+    static bool attr_done = false;
+    if (!attr_done) {
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
+            cudaGetLastError();
+            return LQLORA_ERR_CUDA;
+        }
+        attr_done = true;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * pairs, pl.chunks, pl.ks);
+    cfg.blockDim = dim3(kSwThreads);
+    cfg.dynamicSmemBytes = pl.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;      // a pair, and the slices of its contraction
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = pl.ks;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = (p.steps_d > 0 && after_pre) ? 2 : 1;      // overlap with the rank-r pre-product kernel in front of it
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tX, tT, tF, p);
+    count_launch(1);
+    if (e != cudaSuccess) { cudaGetLastError(); return LQLORA_ERR_CUDA; }
+    return LQLORA_OK;
+}
+
+// Output columns [c_base, c_base + cols) of a call with the plan `pl`; T: the rank-r intermediate [M][r] (r > 0).
+inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const void* A, int M, void* out, const void* T, int* status,
+                    bool backward, const SwapPlan& pl, int c_base, int cols, cudaStream_t st, bool after_pre) {
+    const int C = backward ? q.N : q.K;
+    SwapParams p;
+    p.q = q;
+    p.out = static_cast<__nv_bfloat16*>(out);
+    p.status = status;
+    p.M = M;
+    p.out_cols = backward ? q.K : q.N;
+    p.steps_q = (C + BK - 1) / BK;
+    p.steps_d = (r + BK - 1) / BK;
+    p.c_base = c_base;
+    p.nbox = pl.nbox; p.box = pl.box; p.ss = pl.ss; p.sp = pl.sp; p.tmem_cols = pl.tmem_cols;
+    CUtensorMap tX, tT, tF;
+    if (!make_map(&tX, A, M, C, pl.box / 2)) return LQLORA_ERR_CUDA;
+    if (r > 0) {
+        if (!make_map(&tT, T, M, r, pl.box / 2)) return LQLORA_ERR_CUDA;
+        const bool ok = backward ? make_map(&tF, L2, r, q.K, 64) : make_map(&tF, L1, q.N, r, 128);
+        if (!ok) return LQLORA_ERR_CUDA;
+    } else {
+        tT = tX; tF = tX;
+    }
+    const int pairs = (cols + 255) / 256;
+    switch (q.b0) {
+        case 2: return backward ? launch_swap<2, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<2, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
+        case 3: return backward ? launch_swap<3, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<3, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
+        case 4: return backward ? launch_swap<4, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<4, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
+        default: return backward ? launch_swap<8, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<8, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
+    }
+}
+
+}  // namespace tc
+}  // namespace lq

@@ -572,6 +572,11 @@ tc_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 // backward T = dY L1 (F = L1 [N, r], MN-major B operand).  Grid = (row tiles of 128, splits of the
 // contraction).  Each CTA accumulates its part in tensor memory; with one split it rounds its tile to bf16 and
 // stores it, with several the splits of a tile form a cluster (see CL below).
+// Warps: four that issue the copies (warp w those of the steps w, w + 4, ...: one thread sustains a tensor copy per about
+// 380 clocks, which made the loop 0.4 us per step with a single one), one that issues the MMAs, four for the epilogue.
+constexpr int kLrProducers = 4;
+constexpr int kLrThreads = (kLrProducers + 1 + 4) * 32;
+
 struct PreParams {
     __nv_bfloat16* T;      // [M][r]
     int* status;
@@ -614,9 +619,10 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
     const Ctl ctl{abort_s, p.status};
     const uint32_t tmem_cols = (p.rp <= 64) ? 64u : 128u;
 
-    auto full = [&](int s) { return smem_u32(bars + s); };
-    auto empty = [&](int s) { return smem_u32(bars + 8 + s); };
-    const uint32_t acc_full = smem_u32(bars + 16), drain = smem_u32(bars + 17);
+    const uint32_t bar0 = smem_u32(bars), ring0 = smem_u32(base);
+    auto full = [&](int s) { return bar0 + 8 * s; };
+    auto empty = [&](int s) { return bar0 + 64 + 8 * s; };
+    const uint32_t acc_full = bar0 + 128, drain = bar0 + 136;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < p.stages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
@@ -625,58 +631,65 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
         *abort_s = 0;
         fence_barrier_init();
     }
-    if (warp == 1) { tmem_alloc(smem_u32(tmem_slot), tmem_cols); tmem_relinquish(); }
+    if (warp == kLrProducers) { tmem_alloc(smem_u32(tmem_slot), tmem_cols); tmem_relinquish(); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool cl_ok = false;          // CL: this thread saw the accumulators complete (epilogue warps)
 
-    if (warp == 0) {
-        if (lane == 0) {
-            for (int i = 0; i < total; ++i) {
-                const int s = i % p.stages;
-                const uint32_t ph = (i / p.stages) & 1;
-                if (!wait(empty(s), ph ^ 1, ctl, 11)) break;
-                const uint32_t a_dst = smem_u32(base + static_cast<size_t>(s) * stage_bytes), b_dst = a_dst + A_BYTES;
-                const int c = (s_lo + i) * BK;
+    if (warp < kLrProducers) {
+        int s = warp;                    // stage and pass of step i; advanced without divisions (stages >= kLrProducers)
+        uint32_t ph = 0;
+        for (int i = warp; i < total; i += kLrProducers) {
+            if (!wait(empty(s), ph ^ 1, ctl, 11)) break;
+            const uint32_t a_dst = ring0 + s * stage_bytes, b_dst = a_dst + A_BYTES;
+            const int c = (s_lo + i) * BK;
+            __syncwarp();
+            if (elect_one()) {
                 mbar_expect_tx(full(s), A_BYTES + b_bytes);
                 tma_load_2d(a_dst, &tmA, c, m0, full(s));
                 if (!BWD) tma_load_2d(b_dst, &tmB, c, 0, full(s));                       // [rp rows of L2] x 64 columns
                 else for (int t = 0; t < p.rp / 64; ++t) tma_load_2d(b_dst + t * 8192, &tmB, t * 64, c, full(s));  // 64 rows of L1
             }
+            __syncwarp();
+            s += kLrProducers;
+            if (s >= p.stages) { s -= p.stages; ph ^= 1u; }
         }
         __syncwarp();
-    } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 16) |
-                                   (static_cast<uint32_t>(p.rp >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
-            bool ok = true;
-            for (int i = 0; i < total && ok; ++i) {
-                const int s = i % p.stages;
-                const uint32_t ph = (i / p.stages) & 1;
-                ok = wait(full(s), ph, ctl, 12);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a_src = smem_u32(base + static_cast<size_t>(s) * stage_bytes), b_src = a_src + A_BYTES;
+    } else if (warp == kLrProducers) {
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 16) |
+                               (static_cast<uint32_t>(p.rp >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
+        bool ok = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < total; ++i) {
+            ok = wait(full(s), ph, ctl, 12);
+            if (!ok) break;
+            __syncwarp();
+            tc_fence_after();
+            const uint32_t a_src = ring0 + s * stage_bytes, b_src = a_src + A_BYTES;
+            if (elect_one()) {
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16) {
                     const uint64_t adesc = make_desc(a_src + k16 * 32, 16, 1024);
                     const uint64_t bdesc = BWD ? make_desc(b_src + k16 * 2048, 8192, 1024) : make_desc(b_src + k16 * 32, 16, 1024);
                     tc_mma(tmem, adesc, bdesc, idesc, (i > 0 || k16 > 0) ? 1u : 0u);
                 }
-                tc_commit(empty(s));
+                tc_commit(i + 1 < total ? empty(s) : acc_full);
             }
-            if (ok) tc_commit(acc_full);
-            else {
-                tc_commit(drain);
-                const long long t0 = clock64();
-                while (!mbar_try_wait(drain, 0) && clock64() - t0 < 20000000LL) {}
-            }
+            __syncwarp();
+            if (++s == p.stages) { s = 0; ph ^= 1u; }
+        }
+        if (!ok) {
+            __syncwarp();
+            if (elect_one()) tc_commit(drain);
+            const long long t0 = clock64();
+            while (!mbar_try_wait(drain, 0) && clock64() - t0 < 20000000LL) {}
         }
         __syncwarp();
     } else {
-        // epilogue warps 2..5: TMEM lane quarter = warp % 4
+        // epilogue warps, one per TMEM lane quarter (warp % 4)
         const int quarter = warp & 3;
         const int m = m0 + quarter * 32 + lane;
         const bool ok = (total > 0) ? wait(acc_full, 0, ctl, 13) : true;
@@ -715,7 +728,7 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
         if (nsplit > 1) dec::cluster_wait();           // every CTA of the cluster has started
         const uint32_t recv_addr = smem_u32(recv);
         const int cols_share = p.rp / nsplit;
-        if (warp >= 2 && cl_ok) {
+        if (warp > kLrProducers && cl_ok) {
             tc_fence_after();
             const int quarter = warp & 3;
             const int row = quarter * 32 + lane;
@@ -738,7 +751,7 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
         }
         __syncthreads();
         if (nsplit > 1) dec::cluster_sync_all();
-        for (int item = threadIdx.x; item < 128 * cols_share; item += 192) {
+        for (int item = threadIdx.x; item < 128 * cols_share; item += kLrThreads) {
             const int row = item & 127, cl = item >> 7;
             float sum = 0.0f;
             for (int src = 0; src < nsplit; ++src) sum += recv[(src * cols_share + cl) * 128 + row];
@@ -748,18 +761,18 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, tmem_cols);
+    if (warp == kLrProducers) tmem_dealloc(tmem, tmem_cols);
 }
 
 template <bool BWD>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kLrThreads, 1)
 tc_lowrank_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const PreParams p) {
     lowrank_body<BWD>(tmA, tmB, p, blockIdx.x, blockIdx.y, gridDim.y);
 }
 
 // The same with the splits of a tile as the CTAs of a cluster (grid.y = cluster size, a power of two up to eight).
 template <bool BWD>
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kLrThreads, 1)
 tc_lowrank_cl_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const PreParams p) {
     lowrank_body<BWD, true>(tmA, tmB, p, blockIdx.x, blockIdx.y, gridDim.y);
 }
@@ -767,7 +780,7 @@ tc_lowrank_cl_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 // Both pre-products of one layer in one launch (the weight-gradient path, which has the GPU to itself): grid.z = 0
 // computes T = X L2^T with (tmA0, tmB0, p0), grid.z = 1 computes T' = dY L1 with (tmA1, tmB1, p1); grid.y = splits of
 // the contraction = cluster size (the same for both), reduced through distributed shared memory.
-__global__ void __launch_bounds__(192, 1)
+__global__ void __launch_bounds__(kLrThreads, 1)
 tc_lowrank_both_kernel(const __grid_constant__ CUtensorMap tmA0, const __grid_constant__ CUtensorMap tmB0, const PreParams p0,
                        const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmB1, const PreParams p1) {
     if (blockIdx.z == 0) lowrank_body<false, true>(tmA0, tmB0, p0, blockIdx.x, blockIdx.y, gridDim.y);
@@ -975,7 +988,7 @@ inline int launch_pre(const CUtensorMap& tA, const CUtensorMap& tB, PreParams p,
     // of the linear kernel that runs beside this one find as many free TPCs as the SM count suggests).
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(mtiles, nsplit);
-    cfg.blockDim = dim3(192);
+    cfg.blockDim = dim3(kLrThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];

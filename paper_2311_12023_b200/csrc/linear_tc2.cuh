@@ -7,10 +7,9 @@
 // shared memories.  Compared with the single-CTA kernel each CTA dequantizes half as many weights per MMA
 // flop and its shared memory serves half of the weight-operand traffic.
 //
-// Per CTA: warp 0 lane 0 loads activations (TMA) and packed codes (bulk copies) into a ring; sixteen
+// Per CTA: warp 0 loads activations (TMA) and packed codes (bulk copies) into a ring; sixteen
 // dequantization warps, eight per step (even / odd steps), write the CTA's half of the weight tile into a
-// second ring and arrive on the LEADER's barrier (remote arrive for the second CTA); the leader's MMA
-// thread waits for the sixteen arrivals of a step, issues the MMAs and commits the ring stages back to both
+// second ring; a warp of the second CTA passes the word that its half is complete on to the leader, whose MMA warp issues the MMAs and commits the ring stages back to both
 // CTAs (multicast commit).  Forward and input gradient share the code (K-major / MN-major weight operand)
 // as in the single-CTA kernel; the rank-r term is one more step whose operands come by TMA; the output
 // leaves through shared memory and TMA stores.
@@ -47,11 +46,15 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Arrive on the barrier at local address `bar` of CTA `rank` of the cluster (release at cluster scope).
+// Arrive on the barrier at local address `bar` of CTA `rank` of the cluster.  Sent by the second CTA's messenger warp after
+// it has waited for this CTA's own barrier of the step: the weights are then in this SM's shared memory and visible to the
+// async proxy (every writer has passed fence.proxy.async before it arrived there), and the copies have landed, so nothing is left
+// for a release at cluster scope to order; the tensor core of this SM reads them from this SM's memory.  Spelled with
+// .release.cluster the arrive takes about 1500 clocks, more than a whole step (8192 x 8192, 128 rows: 60 us against 28).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t rank) {
     uint32_t ra;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(bar), "r"(rank));
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(ra) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(ra) : "memory");
 }
 __device__ __forceinline__ uint32_t mbar_try_wait_acq_cluster(uint32_t bar, uint32_t parity) {
     uint32_t ok;
@@ -121,7 +124,8 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < SA; ++s) { mbar_init(full_a(s), 1); mbar_init(empty_a(s), 1); }
-        for (int s = 0; s < SB; ++s) { mbar_init(full_b(s), 16); mbar_init(empty_b(s), 1); mbar_init(dbar(s), 1); }
+        // eight warps per step; leader: also the word of the second CTA that its half is complete
+        for (int s = 0; s < SB; ++s) { mbar_init(full_b(s), rank == 0 ? 9 : 8); mbar_init(empty_b(s), 1); mbar_init(dbar(s), 1); }
         mbar_init(acc_full, 1);
         mbar_init(drain, 1);
         *abort_s = 0;
@@ -139,15 +143,20 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
     if (warp == 0) {
         // ------------------------------------------------------------------ producer: activations + packed codes of this CTA
-        if (lane == 0) {
-            const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
-            RingPos<SA> ra;
-            for (int step = 0; step < total; ++step, ra.advance()) {
-                const int s = ra.s;
-                if (!wait(empty_a(s), ra.ph ^ 1, ctl, 41)) break;
-                const uint32_t a_dst = smem_u32(a_ring) + s * kPairABytes;
-                const uint32_t p_dst = smem_u32(p_ring) + s * P_BYTES;
-                const int my_m = m0 + static_cast<int>(rank) * 128;
+        const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
+        RingPos<SA> ra;
+        for (int step = 0; step < total; ++step, ra.advance()) {
+            const int s = ra.s;
+            if (!wait(empty_a(s), ra.ph ^ 1, ctl, 41)) break;
+            const uint32_t a_dst = smem_u32(a_ring) + s * kPairABytes;
+            const uint32_t p_dst = smem_u32(p_ring) + s * P_BYTES;
+            const int my_m = m0 + static_cast<int>(rank) * 128;
+            if (step == p.steps_q) {
+                pdl_wait();                           // the rank-r intermediate comes from the kernel in front
+                fence_proxy_async_all();
+            }
+            __syncwarp();
+            if (elect_one()) {
                 if (step < p.steps_q) {
                     if (!BWD) {
                         const int tile_row = (c0 >> 7) + static_cast<int>(rank);
@@ -170,57 +179,66 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                         }
                     }
                 } else {
-                    if (step == p.steps_q) {
-                        pdl_wait();                       // the rank-r intermediate comes from the kernel in front
-                        fence_proxy_async_all();
-                    }
                     const int d = step - p.steps_q;
                     mbar_expect_tx(full_a(s), kPairABytes);
                     tma_load_2d(a_dst, &tmA2, d * BK, my_m, full_a(s));
                     tma_load_2d(a_dst + 16384, &tmA2, d * BK, my_m + 256, full_a(s));
                 }
             }
-            if (*abort_s) {
-                for (int s = 0; s < SA; ++s) {
-                    const long long t0 = clock64();
-                    while (!mbar_try_wait(full_a(s), 0) && !mbar_try_wait(full_a(s), 1) && clock64() - t0 < 20000000LL) {}
-                }
+            __syncwarp();
+        }
+        if (*abort_s) {
+            for (int s = 0; s < SA; ++s) {
+                const long long t0 = clock64();
+                while (!mbar_try_wait(full_a(s), 0) && !mbar_try_wait(full_a(s), 1) && clock64() - t0 < 20000000LL) {}
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer (leader CTA only)
-        if (lane == 0 && rank == 0) {
+        // ------------------------------------------------------------------ MMA issuer (leader CTA), messenger (second CTA)
+        if (rank == 1) {
+            // tells the leader that this CTA's half of a step is complete
+            RingPos<SB> rb;
+            for (int step = 0; step < total; ++step, rb.advance()) {
+                if (!wait(full_b(rb.s), rb.ph, ctl, 49)) break;
+                __syncwarp();
+                if (elect_one()) mbar_arrive_cluster(full_b(rb.s), 0);
+            }
+        } else {
             constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 16) |
                                        (static_cast<uint32_t>(BN >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
             bool ok = true;
             RingPos<SA> ra;
             RingPos<SB> rb;
-            for (int step = 0; step < total && ok; ++step, ra.advance(), rb.advance()) {
+            for (int step = 0; step < total; ++step, ra.advance(), rb.advance()) {
                 const int sa = ra.s, sb = rb.s;
-                // sixteen arrivals: the eight warps of this step in each CTA, each after its CTA's copies have landed
+                // the eight warps of this step, each after its CTA's copies have landed, and the second CTA's messenger
                 ok = mbar_try_wait_acq_cluster(full_b(sb), rb.ph) || wait_cluster(full_b(sb), rb.ph, ctl, 42);
                 if (!ok) break;
+                __syncwarp();
                 tc_fence_after();
                 const uint32_t a_src = smem_u32(a_ring) + sa * kPairABytes;
                 const uint32_t b_src = smem_u32(b_ring) + sb * kPairBBytes;
+                if (elect_one()) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
+                    for (int h = 0; h < 2; ++h) {
 #pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16) {
-                        const uint64_t adesc = make_desc(a_src + h * 16384 + k16 * 32, 16, 1024);
-                        const uint64_t bdesc = BWD ? make_desc(b_src + k16 * 2048, 8192, 1024)
-                                                   : make_desc(b_src + k16 * 32, 16, 1024);
-                        tc_mma2(tmem + h * BN, adesc, bdesc, idesc, (step > 0 || k16 > 0) ? 1u : 0u);
+                        for (int k16 = 0; k16 < 4; ++k16) {
+                            const uint64_t adesc = make_desc(a_src + h * 16384 + k16 * 32, 16, 1024);
+                            const uint64_t bdesc = BWD ? make_desc(b_src + k16 * 2048, 8192, 1024)
+                                                       : make_desc(b_src + k16 * 32, 16, 1024);
+                            tc_mma2(tmem + h * BN, adesc, bdesc, idesc, (step > 0 || k16 > 0) ? 1u : 0u);
+                        }
                     }
+                    tc_commit_both(empty_a(sa));
+                    tc_commit_both(empty_b(sb));
+                    if (step + 1 == total) tc_commit_both(acc_full);
                 }
-                tc_commit_both(empty_a(sa));
-                tc_commit_both(empty_b(sb));
+                __syncwarp();
             }
-            if (ok) {
-                tc_commit_both(acc_full);
-            } else {
-                tc_commit_both(drain);
+            if (!ok) {
+                __syncwarp();
+                if (elect_one()) tc_commit_both(drain);
                 const long long t0 = clock64();
                 while (!mbar_try_wait(drain, 0) && clock64() - t0 < 20000000LL) {}
             }
@@ -341,10 +359,7 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                     }
                 }
                 __syncwarp();
-                if (lane == 0) {
-                    if (rank == 0) mbar_arrive(full_b(sb));
-                    else mbar_arrive_cluster(full_b(sb), 0);
-                }
+                if (lane == 0) mbar_arrive(full_b(sb));
                 ra.advance(); ra.advance();
                 rb.advance(); rb.advance();
             }

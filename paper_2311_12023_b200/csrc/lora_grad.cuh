@@ -53,9 +53,10 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
     const Ctl ctl{abort_s, p.status};
     const uint32_t tmem_cols = (p.rp <= 64) ? 64u : 128u;
 
-    auto full = [&](int s) { return smem_u32(bars + s); };
-    auto empty = [&](int s) { return smem_u32(bars + 8 + s); };
-    const uint32_t acc_full = smem_u32(bars + 16), drain = smem_u32(bars + 17);
+    const uint32_t bar0 = smem_u32(bars), ring0 = smem_u32(base);
+    auto full = [&](int s) { return bar0 + 8 * s; };
+    auto empty = [&](int s) { return bar0 + 64 + 8 * s; };
+    const uint32_t acc_full = bar0 + 128, drain = bar0 + 136;
 
     // first phase of the cluster barrier: every CTA of the cluster runs before its shared memory is written remotely
     if (nsplit > 1) dec::cluster_arrive_relaxed();
@@ -74,55 +75,65 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
     bool acc_ok = false;
 
     if (warp == 0) {
-        if (lane == 0) {
-            // The kernel that writes T may still be running (programmatic dependent launch): the tiles of A of the
-            // first ring pass are requested at once, the tiles of T only after that kernel has finished.
-            const int first = min(total, p.stages);
-            for (int i = 0; i < first; ++i) {
-                const uint32_t a_dst = smem_u32(base + static_cast<size_t>(i) * stage_bytes);
-                const int m = (s_lo + i) * BK;               // first token row of the step (rows past M read as zero)
+        // The kernel that writes T may still be running (programmatic dependent launch): the tiles of A of the
+        // first ring pass are requested at once, the tiles of T only after that kernel has finished.
+        const int first = min(total, p.stages);
+        for (int i = 0; i < first; ++i) {
+            const uint32_t a_dst = ring0 + i * stage_bytes;
+            const int m = (s_lo + i) * BK;               // first token row of the step (rows past M read as zero)
+            if (elect_one()) {
                 mbar_expect_tx(full(i), A_BYTES + b_bytes);
                 for (int t = 0; t < 2; ++t) tma_load_2d(a_dst + t * 8192, &tmA, p0 + t * 64, m, full(i));
             }
-            pdl_wait();
-            fence_proxy_async_all();
-            for (int i = 0; i < first; ++i) {
-                const uint32_t b_dst = smem_u32(base + static_cast<size_t>(i) * stage_bytes) + A_BYTES;
-                const int m = (s_lo + i) * BK;
+            __syncwarp();
+        }
+        pdl_wait();
+        fence_proxy_async_all();
+        for (int i = 0; i < first; ++i) {
+            const uint32_t b_dst = ring0 + i * stage_bytes + A_BYTES;
+            const int m = (s_lo + i) * BK;
+            if (elect_one()) {
                 for (int t = 0; t < p.rp / 64; ++t) tma_load_2d(b_dst + t * 8192, &tmT, t * 64, m, full(i));
             }
-            for (int i = first; i < total; ++i) {
-                const int s = i % p.stages;
-                const uint32_t ph = (i / p.stages) & 1;
-                if (!wait(empty(s), ph ^ 1, ctl, 61)) break;
-                const uint32_t a_dst = smem_u32(base + static_cast<size_t>(s) * stage_bytes), b_dst = a_dst + A_BYTES;
-                const int m = (s_lo + i) * BK;
+            __syncwarp();
+        }
+        int s = 0;                        // stage and pass of step i, advanced without divisions
+        uint32_t ph = 1;
+        for (int i = first; i < total; ++i) {
+            if (!wait(empty(s), ph ^ 1, ctl, 61)) break;
+            const uint32_t a_dst = ring0 + s * stage_bytes, b_dst = a_dst + A_BYTES;
+            const int m = (s_lo + i) * BK;
+            __syncwarp();
+            if (elect_one()) {
                 mbar_expect_tx(full(s), A_BYTES + b_bytes);
                 for (int t = 0; t < 2; ++t) tma_load_2d(a_dst + t * 8192, &tmA, p0 + t * 64, m, full(s));
                 for (int t = 0; t < p.rp / 64; ++t) tma_load_2d(b_dst + t * 8192, &tmT, t * 64, m, full(s));
             }
-            if (*abort_s) {
-                // let copies that are still in flight land before the CTA exits (bounded)
-                for (int s = 0; s < p.stages; ++s) {
-                    const long long t0 = clock64();
-                    while (!mbar_try_wait(full(s), 0) && !mbar_try_wait(full(s), 1) && clock64() - t0 < 20000000LL) {}
-                }
+            __syncwarp();
+            if (++s == p.stages) { s = 0; ph ^= 1u; }
+        }
+        if (*abort_s) {
+            // let copies that are still in flight land before the CTA exits (bounded)
+            for (int s = 0; s < p.stages; ++s) {
+                const long long t0 = clock64();
+                while (!mbar_try_wait(full(s), 0) && !mbar_try_wait(full(s), 1) && clock64() - t0 < 20000000LL) {}
             }
         }
         __syncwarp();
     } else if (warp == 1) {
-        if (lane == 0) {
-            // fp32 accumulators, bf16 operands, both MN-major (bits 15 and 16), N = rp, M = 128
-            const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                                   (static_cast<uint32_t>(p.rp >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
-            bool ok = true;
-            for (int i = 0; i < total && ok; ++i) {
-                const int s = i % p.stages;
-                const uint32_t ph = (i / p.stages) & 1;
-                ok = wait(full(s), ph, ctl, 62);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a_src = smem_u32(base + static_cast<size_t>(s) * stage_bytes), b_src = a_src + A_BYTES;
+        // fp32 accumulators, bf16 operands, both MN-major (bits 15 and 16), N = rp, M = 128
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                               (static_cast<uint32_t>(p.rp >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
+        bool ok = true;
+        int s = 0;
+        uint32_t ph = 0;
+        for (int i = 0; i < total; ++i) {
+            ok = wait(full(s), ph, ctl, 62);
+            if (!ok) break;
+            __syncwarp();
+            tc_fence_after();
+            const uint32_t a_src = ring0 + s * stage_bytes, b_src = a_src + A_BYTES;
+            if (elect_one()) {
 #pragma unroll
                 for (int k16 = 0; k16 < 4; ++k16) {
                     // 16 token rows = 2048 bytes down the tile; groups of 64 columns are 8192 bytes apart
@@ -130,14 +141,16 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
                     const uint64_t bdesc = make_desc(b_src + k16 * 2048, 8192, 1024);
                     tc_mma(tmem, adesc, bdesc, idesc, (i > 0 || k16 > 0) ? 1u : 0u);
                 }
-                tc_commit(empty(s));
+                tc_commit(i + 1 < total ? empty(s) : acc_full);
             }
-            if (ok) tc_commit(acc_full);
-            else {
-                tc_commit(drain);
-                const long long t0 = clock64();
-                while (!mbar_try_wait(drain, 0) && clock64() - t0 < 20000000LL) {}
-            }
+            __syncwarp();
+            if (++s == p.stages) { s = 0; ph ^= 1u; }
+        }
+        if (!ok) {
+            __syncwarp();
+            if (elect_one()) tc_commit(drain);
+            const long long t0 = clock64();
+            while (!mbar_try_wait(drain, 0) && clock64() - t0 < 20000000LL) {}
         }
         __syncwarp();
     } else {
@@ -280,7 +293,7 @@ inline int launch_pre_both(const CUtensorMap& tA0, const CUtensorMap& tB0, PrePa
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(mtiles, nsplit, 2);
-    cfg.blockDim = dim3(192);
+    cfg.blockDim = dim3(kLrThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
