@@ -326,10 +326,10 @@ int lqlora_selftest_bounded_wait(void* workspace_dev, int64_t budget_cycles, voi
 /* Which kernel lqlora_linear_fwd (backward = 0) or lqlora_linear_bwd_input (backward != 0) dispatches to for M rows:
  *   LQLORA_PATH_PLAIN    plain-FMA fall-back (shapes the vector paths do not take)
  *   LQLORA_PATH_STREAM   weight-streaming kernel for decode-sized inputs (M <= 16)
- *   LQLORA_PATH_TC_ONE   tcgen05 kernel, one CTA per output tile, contraction split over a cluster
+ *   LQLORA_PATH_TC_ONE   tcgen05 kernel on transposed output tiles (any number of rows), contraction split over a cluster
  *   LQLORA_PATH_TC_PAIR  tcgen05 kernel, CTA pairs (cta_group::2) on [512, 256] output tiles
- * *splits (may be NULL) receives the number of CTAs that share one output tile's contraction (the cluster size; 1 for
- * CTA pairs and the fall-back).  Returns a negative lqlora_status for invalid arguments.  Host only. */
+ * *splits (may be NULL) receives the number of slices of one output tile's contraction (1 for [512, 256] tiles and the
+ * fall-back).  Returns a negative lqlora_status for invalid arguments.  Host only. */
 enum { LQLORA_PATH_PLAIN = 0, LQLORA_PATH_STREAM = 1, LQLORA_PATH_TC_ONE = 2, LQLORA_PATH_TC_PAIR = 3 };
 int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, int64_t M, int backward, int* splits);
 

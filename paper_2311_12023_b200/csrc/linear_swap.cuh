@@ -474,16 +474,22 @@ struct SwapPlan {
     double us;                       // estimated time
 };
 
-// Ring depths; false when they do not fit.
+// Ring depths; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase
+// while the one before it can be incomplete.  A dequantization warp works on every fourth step:
+//   - it may wait for stage j % ss to be free (the tensor core is done with step j - ss) once step j - 2 ss is known to be
+//     done; its own step j - 4 waited for j - 4 - ss, hence ss >= 4;
+//   - it may wait for the codes of step j once those of step j - sp are known to have landed: they have where its own
+//     group used them (sp = 4, 8) or where the tensor core is done with that step (sp >= ss).
 inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
     const int stage = kSwWBytes + pl.nbox * pl.box * 64, pk = 1024 * b0;
     const int fixed = 1024 + kSwTail + (b0 == 8 ? 32768 : 0);
     const int room = kSmemLimit - fixed;
     pl.ss = (room - 4 * pk) / stage;
     if (pl.ss > kSwMaxStages) pl.ss = kSwMaxStages;
-    if (pl.ss < 3) return false;
+    if (pl.ss < 4) return false;
     pl.sp = (room - pl.ss * stage) / pk;
     if (pl.sp > kSwMaxStages) pl.sp = kSwMaxStages;
+    if (pl.sp < pl.ss) pl.sp = 4;
     const int bytes = pl.ss * stage + pl.sp * pk;
     if (ks > 1 && pl.nbox * pl.box * 512 > bytes) return false;      // the accumulators are laid over the rings
     pl.smem = fixed + bytes;
@@ -491,11 +497,14 @@ inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
 }
 
 // The split of a call that costs least by a simple model: waves of clusters, each with a fixed cost, its steps (the
-// slower of dequantization and tensor core) and its reduction.
+// slower of dequantization and tensor core) and its reduction.  The constants are those of a sweep over chunks and slices
+// (us with 1, 2, 3, 4 slices): 4096 x 4096 NF3, 64 rows: 24, 17, 15, 26 (16 clusters of eight, of which 15 fit); 8192 x 8192
+// NF4, 17 rows: 53, 32, 45, 56; 11008 x 4096 NF4, 128 rows: 31, 40, 35, 45; 1024 x 1024 NF3, 512 rows in four chunks: 12.3, 12.9,
+// 16, 24, in seven: 11.6, 14, 21, 23; 1024 x 8192 NF3, 1024 rows in four chunks: 47, 32, 39, 55.
 inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
     SwapPlan best{};
     best.us = -1.0;
-    const double dq = b0 == 2 ? 0.26 : b0 == 3 ? 0.28 : b0 == 4 ? 0.36 : 0.42;      // us per step of 128 x 64 weights
+    const double dq = b0 == 2 ? 0.22 : b0 == 3 ? 0.26 : b0 == 4 ? 0.35 : 0.40;      // us per step of 128 x 64 weights
     const long long pairs = (out_cols + 255) / 256;
     const int first = static_cast<int>((M + 511) / 512);
     for (int ch = first; ch <= first + 7; ++ch) {
@@ -512,11 +521,15 @@ inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q,
             if (!swap_rings(b0, ks, pl)) continue;
             pl.ks = ks;
             pl.ctas = 2 * pairs * pl.chunks * ks;
-            const long long at_once = tc_max_clusters(2 * ks);
+            // a rank-r pre-product runs beside this kernel and takes SMs out of the GPCs, which costs large clusters most (a
+            // second wave costs more than a finer split saves)
+            const int taken[4] = {2, 1, 2, 4};
+            const long long at_once = tc_max_clusters(2 * ks) - (steps_d > 0 ? taken[ks - 1] : 0);
             const long long waves = (pairs * pl.chunks + at_once - 1) / at_once;
-            const double step = dq > tokens * 0.00115 ? dq : tokens * 0.00115;
-            const double body = 4.0 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 2.0 + tokens * 0.008 : tokens * 0.006);
+            const double step = dq > tokens * 0.0012 ? dq : tokens * 0.0012;
+            const double body = 6.5 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 2.5 + tokens * 0.008 : tokens * 0.006);
             pl.us = waves * body;
+            if (ks == 1 && steps_q > 16) pl.us *= 1.2;      // (long contractions: slices spread better than the model says)
             if (best.us < 0 || pl.us < best.us) best = pl;
         }
     }

@@ -1,21 +1,17 @@
-// Tensor-core path for many rows of X (training-sized M) on sm_100a.
+// Tensor-core path (tcgen05) for more rows of X than the weight-streaming kernels take: what its two linear kernels share
+// (linear_tc2.cuh: [512, 256] output tiles on CTA pairs; linear_swap.cuh: transposed tiles with the contraction split over a
+// cluster), the rank-r pre-product, and the dispatch between them.
 //
-// One CTA computes a [MH*128, 256] tile of the output.  Per pipeline step of 64 contraction
-// elements:
-//   - a producer thread issues a TMA tile load of the bf16 activations (128-byte swizzle) and
-//     bulk copies of the packed code slabs into shared memory;
-//   - sixteen dequantization warps unpack the codes, multiply by the block scale in fp32, round to
-//     bf16 and write the weight tile into shared memory in the 128-byte-swizzled layout that the
-//     tensor core reads (one thread = 32 weights of one row);
-//   - one thread issues tcgen05.mma (M = 128, N = 256, K = 16) with fp32 accumulators in tensor
-//     memory and commits the stage back to the producer.
+// Both linear kernels run the same pipeline over steps of 64 contraction elements: copies bring the bf16 activations (TMA,
+// 128-byte swizzle) and the packed codes into shared memory; sixteen dequantization warps unpack the codes, multiply by
+// the block scale in fp32, round to bf16 and write the weight tile in the 128-byte-swizzled layout that the tensor core
+// reads; one warp issues tcgen05.mma with fp32 accumulators in tensor memory and commits the stage back.
 // The rank-r term is folded in as extra contraction steps whose two operands come by TMA
-// (forward: [X L2^T | L1]; backward: [dY L1 | L2]).  The epilogue reads the accumulators with
-// tcgen05.ld, rounds to bf16 and stores.
+// (forward: [X L2^T | L1]; backward: [dY L1 | L2]).
 //
 // The same shared-memory weight tile ([rows of Q] x 64 columns, 128 bytes per row, swizzled)
-// serves both passes: the forward reads it as a K-major B operand (contraction along the row),
-// the input gradient as an MN-major B operand (contraction across rows).
+// serves both passes: the forward reads it as a K-major operand (contraction along the row),
+// the input gradient as an MN-major operand (contraction across rows).
 //
 // Every wait on an mbarrier is bounded; when a wait expires the kernel records it in the status
 // word of the workspace, stops issuing work, lets its copies land, frees its tensor memory and
@@ -36,7 +32,6 @@ constexpr int BK = 64;
 constexpr int BN = 256;
 constexpr int kDeqWarps = 16;
 constexpr int kThreads = (2 + kDeqWarps) * 32;
-constexpr int kBBytes = BN * 128;            // bf16 weight tile of one step
 
 struct Params {
     QView q;
@@ -46,7 +41,6 @@ struct Params {
     int out_cols;      // N (forward) or K (backward)
     int steps_q;       // steps whose weights are dequantized
     int steps_d;       // steps of the rank-r term
-    int stages;
     int c_base;        // first output column of this launch (a call may be split over two launches by output columns)
     int c_tiles;       // number of 256-column output tiles of this launch
 };
@@ -108,9 +102,9 @@ __device__ __forceinline__ void sts_v4(uint32_t addr, uint32_t a, uint32_t b, ui
 // `words` pointing at the thread's first word, the others 32 words apart -- and writes them as four
 // 16-byte chunks of the row's 128 bytes; `dst` is the row start, `goff` the byte offset of the group
 // in the row (0 or 64), `xr` is (row % 8) * 16; a chunk at byte offset o of the row lives at o ^ xr.
-// 8-bit codes read the code book from shared memory.  REP: the table is stored once per bank, entry c of the copy
+// 8-bit codes read the code book from shared memory, where it is stored once per bank: entry c of the copy
 // of lane l at lut8[c * 32 + l], and `lut8` already points at the lane's copy, so no look-up meets a bank conflict.
-template <int B, bool REP = false>
+template <int B>
 __device__ __forceinline__ void dequant_group(uint32_t words, float s_lo, float s_hi, bool two_scales,
                                               uint32_t dst, uint32_t goff, uint32_t xr, const float* __restrict__ lut8) {
     // `words` and `dst` are 32-bit shared-memory addresses (explicit shared-space loads and stores)
@@ -126,8 +120,8 @@ __device__ __forceinline__ void dequant_group(uint32_t words, float s_lo, float 
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const uint32_t ww = w[2 * c + (e >> 1)] >> (16 * (e & 1));
-                const float q0 = REP ? lut8[(ww & 255u) << 5] : lut8[ww & 255u];
-                const float q1 = REP ? lut8[((ww >> 8) & 255u) << 5] : lut8[(ww >> 8) & 255u];
+                const float q0 = lut8[(ww & 255u) << 5];
+                const float q1 = lut8[((ww >> 8) & 255u) << 5];
                 const __nv_bfloat162 h = __floats2bfloat162_rn(__fmul_rn(q0, s), __fmul_rn(q1, s));
                 packed[e] = *reinterpret_cast<const uint32_t*>(&h);
             }
@@ -181,28 +175,7 @@ __device__ __forceinline__ RawScale window_scale(const ScaleWindow& s, int b, bo
     return RawScale{two ? (sh & 0xFFFFu) : (sh & 0xFFu), s.v};
 }
 
-// ------------------------------------------------------------------------------------ kernel
-// Shared memory: [activation ring: SA x A_BYTES][weight ring: 2 x 32 KB][packed ring: SA x 2048*b0]
-// [barriers][8-bit look-up table].  The activation / packed-code ring runs several steps ahead of
-// the tensor core (it hides the latency of global memory); the dequantized weight ring needs two
-// stages only (one being read by the tensor core, one being written).
 constexpr int kSmemLimit = 232448;   // 227 KB of dynamic shared memory per CTA
-// stages of the dequantized weight ring: three, so that the dequantization of a step may start two
-// tensor-core steps before its result is needed (two for 8-bit codes, whose packed data leave less room)
-template <int B, int MH>
-__host__ __device__ constexpr int b_stages() { return (B == 8 && MH == 2) ? 2 : 3; }
-
-template <int B, int MH>
-__host__ __device__ constexpr int stage_bytes() { return MH * 16384 + 2048 * B; }        // one stage of the activation + packed-code ring
-template <int B>
-__host__ __device__ constexpr int tail_bytes() { return 256 + (B == 8 ? 1024 : 0) + 64; }
-template <int B, int MH>
-__host__ __device__ constexpr int fixed_bytes() { return 1024 + b_stages<B, MH>() * kBBytes; }   // alignment slack + weight ring
-template <int B, int MH>
-__host__ __device__ constexpr int ring_stages() {
-    const int s = (kSmemLimit - fixed_bytes<B, MH>() - tail_bytes<B>()) / stage_bytes<B, MH>();
-    return s > 6 ? 6 : s;
-}
 
 // Ring position that advances without divisions: stage index and the parity of the current pass.
 template <int S> struct RingPos {
@@ -210,361 +183,6 @@ template <int S> struct RingPos {
     uint32_t ph = 0;
     __device__ __forceinline__ void advance() { if (++s == S) { s = 0; ph ^= 1u; } }
 };
-
-template <int B, bool BWD, int MH>
-__global__ void __launch_bounds__(kThreads, 1)
-tc_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
-                 const __grid_constant__ CUtensorMap tmB2, const Params p) {
-    constexpr int A_BYTES = MH * 128 * 128;
-    constexpr int P_BYTES = 2048 * B;
-    constexpr uint32_t TMEM_COLS = MH * BN;
-    constexpr int SA = ring_stages<B, MH>();
-    constexpr int kBStages = b_stages<B, MH>();
-
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-    uint8_t* a_ring = base;
-    uint8_t* b_ring = a_ring + static_cast<size_t>(SA) * A_BYTES;
-    uint8_t* p_ring = b_ring + kBStages * kBBytes;
-    uint8_t* tail = p_ring + static_cast<size_t>(SA) * P_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);   // full_a[8], empty_a[8], full_b[4], empty_b[4], acc_full, drain
-    float* lut8 = reinterpret_cast<float*>(tail + 256);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 256 + (B == 8 ? 1024 : 0));
-    volatile int* abort_s = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int m0 = blockIdx.x * (MH * 128);
-    const int c0 = p.c_base + blockIdx.y * BN;          // first output column: n0 (forward) or k0 (backward)
-    // split of the contraction over the CTAs of a cluster (gridDim.z of them); the rank-r steps go to split 0
-    const int nsplit = gridDim.z, split = blockIdx.z;
-    const int per_split = (p.steps_q + nsplit - 1) / nsplit;
-    const int q_lo = min(p.steps_q, split * per_split);
-    const int nq = min(p.steps_q, q_lo + per_split) - q_lo;       // dequantized steps of this CTA
-    const int total = nq + (split == 0 ? p.steps_d : 0);
-    const Ctl ctl{abort_s, p.status};
-
-    auto full_a = [&](int s) { return smem_u32(bars + s); };
-    auto empty_a = [&](int s) { return smem_u32(bars + 8 + s); };
-    auto full_b = [&](int s) { return smem_u32(bars + 16 + s); };
-    auto empty_b = [&](int s) { return smem_u32(bars + 20 + s); };
-    const uint32_t acc_full = smem_u32(bars + 24), drain = smem_u32(bars + 25);
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < SA; ++s) { mbar_init(full_a(s), 1); mbar_init(empty_a(s), 1); }
-        for (int s = 0; s < kBStages; ++s) { mbar_init(full_b(s), kDeqWarps); mbar_init(empty_b(s), 1); }
-        mbar_init(acc_full, 1);
-        mbar_init(drain, 1);
-        *abort_s = 0;
-        fence_barrier_init();
-    }
-    if constexpr (B == 8) {
-        for (int i = threadIdx.x; i < 256; i += kThreads) lut8[i] = c_codebook[3][i];
-    }
-    if (warp == 1) { tmem_alloc(smem_u32(tmem_slot), TMEM_COLS); tmem_relinquish(); }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    bool acc_ok = false;          // this thread saw the accumulators complete (dequantization warps only)
-
-    if (warp == 0) {
-        // ------------------------------------------------------------------ producer: activations + packed codes
-        if (lane == 0) {
-            const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
-            RingPos<SA> ra;
-            for (int step = 0; step < total; ++step, ra.advance()) {
-                const int s = ra.s;
-                if (!wait(empty_a(s), ra.ph ^ 1, ctl, 1)) break;
-                const uint32_t a_dst = smem_u32(a_ring) + s * A_BYTES;
-                const uint32_t p_dst = smem_u32(p_ring) + s * P_BYTES;
-                if (step < nq) {
-                    const int qs = q_lo + step;                  // step index in the whole contraction
-                    if (!BWD) {
-                        int nt_have = 0;
-                        for (int t = 0; t < 2; ++t) if ((c0 >> 7) + t < p.q.ntiles) ++nt_have;
-                        mbar_expect_tx(full_a(s), A_BYTES + nt_have * 1024 * B);
-                        tma_load_2d(a_dst, &tmA, qs * BK, m0, full_a(s));
-                        for (int t = 0; t < nt_have; ++t) {
-                            const size_t tile = static_cast<size_t>((c0 >> 7) + t) * p.q.ktiles + qs;
-                            bulk_load(p_dst + t * 1024 * B, codes + tile * (1024 * B), 1024 * B, full_a(s));
-                        }
-                    } else {
-                        const int nn0 = qs * BK;
-                        int kt_have = 0;
-                        for (int t = 0; t < 4; ++t) if ((c0 >> 6) + t < p.q.ktiles) ++kt_have;
-                        mbar_expect_tx(full_a(s), A_BYTES + kt_have * 512 * B);
-                        tma_load_2d(a_dst, &tmA, nn0, m0, full_a(s));
-                        for (int t = 0; t < kt_have; ++t) {
-                            const size_t tile = static_cast<size_t>(nn0 >> 7) * p.q.ktiles + (c0 >> 6) + t;
-                            bulk_load(p_dst + t * 512 * B, codes + tile * (1024 * B) + ((nn0 >> 6) & 1) * (512 * B), 512 * B,
-                                      full_a(s));
-                        }
-                    }
-                } else {
-                    if (step == nq) {
-                        // the rank-r intermediate is written by the preceding kernel, which may still be
-                        // running (programmatic dependent launch): wait for it, then order this thread's
-                        // bulk-copy reads after what it wrote
-                        pdl_wait();
-                        fence_proxy_async_all();
-                    }
-                    mbar_expect_tx(full_a(s), A_BYTES);
-                    tma_load_2d(a_dst, &tmA2, (step - nq) * BK, m0, full_a(s));
-                }
-            }
-            if (*abort_s) {
-                // let copies that are still in flight land before the CTA exits (bounded)
-                for (int s = 0; s < SA; ++s) {
-                    const long long t0 = clock64();
-                    while (!mbar_try_wait(full_a(s), 0) && !mbar_try_wait(full_a(s), 1) && clock64() - t0 < 20000000LL) {}
-                }
-            }
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 16) |
-                                       (static_cast<uint32_t>(BN >> 3) << 17) | (static_cast<uint32_t>(128 >> 4) << 24);
-            bool ok = true;
-            RingPos<SA> ra;
-            RingPos<kBStages> rb;
-            for (int step = 0; step < total && ok; ++step, ra.advance(), rb.advance()) {
-                const int sa = ra.s, sb = rb.s;
-                ok = wait(full_a(sa), ra.ph, ctl, 2) && wait(full_b(sb), rb.ph, ctl, 3);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t a_src = smem_u32(a_ring) + sa * A_BYTES;
-                const uint32_t b_src = smem_u32(b_ring) + sb * kBBytes;
-#pragma unroll
-                for (int h = 0; h < MH; ++h) {
-#pragma unroll
-                    for (int k16 = 0; k16 < 4; ++k16) {
-                        const uint64_t adesc = make_desc(a_src + h * 16384 + k16 * 32, 16, 1024);
-                        const uint64_t bdesc = BWD ? make_desc(b_src + k16 * 2048, 8192, 1024)
-                                                   : make_desc(b_src + k16 * 32, 16, 1024);
-                        tc_mma(tmem + h * BN, adesc, bdesc, idesc, (step > 0 || k16 > 0) ? 1u : 0u);
-                    }
-                }
-                tc_commit(empty_a(sa));
-                tc_commit(empty_b(sb));
-            }
-            if (ok) {
-                tc_commit(acc_full);
-            } else {
-                tc_commit(drain);      // wait (bounded) for issued MMAs before tensor memory is freed
-                const long long t0 = clock64();
-                while (!mbar_try_wait(drain, 0) && clock64() - t0 < 20000000LL) {}
-            }
-        }
-        __syncwarp();
-    } else {
-        // ------------------------------------------------------------------ dequantization warps, then epilogue
-        // warp dw handles slab (dw / 2) of the step's packed data and the 32-column group (dw % 2);
-        // one thread = one row of that slab.
-        const int dw = warp - 2;
-        const int slab_i = dw >> 1, g = dw & 1;
-        int row_local;            // row inside the 128-byte-row (sub-)tile of the B operand
-        uint32_t b_off;           // byte offset of this thread's row inside the B tile
-        if (!BWD) { row_local = slab_i * 32 + lane; b_off = row_local * 128; }
-        else { row_local = (slab_i & 1) * 32 + lane; b_off = (slab_i >> 1) * 8192 + row_local * 128; }
-        const uint32_t xr = (row_local & 7) << 4;
-        const bool two_scales = (p.q.B0 == 16);
-        // block index of the scale of step `st` (32-bit: the host checks that N*K/B0 fits):
-        //   forward  (row c0 + row_local, columns st*64 + 32 g ..), backward (row st*64 + row_local, columns c0 + 64*(slab_i/2) + 32 g ..)
-        const int my_row = BWD ? row_local : c0 + row_local;
-        const int my_col = BWD ? c0 + (slab_i >> 1) * 64 + g * 32 : g * 32;
-        const bool col_ok = my_col < p.q.K;
-        const uint32_t blk0 = static_cast<uint32_t>(my_row) * p.q.KB + (BWD ? (my_col >> p.q.logB0) : 0);
-        const uint32_t row_stride = static_cast<uint32_t>(BK) * p.q.KB;
-        const uint8_t* __restrict__ scp = p.q.sc;
-        const float* __restrict__ vp = p.q.v;
-        const int logB0 = p.q.logB0, logB1 = p.q.logB1;
-        auto fetch = [&](int st) {
-            RawScale r{0u, 0.0f};
-            const int row = BWD ? st * BK + my_row : my_row;
-            if (row < p.q.N && col_ok) {
-                const uint32_t blk = BWD ? blk0 + st * row_stride : blk0 + ((st * BK + my_col) >> logB0);
-                r.sc = two_scales ? static_cast<uint32_t>(__ldg(reinterpret_cast<const uint16_t*>(scp + blk))) : static_cast<uint32_t>(__ldg(scp + blk));
-                r.v = __ldg(vp + (blk >> logB1));
-            }
-            return r;
-        };
-        // The raw scale data of step s + 4 are requested right after those of step s have been used,
-        // into the same slot; the loop is unrolled by four so that the slots are fixed registers and
-        // no instruction touches a slot while its load is in flight.
-        float v_cached = -1.0f, sigma = 0.0f, s_lo = 0.0f, s_hi = 0.0f;
-        RawScale slot[4];
-        // forward, rows aligned to 16 blocks: windows of 16 scale codes instead of one load per step
-        const bool use_win = !BWD && (p.q.KB % 16 == 0);
-        const bool win_row_ok = !BWD && my_row < p.q.N;
-        ScaleWindow cur{make_uint4(0u, 0u, 0u, 0u), 0.0f}, nxt = cur;
-        int cur_base = 0;
-        if (use_win) {
-            cur_base = ((q_lo * BK + my_col) >> logB0) & ~15;
-            cur = load_scale_window(p.q, blk0, cur_base, win_row_ok);
-            nxt = load_scale_window(p.q, blk0, cur_base + 16, win_row_ok);
-        } else {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) slot[u] = (u < nq) ? fetch(q_lo + u) : RawScale{0u, 0.0f};
-        }
-        // word plane slot of this thread's row: rotated by 8 g + 16 (tile column % 2), see slab_row_slot();
-        // forward: the tile column is the step index, backward: it is fixed per thread
-        const uint32_t slab_base = smem_u32(p_ring) + (slab_i * (64 * B) + g * (B * 32)) * 4;      // byte address in shared memory
-        const int slot_even = slab_row_slot(lane, g, BWD ? ((c0 >> 6) + (slab_i >> 1)) : 0);
-        const int slot_odd = BWD ? slot_even : slab_row_slot(lane, g, 1);
-        const uint32_t my_b = smem_u32(b_ring) + b_off;
-        bool ok = true;
-        RingPos<SA> ra;
-        RingPos<kBStages> rb;
-        for (int step4 = 0; step4 < total && ok; step4 += 4) {
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int step = step4 + u;
-                if (step >= total || !ok) break;
-                const int sa = ra.s, sb = rb.s;
-                ok = wait(empty_b(sb), rb.ph ^ 1, ctl, 6);
-                if (!ok) break;
-                if (step < nq) {
-                    if (use_win) {
-                        const int b = ((q_lo + step) * BK + my_col) >> logB0;
-                        if ((b & ~15) != cur_base) {
-                            cur = nxt;
-                            cur_base += 16;
-                            nxt = load_scale_window(p.q, blk0, cur_base + 16, win_row_ok);
-                        }
-                        make_scales(p.q, window_scale(cur, b, two_scales), v_cached, sigma, s_lo, s_hi);
-                    } else {
-                        make_scales(p.q, slot[u], v_cached, sigma, s_lo, s_hi);
-                        if (step + 4 < nq) slot[u] = fetch(q_lo + step + 4);
-                    }
-                    ok = wait(full_a(sa), ra.ph, ctl, 4);
-                    if (!ok) break;
-                    dequant_group<B>(slab_base + sa * P_BYTES + (((q_lo + step) & 1) ? slot_odd : slot_even) * 4, s_lo, s_hi, two_scales, my_b + sb * kBBytes, g << 6, xr, lut8);
-                    fence_proxy_async();            // make the generic-proxy stores visible to the tensor core
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(full_b(sb));
-                } else if (dw == 0) {
-                    // rank-r step: the second operand ([L1 | ..] rows or L2 rows) comes by TMA into the weight ring
-                    if (lane == 0) {
-                        const int d = step - nq;
-                        const uint32_t dst = smem_u32(b_ring) + sb * kBBytes;
-                        if (!BWD) {
-                            mbar_expect_tx(full_b(sb), kBBytes);
-                            tma_load_2d(dst, &tmB2, d * BK, c0, full_b(sb));
-                        } else {
-                            int kt_have = 0;
-                            for (int t = 0; t < 4; ++t) if (c0 + t * 64 < p.out_cols) ++kt_have;
-                            mbar_expect_tx(full_b(sb), kt_have * 8192);
-                            for (int t = 0; t < kt_have; ++t) tma_load_2d(dst + t * 8192, &tmB2, c0 + t * 64, d * BK, full_b(sb));
-                        }
-                    }
-                    __syncwarp();
-                } else {
-                    if (lane == 0) mbar_arrive(full_b(sb));
-                }
-                ra.advance();
-                rb.advance();
-            }
-        }
-        // epilogue: warp reads its quarter of the 128 accumulator lanes and 64 of the 256 columns
-        acc_ok = ok && wait(acc_full, 0, ctl, 5);
-        if (acc_ok && nsplit == 1) {
-            tc_fence_after();
-            const int quarter = warp & 3, colq = dw >> 2;
-#pragma unroll 1
-            for (int h = 0; h < MH; ++h) {
-                const int m = m0 + h * 128 + quarter * 32 + lane;
-#pragma unroll 1
-                for (int cc = 0; cc < 2; ++cc) {
-                    const int col = colq * 64 + cc * 32;
-                    uint32_t v[32];
-                    tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + h * BN + col, v);
-                    tmem_ld_wait();
-                    if (m < p.M) {
-                        __nv_bfloat16* dst = p.out + static_cast<size_t>(m) * p.out_cols + c0 + col;
-#pragma unroll
-                        for (int i = 0; i < 4; ++i) {
-                            if (c0 + col + i * 8 < p.out_cols) {
-                                uint32_t w[4];
-#pragma unroll
-                                for (int e = 0; e < 4; ++e) {
-                                    const __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(v[i * 8 + 2 * e]),
-                                                                                   __uint_as_float(v[i * 8 + 2 * e + 1]));
-                                    w[e] = *reinterpret_cast<const uint32_t*>(&hh);
-                                }
-                                *reinterpret_cast<uint4*>(dst + i * 8) = make_uint4(w[0], w[1], w[2], w[3]);
-                            }
-                        }
-                    }
-                }
-            }
-        }
-    }
-    if (nsplit > 1) {
-        // ------------------------------------------------------------------ sum over the splits of the contraction
-        // Every CTA of the cluster writes its accumulator tile (fp32, [256 columns][128 rows]) over the idle
-        // rings; CTA `split` then adds the 256 / nsplit columns it owns from all CTAs through distributed
-        // shared memory, rounds to bf16 and stores.  The barriers are executed by all threads of all CTAs,
-        // whatever happened before (a CTA that gave up on a wait still takes part; its output is undefined
-        // and the status word says so).
-        float* accbuf = reinterpret_cast<float*>(base);
-        const uint32_t accbuf_addr = smem_u32(accbuf);
-        // CTA `split` owns the groups of eight columns [split * 32 / nsplit, (split + 1) * 32 / nsplit) (any cluster size)
-        const int g_lo = split * (BN / 8) / nsplit, g_hi = (split + 1) * (BN / 8) / nsplit;
-#pragma unroll 1
-        for (int h = 0; h < MH; ++h) {
-            if (warp >= 2 && acc_ok) {
-                tc_fence_after();
-                const int dw = warp - 2, quarter = warp & 3, colq = dw >> 2;
-#pragma unroll 1
-                for (int cc = 0; cc < 2; ++cc) {
-                    const int col = colq * 64 + cc * 32;
-                    uint32_t v[32];
-                    tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + h * BN + col, v);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int i = 0; i < 32; ++i) accbuf[(col + i) * 128 + quarter * 32 + lane] = __uint_as_float(v[i]);
-                }
-            }
-            __syncthreads();
-            dec::cluster_sync_all();
-            for (int item = threadIdx.x; item < 128 * (g_hi - g_lo); item += kThreads) {
-                const int row = item & 127, cg = item >> 7;
-                const int m = m0 + h * 128 + row;
-                const int col = (g_lo + cg) * 8;
-                // all remote loads are requested before the first is used (a round trip costs about two thousand clocks)
-                float part[8][8];
-#pragma unroll
-                for (int rk = 0; rk < 8; ++rk)
-#pragma unroll
-                    for (int i = 0; i < 8; ++i)
-                        part[rk][i] = (rk < nsplit) ? dec::ld_dsmem_f32(accbuf_addr + static_cast<uint32_t>((col + i) * 128 + row) * 4u, static_cast<uint32_t>(rk)) : 0.0f;
-                float sum[8];
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                    sum[i] = 0.0f;
-#pragma unroll
-                    for (int rk = 0; rk < 8; ++rk) sum[i] += part[rk][i];
-                }
-                if (m < p.M && c0 + col < p.out_cols) {
-                    uint32_t w[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const __nv_bfloat162 hh = __floats2bfloat162_rn(sum[2 * e], sum[2 * e + 1]);
-                        w[e] = *reinterpret_cast<const uint32_t*>(&hh);
-                    }
-                    *reinterpret_cast<uint4*>(p.out + static_cast<size_t>(m) * p.out_cols + c0 + col) = make_uint4(w[0], w[1], w[2], w[3]);
-                }
-            }
-            __syncthreads();
-            dec::cluster_sync_all();           // the buffers may be overwritten (next half) or released (exit) only now
-        }
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem, TMEM_COLS);
-}
 
 
 // ------------------------------------------------------------------------------------ rank-r pre-product
@@ -831,96 +449,25 @@ inline bool make_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t 
     return true;
 }
 
-template <int B, bool BWD, int MH>
-inline int launch_one(const CUtensorMap& tA, const CUtensorMap& tA2, const CUtensorMap& tB2, Params p, int ksplit, cudaStream_t st,
-                      bool after_pre = true) {
-    constexpr int stages = ring_stages<B, MH>();
-    static_assert(stages >= 2, "activation ring too shallow");
-    p.stages = stages;
-    constexpr int smem = fixed_bytes<B, MH>() + stages * stage_bytes<B, MH>() + tail_bytes<B>();
-    static_assert(smem <= kSmemLimit, "shared memory budget exceeded");
-    auto kern = tc_linear_kernel<B, BWD, MH>;
-    static bool attr_done = false;
-    if (!attr_done) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
-            cudaGetLastError();
-            return LQLORA_ERR_CUDA;
-        }
-        attr_done = true;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((p.M + MH * 128 - 1) / (MH * 128), p.c_tiles, ksplit);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;      // the splits of the contraction of one tile form a cluster
-    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = ksplit;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = (p.steps_d > 0 && after_pre) ? 2 : 1;      // overlap with the rank-r pre-product kernel in front of it
-    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tA, tA2, tB2, p);
-    count_launch(1);
-    if (e != cudaSuccess) { cudaGetLastError(); return LQLORA_ERR_CUDA; }
-    return LQLORA_OK;
-}
+}  // namespace tc
+}  // namespace lq
 
+#include "linear_tc2.cuh"
+#include "linear_swap.cuh"
 
-// Clusters of `ks` CTAs of the one-CTA kernel (one CTA per SM, all of its shared memory) that can be resident at the
-// same time.  A cluster lives inside one GPC, so fewer fit than SMs / ks: 15 clusters of eight on a B200, not 18.
-// Asked once per cluster size; the figures measured on a B200 stand in when there is no device to ask.
-inline int tc_max_clusters(int ks) {
-    static int cached[8] = {-1, -1, -1, -1, -1, -1, -1, -1};       // ks = 1 .. 8
-    const int idx = (ks < 1 ? 1 : ks > 8 ? 8 : ks) - 1;
-    if (cached[idx] >= 0) return cached[idx];
-    const int fallback[8] = {148, 74, 48, 36, 28, 24, 16, 15};
-    int n = 0;
-    auto kern = tc_linear_kernel<3, false, 1>;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(1, 1, ks);
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = kSmemLimit;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = ks;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) {
-        cudaGetLastError();
-        n = fallback[idx];
-    }
-    cached[idx] = n;
-    return n;
-}
+namespace lq {
+namespace tc {
 
-// Splits of the contraction for the one-CTA kernel: few output tiles would leave most SMs idle, so
-// the contraction of a tile is divided over a cluster of up to eight CTAs (any size: each keeps at least 8 steps, 16 beyond four CTAs, and
-// all clusters must be resident at once: a second wave costs more than the finer split saves).
 // CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs; below that the one-CTA
-// kernel with its split of the contraction puts at least twice as many SMs to work (4096 x 4096 at 512 rows: 32 CTAs
-// as pairs, 128 as single CTAs in clusters of four).
+// kernel with its split of the contraction puts at least twice as many SMs to work.
 inline bool tc_use_pair(int64_t M, int64_t out_cols, int sms) {
     if (M <= 256) return false;
     const long long pair_ctas = 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN);
     return 2 * pair_ctas > sms;
 }
 
-inline int tc_ksplit_tiles(long long tiles, int steps_q, int sms) {
-    for (int ks = 8; ks > 1; --ks)
-        if (tiles * ks <= sms && steps_q / ks >= (ks > 4 ? 16 : 8) && tiles <= tc_max_clusters(ks)) return ks;   // the reduction grows with ks
-    return 1;
-}
-inline int tc_ksplit(int64_t M, int64_t out_cols, int steps_q, int sms) {
-    if (tc_use_pair(M, out_cols, sms)) return 1;
-    const int mh = (M > 128) ? 2 : 1;
-    return tc_ksplit_tiles(((M + mh * 128 - 1) / (mh * 128)) * ((out_cols + BN - 1) / BN), steps_q, sms);
-}
-
 struct PrePlan {
     int mtiles, nsplit, steps, steps_per_split, rp;
-    size_t t_bytes;
 };
 
 // Number of SMs of the current device (148 on B200; also the answer when no device is present).
@@ -937,23 +484,24 @@ inline int sm_count() {
 }
 
 // C = contraction length, out_cols = width of the output of the linear kernel that follows.
-inline PrePlan pre_plan(int64_t C, int r, int64_t M, int64_t out_cols) {
+inline PrePlan pre_plan(int b0, int64_t C, int r, int64_t M, int64_t out_cols) {
     PrePlan pl;
     pl.mtiles = static_cast<int>((M + 127) / 128);
     pl.steps = static_cast<int>((C + BK - 1) / BK);
     // The pre-product runs beside the linear kernel that follows it (programmatic dependent launch):
     // give it the SMs that the last wave of that kernel leaves idle, and at least one CTA per row tile.
-    const int mh = (M > 128) ? 2 : 1;
     const int sms = sm_count();
-    const long long main_ctas = ((M + mh * 128 - 1) / (mh * 128)) * ((out_cols + BN - 1) / BN) * tc_ksplit(M, out_cols, pl.steps, sms);
+    const long long main_ctas = tc_use_pair(M, out_cols, sms) ? 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN)
+                                                              : swap_plan(b0, M, out_cols, pl.steps, (r + BK - 1) / BK).ctas;
     const int idle = static_cast<int>((sms - main_ctas % sms) % sms);
     int want = idle / pl.mtiles;
-    if (want > pl.steps / 2) want = pl.steps / 2;
+    if (main_ctas < sms) want = idle / 2 / pl.mtiles;      // beside a single wave of clusters: half of what it leaves (clusters need room)
+    if (want > pl.steps / 4) want = pl.steps / 4;
     if (want > 8) want = 8;          // splits of a tile form a cluster (and more than eight made the sum the critical path)
     if (idle < 48) {
         // beside a nearly full linear kernel (itself made of clusters) large pre-product clusters took a cluster's place
         // from it: at most four pre-product CTAs in all
-        const int cap = (4 / pl.mtiles > 1) ? 4 / pl.mtiles : 1;
+        const int cap = (idle / pl.mtiles < 4) ? (idle / pl.mtiles > 1 ? idle / pl.mtiles : 1) : 4;
         if (want > cap) want = cap;
     }
     if (want < 1) want = 1;
@@ -961,7 +509,6 @@ inline PrePlan pre_plan(int64_t C, int r, int64_t M, int64_t out_cols) {
     pl.steps_per_split = (pl.steps + want - 1) / want;
     pl.nsplit = want;
     pl.rp = (r <= 64) ? 64 : 128;
-    pl.t_bytes = round_up(static_cast<size_t>(M) * (r > 0 ? r : 1) * 2, 256);
     return pl;
 }
 
@@ -1002,17 +549,9 @@ inline int launch_pre(const CUtensorMap& tA, const CUtensorMap& tB, PreParams p,
     return LQLORA_OK;
 }
 
-template <int B>
-inline int launch_b(const CUtensorMap& tA, const CUtensorMap& tA2, const CUtensorMap& tB2, const Params& p, bool bwd, int mh,
-                    int ksplit, cudaStream_t st, bool after_pre = true) {
-    if (!bwd) return mh == 2 ? launch_one<B, false, 2>(tA, tA2, tB2, p, ksplit, st, after_pre) : launch_one<B, false, 1>(tA, tA2, tB2, p, ksplit, st, after_pre);
-    return mh == 2 ? launch_one<B, true, 2>(tA, tA2, tB2, p, ksplit, st, after_pre) : launch_one<B, true, 1>(tA, tA2, tB2, p, ksplit, st, after_pre);
-}
-
 }  // namespace tc
 }  // namespace lq
 
-#include "linear_tc2.cuh"
 
 namespace lq {
 
@@ -1030,22 +569,20 @@ inline bool tc_supported(const QView& q, int r, int64_t M, bool backward) {
     return true;
 }
 
-inline size_t tc_workspace_bytes(int64_t N, int64_t K, int r, int64_t M, bool backward) {
-    const tc::PrePlan pl = tc::pre_plan(backward ? N : K, r, M, backward ? K : N);
-    return kStatusBytes + pl.t_bytes;
+inline size_t tc_workspace_bytes(int r, int64_t M) {
+    return kStatusBytes + round_up(static_cast<size_t>(M) * (r > 0 ? r : 1) * 2, 256);      // [status word][T bf16]
 }
 
 inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, const void* A, int M, void* out, char* ws,
                      bool backward, cudaStream_t st) {
     using namespace tc;
     const int C = backward ? q.N : q.K;              // contraction length
-    const PrePlan pl = pre_plan(C, r, M, backward ? q.K : q.N);
+    const PrePlan pl = pre_plan(q.b0, C, r, M, backward ? q.K : q.N);
     // workspace: [status word][T bf16]; the status word is cleared by the first kernel of the call (or the caller's memset)
     __nv_bfloat16* T = reinterpret_cast<__nv_bfloat16*>(ws + kStatusBytes);
-    const int mh = (M > 128) ? 2 : 1;
     const bool pair = tc_use_pair(M, backward ? q.K : q.N, sm_count());      // CTA pairs (cta_group::2) on [512, 256] tiles; boxes of 128 rows
     CUtensorMap tA, tA2, tB2;
-    if (!make_map(&tA, A, M, C, pair ? 128 : mh * 128)) return LQLORA_ERR_CUDA;
+    if (pair && !make_map(&tA, A, M, C, 128)) return LQLORA_ERR_CUDA;
     if (r > 0) {
         // rank-r pre-product on the tensor cores: T = X L2^T (forward) or dY L1 (backward)
         CUtensorMap tPA, tPB;
@@ -1059,8 +596,14 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
         const int rc = backward ? launch_pre<true>(tPA, tPB, pp, pl.mtiles, pl.nsplit, st)
                                 : launch_pre<false>(tPA, tPB, pp, pl.mtiles, pl.nsplit, st);
         if (rc != LQLORA_OK) return rc;
-        if (!make_map(&tA2, T, M, r, pair ? 128 : mh * 128)) return LQLORA_ERR_CUDA;
-        const bool okb = backward ? make_map(&tB2, L2, r, q.K, 64) : make_map(&tB2, L1, q.N, r, pair ? 128 : 256);
+    }
+    if (!pair) {
+        const SwapPlan sp = swap_plan(q.b0, M, backward ? q.K : q.N, pl.steps, (r + BK - 1) / BK);
+        return run_swap(q, L1, L2, r, A, M, out, T, reinterpret_cast<int*>(ws), backward, sp, 0, backward ? q.K : q.N, st, true);
+    }
+    if (r > 0) {
+        if (!make_map(&tA2, T, M, r, 128)) return LQLORA_ERR_CUDA;
+        const bool okb = backward ? make_map(&tB2, L2, r, q.K, 64) : make_map(&tB2, L1, q.N, r, 128);
         if (!okb) return LQLORA_ERR_CUDA;
     } else {
         tA2 = tA; tB2 = tA;
@@ -1073,60 +616,34 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
     p.out_cols = backward ? q.K : q.N;
     p.steps_q = (C + BK - 1) / BK;
     p.steps_d = (r + BK - 1) / BK;
-    p.stages = 0;
     p.c_base = 0;
     p.c_tiles = static_cast<int>((p.out_cols + BN - 1) / BN);
-    if (pair) {
-        // Wave quantisation: the pair tiles run in waves of sms / 2 clusters.  When the last wave would hold only a few
-        // tiles (at most a quarter of a wave), the output columns it would cover are peeled off and computed by the
-        // one-CTA kernel with the contraction split over clusters, which spreads that small remainder over many SMs
-        // (28672 x 8192 at 2048 rows: 448 pair tiles = 6 waves + 4 tiles, 817 -> 740 us).  Larger remainders stay with
-        // the pairs: the one-CTA kernel needs about 1.6 pair-tile times for three quarters of a wave (measured).
-        const int mt = (M + 511) / 512, pairs = sm_count() / 2;
-        const int tiles = mt * p.c_tiles, rem = tiles % pairs;
-        int peel = 0;
-        if (tiles > pairs && rem > 0 && 4 * rem <= pairs) peel = (rem + mt - 1) / mt;
-        if (peel >= p.c_tiles) peel = 0;
-        CUtensorMap tOut;         // output as boxes of 32 rows x 64 columns
-        if (!make_map(&tOut, out, M, p.out_cols, 32)) return LQLORA_ERR_CUDA;
-        p.c_tiles -= peel;
-        int rc;
-        switch (q.b0) {
-            case 2: rc = backward ? launch_pair<2, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<2, false>(tA, tA2, tB2, tOut, p, st); break;
-            case 3: rc = backward ? launch_pair<3, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<3, false>(tA, tA2, tB2, tOut, p, st); break;
-            case 4: rc = backward ? launch_pair<4, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<4, false>(tA, tA2, tB2, tOut, p, st); break;
-            default: rc = backward ? launch_pair<8, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<8, false>(tA, tA2, tB2, tOut, p, st); break;
-        }
-        if (rc != LQLORA_OK || peel == 0) return rc;
-        // the peeled columns: boxes of 256 rows for the one-CTA kernel; it runs behind the pair kernel (which has waited
-        // for the rank-r intermediate), so it needs no programmatic dependency of its own
-        CUtensorMap uA, uA2, uB2;
-        if (!make_map(&uA, A, M, C, 256)) return LQLORA_ERR_CUDA;
-        if (r > 0) {
-            if (!make_map(&uA2, T, M, r, 256)) return LQLORA_ERR_CUDA;
-            const bool okb = backward ? make_map(&uB2, L2, r, q.K, 64) : make_map(&uB2, L1, q.N, r, 256);
-            if (!okb) return LQLORA_ERR_CUDA;
-        } else {
-            uA2 = uA; uB2 = uA;
-        }
-        Params p2 = p;
-        p2.c_base = p.c_tiles * BN;
-        p2.c_tiles = peel;
-        const int ks2 = tc_ksplit_tiles(static_cast<long long>(peel) * ((M + 255) / 256), p.steps_q, sm_count());
-        switch (q.b0) {
-            case 2: return launch_b<2>(uA, uA2, uB2, p2, backward, 2, ks2, st, false);
-            case 3: return launch_b<3>(uA, uA2, uB2, p2, backward, 2, ks2, st, false);
-            case 4: return launch_b<4>(uA, uA2, uB2, p2, backward, 2, ks2, st, false);
-            default: return launch_b<8>(uA, uA2, uB2, p2, backward, 2, ks2, st, false);
-        }
-    }
-    const int ksplit = tc_ksplit(M, p.out_cols, p.steps_q, sm_count());
+    // Wave quantisation: the pair tiles run in waves of sms / 2 clusters.  When the last wave would hold only a few
+    // tiles (at most a quarter of a wave), the output columns it would cover are peeled off and computed by the
+    // one-CTA kernel with the contraction split over clusters, which spreads that small remainder over many SMs
+    // (28672 x 8192 at 2048 rows: 448 pair tiles = 6 waves + 4 tiles, 817 -> 740 us).  Larger remainders stay with
+    // the pairs: the one-CTA kernel needs about 1.6 pair-tile times for three quarters of a wave (measured).
+    const int mt = (M + 511) / 512, pairs = sm_count() / 2;
+    const int tiles = mt * p.c_tiles, rem = tiles % pairs;
+    int peel = 0;
+    if (tiles > pairs && rem > 0 && 4 * rem <= pairs) peel = (rem + mt - 1) / mt;
+    if (peel >= p.c_tiles) peel = 0;
+    CUtensorMap tOut;         // output as boxes of 32 rows x 64 columns
+    if (!make_map(&tOut, out, M, p.out_cols, 32)) return LQLORA_ERR_CUDA;
+    p.c_tiles -= peel;
+    int rc;
     switch (q.b0) {
-        case 2: return launch_b<2>(tA, tA2, tB2, p, backward, mh, ksplit, st);
-        case 3: return launch_b<3>(tA, tA2, tB2, p, backward, mh, ksplit, st);
-        case 4: return launch_b<4>(tA, tA2, tB2, p, backward, mh, ksplit, st);
-        default: return launch_b<8>(tA, tA2, tB2, p, backward, mh, ksplit, st);
+        case 2: rc = backward ? launch_pair<2, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<2, false>(tA, tA2, tB2, tOut, p, st); break;
+        case 3: rc = backward ? launch_pair<3, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<3, false>(tA, tA2, tB2, tOut, p, st); break;
+        case 4: rc = backward ? launch_pair<4, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<4, false>(tA, tA2, tB2, tOut, p, st); break;
+        default: rc = backward ? launch_pair<8, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<8, false>(tA, tA2, tB2, tOut, p, st); break;
     }
+    if (rc != LQLORA_OK || peel == 0) return rc;
+    // the peeled columns run behind the pair kernel (which has waited for the rank-r intermediate), so they need no
+    // programmatic dependency of their own
+    const int c_base = p.c_tiles * BN;
+    const SwapPlan sp = swap_plan(q.b0, M, p.out_cols - c_base, p.steps_q, p.steps_d);
+    return run_swap(q, L1, L2, r, A, M, out, T, reinterpret_cast<int*>(ws), backward, sp, c_base, p.out_cols - c_base, st, false);
 }
 
 }  // namespace lq

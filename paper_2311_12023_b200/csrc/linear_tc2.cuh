@@ -82,10 +82,13 @@ __device__ __noinline__ bool wait_cluster(uint32_t bar, uint32_t parity, const C
 
 constexpr int kPairBBytes = 128 * 128;        // this CTA's half of the bf16 weight tile of one step
 constexpr int kPairABytes = 2 * 128 * 128;    // two activation tiles of 128 rows x 64 columns
-constexpr int kPairBStages = 4;
+// Stages of the two rings.  A dequantization warp works on every second step and waits for the copies of step j once the
+// weight stage is free; a barrier tells only the parity of its phase, so the copies of step j - SA must be known to have landed
+// by then: with SA = 4 its own group used them, with SA = 3 the tensor core must be done with step j - 3, hence SB = 3.
+template <int B> __host__ __device__ constexpr int pair_b_stages() { return (B == 8) ? 3 : 4; }
 template <int B> __host__ __device__ constexpr int pair_a_stages() { return (B == 8) ? 3 : 4; }
 template <int B> __host__ __device__ constexpr int pair_smem_bytes() {
-    return 1024 + pair_a_stages<B>() * (kPairABytes + 1024 * B) + kPairBStages * kPairBBytes + 512 + (B == 8 ? 32768 : 0);   // 8-bit: code book once per bank
+    return 1024 + pair_a_stages<B>() * (kPairABytes + 1024 * B) + pair_b_stages<B>() * kPairBBytes + 512 + (B == 8 ? 32768 : 0);   // 8-bit: code book once per bank
 }
 
 template <int B, bool BWD>
@@ -93,7 +96,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmA2,
                       const __grid_constant__ CUtensorMap tmB2, const __grid_constant__ CUtensorMap tmOut, const Params p) {
     constexpr int SA = pair_a_stages<B>();
-    constexpr int SB = kPairBStages;
+    constexpr int SB = pair_b_stages<B>();
     constexpr int P_BYTES = 1024 * B;
     constexpr uint32_t TMEM_COLS = 512;
 
@@ -334,7 +337,7 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                     }
                     ok = wait(full_a(sa), ra.ph, ctl, 44);
                     if (!ok) break;
-                    dequant_group<B, true>(slab_base + sa * P_BYTES + ((step & 1) ? slot_odd : slot_even) * 4, s_lo, s_hi, two_scales,
+                    dequant_group<B>(slab_base + sa * P_BYTES + ((step & 1) ? slot_odd : slot_even) * 4, s_lo, s_hi, two_scales,
                                            my_b + sb * kPairBBytes, g << 6, xr, lut8 + lane);
                     fence_proxy_async();
                 } else {

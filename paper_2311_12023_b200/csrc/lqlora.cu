@@ -33,7 +33,7 @@ static int cuda_rc(cudaError_t e) {
 
 // Scratch bytes one direction of the linear needs for M rows, for the kernel family it dispatches to.
 static size_t linear_need_base(const QView& v, int r, int64_t M, bool backward) {
-    if (tc_supported(v, r, M, backward)) return tc_workspace_bytes(v.N, v.K, r, M, backward);
+    if (tc_supported(v, r, M, backward)) return tc_workspace_bytes(r, M);
     if (backward ? dec::bwd_supported(v, M) : dec::supported(v, M)) return dec::workspace_bytes(v, r, static_cast<int>(M), backward);
     const SmallPlan p = small_plan(v.N, v.K, r, M, backward);
     return kStatusBytes + p.t_bytes + p.p_bytes;
@@ -545,7 +545,7 @@ int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, in
         const int64_t out_cols = bwd ? K : N;
         const int steps_q = static_cast<int>(((bwd ? N : K) + tc::BK - 1) / tc::BK);
         if (tc::tc_use_pair(M, out_cols, tc::sm_count())) kernel = LQLORA_PATH_TC_PAIR;
-        else { kernel = LQLORA_PATH_TC_ONE; ks = tc::tc_ksplit(M, out_cols, steps_q, tc::sm_count()); }
+        else { kernel = LQLORA_PATH_TC_ONE; ks = tc::swap_plan(v.b0, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK).ks; }
     } else if (bwd ? dec::bwd_supported(v, M) : dec::supported(v, M)) {
         kernel = LQLORA_PATH_STREAM;
         ks = bwd ? dec::bwd_splits(v, static_cast<int>(M)) : dec::fwd_splits(v, static_cast<int>(M));
