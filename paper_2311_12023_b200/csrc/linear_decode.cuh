@@ -414,6 +414,7 @@ decode_fwd_kernel(const Params p) {
     }
 
     // ---------------------------------------------------------------------- rank-r term, reduction, output
+    pdl_launch_dependents();      // the next call's pre-product may take its place on the SMs (it waits for this kernel)
     __syncthreads();
     if (*abort_s) {
         // a wait gave up: let copies that are still in flight land before the CTA exits (bounded)
@@ -786,6 +787,7 @@ decode_bwd_kernel(const BwdParams p) {
     // tree: the upper half of the active warps writes its accumulators to the idle ring, the lower half adds them
     float* red = reinterpret_cast<float*>(ring);
     static_assert(4 * KF * 32 * 4 <= NS * STAGE, "reduction buffer must fit into the ring");
+    pdl_launch_dependents();      // the next call's pre-product may take its place on the SMs (it waits for this kernel)
     __syncthreads();
     if (*abort_s) {
         // a wait gave up: let copies that are still in flight land before the ring is reused (bounded)
@@ -925,6 +927,7 @@ __global__ void __launch_bounds__(kPreThreads) decode_pre_kernel(const PreParams
     __nv_bfloat16* as = reinterpret_cast<__nv_bfloat16*>(pre_smem);
     float* red = reinterpret_cast<float*>(pre_smem + static_cast<size_t>(MP) * p.chunk * 2);
     float* part = red + kPrePhases * 16 * kPreJ;
+    pdl_wait();                   // started while the previous kernel of the stream ends; everything below comes after it
     pdl_launch_dependents();
     if (blockIdx.x == 0 && blockIdx.y == 0) {
         if (threadIdx.x == 0) *p.status = 0;
@@ -1158,11 +1161,13 @@ inline cudaError_t launch_pre(const __nv_bfloat16* A, const __nv_bfloat16* F, __
     cfg.blockDim = dim3(kPreThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = nranks; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // the launch overlaps the end of the kernel in front
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     count_launch(1);
     return cudaLaunchKernelEx(&cfg, kern, pp);
 }

@@ -375,6 +375,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             }
         }
         // ------------------------------------------------------------------ epilogue: warp = 32 output columns x every fourth chunk of 32 tokens
+        pdl_launch_dependents();      // the next call's pre-product may take its place on the SMs (it waits for this kernel)
         acc_ok = ok && wait(acc_full, 0, ctl, 58);
         if (acc_ok) {
             tc_fence_after();

@@ -226,6 +226,7 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
     // The CTAs of a cluster write into each other's shared memory at the end; that is allowed once every CTA of the
     // cluster runs, which the first phase of the cluster barrier establishes: arrive here, wait before the first store.
     if (CL && nsplit > 1) dec::cluster_arrive_relaxed();
+    pdl_wait();                   // started while the previous kernel of the stream ends; everything below comes after it
     // cleared before this CTA lets the dependent kernel start: that kernel is launched once all CTAs have passed here
     if (p.clear_status && tile == 0 && split == 0 && threadIdx.x == 0) *p.status = 0;
     pdl_launch_dependents();      // the linear kernel behind this one needs T only in its last steps
@@ -538,11 +539,13 @@ inline int launch_pre(const CUtensorMap& tA, const CUtensorMap& tB, PreParams p,
     cfg.blockDim = dim3(kLrThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = (!cl && mtiles % 2 == 0) ? 2 : 1; attr[0].val.clusterDim.y = cl ? nsplit : 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // the launch overlaps the end of the kernel in front
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tA, tB, p);
     count_launch(1);
     if (e != cudaSuccess) { cudaGetLastError(); return LQLORA_ERR_CUDA; }

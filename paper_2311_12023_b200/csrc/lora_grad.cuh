@@ -228,7 +228,7 @@ inline int wgrad_splits(int ptiles, int steps) {
 
 // dL1 [N, r] = dY^T T and dL2 [r, K] = T'^T X in one launch.
 inline int launch_wgrad(const void* dY, const void* X, int64_t M, int64_t N, int64_t K, const void* T, const void* Tp, int r,
-                        float* dL1, float* dL2, int* status, cudaStream_t st) {
+                        float* dL1, float* dL2, int* status, bool after_pre, cudaStream_t st) {
     WgradParams p0, p1;
     p0.out = dL1; p0.status = status; p0.M = static_cast<int>(M); p0.P = static_cast<int>(N); p0.r = r; p0.rp = (r <= 64) ? 64 : 128;
     p0.steps = static_cast<int>((M + BK - 1) / BK);
@@ -263,10 +263,12 @@ inline int launch_wgrad(const void* dY, const void* X, int64_t M, int64_t N, int
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 1; attr[0].val.clusterDim.y = ns; attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // overlaps the end of the pre-product kernel
+    // Overlaps the end of the pre-product kernel.  Only behind that one: the kernel reads X and dY before it waits for its
+    // predecessor, which behind any other kernel (a linear call that lets its successor start early) may still write them.
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = after_pre ? 2 : 1;
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tA0, tT0, p0, tA1, tT1, p1);
     count_launch(1);
     if (e != cudaSuccess) { cudaGetLastError(); return LQLORA_ERR_CUDA; }
@@ -354,7 +356,7 @@ inline int lora_grads_launch(const void* L1, const void* L2, int r, int64_t N, i
     p1.T = Tp; p1.steps = g.steps_y; p1.steps_per_split = g.sps_y; p1.clear_status = 0;
     const int rc = launch_pre_both(tA0, tB0, p0, tA1, tB1, p1, g.nsplit, g.mtiles, st);
     if (rc != LQLORA_OK) return rc;
-    return launch_wgrad(dY, X, M, N, K, T, Tp, r, dL1, dL2, status, st);
+    return launch_wgrad(dY, X, M, N, K, T, Tp, r, dL1, dL2, status, true, st);
 }
 
 }  // namespace tc

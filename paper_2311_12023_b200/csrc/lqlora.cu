@@ -424,7 +424,7 @@ int lqlora_lora_grads_from(const void* T_dev, const void* Tp_dev, int r, int64_t
     if (workspace_bytes < static_cast<size_t>(kStatusBytes)) return LQLORA_ERR_WORKSPACE_TOO_SMALL;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(workspace_dev, 0, kStatusBytes, st) != cudaSuccess) return cuda_rc(cudaGetLastError());
-    return tc::launch_wgrad(dY_dev, X_dev, M, N, K, T_dev, Tp_dev, r, dL1_dev, dL2_dev, static_cast<int*>(workspace_dev), st);
+    return tc::launch_wgrad(dY_dev, X_dev, M, N, K, T_dev, Tp_dev, r, dL1_dev, dL2_dev, static_cast<int*>(workspace_dev), false, st);
 }
 
 int lqlora_lq_workspace_bytes(int64_t N, int64_t K, const lqlora_config* cfg, int r, int oversample, size_t* bytes) {
