@@ -1070,8 +1070,23 @@ inline double grid_cost(long n, double work, int per_sm, int sms, double fixed) 
     return t + fixed + 0.25 * fixed * static_cast<double>(nw - 1);
 }
 
+// Plans of the last few shapes, kept by the calling thread (pure host arithmetic; a call asks for its plan four times).
+template <typename P, typename F>
+inline P cached_plan(const QView& q, int M, F&& make) {
+    struct Entry { int N = 0, K = 0, logB0 = 0, logB1 = 0, M = 0; P plan; };
+    constexpr int kEntries = 16;
+    thread_local Entry cache[kEntries];
+    Entry& e = cache[(static_cast<uint32_t>(q.N) * 2654435761u + static_cast<uint32_t>(q.K) * 2246822519u +
+                      static_cast<uint32_t>(M * 64 + q.logB0 * 8 + q.logB1) * 3266489917u) >> 28];
+    if (e.N != q.N || e.K != q.K || e.logB0 != q.logB0 || e.logB1 != q.logB1 || e.M != M) {
+        e.plan = make();
+        e.N = q.N; e.K = q.K; e.logB0 = q.logB0; e.logB1 = q.logB1; e.M = M;
+    }
+    return e.plan;
+}
+
 template <int B>
-inline Plan make_plan(const QView& q, int M) {
+inline Plan compute_plan(const QView& q, int M) {
     Plan best{};
     best.ok = false;
     const int NT = (M <= 8) ? 1 : 2;
@@ -1107,6 +1122,9 @@ inline Plan make_plan(const QView& q, int M) {
     }
     return best;
 }
+
+template <int B>
+inline Plan make_plan(const QView& q, int M) { return cached_plan<Plan>(q, M, [&] { return compute_plan<B>(q, M); }); }
 
 template <int B>
 inline size_t fwd_workspace(const QView& q, int r, int M) {
@@ -1258,7 +1276,7 @@ inline BwdPlan make_bwd_plan_t(const QView& q, int M, int trps, bool allow_compa
 // A unit of work is one tile row of the window (128 x 256 weights); the compact table costs a few conversions per use
 // (about 4 %) and wins where the fp32 table would force more slices or a single CTA per SM.
 template <int B>
-inline BwdPlan make_bwd_plan(const QView& q, int M) {
+inline BwdPlan compute_bwd_plan(const QView& q, int M) {
     BwdPlan best{};
     double best_cost = 0.0;
     const int NT = (M <= 8) ? 1 : 2;
@@ -1283,6 +1301,9 @@ inline BwdPlan make_bwd_plan(const QView& q, int M) {
     }
     return best;
 }
+
+template <int B>
+inline BwdPlan make_bwd_plan(const QView& q, int M) { return cached_plan<BwdPlan>(q, M, [&] { return compute_bwd_plan<B>(q, M); }); }
 
 template <int B>
 inline size_t bwd_workspace(const QView& q, int r, int M) {
