@@ -497,6 +497,14 @@ inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
     return true;
 }
 
+// Tokens of the largest chunk whose rings fit: 512, and 384 for 8-bit codes (their code book takes 32 KB of shared memory).
+inline int swap_max_tokens(int b0) {
+    SwapPlan pl{};
+    pl.nbox = 2;
+    for (pl.box = 256; pl.box > 16 && !swap_rings(b0, 1, pl); pl.box -= 16) {}
+    return 2 * pl.box;
+}
+
 // The split of a call that costs least by a simple model: waves of clusters, each with a fixed cost, its steps (the
 // slower of dequantization and tensor core) and its reduction.  The constants are those of a sweep over chunks and slices
 // (us with 1, 2, 3, 4 slices): 4096 x 4096 NF3, 64 rows: 24, 17, 15, 26 (16 clusters of eight, of which 15 fit); 8192 x 8192
@@ -507,7 +515,11 @@ inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q,
     best.us = -1.0;
     const double dq = b0 == 2 ? 0.22 : b0 == 3 ? 0.26 : b0 == 4 ? 0.35 : 0.40;      // us per step of 128 x 64 weights
     const long long pairs = (out_cols + 255) / 256;
-    const int first = static_cast<int>((M + 511) / 512);
+    int first = static_cast<int>((M + 511) / 512);
+    // The search covers eight numbers of chunks.  Where the chunks of all of them are too large for the rings (8-bit codes
+    // above 11136 rows), it starts at the fewest that are not: a plan exists for every number of rows.
+    const int tokens_max = swap_max_tokens(b0), fit = static_cast<int>((M + tokens_max - 1) / tokens_max);
+    if (fit > first + 7) first = fit;
     for (int ch = first; ch <= first + 7; ++ch) {
         SwapPlan pl{};
         const int per = static_cast<int>((M + ch - 1) / ch);

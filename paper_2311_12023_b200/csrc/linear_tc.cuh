@@ -484,6 +484,30 @@ inline int sm_count() {
     return n;
 }
 
+// Wave quantisation of the pair kernel: its tiles run in waves of sms / 2 clusters.  When the last wave would hold only a few
+// tiles (at most a quarter of a wave), the output columns it would cover are peeled off and computed by the
+// one-CTA kernel with the contraction split over clusters, which spreads that small remainder over many SMs
+// (28672 x 8192 at 2048 rows: 448 pair tiles = 6 waves + 4 tiles, 817 -> 740 us).  Larger remainders stay with
+// the pairs: the one-CTA kernel needs about 1.6 pair-tile times for three quarters of a wave (measured).
+// Returns the number of 256-column tiles to peel off.
+inline int pair_peel(int64_t M, int64_t out_cols) {
+    const int mt = static_cast<int>((M + 511) / 512), pairs = sm_count() / 2, c_tiles = static_cast<int>((out_cols + BN - 1) / BN);
+    const long long tiles = static_cast<long long>(mt) * c_tiles;
+    const int rem = static_cast<int>(tiles % pairs);
+    const int peel = (tiles > pairs && rem > 0 && 4 * rem <= pairs) ? (rem + mt - 1) / mt : 0;
+    return peel >= c_tiles ? 0 : peel;
+}
+
+// The launch on transposed tiles that a call needs: the whole of it, or the output columns from *c_base on that the pair
+// kernel leaves (none where *c_base is not below out_cols).
+inline SwapPlan call_swap_plan(int b0, bool pair, int64_t M, int64_t out_cols, int steps_q, int steps_d, int* c_base) {
+    *c_base = 0;
+    if (!pair) return swap_plan(b0, M, out_cols, steps_q, steps_d);
+    const int peel = pair_peel(M, out_cols);
+    *c_base = (static_cast<int>((out_cols + BN - 1) / BN) - peel) * BN;
+    return peel > 0 ? swap_plan(b0, M, out_cols - *c_base, steps_q, steps_d) : SwapPlan{};
+}
+
 // C = contraction length, out_cols = width of the output of the linear kernel that follows.
 inline PrePlan pre_plan(int b0, int64_t C, int r, int64_t M, int64_t out_cols) {
     PrePlan pl;
@@ -584,6 +608,10 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
     // workspace: [status word][T bf16]; the status word is cleared by the first kernel of the call (or the caller's memset)
     __nv_bfloat16* T = reinterpret_cast<__nv_bfloat16*>(ws + kStatusBytes);
     const bool pair = tc_use_pair(M, backward ? q.K : q.N, sm_count());      // CTA pairs (cta_group::2) on [512, 256] tiles; boxes of 128 rows
+    const int out_cols = backward ? q.K : q.N;
+    int c_base = 0;
+    const SwapPlan sp = call_swap_plan(q.b0, pair, M, out_cols, pl.steps, (r + BK - 1) / BK, &c_base);
+    if (c_base < out_cols && sp.ks < 1) return LQLORA_ERR_INVALID_SHAPE;      // (never: a plan exists for every shape) before any launch
     CUtensorMap tA, tA2, tB2;
     if (pair && !make_map(&tA, A, M, C, 128)) return LQLORA_ERR_CUDA;
     if (r > 0) {
@@ -600,10 +628,7 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
                                 : launch_pre<false>(tPA, tPB, pp, pl.mtiles, pl.nsplit, st);
         if (rc != LQLORA_OK) return rc;
     }
-    if (!pair) {
-        const SwapPlan sp = swap_plan(q.b0, M, backward ? q.K : q.N, pl.steps, (r + BK - 1) / BK);
-        return run_swap(q, L1, L2, r, A, M, out, T, reinterpret_cast<int*>(ws), backward, sp, 0, backward ? q.K : q.N, st, true);
-    }
+    if (!pair) return run_swap(q, L1, L2, r, A, M, out, T, reinterpret_cast<int*>(ws), backward, sp, 0, out_cols, st, true);
     if (r > 0) {
         if (!make_map(&tA2, T, M, r, 128)) return LQLORA_ERR_CUDA;
         const bool okb = backward ? make_map(&tB2, L2, r, q.K, 64) : make_map(&tB2, L1, q.N, r, 128);
@@ -616,24 +641,13 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
     p.out = static_cast<__nv_bfloat16*>(out);
     p.status = reinterpret_cast<int*>(ws);
     p.M = M;
-    p.out_cols = backward ? q.K : q.N;
+    p.out_cols = out_cols;
     p.steps_q = (C + BK - 1) / BK;
     p.steps_d = (r + BK - 1) / BK;
     p.c_base = 0;
-    p.c_tiles = static_cast<int>((p.out_cols + BN - 1) / BN);
-    // Wave quantisation: the pair tiles run in waves of sms / 2 clusters.  When the last wave would hold only a few
-    // tiles (at most a quarter of a wave), the output columns it would cover are peeled off and computed by the
-    // one-CTA kernel with the contraction split over clusters, which spreads that small remainder over many SMs
-    // (28672 x 8192 at 2048 rows: 448 pair tiles = 6 waves + 4 tiles, 817 -> 740 us).  Larger remainders stay with
-    // the pairs: the one-CTA kernel needs about 1.6 pair-tile times for three quarters of a wave (measured).
-    const int mt = (M + 511) / 512, pairs = sm_count() / 2;
-    const int tiles = mt * p.c_tiles, rem = tiles % pairs;
-    int peel = 0;
-    if (tiles > pairs && rem > 0 && 4 * rem <= pairs) peel = (rem + mt - 1) / mt;
-    if (peel >= p.c_tiles) peel = 0;
+    p.c_tiles = c_base / BN;
     CUtensorMap tOut;         // output as boxes of 32 rows x 64 columns
     if (!make_map(&tOut, out, M, p.out_cols, 32)) return LQLORA_ERR_CUDA;
-    p.c_tiles -= peel;
     int rc;
     switch (q.b0) {
         case 2: rc = backward ? launch_pair<2, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<2, false>(tA, tA2, tB2, tOut, p, st); break;
@@ -641,11 +655,9 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
         case 4: rc = backward ? launch_pair<4, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<4, false>(tA, tA2, tB2, tOut, p, st); break;
         default: rc = backward ? launch_pair<8, true>(tA, tA2, tB2, tOut, p, st) : launch_pair<8, false>(tA, tA2, tB2, tOut, p, st); break;
     }
-    if (rc != LQLORA_OK || peel == 0) return rc;
+    if (rc != LQLORA_OK || c_base >= out_cols) return rc;
     // the peeled columns run behind the pair kernel (which has waited for the rank-r intermediate), so they need no
     // programmatic dependency of their own
-    const int c_base = p.c_tiles * BN;
-    const SwapPlan sp = swap_plan(q.b0, M, p.out_cols - c_base, p.steps_q, p.steps_d);
     return run_swap(q, L1, L2, r, A, M, out, T, reinterpret_cast<int*>(ws), backward, sp, c_base, p.out_cols - c_base, st, false);
 }
 

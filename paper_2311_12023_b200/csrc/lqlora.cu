@@ -544,8 +544,12 @@ int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, in
     if (tc_supported(v, r, M, bwd)) {
         const int64_t out_cols = bwd ? K : N;
         const int steps_q = static_cast<int>(((bwd ? N : K) + tc::BK - 1) / tc::BK);
-        if (tc::tc_use_pair(M, out_cols, tc::sm_count())) kernel = LQLORA_PATH_TC_PAIR;
-        else { kernel = LQLORA_PATH_TC_ONE; ks = tc::swap_plan(v.b0, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK).ks; }
+        const bool pair = tc::tc_use_pair(M, out_cols, tc::sm_count());
+        int c_base = 0;
+        const tc::SwapPlan sp = tc::call_swap_plan(v.b0, pair, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK, &c_base);
+        if (c_base < out_cols && sp.ks < 1) return LQLORA_ERR_INVALID_SHAPE;      // as the call itself
+        kernel = pair ? LQLORA_PATH_TC_PAIR : LQLORA_PATH_TC_ONE;
+        if (!pair) ks = sp.ks;
     } else if (bwd ? dec::bwd_supported(v, M) : dec::supported(v, M)) {
         kernel = LQLORA_PATH_STREAM;
         ks = bwd ? dec::bwd_splits(v, static_cast<int>(M)) : dec::fwd_splits(v, static_cast<int>(M));

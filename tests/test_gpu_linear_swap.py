@@ -27,3 +27,14 @@ def test_rank_steps(r):
     A = inputs.student_t(1650, (N, K), 5.0, 0.02)
     l1b, l2b = inputs.lowrank_factors(1651, N, K, r, 0.03) if r else (None, None)
     run_case(A, l1b, l2b, C(3, 64, 8, 256, 32), M, seed=1750 + r)
+
+
+# 8-bit codes take the most shared memory (token chunks of at most 384 rows): many rows on a narrow output, and on the columns
+# that the pair kernel peels off (4096 columns at 12288 rows: 384 pair tiles, 14 of them in the last wave), both passes
+@pytest.mark.parametrize("N,K", [(256, 512), (512, 256), (4096, 512), (512, 4096)])
+def test_8_bit_codes_many_rows(N, K):
+    M = 12288
+    A = inputs.gaussian(1800 + N, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(1801 + K, N, K, 64, 0.01)
+    route = {256: binding.PATH_TC_ONE, 4096: binding.PATH_TC_PAIR}.get(N)
+    run_case(A, l1b, l2b, C(8, 64, 8, 64, 32), M, seed=1810, rows=inputs.sample_rows(1811, M, count=24, tile=384), route=route)

@@ -170,3 +170,19 @@ def test_budgeted_assignment_matches_exhaustive_search(binding):
     E = np.array([[5.0, 7.0, 1.0]])
     assert binding.assign_configs(E, S, 2.5)[0] == [0]
     assert binding.assign_configs(E, S, 3.0)[0] == [2]
+
+
+@pytest.mark.parametrize("b0", [2, 3, 4, 8])
+def test_every_number_of_rows_has_a_plan_on_the_tensor_core_kernels(binding, b0):
+    """The route of a call names at least one slice of the contraction for any number of rows, on narrow outputs (all of
+    them on transposed tiles) and where the pair kernel peels columns off (an error without a plan for those).  8-bit codes
+    take the most shared memory: their token chunks end at 384 instead of 512 rows."""
+    cfg = inputs.QuantConfig(b0, 64, 8, 256, 32)
+    g = inputs.rng(77 + b0)
+    edges = [m + d for m in (512, 3072, 11136, 11264, 11520, 11776, 12288, 14336, 16384, 18944, 28672, 1 << 20, 1 << 24) for d in (-1, 0, 1)]
+    rows = sorted({m for m in edges + list(range(17, 19200, 37)) + [int(2 ** x) for x in g.uniform(4.1, 24.0, 400)] if 17 <= m <= 1 << 24})
+    for N, K in ((256, 4096), (64, 512), (4096, 512), (8192, 1024), (14336, 4096), (28672, 8192)):
+        for M in rows:
+            for r, backward in ((64, False), (0, False), (128, True)):
+                kernel, splits = binding.linear_route(N, K, cfg, r, M, backward)
+                assert kernel in (binding.PATH_TC_ONE, binding.PATH_TC_PAIR) and 1 <= splits <= 4, (N, K, M, r, backward)
