@@ -59,7 +59,10 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 
 constexpr long long kWaitCycles = 4000000000LL;   // about two seconds
 
-// Bounded wait.  Returns false when the wait was abandoned (another thread aborted, or time ran out).
+// Bounded wait of a whole (converged) warp.  Returns false when the wait was abandoned (another thread aborted, or time ran
+// out).  The verdict is the warp's: every lane polls the barrier, the abort flag and the clock for itself, so near a time-out
+// lanes can disagree, and what follows a wait (elect.sync, __syncwarp, tcgen05.ld, shuffles) needs all of them on one path.
+// The wait holds when it held for all lanes.
 struct Ctl {
     volatile int* abort_s;
     int* status_g;
@@ -80,8 +83,9 @@ __device__ __noinline__ bool wait_slow(uint32_t bar, uint32_t parity, const Ctl&
     }
 }
 __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
-    if (mbar_try_wait(bar, parity)) return true;
-    return wait_slow(bar, parity, c, where);
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const bool ok = wait_slow(bar, parity, c, where);
+    return __all_sync(0xffffffffu, ok);
 }
 
 // ------------------------------------------------------------------------------------ dequantization tables

@@ -259,7 +259,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             uint32_t acc = 0;
             RingAt r(0, p.ss);
             for (int step = 0; step < total; ++step, r.advance(1, p.ss)) {
-                ok = mbar_try_wait_acq_cluster(full(r.s), r.ph) || wait_cluster(full(r.s), r.ph, ctl, 53);
+                ok = wait_cluster(full(r.s), r.ph, ctl, 53);
                 if (!ok) break;
                 __syncwarp();
                 tc_fence_after();

@@ -65,19 +65,25 @@ __device__ __forceinline__ uint32_t mbar_try_wait_acq_cluster(uint32_t bar, uint
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok;
 }
-__device__ __noinline__ bool wait_cluster(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
+__device__ __noinline__ bool wait_cluster_slow(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
     const long long t0 = clock64();
     for (int it = 0;; ++it) {
         if (mbar_try_wait_acq_cluster(bar, parity)) return true;
         if ((it & 63) == 63) {
             if (*c.abort_s) return false;
-            if (clock64() - t0 > kWaitCycles) {
+            if (clock64() - t0 > c.budget) {
                 *c.abort_s = 1;
                 atomicCAS(c.status_g, 0, where);
                 return false;
             }
         }
     }
+}
+// wait() for a barrier that a thread of the other CTA arrives on
+__device__ __forceinline__ bool wait_cluster(uint32_t bar, uint32_t parity, const Ctl& c, int where) {
+    if (__all_sync(0xffffffffu, mbar_try_wait_acq_cluster(bar, parity))) return true;
+    const bool ok = wait_cluster_slow(bar, parity, c, where);
+    return __all_sync(0xffffffffu, ok);
 }
 
 constexpr int kPairBBytes = 128 * 128;        // this CTA's half of the bf16 weight tile of one step
@@ -216,7 +222,7 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             for (int step = 0; step < total; ++step, ra.advance(), rb.advance()) {
                 const int sa = ra.s, sb = rb.s;
                 // the eight warps of this step, each after its CTA's copies have landed, and the second CTA's messenger
-                ok = mbar_try_wait_acq_cluster(full_b(sb), rb.ph) || wait_cluster(full_b(sb), rb.ph, ctl, 42);
+                ok = wait_cluster(full_b(sb), rb.ph, ctl, 42);
                 if (!ok) break;
                 __syncwarp();
                 tc_fence_after();

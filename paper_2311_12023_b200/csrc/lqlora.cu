@@ -141,17 +141,22 @@ static int static_scratch_ptr(void** out) {
     return LQLORA_OK;
 }
 
-// Self-test of the bounded waits: a CTA arms an mbarrier for bytes that nobody delivers and waits on it with the same
-// helper (and the same status word) as the linear kernels, holding a tensor-memory allocation meanwhile; when the
+// Self-test of the bounded waits: a warp arms an mbarrier for bytes that nobody delivers and waits on it with the same
+// helper (and the same status word) as the linear kernels, while the CTA holds a tensor-memory allocation; when the
 // budget runs out the wait is abandoned, the status word is set, tensor memory is freed and the kernel returns.
-__global__ void __launch_bounds__(64) bounded_wait_selftest_kernel(int* status, long long budget) {
-    __shared__ uint64_t bar;
+// Then a wait whose lanes cannot agree by themselves: lane 0 has a short budget and the others a long one, and the barrier is
+// completed as soon as lane 0 has given up.  Word 32 + lane receives 1 where the lane's verdict was "abandoned".
+__global__ void __launch_bounds__(96) bounded_wait_selftest_kernel(int* status, long long budget) {
+    __shared__ uint64_t bars[2];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_s;
-    const int warp = threadIdx.x >> 5;
+    __shared__ int abort_s, abort2_s;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t never = dev::smem_u32(bars), late = dev::smem_u32(bars + 1);
     if (threadIdx.x == 0) {
-        dev::mbar_init(dev::smem_u32(&bar), 1);
+        dev::mbar_init(never, 1);
+        dev::mbar_init(late, 1);
         abort_s = 0;
+        abort2_s = 0;
         dev::fence_barrier_init();
     }
     if (warp == 1) { tc::tmem_alloc(dev::smem_u32(&tmem_slot), 32); tc::tmem_relinquish(); }
@@ -159,10 +164,18 @@ __global__ void __launch_bounds__(64) bounded_wait_selftest_kernel(int* status, 
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = tmem_slot;
-    if (threadIdx.x == 0) {
-        dev::Ctl ctl{&abort_s, status, budget};
-        dev::mbar_expect_tx(dev::smem_u32(&bar), 128);           // 128 bytes that never arrive
-        dev::wait(dev::smem_u32(&bar), 0, ctl, 99);
+    constexpr long long kShort = 100000;      // clock cycles
+    if (warp == 0) {
+        const dev::Ctl ctl{&abort_s, status, budget};
+        if (lane == 0) dev::mbar_expect_tx(never, 128);          // 128 bytes that never arrive
+        __syncwarp();
+        dev::wait(never, 0, ctl, 99);
+        const dev::Ctl ctl2{&abort2_s, status, lane == 0 ? kShort : 100 * kShort};
+        status[32 + lane] = dev::wait(late, 0, ctl2, 98) ? 0 : 1;
+    } else if (warp == 2 && lane == 0) {
+        const long long t0 = clock64();
+        while (!*const_cast<volatile int*>(&abort2_s) && clock64() - t0 < 2 * budget + 100 * kShort) {}
+        dev::mbar_arrive(late);
     }
     tc::tc_fence_before();
     __syncthreads();
@@ -178,7 +191,7 @@ int lqlora_selftest_bounded_wait(void* workspace_dev, int64_t budget_cycles, voi
     if (budget_cycles < 1000 || budget_cycles > 2000000000LL) return LQLORA_ERR_INVALID_SHAPE;     // at most about a second
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaMemsetAsync(workspace_dev, 0, lq::kStatusBytes, st) != cudaSuccess) return lq::cuda_rc(cudaGetLastError());
-    lq::bounded_wait_selftest_kernel<<<1, 64, 0, st>>>(static_cast<int*>(workspace_dev), budget_cycles);
+    lq::bounded_wait_selftest_kernel<<<1, 96, 0, st>>>(static_cast<int*>(workspace_dev), budget_cycles);
     lq::count_launch(1);
     return lq::cuda_rc(cudaGetLastError());
 }

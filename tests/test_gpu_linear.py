@@ -325,3 +325,13 @@ def test_a_bounded_wait_that_runs_out_sets_the_status_and_leaves_the_device_usab
     Y = binding.linear_fwd(q, L1, L2, binding.bf16_from_bits(xb), workspace=ws)
     assert binding.workspace_status(ws) == 0
     check_close(to_np(Y[torch.from_numpy(rows).cuda()]), oracle.linear_fwd(ref["d32"], l1b, l2b, xb, rows), "Y after the time-outs")
+
+
+def test_the_lanes_of_a_warp_agree_on_a_wait_that_runs_out():
+    """A barrier that is completed after lane 0 has given up and before the other lanes have: what follows a wait (elections,
+    shuffles, tensor-memory loads) needs the whole warp on one path, so the verdict has to be the warp's."""
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        binding.selftest_bounded_wait(ws, 100_000)
+        assert binding.workspace_status(ws) == -7
+        assert ws.view(torch.int32)[32:].tolist() == [1] * 32
