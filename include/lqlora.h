@@ -321,7 +321,8 @@ int lqlora_workspace_status(const void* workspace_dev, void* stream);
  * budget_cycles SM clocks (1e3 .. 2e9) the wait is abandoned: the kernel records the time-out in the status word at the
  * head of workspace_dev (at least 256 bytes), frees its tensor memory and returns, so lqlora_workspace_status then
  * reports LQLORA_ERR_TIMEOUT while the context stays usable.  A second wait is completed just after one lane of the warp has
- * given up on it: 32-bit words 32 .. 63 of the workspace receive the verdicts of the 32 lanes (1 = abandoned), which agree.
+ * given up on it: 32-bit words 32 .. 63 of the workspace receive the verdicts of the 32 lanes (1 = abandoned), which agree;
+ * word 1 receives 1 if the wait for copies in flight, on the way out of a kernel that gave up, waits for the step issued last.
  * Nothing traps, faults or spins without bound. */
 int lqlora_selftest_bounded_wait(void* workspace_dev, int64_t budget_cycles, void* stream);
 

@@ -88,6 +88,20 @@ __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, const Ctl& c
     return __all_sync(0xffffffffu, ok);
 }
 
+// On the way out of a kernel that gave up: copies in flight have to land before the CTA exits.  A barrier tells only the parity
+// of its phase (of the two parities one always reads as complete), so the caller names the phase of the copies that it
+// knows to have been issued.  Waits about ten milliseconds at most.
+__device__ __noinline__ void let_land(uint32_t bar, uint32_t parity) {
+    const long long t0 = clock64();
+    while (!mbar_try_wait(bar, parity) && clock64() - t0 < 20000000LL) {}
+}
+// The same for a ring of which `issued` steps have been issued: step i on the barrier bar0 + 8 (i % stages), in its phase
+// i / stages.  The barriers count these copies alone (and the arrival that announces them), and a stage was issued again only
+// after its last copies had landed.
+__device__ __forceinline__ void drain_ring(uint32_t bar0, int issued, int stages) {
+    for (int i = max(0, issued - stages); i < issued; ++i) let_land(bar0 + 8 * (i % stages), (i / stages) & 1);
+}
+
 // ------------------------------------------------------------------------------------ dequantization tables
 // The 2^b0 products fl32(q~[c] * s~) of one block, rounded to bf16, are kept in registers as a
 // byte table: lo[] holds the low bytes, hi[] the high bytes, four entries per register.  One

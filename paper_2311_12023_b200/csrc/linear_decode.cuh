@@ -192,8 +192,9 @@ decode_fwd_kernel(const Params p) {
     uint8_t* ring = base;
     float* recv = reinterpret_cast<float*>(ring + NS * STAGE);        // [2 windows][MT][128 rows] sums of the two warps of a row
     float* lut8 = recv + 2 * 128 * MT;                                 // 256 floats (8-bit codes only)
-    uint64_t* bars = reinterpret_cast<uint64_t*>(lut8 + (B == 8 ? 256 : 0));   // full[NS], then NS counters of warps done with a slot
+    uint64_t* bars = reinterpret_cast<uint64_t*>(lut8 + (B == 8 ? 256 : 0));   // full[NS], NS counters of warps done with a slot, NS steps last issued into it
     uint32_t* done = reinterpret_cast<uint32_t*>(bars + NS);
+    int* issued = reinterpret_cast<int*>(done + NS);
     volatile int* abort_s = reinterpret_cast<volatile int*>(bars + 2 * NS);
     volatile int* last_s = abort_s + 1;
     float* stab = reinterpret_cast<float*>(bars + 2 * NS + 2);         // [nkb][kStabStride] block scales s~ (fp32 table)
@@ -214,7 +215,7 @@ decode_fwd_kernel(const Params p) {
     auto full = [&](int s) { return smem_u32(bars + s); };
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NS; ++s) { mbar_init(full(s), 1); done[s] = 0u; }
+        for (int s = 0; s < NS; ++s) { mbar_init(full(s), 1); done[s] = 0u; issued[s] = -1; }
         *abort_s = 0;
         *last_s = 0;
         fence_barrier_init();
@@ -231,6 +232,7 @@ decode_fwd_kernel(const Params p) {
         const int nt = min(kStageTiles, ntiles_cta - it * kStageTiles);
         const uint32_t dst = smem_u32(ring + s * STAGE);
         if (ln == 0) {
+            issued[s] = it;
             mbar_expect_tx(full(s), nt * 1024 * B + p.M * nt * (kTileCols * 2));
             bulk_load(dst, codes + static_cast<size_t>(it) * (kStageTiles * 1024 * B), nt * 1024 * B, full(s));
         } else if (ln <= p.M) {
@@ -419,10 +421,8 @@ decode_fwd_kernel(const Params p) {
     if (*abort_s) {
         // a wait gave up: let copies that are still in flight land before the CTA exits (bounded)
         if (threadIdx.x == 0) {
-            for (int s = 0; s < NS; ++s) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(full(s), 0) && !mbar_try_wait(full(s), 1) && clock64() - t0 < 20000000LL) {}
-            }
+            for (int s = 0; s < NS; ++s)
+                if (issued[s] >= 0) let_land(full(s), (issued[s] / NS) & 1);
         }
         __syncthreads();
     }
@@ -538,8 +538,9 @@ decode_bwd_kernel(const BwdParams p) {
     uint8_t* ring = base;
     float* outs = reinterpret_cast<float*>(ring + NS * STAGE);        // [8 NT tokens][256 columns] sums of the CTA
     float* lut8 = outs + KF * 32;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(lut8 + (B == 8 ? 256 : 0));   // full[NS], then NS counters of warps done with a slot
+    uint64_t* bars = reinterpret_cast<uint64_t*>(lut8 + (B == 8 ? 256 : 0));   // full[NS], NS counters of warps done with a slot, NS steps last issued into it
     uint32_t* done = reinterpret_cast<uint32_t*>(bars + NS);
+    int* issued = reinterpret_cast<int*>(done + NS);
     volatile int* abort_s = reinterpret_cast<volatile int*>(bars + 2 * NS);
     volatile int* last_s = abort_s + 1;
     float* stab = reinterpret_cast<float*>(bars + 2 * NS + 2);         // [nkb][rows_stride] block scales s~
@@ -558,7 +559,7 @@ decode_bwd_kernel(const BwdParams p) {
     auto full = [&](int s) { return smem_u32(bars + s); };
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NS; ++s) { mbar_init(full(s), 1); done[s] = 0u; }
+        for (int s = 0; s < NS; ++s) { mbar_init(full(s), 1); done[s] = 0u; issued[s] = -1; }
         *abort_s = 0;
         fence_barrier_init();
     }
@@ -573,7 +574,10 @@ decode_bwd_kernel(const BwdParams p) {
         const uint32_t dst = smem_u32(ring + s * STAGE);
         const int row0 = (tr0 + 2 * it) * 128;
         const int nrows = min(ntr * 128, q.N - row0);             // entries of dY that exist (a multiple of 8)
-        if (ln == 0) mbar_expect_tx(full(s), ntr * ncol_tiles * 1024 * B + p.M * nrows * 2);
+        if (ln == 0) {
+            issued[s] = it;
+            mbar_expect_tx(full(s), ntr * ncol_tiles * 1024 * B + p.M * nrows * 2);
+        }
         if (ln < ntr)
             bulk_load(dst + ln * (4 * 1024 * B), codes + (static_cast<size_t>(tr0 + 2 * it + ln) * q.ktiles + kt_first) * (1024 * B),
                       ncol_tiles * 1024 * B, full(s));
@@ -792,10 +796,8 @@ decode_bwd_kernel(const BwdParams p) {
     if (*abort_s) {
         // a wait gave up: let copies that are still in flight land before the ring is reused (bounded)
         if (threadIdx.x == 0) {
-            for (int s = 0; s < NS; ++s) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(full(s), 0) && !mbar_try_wait(full(s), 1) && clock64() - t0 < 20000000LL) {}
-            }
+            for (int s = 0; s < NS; ++s)
+                if (issued[s] >= 0) let_land(full(s), (issued[s] / NS) & 1);
         }
         __syncthreads();
     }

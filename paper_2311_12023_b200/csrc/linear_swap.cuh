@@ -129,8 +129,8 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     const int stage_bytes = kSwWBytes + x_bytes;                         // [weight tile][token boxes]
     uint8_t* p_ring = base + p.ss * stage_bytes;
     uint8_t* tail = p_ring + p.sp * P_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);     // full[8], empty[8], full_p[8], empty_p[8], fbar[2], acc_full, drain
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 36 * 8);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);     // full[8], empty[8], full_p[8], empty_p[8], fbar[2], acc_full, drain, box_full[2][8]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 52 * 8);
     volatile int* abort_s = reinterpret_cast<volatile int*>(tmem_slot + 1);
     float* lut8 = reinterpret_cast<float*>(tail + kSwTail);
 
@@ -152,11 +152,14 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     auto empty_p = [&](int s) { return bar0 + 192 + 8 * s; };
     auto fbar = [&](int d) { return bar0 + 256 + 8 * d; };
     const uint32_t acc_full = bar0 + 272, drain = bar0 + 280;
+    auto box_full = [&](int b, int s) { return bar0 + 288 + 64 * b + 8 * s; };      // token box b has landed
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kSwMaxStages; ++s) {
-            // token boxes and four dequantization warps; leader: also the word of the second CTA that its step is complete
-            mbar_init(full(s), p.nbox + 4 + (rank == 0 ? 1 : 0));
+            // four dequantization warps; leader: also the word of the second CTA that its step is complete
+            mbar_init(full(s), 4 + (rank == 0 ? 1 : 0));
+            mbar_init(box_full(0, s), 1);
+            mbar_init(box_full(1, s), 1);
             mbar_init(empty(s), 1);
             mbar_init(full_p(s), 1);
             mbar_init(empty_p(s), 4);
@@ -178,6 +181,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool acc_ok = false;
+    int issued = 0;               // steps whose copies this warp has requested (warps 0..2)
 
     if (warp < p.nbox) {
         // ------------------------------------------------------------------ this CTA's half of token box `warp`
@@ -194,19 +198,14 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             }
             __syncwarp();
             if (elect_one()) {
-                mbar_expect_tx(full(r.s), half_bytes);
-                if (step < nq) tma_load_2d(dst0 + r.s * stage_bytes, &tmX, k, row, full(r.s));
-                else tma_load_2d(dst0 + r.s * stage_bytes, &tmT, (step - nq) * BK, row, full(r.s));
+                const uint32_t bar = box_full(warp, r.s);
+                mbar_expect_tx(bar, half_bytes);
+                if (step < nq) tma_load_2d(dst0 + r.s * stage_bytes, &tmX, k, row, bar);
+                else tma_load_2d(dst0 + r.s * stage_bytes, &tmT, (step - nq) * BK, row, bar);
             }
             __syncwarp();
+            issued = step + 1;
         }
-        if (*abort_s && warp == 0) {
-            for (int s = 0; s < p.ss; ++s) {          // let copies in flight land before the CTA exits (bounded)
-                const long long t0 = clock64();
-                while (!mbar_try_wait(full(s), 0) && !mbar_try_wait(full(s), 1) && clock64() - t0 < 20000000LL) {}
-            }
-        }
-        __syncwarp();
     } else if (warp == 2) {
         // ------------------------------------------------------------------ packed codes
         const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
@@ -230,14 +229,8 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                 }
             }
             __syncwarp();
+            issued = step + 1;
         }
-        if (*abort_s) {
-            for (int s = 0; s < p.sp; ++s) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(full_p(s), 0) && !mbar_try_wait(full_p(s), 1) && clock64() - t0 < 20000000LL) {}
-            }
-        }
-        __syncwarp();
     } else if (warp == 3) {
         // ------------------------------------------------------------------ MMA issuer (leader), messenger (second CTA)
         if (rank == 1) {
@@ -366,9 +359,15 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                             }
                         }
                         ok = wait(fbar(d), 0, ctl, 59);
-                        if (!ok) break;
+                        if (!ok) { let_land(fbar(d), 0); break; }
                     }
                     __syncwarp();
+                }
+                // The token boxes are on barriers of their own, which count copies alone (a kernel that gives up can wait for them); one of
+                // the four warps answers for each box.
+                if (wi < p.nbox) {
+                    ok = wait(box_full(wi, rw.s), rw.ph, ctl, 54);
+                    if (!ok) break;
                 }
                 if (lane == 0) mbar_arrive(full(rw.s));
                 rw.advance(4, p.ss);
@@ -434,6 +433,11 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     }
     tc_fence_before();
     __syncthreads();
+    if (*abort_s) {               // copies in flight land before the CTA exits
+        if (warp < p.nbox) drain_ring(box_full(warp, 0), issued, p.ss);
+        else if (warp == 2) drain_ring(full_p(0), issued, p.sp);
+        __syncwarp();
+    }
     cluster_barrier();            // tensor and shared memory are released only when no CTA of the cluster uses them any more
     if (warp == 3) tmem_dealloc2(tmem, p.tmem_cols);
 }

@@ -222,6 +222,7 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);      // full[8], empty[8], acc_full, drain
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 160);
     volatile int* abort_s = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    int* issued = reinterpret_cast<int*>(tmem_slot + 2);      // [kLrProducers] next step of each producer warp
 
     // The CTAs of a cluster write into each other's shared memory at the end; that is allowed once every CTA of the
     // cluster runs, which the first phase of the cluster barrier establishes: arrive here, wait before the first store.
@@ -260,7 +261,8 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
     if (warp < kLrProducers) {
         int s = warp;                    // stage and pass of step i; advanced without divisions (stages >= kLrProducers)
         uint32_t ph = 0;
-        for (int i = warp; i < total; i += kLrProducers) {
+        int i = warp;
+        for (; i < total; i += kLrProducers) {
             if (!wait(empty(s), ph ^ 1, ctl, 11)) break;
             const uint32_t a_dst = ring0 + s * stage_bytes, b_dst = a_dst + A_BYTES;
             const int c = (s_lo + i) * BK;
@@ -275,6 +277,7 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
             s += kLrProducers;
             if (s >= p.stages) { s -= p.stages; ph ^= 1u; }
         }
+        if (lane == 0) issued[warp] = i;
         __syncwarp();
     } else if (warp == kLrProducers) {
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 16) |
@@ -380,6 +383,15 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
     }
     tc_fence_before();
     __syncthreads();
+    if (*abort_s && warp == 0) {
+        // copies in flight land before the CTA exits: the last step issued into every stage (the producer warps are at most a
+        // ring apart, so it is among the last two rings of steps)
+        int top = 0;
+        for (int w = 0; w < kLrProducers; ++w) top = max(top, min(total, issued[w]));
+        for (int i = max(0, top - 2 * p.stages); i < top; ++i)
+            if (i < issued[i % kLrProducers] && (i + p.stages >= total || i + p.stages >= issued[(i + p.stages) % kLrProducers]))
+                let_land(full(i % p.stages), (i / p.stages) & 1);
+    }
     if (warp == kLrProducers) tmem_dealloc(tmem, tmem_cols);
 }
 

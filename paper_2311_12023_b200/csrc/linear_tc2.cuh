@@ -150,6 +150,8 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    int issued = 0;               // steps whose copies warp 0 has requested
+
     if (warp == 0) {
         // ------------------------------------------------------------------ producer: activations + packed codes of this CTA
         const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
@@ -195,14 +197,8 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                 }
             }
             __syncwarp();
+            issued = step + 1;
         }
-        if (*abort_s) {
-            for (int s = 0; s < SA; ++s) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(full_a(s), 0) && !mbar_try_wait(full_a(s), 1) && clock64() - t0 < 20000000LL) {}
-            }
-        }
-        __syncwarp();
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer (leader CTA), messenger (second CTA)
         if (rank == 1) {
@@ -363,8 +359,9 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
                                     tma_load_2d(dst + t * 8192, &tmB2, c0 + static_cast<int>(rank) * 128 + t * 64, d * BK, dbar(sb));
                             }
                         }
-                        ok = wait(dbar(sb), ((step - p.steps_q) / SB) & 1, ctl, 47) && wait(full_a(sa), ra.ph, ctl, 48);
-                        if (!ok) break;
+                        const uint32_t dpar = ((step - p.steps_q) / SB) & 1;
+                        ok = wait(dbar(sb), dpar, ctl, 47) && wait(full_a(sa), ra.ph, ctl, 48);
+                        if (!ok) { let_land(dbar(sb), dpar); break; }
                     }
                 }
                 __syncwarp();
@@ -419,6 +416,8 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
     }
     tc_fence_before();
     __syncthreads();
+    if (*abort_s && warp == 0) drain_ring(full_a(0), issued, SA);      // copies in flight land before the CTA exits
+    __syncwarp();
     cluster_barrier();            // neither CTA frees tensor memory or exits while the other may still use its shared memory
     if (warp == 1) tmem_dealloc2(tmem, TMEM_COLS);
 }

@@ -73,6 +73,7 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool acc_ok = false;
+    int issued = 0;              // steps whose copies this warp has requested (warp 0)
 
     if (warp == 0) {
         // The kernel that writes T may still be running (programmatic dependent launch): the tiles of A of the
@@ -99,6 +100,7 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
         }
         int s = 0;                        // stage and pass of step i, advanced without divisions
         uint32_t ph = 1;
+        issued = first;
         for (int i = first; i < total; ++i) {
             if (!wait(empty(s), ph ^ 1, ctl, 61)) break;
             const uint32_t a_dst = ring0 + s * stage_bytes, b_dst = a_dst + A_BYTES;
@@ -110,16 +112,9 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
                 for (int t = 0; t < p.rp / 64; ++t) tma_load_2d(b_dst + t * 8192, &tmT, t * 64, m, full(s));
             }
             __syncwarp();
+            issued = i + 1;
             if (++s == p.stages) { s = 0; ph ^= 1u; }
         }
-        if (*abort_s) {
-            // let copies that are still in flight land before the CTA exits (bounded)
-            for (int s = 0; s < p.stages; ++s) {
-                const long long t0 = clock64();
-                while (!mbar_try_wait(full(s), 0) && !mbar_try_wait(full(s), 1) && clock64() - t0 < 20000000LL) {}
-            }
-        }
-        __syncwarp();
     } else if (warp == 1) {
         // fp32 accumulators, bf16 operands, both MN-major (bits 15 and 16), N = rp, M = 128
         const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
@@ -201,6 +196,7 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
     }
     tc_fence_before();
     __syncthreads();
+    if (*abort_s && warp == 0) drain_ring(full(0), issued, p.stages);      // copies in flight land before the CTA exits
     if (warp == 1) tmem_dealloc(tmem, tmem_cols);
 }
 

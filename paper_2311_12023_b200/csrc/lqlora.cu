@@ -146,15 +146,20 @@ static int static_scratch_ptr(void** out) {
 // budget runs out the wait is abandoned, the status word is set, tensor memory is freed and the kernel returns.
 // Then a wait whose lanes cannot agree by themselves: lane 0 has a short budget and the others a long one, and the barrier is
 // completed as soon as lane 0 has given up.  Word 32 + lane receives 1 where the lane's verdict was "abandoned".
+// Then the wait for copies in flight on the way out: a ring of two stages with three steps issued, of which the last one (the second
+// phase of stage 0) completes late.  Word 1 receives 1 where the drain returned after that.
 __global__ void __launch_bounds__(96) bounded_wait_selftest_kernel(int* status, long long budget) {
-    __shared__ uint64_t bars[2];
+    __shared__ uint64_t bars[4];
     __shared__ uint32_t tmem_slot;
-    __shared__ int abort_s, abort2_s;
+    __shared__ int abort_s, abort2_s, landed_s;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint32_t never = dev::smem_u32(bars), late = dev::smem_u32(bars + 1);
+    const uint32_t never = dev::smem_u32(bars), late = dev::smem_u32(bars + 1), ring = dev::smem_u32(bars + 2);
     if (threadIdx.x == 0) {
         dev::mbar_init(never, 1);
         dev::mbar_init(late, 1);
+        dev::mbar_init(ring, 1);
+        dev::mbar_init(ring + 8, 1);
+        landed_s = 0;
         abort_s = 0;
         abort2_s = 0;
         dev::fence_barrier_init();
@@ -176,6 +181,18 @@ __global__ void __launch_bounds__(96) bounded_wait_selftest_kernel(int* status, 
         const long long t0 = clock64();
         while (!*const_cast<volatile int*>(&abort2_s) && clock64() - t0 < 2 * budget + 100 * kShort) {}
         dev::mbar_arrive(late);
+        dev::mbar_arrive(ring);                  // steps 0 and 1 have landed
+        dev::mbar_arrive(ring + 8);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        dev::drain_ring(ring, 3, 2);
+        if (lane == 0) status[1] = *const_cast<volatile int*>(&landed_s);
+    } else if (warp == 2 && lane == 0) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < kShort) {}
+        *const_cast<volatile int*>(&landed_s) = 1;
+        dev::mbar_arrive(ring);                  // step 2
     }
     tc::tc_fence_before();
     __syncthreads();

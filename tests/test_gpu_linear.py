@@ -335,3 +335,13 @@ def test_the_lanes_of_a_warp_agree_on_a_wait_that_runs_out():
         binding.selftest_bounded_wait(ws, 100_000)
         assert binding.workspace_status(ws) == -7
         assert ws.view(torch.int32)[32:].tolist() == [1] * 32
+
+
+def test_the_wait_for_copies_in_flight_waits_for_the_step_issued_last():
+    """On the way out of a kernel that gave up: a ring whose last step lands late (its stage has landed before, so the other
+    parity of its barrier reads as complete all along)."""
+    ws = torch.zeros(256, dtype=torch.uint8, device="cuda")
+    for _ in range(3):
+        binding.selftest_bounded_wait(ws, 100_000)
+        torch.cuda.synchronize()
+        assert ws.view(torch.int32)[1].item() == 1

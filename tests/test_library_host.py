@@ -186,3 +186,13 @@ def test_every_number_of_rows_has_a_plan_on_the_tensor_core_kernels(binding, b0)
             for r, backward in ((64, False), (0, False), (128, True)):
                 kernel, splits = binding.linear_route(N, K, cfg, r, M, backward)
                 assert kernel in (binding.PATH_TC_ONE, binding.PATH_TC_PAIR) and 1 <= splits <= 4, (N, K, M, r, backward)
+
+
+def test_no_kernel_polls_a_barrier_for_both_parities():
+    """try_wait.parity succeeds for the parity of the phase before the current one, so "neither parity" is never true and a loop
+    on it waits for nothing: copies in flight are awaited by the phase they were issued in (let_land, drain_ring)."""
+    import glob
+    import re
+    for f in glob.glob(os.path.join(ROOT, "paper_2311_12023_b200", "csrc", "*")):
+        for args in re.findall(r"!mbar_try_wait\((.*?), 0\) && !mbar_try_wait\(.*?, 1\)", open(f).read()):
+            raise AssertionError(f"{os.path.basename(f)}: {args}")
