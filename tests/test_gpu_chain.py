@@ -1,0 +1,131 @@
+"""Calls enqueued one behind the other without a synchronisation: the first kernel of a call starts while the last one of the call
+before it ends, so each has to wait before it reads what that one writes (the result, the workspace) or overwrites it."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2311_12023_b200 import binding, inputs
+from test_gpu_linear import C
+
+pytestmark = pytest.mark.gpu
+
+M, R = 2100, 64
+
+
+class Layer:
+    def __init__(self, seed, N, K, cfg, r=R):
+        self.q = binding.encode(torch.from_numpy(inputs.gaussian(seed, (N, K), 0.04)).cuda(), cfg)
+        self.r = r
+        self.L1 = self.L2 = None
+        if r:
+            l1b, l2b = inputs.lowrank_factors(seed + 1, N, K, r, 0.02)
+            self.L1, self.L2 = binding.bf16_from_bits(l1b), binding.bf16_from_bits(l2b)
+
+    def path(self, rows, backward):
+        return binding.linear_path(self.q.N, self.q.K, self.q.cfg, self.r, rows, backward)
+
+
+class Chain:
+    """The calls of one run, in order; every result goes into a buffer that a later call reads."""
+
+    def __init__(self):
+        wide, narrow = Layer(9000, 2560, 512, C(3, 64, 8, 256, 32)), Layer(9010, 512, 2560, C(4, 32, 8, 64, 32))
+        square, plain = Layer(9020, 512, 512, C(2, 64, 8, 64, 32)), Layer(9030, 512, 512, C(8, 64, 8, 64, 32), r=0)
+        packed = Layer(9040, 512, 512, C(3, 64, 4, 64, 16))
+        nf8 = C(8, 64, 8, 256, 32)
+        f1, f2 = (binding.encode(x.float().contiguous(), nf8) for x in (square.L1, square.L2))
+        S, ONE, PAIR = binding.PATH_STREAM, binding.PATH_TC_ONE, binding.PATH_TC_PAIR
+        assert wide.path(M, False) == PAIR and narrow.path(M, False) == ONE and square.path(8, False) == S
+        assert square.path(100, True) == ONE and narrow.path(M, True) == PAIR and wide.path(M, True) == ONE
+
+        def bf(rows, cols):
+            return torch.empty(rows, cols, dtype=torch.bfloat16, device="cuda")
+
+        self.src = binding.bf16_from_bits(inputs.activations(9100, M, 512))
+        X, Y1, Y2, Y3, dY1, dX1 = bf(M, 512), bf(M, 2560), bf(M, 512), bf(M, 512), bf(M, 2560), bf(M, 512)
+        s = [bf(100, 512) for _ in range(10)]
+        g = [torch.empty(*shape, dtype=torch.float32, device="cuda") for shape in ((2560, R), (R, 512), (512, R), (R, 2560))]
+        need = max(binding.linear_workspace_bytes(l.q.N, l.q.K, l.q.cfg, l.r, rows) for l in (wide, narrow, square, plain, packed)
+                   for rows in (8, 100, M))
+        need = max(need, binding.lora_grads_workspace_bytes(2560, 512, R, M))
+        ws = torch.empty(need, dtype=torch.uint8, device="cuda")               # one workspace for every call
+        ws_f, ws_b = torch.empty_like(ws), torch.empty_like(ws)                # ... but for the two whose intermediates are used
+        self.X = X
+        self.poisoned = [Y1, Y2, Y3, dY1, dX1] + s + g
+        self.results = self.poisoned
+
+        def fwd(l, x, out, w=ws):
+            return lambda: binding.linear_fwd(l.q, l.L1, l.L2, x, out=out, workspace=w)
+
+        def bwd(l, dy, out, w=ws):
+            return lambda: binding.linear_bwd_input(l.q, l.L1, l.L2, dy, out=out, workspace=w)
+
+        def qfactors(x, out, backward):
+            return lambda: out.copy_(binding.linear_qfactors(square.q, f1, f2, x, backward=backward))
+
+        def grads_from():
+            T = binding.linear_intermediate(ws_f, 512, 2560, narrow.q.cfg, R, M, False)
+            Tp = binding.linear_intermediate(ws_b, 512, 2560, narrow.q.cfg, R, M, True)
+            binding.lora_grads_from(T, Tp, 512, 2560, Y1, Y3, out=(g[2], g[3]), workspace=ws[:256])
+
+        self.calls = [
+            fwd(wide, X, Y1),                                        # pair kernel
+            fwd(narrow, Y1, Y2),                                     # transposed tiles, reads what the pair kernel wrote
+            fwd(square, Y2[:8], s[0][:8]),                           # weight streaming
+            bwd(square, s[0][:8], s[1][:8]),
+            fwd(plain, s[1][:8], s[2][:8]),                          # no rank-r term: no pre-product in front
+            fwd(packed, s[2][:8], s[3][:8]),                         # scales expanded inside the call
+            qfactors(s[3][:8], s[4][:8], False),                     # factors dequantized inside the call
+            fwd(square, Y2[:100], s[5]),                             # transposed tiles, few rows
+            bwd(square, s[5], s[6]),
+            fwd(packed, s[6], s[7]),
+            qfactors(s[7], s[8], True),
+            bwd(plain, s[8], s[9]),
+            bwd(narrow, Y2, dY1),                                    # pair kernel
+            bwd(wide, dY1, dX1),
+            lambda: binding.lora_grads(wide.L1, wide.L2, X, dY1, out=(g[0], g[1]), workspace=ws),
+            bwd(narrow, dX1, dY1, ws_b),                             # T', T of the gradients below stay in their workspaces
+            fwd(narrow, Y1, Y3, ws_f),                               # writes the dY that the next call reads
+            grads_from,
+            fwd(square, Y3[:8], s[0][8:16]),                         # streaming behind the weight gradients
+            fwd(square, s[0][8:16], X[:8]),                          # and into the first call's input
+            fwd(wide, X, Y1),
+        ]
+
+    def run(self, synchronize=False):
+        self.X.copy_(self.src)
+        for t in self.poisoned:
+            t.fill_(float("nan"))
+        for call in self.calls:
+            call()
+            if synchronize:
+                torch.cuda.synchronize()
+
+    def take(self):
+        torch.cuda.synchronize()
+        return [t.clone() for t in self.results]
+
+
+def same_bits(a, b):
+    return torch.equal(a.view(torch.int16), b.view(torch.int16))
+
+
+def test_chained_calls_give_the_bits_of_synchronised_ones():
+    chain = Chain()
+    chain.run(synchronize=True)
+    want = chain.take()
+    written = [0, 1, 2, 3, 4] + list(range(5, 19))
+    assert all(bool(torch.isfinite(want[i][:8].float()).all()) for i in written)
+    for _ in range(20):
+        chain.run()
+        got = chain.take()
+        assert [i for i in written if not same_bits(want[i], got[i])] == []
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain.run()
+    for _ in range(10):
+        for t in chain.poisoned:
+            t.fill_(float("nan"))
+        graph.replay()
+        got = chain.take()
+        assert [i for i in written if not same_bits(want[i], got[i])] == []
