@@ -129,9 +129,10 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     const int stage_bytes = kSwWBytes + x_bytes;                         // [weight tile][token boxes]
     uint8_t* p_ring = base + p.ss * stage_bytes;
     uint8_t* tail = p_ring + p.sp * P_BYTES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);     // full[8], empty[8], full_p[8], empty_p[8], fbar[2], acc_full, drain, box_full[2][8]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 52 * 8);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);     // full[8], empty[8], full_p[8], empty_p[8], fbar[2], acc_full, drain
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 36 * 8);
     volatile int* abort_s = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    int* reached = reinterpret_cast<int*>(tmem_slot + 2);    // [20] per warp: the first step that it has not (issued or) arrived at
     float* lut8 = reinterpret_cast<float*>(tail + kSwTail);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -152,14 +153,11 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     auto empty_p = [&](int s) { return bar0 + 192 + 8 * s; };
     auto fbar = [&](int d) { return bar0 + 256 + 8 * d; };
     const uint32_t acc_full = bar0 + 272, drain = bar0 + 280;
-    auto box_full = [&](int b, int s) { return bar0 + 288 + 64 * b + 8 * s; };      // token box b has landed
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kSwMaxStages; ++s) {
-            // four dequantization warps; leader: also the word of the second CTA that its step is complete
-            mbar_init(full(s), 4 + (rank == 0 ? 1 : 0));
-            mbar_init(box_full(0, s), 1);
-            mbar_init(box_full(1, s), 1);
+            // token boxes and four dequantization warps; leader: also the word of the second CTA that its step is complete
+            mbar_init(full(s), p.nbox + 4 + (rank == 0 ? 1 : 0));
             mbar_init(empty(s), 1);
             mbar_init(full_p(s), 1);
             mbar_init(empty_p(s), 4);
@@ -181,7 +179,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool acc_ok = false;
-    int issued = 0;               // steps whose copies this warp has requested (warps 0..2)
+    int issued = 0;               // steps whose codes have been requested (warp 2)
 
     if (warp < p.nbox) {
         // ------------------------------------------------------------------ this CTA's half of token box `warp`
@@ -189,7 +187,8 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         const int row = m0 + warp * p.box + static_cast<int>(rank) * half_box;
         uint32_t dst0 = ring + kSwWBytes + warp * half_bytes;
         int k = q_lo * BK;
-        for (int step = 0; step < total; ++step, r.advance(1, p.ss), k += BK) {
+        int step = 0;
+        for (; step < total; ++step, r.advance(1, p.ss), k += BK) {
             if (!wait(empty(r.s), r.ph ^ 1, ctl, 51)) break;
             if (step == nq) {
                 // the rank-r intermediate comes from the kernel in front (programmatic dependent launch)
@@ -198,14 +197,13 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             }
             __syncwarp();
             if (elect_one()) {
-                const uint32_t bar = box_full(warp, r.s);
-                mbar_expect_tx(bar, half_bytes);
-                if (step < nq) tma_load_2d(dst0 + r.s * stage_bytes, &tmX, k, row, bar);
-                else tma_load_2d(dst0 + r.s * stage_bytes, &tmT, (step - nq) * BK, row, bar);
+                mbar_expect_tx(full(r.s), half_bytes);
+                if (step < nq) tma_load_2d(dst0 + r.s * stage_bytes, &tmX, k, row, full(r.s));
+                else tma_load_2d(dst0 + r.s * stage_bytes, &tmT, (step - nq) * BK, row, full(r.s));
             }
             __syncwarp();
-            issued = step + 1;
         }
+        if (lane == 0) reached[warp] = step;
     } else if (warp == 2) {
         // ------------------------------------------------------------------ packed codes
         const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
@@ -236,11 +234,13 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         if (rank == 1) {
             // tells the leader that this CTA's half of a step is complete
             RingAt r(0, p.ss);
-            for (int step = 0; step < total; ++step, r.advance(1, p.ss)) {
+            int step = 0;
+            for (; step < total; ++step, r.advance(1, p.ss)) {
                 if (!wait(full(r.s), r.ph, ctl, 60)) break;
                 __syncwarp();
                 if (elect_one()) mbar_arrive_cluster(full(r.s), cluster_rank() & ~1u);
             }
+            if (lane == 0) dec::st_dsmem_f32(smem_u32(reached + 3), cluster_rank() & ~1u, __int_as_float(step));     // to the leader
         } else {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 15) |
                                    (static_cast<uint32_t>(p.box >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
@@ -314,6 +314,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         slot[1] = (grp + 4 < nq) ? fetch(q_lo + grp + 4) : RawScale{0u, 0.0f};
         RingAt rw(grp, p.ss), rp(grp, p.sp);
         bool ok = true;
+        int next = grp;
         for (int step8 = grp; step8 < total && ok; step8 += 8) {
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
@@ -363,16 +364,12 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     }
                     __syncwarp();
                 }
-                // The token boxes are on barriers of their own, which count copies alone (a kernel that gives up can wait for them); one of
-                // the four warps answers for each box.
-                if (wi < p.nbox) {
-                    ok = wait(box_full(wi, rw.s), rw.ph, ctl, 54);
-                    if (!ok) break;
-                }
                 if (lane == 0) mbar_arrive(full(rw.s));
+                next = step + 4;
                 rw.advance(4, p.ss);
             }
         }
+        if (lane == 0) reached[warp] = next;
         // ------------------------------------------------------------------ epilogue: warp = 32 output columns x every fourth chunk of 32 tokens
         pdl_launch_dependents();      // the next call's pre-product may take its place on the SMs (it waits for this kernel)
         acc_ok = ok && wait(acc_full, 0, ctl, 58);
@@ -433,12 +430,24 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     }
     tc_fence_before();
     __syncthreads();
-    if (*abort_s) {               // copies in flight land before the CTA exits
-        if (warp < p.nbox) drain_ring(box_full(warp, 0), issued, p.ss);
-        else if (warp == 2) drain_ring(full_p(0), issued, p.sp);
-        __syncwarp();
-    }
     cluster_barrier();            // tensor and shared memory are released only when no CTA of the cluster uses them any more
+    if (*abort_s) {
+        // copies in flight land before the CTA exits.  The barrier of a step counts its token boxes, the warps of its weights and
+        // the second CTA's word: those that have not come will not (everybody has left the loops), so they are made up for here, and
+        // the phase then waits for the boxes alone.  A box of step j is issued behind the end of step j - ss, so the last ss steps
+        // that any box was issued for are the ones that can be open, each in the phase j / ss of its stage.
+        if (warp == 0) {
+            const int top = p.nbox == 2 ? max(reached[0], reached[1]) : reached[0];
+            for (int j = max(0, top - p.ss); j < top; ++j) {
+                int missing = (j >= reached[0] ? 1 : 0) + (p.nbox == 2 && j >= reached[1] ? 1 : 0) + (rank == 0 && j >= reached[3] ? 1 : 0);
+                for (int w = 0; w < 4; ++w) missing += (j >= reached[kSwFirstDeq + 4 * (j & 3) + w] ? 1 : 0);
+                if (lane < missing) mbar_arrive(full(j % p.ss));
+                let_land(full(j % p.ss), (j / p.ss) & 1);
+            }
+        } else if (warp == 2) {
+            drain_ring(full_p(0), issued, p.sp);
+        }
+    }
     if (warp == 3) tmem_dealloc2(tmem, p.tmem_cols);
 }
 
