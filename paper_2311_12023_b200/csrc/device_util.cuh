@@ -88,6 +88,14 @@ __device__ __forceinline__ bool wait(uint32_t bar, uint32_t parity, const Ctl& c
     return __all_sync(0xffffffffu, ok);
 }
 
+// wait() for two barriers, the second one asked after the first (its phase may be unambiguous only then), with one vote where
+// both are complete.
+__device__ __forceinline__ bool wait2(uint32_t bar, uint32_t parity, uint32_t bar2, uint32_t parity2, const Ctl& c, int where, int where2) {
+    const uint32_t a = mbar_try_wait(bar, parity), b = mbar_try_wait(bar2, parity2);
+    if (__all_sync(0xffffffffu, (a & b) != 0u)) return true;
+    return wait(bar, parity, c, where) && wait(bar2, parity2, c, where2);
+}
+
 // On the way out of a kernel that gave up: copies in flight have to land before the CTA exits.  A barrier tells only the parity
 // of its phase (of the two parities one always reads as complete), so the caller names the phase of the copies that it
 // knows to have been issued.  Waits about ten milliseconds at most.

@@ -336,7 +336,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     }
                     const int kt = BWD ? (my_col >> 6) : q_lo + step;
                     const uint32_t src = wsrc + rp.s * P_BYTES;
-                    ok = wait(empty(rw.s), rw.ph ^ 1, ctl, 55) && wait(full_p(rp.s), rp.ph, ctl, 56);
+                    ok = wait2(empty(rw.s), rw.ph ^ 1, full_p(rp.s), rp.ph, ctl, 55, 56);
                     if (!ok) break;
                     dequant_row64<B>(src + slab_row_slot(lane, 0, kt) * 4, src + (B * 32 + slab_row_slot(lane, 1, kt)) * 4, s, nsc,
                                      dst0 + stage, xr, lut8 + lane);
