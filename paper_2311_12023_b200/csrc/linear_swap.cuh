@@ -555,7 +555,10 @@ inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q,
             const double step = dq > tokens * 0.0012 ? dq : tokens * 0.0012;
             const double body = 6.5 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 2.5 + tokens * 0.008 : tokens * 0.006);
             pl.us = waves * body;
-            if (ks == 1 && steps_q > 16) pl.us *= 1.2;      // (long contractions: slices spread better than the model says)
+            // A single slice of a long contraction is made 20 % dearer than the model has it.  Both sides (us as a graph, with / without):
+            // 8192 x 8192 at 384 rows 45 / 48 (NF2), 45 / 50 (NF3); but 8192 x 28672 NF3 at 512 rows 198 / 168, 5120 x 5120 NF4 at 512 rows
+            // 49 / 40, 2048 x 2048 NF3 at 1024 rows 20 / 18: right for chunks of fewer than 512 tokens only.
+            if (ks == 1 && steps_q > 16) pl.us *= 1.2;
             if (best.us < 0 || pl.us < best.us) best = pl;
         }
     }

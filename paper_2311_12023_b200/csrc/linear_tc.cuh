@@ -471,8 +471,11 @@ inline bool make_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t 
 namespace lq {
 namespace tc {
 
-// CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs; below that the one-CTA
-// kernel with its split of the contraction puts at least twice as many SMs to work.
+// CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs.  The line was drawn against a kernel with the
+// tokens as rows of its tiles; the transposed tiles that took that kernel's place pad to 16 rows instead of 512 and hold out
+// longer (us as a graph, pair / transposed): 8192 x 8192 NF3 at 512 rows 84 / 54 (transposed by this rule), 600 87 / 61, 800
+// 90 / 77, 1024 93 / 93, 1100 172 / 138, 1536 174 / 144; input gradient 4096 x 4096 NF4 at 1024 rows 49 / 36 (transposed),
+// 1100 50 / 40, 1536 50 / 44, 2048 53 / 56; 28672 x 8192 NF3, blocks of 16, at 300 rows 172 / 122, 600 301 / 263.
 inline bool tc_use_pair(int64_t M, int64_t out_cols, int sms) {
     if (M <= 256) return false;
     const long long pair_ctas = 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN);
@@ -497,10 +500,12 @@ inline int sm_count() {
 }
 
 // Wave quantisation of the pair kernel: its tiles run in waves of sms / 2 clusters.  When the last wave would hold only a few
-// tiles (at most a quarter of a wave), the output columns it would cover are peeled off and computed by the
-// one-CTA kernel with the contraction split over clusters, which spreads that small remainder over many SMs
-// (28672 x 8192 at 2048 rows: 448 pair tiles = 6 waves + 4 tiles, 817 -> 740 us).  Larger remainders stay with
-// the pairs: the one-CTA kernel needs about 1.6 pair-tile times for three quarters of a wave (measured).
+// tiles (at most a quarter of a wave), the output columns it would cover are peeled off and computed on
+// transposed tiles with the contraction split over clusters, which spreads that small remainder over many SMs (us as a graph,
+// all on pairs / peeled: 28672 x 8192 NF3 at 2048 rows, 6 waves + 4 tiles, 674 / 637; 4096 x 4096 NF3 at 2560 rows, 1 wave + 6,
+// 95 / 91).  Remainders of three quarters of a wave stay with the pairs (8192 x 8192 at 2048 rows, 1 wave + 54: NF3 186 / 209, 8-bit
+// codes 236 / 368; 4096 x 11008 NF4 at 4096 rows, the same: 266 / 297).  In between the line predates the transposed tiles: remainders of
+// 22 and 34 of 74 would gain (8192 x 8192 at 1536 rows 176 / 162, 6912 x 8192 at 2048 rows 176 / 167).
 // Returns the number of 256-column tiles to peel off.
 inline int pair_peel(int64_t M, int64_t out_cols) {
     const int mt = static_cast<int>((M + 511) / 512), pairs = sm_count() / 2, c_tiles = static_cast<int>((out_cols + BN - 1) / BN);
@@ -599,8 +604,11 @@ constexpr int kTcMinRowsBwd = 9;  // input gradient of matrices with at least 20
 
 inline bool tc_supported(const QView& q, int r, int64_t M, bool backward) {
     (void)r;
-    // The input gradient of 9..16 rows is faster here than in the weight-streaming kernel (which then runs one CTA of
-    // eight warps per SM) unless the matrix has few rows: 8192 x 8192 at 16 rows 49 -> 41 us, 8192 x 28672 162 -> 100 us.
+    // Both lines were drawn against a kernel with the tokens as rows of its tiles, which the transposed tiles replaced; these would win
+    // earlier (us as a graph, streaming / transposed, 2-, 3-, 4- and 8-bit codes of 8192 x 8192): forward 1 row 20 / 25, 22 / 26,
+    // 30 / 32, 44 / 45; 8 rows 26 / 25, 28 / 26, 35 / 32, 50 / 46; 16 rows 34 / 25, 35 / 26, 43 / 32, 62 / 46; input gradient 1 row 27 / 26,
+    // 29 / 27, 40 / 33, 60 / 46; 8 rows 33 / 26, 36 / 27, 46 / 33, 62 / 46.  One row of a larger matrix stays with the streaming kernel:
+    // 28672 x 8192 NF3 forward 70 / 91 (16 rows 104 / 91), 8192 x 28672 NF2 63 / 68 and 81 / 85 (input gradient).
     const int min_rows = (backward && q.N >= 2048) ? kTcMinRowsBwd : kTcMinRows;
     if (M < min_rows) return false;
     if (q.N % 8 != 0 || q.K % 8 != 0) return false;

@@ -4,14 +4,13 @@
 // 2 x 128 rows of the activations (two accumulators of 128 lanes x 256 fp32 columns in its tensor memory)
 // and HALF of the weight tile of a step (128 of the 256 output columns).  One thread of the leader CTA issues
 // tcgen05.mma with M = 256: the tensor cores of both CTAs read the two halves of the weight tile from both
-// shared memories.  Compared with the single-CTA kernel each CTA dequantizes half as many weights per MMA
-// flop and its shared memory serves half of the weight-operand traffic.
+// shared memories, so a CTA dequantizes half of the weights that it multiplies with.
 //
 // Per CTA: warp 0 loads activations (TMA) and packed codes (bulk copies) into a ring; sixteen
 // dequantization warps, eight per step (even / odd steps), write the CTA's half of the weight tile into a
-// second ring; a warp of the second CTA passes the word that its half is complete on to the leader, whose MMA warp issues the MMAs and commits the ring stages back to both
-// CTAs (multicast commit).  Forward and input gradient share the code (K-major / MN-major weight operand)
-// as in the single-CTA kernel; the rank-r term is one more step whose operands come by TMA; the output
+// second ring; a warp of the second CTA passes the word that its half is complete on to the leader, whose MMA warp issues the
+// MMAs and commits the ring stages back to both CTAs (multicast commit).  Forward and input gradient share the code (K-major /
+// MN-major weight operand); the rank-r term is one more step whose operands come by TMA; the output
 // leaves through shared memory and TMA stores.
 // Every wait is bounded; both CTAs meet at a cluster barrier before tensor memory is freed.
 #pragma once
@@ -48,8 +47,10 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 // Arrive on the barrier at local address `bar` of CTA `rank` of the cluster.  Sent by the second CTA's messenger warp after
 // it has waited for this CTA's own barrier of the step: the weights are then in this SM's shared memory and visible to the
-// async proxy (every writer has passed fence.proxy.async before it arrived there), and the copies have landed, so nothing is left
-// for a release at cluster scope to order; the tensor core of this SM reads them from this SM's memory.  Spelled with
+// async proxy (every writer has passed fence.proxy.async before it arrived there), and the copies have landed; the tensor core of
+// this SM reads them from this SM's memory, so nothing is left for a release at cluster scope to order.  That is the ground this
+// rests on: without a scope the arrive is a release at CTA scope, and the PTX memory model does not order the weights for the thread of
+// the other CTA that issues the MMA.  (CUTLASS signals the leader of a CTA pair with the same instruction.)  Spelled with
 // .release.cluster the arrive takes about 1500 clocks, more than a whole step (8192 x 8192, 128 rows: 60 us against 28).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t rank) {
     uint32_t ra;

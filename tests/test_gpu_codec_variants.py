@@ -58,7 +58,7 @@ def test_codec_variant_ragged_block_count():
 @pytest.mark.parametrize("cfg", [C(3, 64, 4, 256, BF16), C(4, 32, 3, 64, FP16), C(2, 16, 2, 16, FP32)])
 @pytest.mark.parametrize("M", [3, 16, 100, 600])
 def test_linear_with_variant_scales(cfg, M):
-    """Every kernel family (weight-streaming, one-CTA and CTA-pair tcgen05) reads the expanded scales."""
+    """Every kernel family (weight-streaming, transposed-tile and CTA-pair tcgen05) reads the expanded scales."""
     N, K = 1152, 1536
     A = inputs.gaussian(500 + cfg.b1, (N, K), 0.02)
     l1b, l2b = inputs.lowrank_factors(501, N, K, 64, 0.01)

@@ -90,8 +90,8 @@ def test_linear_single_row_with_odd_feature_count_uses_the_fallback():
 @pytest.mark.parametrize("N,K,M", [(640, 1088, 1000), (328, 704, 513), (896, 320, 700)])
 @pytest.mark.parametrize("b0,B0", [(3, 64), (4, 32)])
 def test_linear_many_rows_few_tiles(N, K, M, b0, B0):
-    """More than 256 rows on matrices whose CTA-pair tiles would fill few SMs: the one-CTA kernel with several row
-    tiles (grid.x > 1), split contraction, M, N, K not multiples of the tile."""
+    """More than 256 rows on matrices whose CTA-pair tiles would fill few SMs: the transposed-tile kernel with several
+    chunks of tokens, split contraction, M, N, K not multiples of the tile."""
     A = inputs.gaussian(600 + N, (N, K), 0.02)
     l1b, l2b = inputs.lowrank_factors(601 + K, N, K, 64, 0.01)
     kernel, splits = binding.linear_route(N, K, C(b0, B0, 8, 64, 32), 64, M, False)
@@ -116,7 +116,7 @@ def test_linear_pair_kernel_ragged_tiles(N, K, M, b0, B0):
 @pytest.mark.parametrize("b0,B0,r", [(3, 64, 64), (8, 32, 0)])
 def test_linear_pair_kernel_with_peeled_last_wave(b0, B0, r):
     """80 pair tiles on 74 CTA pairs: the six tiles of the second wave are peeled off as two output column tiles and run
-    on the one-CTA kernel (forward: N = 4096 at 2560 rows; the input gradient of the transposed shape likewise)."""
+    on transposed tiles (forward: N = 4096 at 2560 rows; the input gradient of the transposed shape likewise)."""
     M = 2560
     for N, K in ((4096, 512), (512, 4096)):
         A = inputs.gaussian(670 + N, (N, K), 0.02)
@@ -241,7 +241,7 @@ def test_config4_remaining_matrices(name):
 
 @pytest.mark.parametrize("b0,B0", [(2, 16), (3, 64), (4, 128), (8, 16), (8, 256)])
 def test_config5_sweep_points(b0, B0):
-    """Points of the 8192 x 8192 sweep at every M of the sweep (decode kernels, one-CTA and CTA-pair tensor-core
+    """Points of the 8192 x 8192 sweep at every M of the sweep (decode kernels, transposed-tile and CTA-pair tensor-core
     kernels; 8192 rows = 16 x 32 pair tiles), whole-height bit-exact codec parity included (encode_both)."""
     A = inputs.gaussian(5000, (8192, 8192), 0.02)
     l1b, l2b = inputs.lowrank_factors(5700, 8192, 8192, 64, 0.01)

@@ -48,7 +48,7 @@ def test_lora_grads_training_shape_and_repeatability():
                                            (384, 640, 1000, 128, 3, 32)])
 def test_lora_grads_from_the_intermediates_of_the_other_passes(N, K, M, r, b0, B0):
     """The layer's three passes on the same X and dY: forward, input gradient, then lqlora_lora_grads_from with the
-    intermediates T, T' the first two left in their workspaces (CTA-pair kernel, one-CTA kernel, weight-streaming
+    intermediates T, T' the first two left in their workspaces (CTA-pair kernel, transposed-tile kernel, weight-streaming
     kernel, rank padded to 128).  Same tolerance against the fp64 oracle as lqlora_lora_grads."""
     from gpu_util import encode_both
     cfg = inputs.QuantConfig(b0, B0, 8, 64, 32)
