@@ -11,10 +11,10 @@ configurations averaging about 2.73 bits per parameter; rank 64):
 
 `value` is the algorithmic TFLOP/s of the whole step: 2 M (N K + r K + N r) flop per linear call, summed
 over the 28 calls, divided by the device time of the step (CUDA events).  The JSON line also carries the
-roofline of the dominant kernel (the CTA-pair tcgen05 kernel on the 28672x8192 gate projection), per-call
-figures of the step, the other seeded workloads (RoBERTa projection, LLaMA-2-7B attention projection and MLP
-block, points of the 8192x8192 sweep) measured beside it, the end-to-end number through the host-buffer
-C ABI, and the CPU oracle timed on the host as a baseline.
+roofline of the dominant kernel (the CTA-pair tcgen05 kernel on the 28672x8192 gate projection), the times of the
+five phases of the step, the end-to-end number through the host-buffer C ABI, and the CPU oracle timed on the
+host as a baseline.  Per-call figures of the step and the other seeded workloads (RoBERTa projection, LLaMA-2-7B
+attention projection and MLP block, points of the 8192x8192 sweep), measured beside it, go to the file of --breakdown.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
     python bench.py --sweep                      # the whole b0 x B0 x M table of the 8192x8192 sweep
@@ -185,6 +185,16 @@ def run_reference(args):
         "gpu_launches": 0,
     }
     print(json.dumps(line), flush=True)
+
+
+def short(x):
+    """The same with floats at six digits: the line has to fit where only the last few thousand characters of the output are
+    kept (the per-call figures go to a file of their own)."""
+    if isinstance(x, float):
+        return float(f"{x:.6g}")
+    if isinstance(x, dict):
+        return {k: short(v) for k, v in x.items()}
+    return [short(v) for v in x] if isinstance(x, (list, tuple)) else x
 
 
 # ------------------------------------------------------------------------------------- ranks
@@ -541,12 +551,10 @@ def run_device(args):
     sustained = pk.get("bf16_tflops_sustained", pk["bf16_tflops"])
     roofline = {"bound": "tensor", "achieved": achieved, "peak": sustained, "unit": "TFLOP/s", "frac": achieved / sustained,
                 "traffic": DOMINANT_TRAFFIC_BYTES,
-                "kernel": f"tc_pair_linear_kernel<{gate.cfg.b0}, forward> on gate {gate.N}x{gate.K} at M=2048 (with the rank-r pre-product kernel "
-                          "that runs beside it); duration = mean over the timed steps of the CUDA-event interval around the call",
-                "ms_per_launch": g_ms, "ms_per_launch_median": float(np.median(call_ms[:, gi])),
-                "ms_per_launch_min_max": [float(call_ms[:, gi].min()), float(call_ms[:, gi].max())],
-                "flop_per_launch": linear_flops(2048, gate.N, gate.K, r),
-                "peak_kind": pk_kind + " cuBLAS bf16, sustained figure (the kernel is timed inside a long step)",
+                "kernel": f"tc_pair_linear_kernel<{gate.cfg.b0}, forward> on gate {gate.N}x{gate.K} at M=2048, mean CUDA-event interval around the "
+                          "call in the timed steps",
+                "ms_per_launch": g_ms, "ms_per_launch_min_max": [float(call_ms[:, gi].min()), float(call_ms[:, gi].max())],
+                "flop_per_launch": linear_flops(2048, gate.N, gate.K, r), "peak_kind": pk_kind + " cuBLAS bf16, sustained",
                 "frac_of_burst_" + pk_kind: achieved / pk["bf16_tflops"], "frac_of_nominal_2250": achieved / NOMINAL["bf16_tflops"]}
 
     # ---- the decode-sized calls of the layer once more, each matrix alone over cold copies as one CUDA graph
@@ -619,8 +627,7 @@ def run_device(args):
         "data": "synthetic",
         "config": {"workload": WORKLOAD, "rank": r, "M": list(MS), "calls_per_step": ncalls,
                    "parallelism": f"dp{world} over tokens, weights replicated, no collective",
-                   "l2": "inputs larger than L2: a step reads 3.4 GB of fp32 weights, 0.29 GB of packed codes per pass and 0.5 GB of "
-                         "activations, and no buffer is touched twice within 126 MB of traffic except the shared inputs of q/k/v and gate/up",
+                   "l2": "inputs larger than L2 (3.4 GB of weights, 0.29 GB of codes per pass, 0.5 GB of activations per step)",
                    "ms_per_step_median": float(statistics.median(step_ms)), "ms_per_step_min_max": [min(step_ms), max(step_ms)],
                    "wall_ms_per_step": t_wall / args.steps * 1e3},
         "clocks": clocks,
@@ -629,9 +636,13 @@ def run_device(args):
         "gpu_launches": int(launches),
         "roofline": roofline,
         "cpu_baseline": cpu,
-        "breakdown": {"phases": phases, "calls": layer, "decode_calls_alone": decode, "extra": extra, "other_configs": other},
+        "phases_ms": {ph: ent["ms"] for ph, ent in phases.items()},
     }
-    print(json.dumps(line), flush=True)
+    if args.breakdown:
+        os.makedirs(os.path.dirname(os.path.abspath(args.breakdown)), exist_ok=True)
+        with open(args.breakdown, "w") as f:
+            json.dump({"phases": phases, "calls": layer, "decode_calls_alone": decode, "extra": extra, "other_configs": other}, f)
+    print(json.dumps(short(line)), flush=True)
     if world > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
@@ -750,6 +761,8 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-configs", action="store_true", help="skip the per-config figures measured beside the step")
+    ap.add_argument("--breakdown", default=os.path.join(ROOT, "build", "bench_breakdown.json"),
+                    help="file for the per-call figures and the other workloads ('' writes none)")
     ap.add_argument("--dry-run", action="store_true", help="host logic of the multi-rank path only (gloo, no device work)")
     ap.add_argument("--sweep", action="store_true", help="print the b0 x B0 x M table of the 8192 x 8192 sweep instead")
     ap.add_argument("--sweep-ms", default="1,16,128,2048,8192")

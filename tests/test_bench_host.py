@@ -108,3 +108,8 @@ def test_gpus_flag_starts_the_ranks_itself_and_reports_their_number():
     out = subprocess.run([sys.executable, os.path.join(ROOT, "bench.py"), "--gpus", "1", "--dry-run"], env=env, capture_output=True,
                          text=True, timeout=300)
     assert out.returncode == 0 and json.loads(out.stdout.strip().splitlines()[-1])["n_gpus"] == 1
+
+
+def test_floats_of_the_line_are_shortened_and_nothing_else():
+    line = {"a": 1.23456789012, "b": [0.1 + 0.2, 3, None, "x"], "c": {"d": 123456789.0, "e": True}, "f": 4123456789}
+    assert bench.short(line) == {"a": 1.23457, "b": [0.3, 3, None, "x"], "c": {"d": 123457000.0, "e": True}, "f": 4123456789}
