@@ -17,6 +17,8 @@
 // weights of a row and warp).
 #pragma once
 
+#include <atomic>
+
 namespace lq {
 namespace tc {
 
@@ -453,13 +455,14 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 
 // ------------------------------------------------------------------------------------ host side
 // Clusters of `n` CTAs (one CTA per SM, all of its shared memory) that can be resident at the same time.  A cluster lives
-// inside one GPC, so fewer fit than SMs / n: 15 clusters of eight on a B200, not 18.  Asked once per cluster size; the
-// figures measured on a B200 stand in when there is no device to ask.
+// inside one GPC, so fewer fit than SMs / n: 15 clusters of eight on a B200, not 18.  Asked once per cluster size; what the
+// driver answered on a B200 (74, 33, 22, 15) stands in when there is no device to ask.
 inline int tc_max_clusters(int n) {
-    static int cached[4] = {-1, -1, -1, -1};       // n = 2, 4, 6, 8
+    static std::atomic<int> cached[4] = {-1, -1, -1, -1};       // n = 2, 4, 6, 8 (threads that ask at the same time get the same answer)
     const int idx = n / 2 - 1;
-    if (cached[idx] >= 0) return cached[idx];
-    const int fallback[4] = {74, 36, 24, 15};
+    const int known = cached[idx].load(std::memory_order_relaxed);
+    if (known >= 0) return known;
+    const int fallback[4] = {74, 33, 22, 15};
     int got = 0;
     auto kern = tc_swap_linear_kernel<3, false>;
     cudaLaunchConfig_t cfg = {};
@@ -476,7 +479,7 @@ inline int tc_max_clusters(int n) {
         cudaGetLastError();
         got = fallback[idx];
     }
-    cached[idx] = got;
+    cached[idx].store(got, std::memory_order_relaxed);
     return got;
 }
 
