@@ -337,9 +337,10 @@ int lqlora_selftest_bounded_wait(void* workspace_dev, int64_t budget_cycles, voi
 enum { LQLORA_PATH_PLAIN = 0, LQLORA_PATH_STREAM = 1, LQLORA_PATH_TC_ONE = 2, LQLORA_PATH_TC_PAIR = 3 };
 int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, int64_t M, int backward, int* splits);
 
-/* lqlora_encode finds the nearest code (Sec. 2.2: c_j = argmin_k |q~_k - u_j / s_i|) with a bin table over [-1, 1]:
+/* lqlora_encode finds the nearest 8-bit code (Sec. 2.2: c_j = argmin_k |q~_k - u_j / s_i|) with a bin table over [-1, 1]:
  * every bin holds at most one decision threshold (the midpoint of two neighbouring code-book entries), and inputs
- * closer than 1e-6 to a threshold are decided with the exact IEEE quotient.  This returns the smallest distance
+ * closer than 1e-6 to a threshold are decided with the exact IEEE quotient.  (2-, 3- and 4-bit codes are found on a curve through
+ * the thresholds, with the same exact decision next to them.)  This returns the smallest distance
  * between a threshold and a bin edge for the b0-bit table; it must exceed that 1e-6 by a wide margin for the
  * fast and the exact route to agree (checked by the host tests).  Negative for an invalid b0.  Host only. */
 double lqlora_encode_search_clearance(int b0);

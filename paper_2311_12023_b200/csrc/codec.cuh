@@ -6,6 +6,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "device_util.cuh"
 
 namespace lq {
 
@@ -29,69 +30,109 @@ __device__ __forceinline__ uint32_t nearest_code(float x, const float* __restric
     }
 }
 
-// Fast search for 2- and 3-bit codes without compares or selects (the compare / select pipe is the encoder's
-// bottleneck; this runs on the fused-multiply-add pipe).  For x^ and threshold T_k, f_k = saturate(x^ * S + b_k) with
-// S = kSatScale, b_k = fl(0.5 - T_k S) is exactly 0 when x^ < T_k - 0.5/S, exactly 1 when x^ > T_k + 0.5/S, so the code
-// is f_1 + ... + f_n whenever x^ is not that close to a threshold.  The sum starts from a power of two chosen so that
-// the code lands in the mantissa bits that are the code's field of the packed word, seven bits above the bottom of the
-// word's 16-bit half: all bits below the field are zero unless some f_k was fractional (to 2^-8), i.e. unless x^ lies
-// within (0.5 - 2^-8 - 2^-5) / S = 8.9e-7 of a threshold (2^-5 bounds the rounding of b_k) -- more than the 2.4e-7 that x^ can
-// differ from the quotient.  Those bits are collected in `danger`; the caller then decides every code of the thread
-// exactly.  field_bits: position p (0, 2, .. 14) of the field in its half-word.
-template <int B>
-__device__ __forceinline__ uint32_t sat_count(float xh, float start) {
-    float acc = start;
-#pragma unroll
-    for (int k = 0; k < (1 << B) - 1; ++k) {
-        float f;
-        asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(f) : "f"(xh), "f"(kSatScale), "f"(c_satbias[B - 2][k]));
-        acc += f;
-    }
-    return __float_as_uint(acc);
+// Fast search for 2-, 3- and 4-bit codes: no compares, selects, look-ups or conversions.  The code is the integer part of a curve
+// P(x) = E(|x|) + x O(|x|) through the points (T_k, k) at the thresholds T_1 < T_2 < ... (two polynomials, because the quantiles are
+// spaced differently on the two sides of zero; 3-bit codes take one more point, (1, 7.55), without which the curve bends back).  The
+// coefficients come from HostTables; 2^B is added to E, so the integer part stands in the top B mantissa bits, and half of kLim units in
+// the last place are added too, so that the fraction bits below kLim mean "within about 1e-6 of a threshold": those elements are decided
+// exactly.  Evaluated in fp32 for every float in [-1 - 4 ulp, 1 + 4 ulp]: every other x gives the right code, and lies at least 8.2e-7
+// from any threshold (x^ below differs from the quotient by at most 2.4e-7).  Two elements per instruction (fma.f32x2).
+//
+// What bounds the kernel: loads in flight (a CTA loads, then computes, then stores) and instruction issue, 18 instructions per 3-bit weight
+// (25.6 before, with a saturating sum over the thresholds; 4-bit codes looked a bin table up in shared memory).  us per call with the
+// scale kernel, before / now: 8192 x 8192 2 bits 61 / 59, 3 bits 75 / 70, blocks of 16 82 / 75, 4 bits 91 / 81; 11008 x 4096 4 bits
+// 65.5 / 58.  The scalar form of the same polynomials: 4 bits 88 and 63.
+template <int B> struct Curve {
+    static constexpr int NE = B == 2 ? 2 : B == 3 ? 4 : 8, NO = B == 2 ? 1 : B == 3 ? 4 : 7;
+    static constexpr uint32_t kMask = (1u << (23 - B)) - 1u;               // fraction bits
+    static constexpr uint32_t kLim = curve_limit(B);
+};
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(a), "f"(b));
+    return d;
 }
-// The B words of 32 codes from u * (r_lo | r_hi), layout of deposit_code<B>.
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+// The bits of P for the two halves of x.
 template <int B>
-__device__ __forceinline__ void sat_encode(const float (&u)[32], float r_lo, float r_hi, uint32_t (&words)[B], uint32_t& danger) {
-    static_assert(B == 2 || B == 3, "2- and 3-bit codes");
-    constexpr uint32_t cmask = (1u << B) - 1u;
-    if constexpr (B == 3) {
-        uint32_t V = 0;
+__device__ __forceinline__ void curve_bits(uint64_t x, uint32_t& b0, uint32_t& b1) {
+    using C = Curve<B>;
+    const float2* c = c_curve[B - 2];
+    const uint64_t y = x & 0x7fffffff7fffffffull;
+    uint64_t e = pack2(c[C::NE - 1].x, c[C::NE - 1].y), o = pack2(c[C::NE + C::NO - 1].x, c[C::NE + C::NO - 1].y);
 #pragma unroll
-        for (int w = 0; w < 4; ++w) {
-            uint32_t H[2] = {0u, 0u};
+    for (int i = C::NE - 2; i >= 0; --i) e = fma2(e, y, pack2(c[i].x, c[i].y));
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
+    for (int i = C::NO - 2; i >= 0; --i) o = fma2(o, y, pack2(c[C::NE + i].x, c[C::NE + i].y));
+    const uint64_t p = fma2(x, o, e);
+    b0 = static_cast<uint32_t>(p);
+    b1 = static_cast<uint32_t>(p >> 32);
+}
+// Third bytes of four words: exponent bit, code, leading fraction bits.
+__device__ __forceinline__ uint32_t third_bytes(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0062), __byte_perm(c, d, 0x0062), 0x5410);
+}
+// Words of 32 codes (layout of deposit_code<B>) from u * (r_lo | r_hi); `closest` = smallest fraction seen.
+template <int B>
+__device__ __forceinline__ void curve_encode(const float (&u)[32], float r_lo, float r_hi, uint32_t (&words)[B], uint32_t& closest) {
+    constexpr uint32_t kMask = Curve<B>::kMask;
+    constexpr int kSpan = B == 2 ? 16 : 8;                   // elements per word
+    uint32_t word[32 / kSpan];
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) {
-                    const int j = 8 * w + 4 * h + jj, p = 4 * jj;
-                    const uint32_t bits = sat_count<3>(u[j] * ((j < 16) ? r_lo : r_hi), static_cast<float>(1u << (16 - p)));
-                    H[h] |= bits & (cmask << (7 + p));
-                    danger |= bits & ((1u << (7 + p)) - 1u);
-                }
-            }
-            const uint32_t word = (H[0] >> 7) | (H[1] << 9);
-            if (w < 3) words[w] = word;
-            else V = word;                 // codes 24..31 as 4-bit fields: their bits go to the spare fourth bits
+    for (int w = 0; w < 32 / kSpan; ++w) {
+        uint32_t bits[kSpan];
+#pragma unroll
+        for (int i = 0; i < kSpan; i += 2) {
+            const int j = w * kSpan + i;
+            const float r = j < 16 ? r_lo : r_hi;
+            uint64_t x;
+            asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(x) : "l"(pack2(u[j], u[j + 1])), "l"(pack2(r, r)));
+            curve_bits<B>(x, bits[i], bits[i + 1]);
+            closest = min(closest, min(bits[i] & kMask, bits[i + 1] & kMask));
         }
-        words[0] |= (V & 0x11111111u) << 3;
-        words[1] |= ((V >> 1) & 0x11111111u) << 3;
-        words[2] |= ((V >> 2) & 0x11111111u) << 3;
-    } else {
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            uint32_t H[2] = {0u, 0u};
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                for (int t2 = 0; t2 < 8; ++t2) {
-                    const int j = 16 * w + (t2 >> 2) * 8 + 4 * h + (t2 & 3), p = 4 * (t2 & 3) + 2 * (t2 >> 2);
-                    const uint32_t bits = sat_count<2>(u[j] * ((j < 16) ? r_lo : r_hi), static_cast<float>(1u << (16 - p)));
-                    H[h] |= bits & (cmask << (7 + p));
-                    danger |= bits & ((1u << (7 + p)) - 1u);
-                }
-            }
-            words[w] = (H[0] >> 7) | (H[1] << 9);
+        const uint32_t even = third_bytes(bits[0], bits[2], bits[4], bits[6]), odd = third_bytes(bits[1], bits[3], bits[5], bits[7]);
+        if constexpr (B == 4) {
+            word[w] = ((even >> 3) & 0x0F0F0F0Fu) | ((odd << 1) & 0xF0F0F0F0u);
+        } else if constexpr (B == 3) {
+            word[w] = ((even >> 4) & 0x07070707u) | (odd & 0x70707070u);
+        } else {
+            const uint32_t even2 = third_bytes(bits[8], bits[10], bits[12], bits[14]), odd2 = third_bytes(bits[9], bits[11], bits[13], bits[15]);
+            word[w] = ((even >> 5) & 0x03030303u) | ((even2 >> 3) & 0x0C0C0C0Cu) | ((odd >> 1) & 0x30303030u) | ((odd2 << 1) & 0xC0C0C0C0u);
         }
+    }
+#pragma unroll
+    for (int w = 0; w < B; ++w) words[w] = word[w];
+    if constexpr (B == 3) {                                  // codes 24..31: their bits go to the spare fourth bits
+        words[0] |= (word[3] & 0x11111111u) << 3;
+        words[1] |= (word[3] & 0x22222222u) << 2;
+        words[2] |= (word[3] & 0x44444444u) << 1;
+    }
+}
+// The same for a thread with an element close to a threshold, or a reciprocal that is not a normal number: element by element (a
+// loop over the thread's row in shared memory, `at(j)`), the close ones with the IEEE quotient and the full search.
+template <int B, typename F>
+__device__ __forceinline__ void curve_encode_exact(F at, float s_lo, float s_hi, float r_lo, float r_hi, uint32_t (&words)[B]) {
+    constexpr uint32_t zero_code = (1u << (B - 1)) - 1u;
+#pragma unroll
+    for (int w = 0; w < B; ++w) words[w] = 0u;
+#pragma unroll 1
+    for (int j = 0; j < 32; ++j) {
+        const float u = at(j), s = j < 16 ? s_lo : s_hi, r = j < 16 ? r_lo : r_hi;
+        uint32_t b0, b1;
+        curve_bits<B>(pack2(__fmul_rn(u, r), 0.0f), b0, b1);
+        uint32_t c = (b0 >> (23 - B)) & ((1u << B) - 1u);
+        if ((b0 & Curve<B>::kMask) < Curve<B>::kLim || !(r == r)) {
+            c = zero_code;
+            if (s != 0.0f) c = nearest_code<B>(__fdiv_rn(u, s), nullptr);
+        }
+        uint32_t one[B] = {};
+        deposit_code<B>(one, j, c);
+#pragma unroll
+        for (int w = 0; w < B; ++w) words[w] |= one[w];
     }
 }
 
@@ -111,14 +152,13 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
                                                            float* __restrict__ absmax, int N, int K, int B0, int logB0) {
     __shared__ float red[8][33];
     __shared__ __align__(16) float4 tile[8][32 * 8];   // per warp: 32 rows x 32 columns
-    __shared__ float th8[256];
-    __shared__ float2 bins[kMaxBins + 1];        // (threshold of the bin or +inf, number of thresholds below the bin)
+    __shared__ float th8[B == 8 ? 256 : 1];
+    __shared__ float2 bins[B == 8 ? kMaxBins + 1 : 1];        // (threshold of the bin or +inf, number of thresholds below the bin)
     if constexpr (B == 8) {
         th8[threadIdx.x] = c_threshold[3][threadIdx.x];
     }
-    // 4- and 8-bit codes (15 / 255 thresholds) find their code through a bin table; 2- and 3-bit codes by a binary
-    // search among constants
-    constexpr bool kUseBins = (B >= 4);
+    // 8-bit codes (255 thresholds) find their code through a bin table, the others on a curve through the thresholds
+    constexpr bool kUseBins = (B == 8);
     const int nb = kUseBins ? c_nbins[bits_index(B)] : 0;
     if constexpr (kUseBins) {
         for (int i = threadIdx.x; i <= nb; i += 256) {
@@ -127,6 +167,7 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
         }
     }
     const float bin_scale = 0.5f * static_cast<float>(nb);
+    dev::pdl_wait();                             // started while the kernel in front ends; everything that it may touch comes below
     const int rl = threadIdx.x & 31, grp = threadIdx.x >> 5;
     const int row = blockIdx.x * 32 + rl;
     const int k0 = blockIdx.y * 256 + grp * 32;
@@ -171,7 +212,7 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
     float m0 = 0.0f, m1 = 0.0f;
 #pragma unroll
     for (int i = 0; i < 16; ++i) { m0 = fmaxf(m0, fabsf(u[i])); m1 = fmaxf(m1, fabsf(u[16 + i])); }
-    if constexpr (B >= 4) __syncthreads();       // the search tables in shared memory are complete
+    if constexpr (kUseBins) __syncthreads();     // the search tables in shared memory are complete
     float s_lo, s_hi;   // block absmax for columns 0..15 and 16..31 of this thread's group
     if (B0 == 16) { s_lo = m0; s_hi = m1; }
     else if (B0 == 32) { s_lo = s_hi = fmaxf(m0, m1); }
@@ -198,32 +239,21 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
     uint32_t words[B];
 #pragma unroll
     for (int i = 0; i < B; ++i) words[i] = 0u;
-    // Fast search: x^ = u * fl(1/s) is within 2 ulp (2.4e-7) of the quotient fl(u/s) that defines the code.  The code
-    // is found from x^ (bin table: the bin of x^ holds at most one threshold, code = thresholds below the bin plus
-    // (x^ > threshold); 2/3-bit codes: binary search).  When x^ comes within 1e-6 of a threshold it was compared with
-    // (or is not a number in [-1, 1]) the decision is taken exactly, with the IEEE quotient and the full search.  No
-    // threshold lies that close to a bin edge (the bin count is chosen on the host for the largest clearance), so
-    // the two routes agree.
+    // Fast search: x^ = u * fl(1/s) is within 2 ulp (2.4e-7) of the quotient fl(u/s) that defines the code.  Where x^ comes
+    // within about 1e-6 of a threshold (or a reciprocal is not a normal number) the decision is taken exactly, with the
+    // IEEE quotient and the full search.
     const float r_lo = search_reciprocal(s_lo);
     const float r_hi = search_reciprocal(s_hi);
-    if constexpr (B <= 3) {
-        // codes by saturating arithmetic; exact route for the whole thread when some x^ came close to a threshold or a
-        // reciprocal is not a normal number
-        uint32_t danger = (r_lo == r_lo && r_hi == r_hi) ? 0u : 1u;
-        if (danger == 0u) sat_encode<B>(u, r_lo, r_hi, words, danger);
-        if (danger != 0u) {
-#pragma unroll
-            for (int i = 0; i < B; ++i) words[i] = 0u;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float s = (j < 16) ? s_lo : s_hi;
-                uint32_t c = zero_code;
-                if (s != 0.0f) c = nearest_code<B>(__fdiv_rn(u[j], s), th8);
-                deposit_code<B>(words, j, c);
-            }
+    if constexpr (B <= 4) {
+        uint32_t closest = (r_lo == r_lo && r_hi == r_hi) ? Curve<B>::kMask : 0u;
+        curve_encode<B>(u, r_lo, r_hi, words, closest);
+        if (closest < Curve<B>::kLim) {
+            const float* mine = reinterpret_cast<const float*>(tile[grp] + rl * 8);
+            curve_encode_exact<B>([&](int j) { return mine[(((j >> 2) ^ (rl & 7)) << 2) + (j & 3)]; }, s_lo, s_hi, r_lo, r_hi, words);
         }
     } else {
-        // Bin table: the bin of x^ holds at most one threshold, code = thresholds below the bin plus (x^ > threshold).
+        // Bin table: the bin of x^ holds at most one threshold, and none lies close to a bin edge (the bin count is chosen on the
+        // host for the largest clearance); code = thresholds below the bin plus (x^ > threshold).
         // First all 32 codes without a branch (32 independent chains for the scheduler), keeping the smallest distance
         // between an x^ and the threshold it was compared with; only a thread where that distance is within 1e-6 (or a
         // reciprocal is not a normal number) goes through its elements again and decides the close ones exactly.
@@ -256,6 +286,7 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
             }
         }
     }
+    dev::pdl_launch_dependents();                // the scale kernel may take its place (it waits for this one)
     uint32_t* dst = codes + slab_word_base(row, k0 >> 6, K >> 6, B);
     const int g = (k0 >> 5) & 1;
 #pragma unroll
@@ -285,6 +316,7 @@ __global__ void __launch_bounds__(256) encode_scales_span_kernel(const float* __
                                                                  float* __restrict__ v, long long nblk, long long ngrp, int B1, int logB1,
                                                                  float levels) {
     const long long base = (static_cast<long long>(blockIdx.x) * 8 + (threadIdx.x >> 5)) * 256;
+    dev::pdl_wait();                             // launched while the kernel that writes the maxima ends
     if (base >= nblk) return;
     const int lane = threadIdx.x & 31;
     float2 a[4];
@@ -293,8 +325,8 @@ __global__ void __launch_bounds__(256) encode_scales_span_kernel(const float* __
     for (int e = 0; e < 4; ++e) {
         const long long blk = base + 2 * (e * 32 + lane);
         a[e] = make_float2(0.0f, 0.0f);
-        if (blk + 1 < nblk) a[e] = *reinterpret_cast<const float2*>(absmax + blk);
-        else if (blk < nblk) a[e].x = absmax[blk];
+        if (blk + 1 < nblk) a[e] = __ldcg(reinterpret_cast<const float2*>(absmax + blk));
+        else if (blk < nblk) a[e].x = __ldcg(absmax + blk);
     }
 #pragma unroll
     for (int e = 0; e < 4; ++e) m[e] = fmaxf(a[e].x, a[e].y);
@@ -477,10 +509,25 @@ __global__ void __launch_bounds__(256) export_kernel(QView q, uint8_t* __restric
     }
 }
 
+// Launch that may overlap the end of the kernel in front of it (which the kernel waits for).
+template <typename... P, typename... A>
+inline void launch_behind(void (*kern)(P...), dim3 grid, int threads, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);      // (an error is reported by the caller's cudaGetLastError)
+}
+
 inline void launch_encode_scales(const float* absmax, uint8_t* sc, float* v, long long nblk, long long ngrp, int B1, float levels, cudaStream_t st) {
     if (B1 <= 256) {
         const long long spans = (nblk + 255) / 256;
-        encode_scales_span_kernel<<<static_cast<unsigned>((spans + 7) / 8), 256, 0, st>>>(absmax, sc, v, nblk, ngrp, B1, ilog2(B1), levels);
+        launch_behind(encode_scales_span_kernel, dim3(static_cast<unsigned>((spans + 7) / 8)), 256, st, absmax, sc, v, nblk, ngrp, B1, ilog2(B1), levels);
     } else {
         encode_scales_kernel<<<static_cast<unsigned>((ngrp + 7) / 8), 256, 0, st>>>(absmax, sc, v, nblk, ngrp, B1, levels);
     }
@@ -491,8 +538,7 @@ inline cudaError_t launch_encode(const float* W, const lqlora_qmatrix* out, floa
     const int N = static_cast<int>(out->N), K = static_cast<int>(out->K);
     const int Np = (N + kTileRows - 1) / kTileRows * kTileRows;
     dim3 grid(Np / 32, (K + 255) / 256);
-    encode_codes_kernel<B><<<grid, 256, 0, st>>>(W, static_cast<uint32_t*>(out->codes), absmax, N, K, out->cfg.B0,
-                                                 ilog2(out->cfg.B0));
+    launch_behind(encode_codes_kernel<B>, grid, 256, st, W, static_cast<uint32_t*>(out->codes), absmax, N, K, out->cfg.B0, ilog2(out->cfg.B0));
     const long long nblk = static_cast<long long>(N) * K / out->cfg.B0;
     const long long ngrp = (nblk + out->cfg.B1 - 1) / out->cfg.B1;
     const float levels = static_cast<float>(scale_levels(out->cfg.b1));

@@ -145,12 +145,13 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) { return __uint_
 // neighbouring code-book entries (x > midpoint  <=>  x > threshold for fp32 x).
 __constant__ float c_codebook[4][256];
 __constant__ float c_threshold[4][256];
-// 2- and 3-bit encoder: fl(0.5 - threshold * kSatScale) per threshold; saturate(x * kSatScale + bias) is 0 below the
-// threshold, 1 above it and in between only within 0.5 / kSatScale = 9.5e-7 of it.
-constexpr float kSatScale = 524288.0f;
-__constant__ float c_satbias[2][8];
+// 2-, 3- and 4-bit encoder: coefficients of the curve through the thresholds (E, then O; each twice, for two elements per
+// instruction), and the fraction (in units of the last place) below which a value counts as close to a threshold.
+constexpr int kCurveCoefs = 15;
+__host__ __device__ constexpr uint32_t curve_limit(int b0) { return b0 == 2 ? 10u : b0 == 3 ? 16u : 12u; }
+__constant__ float2 c_curve[3][kCurveCoefs + 1];
 
-// Bin table for the nearest-code search of the encoder: [-1, 1] is cut into `nb` equal bins chosen so that every
+// Bin table for the nearest-code search of the 8-bit encoder: [-1, 1] is cut into `nb` equal bins chosen so that every
 // bin holds at most one threshold and no threshold lies near a bin edge.  Entry k = (threshold in the bin or +inf,
 // number of thresholds below the bin); entry nb serves x slightly above 1.
 constexpr int kMaxBins = 1280;

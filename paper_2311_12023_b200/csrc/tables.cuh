@@ -5,6 +5,7 @@
 #include <atomic>
 #include <cmath>
 #include <mutex>
+#include <utility>
 
 #include "common.cuh"
 
@@ -35,7 +36,7 @@ struct HostTables {
     float threshold[4][256];
     BinEntry bins[4][kMaxBins + 1];
     int nbins[4];
-    float satbias[2][8];
+    float2 curve[3][kCurveCoefs + 1];
     // Bin count for `n - 1` thresholds: the candidate with the largest distance between any threshold and any
     // bin edge among those with at most one threshold per bin.
     void build_bins(int t, int n) {
@@ -71,6 +72,38 @@ struct HostTables {
         }
         bin_clearance[t] = best_clear;
     }
+    // Coefficients of P(x) = E(|x|) + x O(|x|), P(T_k) = k at the thresholds (3-bit codes: and P(1) = 7.55), by Gaussian
+    // elimination with row pivoting; 2^b0 and half of the "close to a threshold" range are added to the constant term.
+    void build_curve(int b0) {
+        const int t = bits_index(b0), n = 1 << b0;
+        const int ne = b0 == 2 ? 2 : b0 == 3 ? 4 : 8, no = b0 == 2 ? 1 : b0 == 3 ? 4 : 7, m = ne + no;
+        double A[kCurveCoefs][kCurveCoefs + 1];
+        for (int i = 0; i < m; ++i) {
+            const double x = i + 1 < n ? 0.5 * (static_cast<double>(codebook[t][i]) + static_cast<double>(codebook[t][i + 1])) : 1.0;
+            const double y = std::fabs(x);
+            double p = 1.0;
+            for (int j = 0; j < ne; ++j, p *= y) A[i][j] = p;
+            p = x;
+            for (int j = 0; j < no; ++j, p *= y) A[i][ne + j] = p;
+            A[i][m] = i + 1 < n ? i + 1.0 : 7.55;
+        }
+        for (int c = 0; c < m; ++c) {
+            int pv = c;
+            for (int r = c + 1; r < m; ++r) if (std::fabs(A[r][c]) > std::fabs(A[pv][c])) pv = r;
+            for (int k = 0; k <= m; ++k) std::swap(A[c][k], A[pv][k]);
+            for (int r = 0; r < m; ++r) {
+                if (r == c) continue;
+                const double f = A[r][c] / A[c][c];
+                for (int k = c; k <= m; ++k) A[r][k] -= f * A[c][k];
+            }
+        }
+        for (int j = 0; j < m; ++j) {
+            double v = A[j][m] / A[j][j];
+            if (j == 0) v += n + std::ldexp(0.5 * curve_limit(b0), b0 - 23);
+            curve[t][j] = make_float2(static_cast<float>(v), static_cast<float>(v));
+        }
+        for (int j = m; j <= kCurveCoefs; ++j) curve[t][j] = make_float2(0.0f, 0.0f);
+    }
     double bin_clearance[4];
     HostTables() {
         const int bits[4] = {2, 3, 4, 8};
@@ -96,9 +129,7 @@ struct HostTables {
             }
             build_bins(t, n);
         }
-        for (int t = 0; t < 2; ++t)
-            for (int i = 0; i < 8; ++i)
-                satbias[t][i] = (i + 1 < (4 << t)) ? static_cast<float>(0.5 - static_cast<double>(threshold[t][i]) * static_cast<double>(kSatScale)) : 0.0f;
+        for (int b0 = 2; b0 <= 4; ++b0) build_curve(b0);
     }
 };
 
@@ -121,7 +152,7 @@ int ensure_tables() {
     const detail::HostTables& t = detail::host_tables();
     if (cudaMemcpyToSymbol(c_codebook, t.codebook, sizeof(t.codebook)) != cudaSuccess ||
         cudaMemcpyToSymbol(c_threshold, t.threshold, sizeof(t.threshold)) != cudaSuccess ||
-        cudaMemcpyToSymbol(c_satbias, t.satbias, sizeof(t.satbias)) != cudaSuccess ||
+        cudaMemcpyToSymbol(c_curve, t.curve, sizeof(t.curve)) != cudaSuccess ||
         cudaMemcpyToSymbol(g_bins, t.bins, sizeof(t.bins)) != cudaSuccess ||
         cudaMemcpyToSymbol(c_nbins, t.nbins, sizeof(t.nbins)) != cudaSuccess) {
         cudaGetLastError();
