@@ -6,6 +6,7 @@
 #include "tables.cuh"
 #include "codec.cuh"
 #include "linear_decode.cuh"
+#include "linear_stream.cuh"
 #include "linear_small.cuh"
 #include "linear_tc.cuh"
 #include "lora_grad.cuh"
@@ -34,7 +35,7 @@ static int cuda_rc(cudaError_t e) {
 // Scratch bytes one direction of the linear needs for M rows, for the kernel family it dispatches to.
 static size_t linear_need_base(const QView& v, int r, int64_t M, bool backward) {
     if (tc_supported(v, r, M, backward)) return tc_workspace_bytes(r, M);
-    if (backward ? dec::bwd_supported(v, M) : dec::supported(v, M)) return dec::workspace_bytes(v, r, static_cast<int>(M), backward);
+    if (stream_supported(v, r, M, backward)) return stream::workspace_bytes(v, r, static_cast<int>(M), backward);
     const SmallPlan p = small_plan(v.N, v.K, r, M, backward);
     return kStatusBytes + p.t_bytes + p.p_bytes;
 }
@@ -75,12 +76,12 @@ static int run_linear(const lqlora_qmatrix* q, const void* L1, const void* L2, i
         if (expand_scales(q, &v, static_cast<char*>(ws) + base, st) != cudaSuccess) return cuda_rc(cudaGetLastError());
     }
     const bool use_tc = tc_supported(v, r, M, backward);
-    const bool use_decode = !use_tc && (backward ? dec::bwd_supported(v, M) : dec::supported(v, M));
+    const bool use_decode = !use_tc && stream_supported(v, r, M, backward);
     // With a rank-r term the first kernel of the call (the pre-product) clears what has to start at zero (the status
     // word, and the arrival counters of the weight-streaming kernels); otherwise a memset does.
     const bool first_kernel_clears = r > 0 && (use_decode || use_tc);
     if (!first_kernel_clears) {
-        const size_t n = use_decode ? dec::clear_bytes(v, backward) : static_cast<size_t>(kStatusBytes);
+        const size_t n = use_decode ? stream::clear_bytes(v, backward) : static_cast<size_t>(kStatusBytes);
         if (cudaMemsetAsync(ws, 0, n, st) != cudaSuccess) return cuda_rc(cudaGetLastError());
     }
     cudaError_t e = cudaSuccess;
@@ -92,17 +93,17 @@ static int run_linear(const lqlora_qmatrix* q, const void* L1, const void* L2, i
         const int m = static_cast<int>(M);
         if (!backward) {
             switch (v.b0) {
-                case 2: e = dec::launch_fwd<2>(v, L1, L2, r, A, m, out, w, st); break;
-                case 3: e = dec::launch_fwd<3>(v, L1, L2, r, A, m, out, w, st); break;
-                case 4: e = dec::launch_fwd<4>(v, L1, L2, r, A, m, out, w, st); break;
-                default: e = dec::launch_fwd<8>(v, L1, L2, r, A, m, out, w, st); break;
+                case 2: e = stream::launch_fwd<2>(v, L1, L2, r, A, m, out, w, st); break;
+                case 3: e = stream::launch_fwd<3>(v, L1, L2, r, A, m, out, w, st); break;
+                case 4: e = stream::launch_fwd<4>(v, L1, L2, r, A, m, out, w, st); break;
+                default: e = stream::launch_fwd<8>(v, L1, L2, r, A, m, out, w, st); break;
             }
         } else {
             switch (v.b0) {
-                case 2: e = dec::launch_bwd<2>(v, L1, L2, r, A, m, out, w, st); break;
-                case 3: e = dec::launch_bwd<3>(v, L1, L2, r, A, m, out, w, st); break;
-                case 4: e = dec::launch_bwd<4>(v, L1, L2, r, A, m, out, w, st); break;
-                default: e = dec::launch_bwd<8>(v, L1, L2, r, A, m, out, w, st); break;
+                case 2: e = stream::launch_bwd<2>(v, L1, L2, r, A, m, out, w, st); break;
+                case 3: e = stream::launch_bwd<3>(v, L1, L2, r, A, m, out, w, st); break;
+                case 4: e = stream::launch_bwd<4>(v, L1, L2, r, A, m, out, w, st); break;
+                default: e = stream::launch_bwd<8>(v, L1, L2, r, A, m, out, w, st); break;
             }
         }
         return cuda_rc(e);
@@ -436,7 +437,7 @@ int lqlora_linear_intermediate_offset(int64_t N, int64_t K, const lqlora_config*
     const bool bwd = backward != 0;
     // the tensor-core and the plain kernels keep [status][T]; the weight-streaming kernels [status][arrival counters][T]
     size_t off = kStatusBytes;
-    if (!tc_supported(v, r, M, bwd) && (bwd ? dec::bwd_supported(v, M) : dec::supported(v, M))) off = dec::clear_bytes(v, bwd);
+    if (!tc_supported(v, r, M, bwd) && stream_supported(v, r, M, bwd)) off = stream::clear_bytes(v, bwd);
     *offset = off;
     return LQLORA_OK;
 }
@@ -580,9 +581,9 @@ int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, in
         if (c_base < out_cols && sp.ks < 1) return LQLORA_ERR_INVALID_SHAPE;      // as the call itself
         kernel = pair ? LQLORA_PATH_TC_PAIR : LQLORA_PATH_TC_ONE;
         if (!pair) ks = sp.ks;
-    } else if (bwd ? dec::bwd_supported(v, M) : dec::supported(v, M)) {
+    } else if (stream_supported(v, r, M, bwd)) {
         kernel = LQLORA_PATH_STREAM;
-        ks = bwd ? dec::bwd_splits(v, static_cast<int>(M)) : dec::fwd_splits(v, static_cast<int>(M));
+        ks = stream::slots(v, r, static_cast<int>(M), bwd);
     }
     if (splits) *splits = ks;
     return kernel;

@@ -1,0 +1,31 @@
+"""Weight-streaming kernels: edges of units, runs, scale runs, second-level groups and rank-r units."""
+import pytest
+
+from paper_2311_12023_b200 import binding, inputs
+from test_gpu_linear import C, run_case
+
+pytestmark = pytest.mark.gpu
+
+
+# one tile of a unit / of a window, a ragged last unit, a partial tile row and slab; rows of blocks that are not whole vectors of scale
+# codes (odd numbers of blocks, groups of 16 blocks that end inside a vector); tokens on both sides of 8; fewer units than SMs, one tile
+# row shared by all runs (40960 columns), runs over three tile rows (40000 rows)
+@pytest.mark.parametrize("N,K,M", [(8, 64, 1), (40, 192, 8), (136, 1088, 7), (392, 1984, 9), (1000, 320, 16), (264, 2368, 3),
+                                   (64, 40960, 2), (40000, 64, 5)])
+@pytest.mark.parametrize("b0,B0,B1,r", [(2, 16, 64, 16), (2, 64, 16, 80), (3, 64, 16, 64), (3, 32, 256, 128), (4, 16, 16, 48), (4, 64, 64, 0), (8, 64, 16, 16)])
+def test_unit_run_and_scale_edges(N, K, M, b0, B0, B1, r):
+    cfg = C(b0, B0, 8, B1, 32)
+    assert binding.linear_path(N, K, cfg, r, M, False) == binding.PATH_STREAM
+    A = inputs.gaussian(6100 + N, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(6101 + K, N, K, r, 0.05) if r else (None, None)
+    run_case(A, l1b, l2b, cfg, M, seed=6200 + M)
+
+
+# blocks wider than a tile and than a window, on a matrix whose runs end inside a tile row, both sides of eight tokens
+@pytest.mark.parametrize("M", [1, 8, 9, 16])
+@pytest.mark.parametrize("b0,B0", [(2, 128), (3, 256), (4, 128), (8, 256)])
+def test_wide_blocks(b0, B0, M):
+    N, K = 1928, 2304
+    A = inputs.student_t(6300 + b0, (N, K), 5.0, 0.02)
+    l1b, l2b = inputs.lowrank_factors(6301, N, K, 64, 0.03)
+    run_case(A, l1b, l2b, C(b0, B0, 8, 16, 32), M, seed=6400 + M)
