@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from dataclasses import dataclass
 from typing import Optional, Tuple
 
@@ -49,6 +50,9 @@ class CQMatrix(ctypes.Structure):
                 ("N", ctypes.c_int64), ("K", ctypes.c_int64), ("cfg", CConfig)]
 
 
+_QSTRUCT = struct.Struct("@PPPqq5i4x")       # layout of CQMatrix
+assert _QSTRUCT.size == ctypes.sizeof(CQMatrix)
+
 _lib = None
 
 
@@ -70,8 +74,9 @@ def lib() -> ctypes.CDLL:
         L.lqlora_unpack.argtypes = [ctypes.POINTER(CQMatrix), vp, vp]
         L.lqlora_dequant.argtypes = [ctypes.POINTER(CQMatrix), vp, vp, vp]
         L.lqlora_linear_workspace_bytes.argtypes = [i64, i64, ctypes.POINTER(CConfig), ci, i64, ctypes.POINTER(sz)]
-        L.lqlora_linear_fwd.argtypes = [ctypes.POINTER(CQMatrix), vp, vp, ci, vp, i64, vp, vp, sz, vp]
-        L.lqlora_linear_bwd_input.argtypes = [ctypes.POINTER(CQMatrix), vp, vp, ci, vp, i64, vp, vp, sz, vp]
+        # (the quantized matrix as a plain pointer: byref of a CQMatrix, or the bytes of one)
+        L.lqlora_linear_fwd.argtypes = [vp, vp, vp, ci, vp, i64, vp, vp, sz, vp]
+        L.lqlora_linear_bwd_input.argtypes = [vp, vp, vp, ci, vp, i64, vp, vp, sz, vp]
         L.lqlora_lora_grads_workspace_bytes.argtypes = [i64, i64, ci, i64, ctypes.POINTER(sz)]
         L.lqlora_lora_grads.argtypes = [vp, vp, ci, i64, i64, vp, vp, i64, vp, vp, vp, sz, vp]
         L.lqlora_linear_intermediate_offset.argtypes = [i64, i64, ctypes.POINTER(CConfig), ci, i64, ci, ctypes.POINTER(sz)]
@@ -191,6 +196,15 @@ class QMatrix:
         return CQMatrix(self.codes.data_ptr(), self.scale_codes.data_ptr(), self.scale2.data_ptr(),
                         self.N, self.K, _cfg(self.cfg))
 
+    def cbytes(self) -> bytes:
+        """The same struct as bytes (a third of the time of the ctypes object, for the calls of the layer)."""
+        c = self.cfg
+        try:
+            return _QSTRUCT.pack(self.codes.data_ptr(), self.scale_codes.data_ptr(), self.scale2.data_ptr(), self.N, self.K,
+                                 c.b0, c.B0, c.b1, c.B1, c.b2)
+        except struct.error:                   # fields that are not integers: as cstruct converts them
+            return bytes(self.cstruct())
+
     @property
     def packed_bytes(self) -> int:
         return self.codes.numel() + self.scale_codes.numel() + self.scale2.numel() * self.scale2.element_size()
@@ -274,13 +288,12 @@ def _linear(fn, name, q, L1, L2, A, out_cols, out, workspace):
     r = 0 if L1 is None else L1.shape[1]
     if r:
         assert L1.dtype == torch.bfloat16 and L2.dtype == torch.bfloat16 and L1.is_contiguous() and L2.is_contiguous()
-        assert tuple(L1.shape) == (q.N, r) and tuple(L2.shape) == (r, q.K)
+        assert L1.shape == (q.N, r) and L2.shape == (r, q.K)
     if out is None:
-        out = torch.empty((M, out_cols), dtype=torch.bfloat16, device=A.device)
+        out = A.new_empty((M, out_cols))
     if workspace is None:
         workspace = alloc_workspace(q, r, M)
-    cs = q.cstruct()
-    _check(fn(ctypes.byref(cs), _ptr(L1), _ptr(L2), r, A.data_ptr(), M, out.data_ptr(), workspace.data_ptr(),
+    _check(fn(q.cbytes(), _ptr(L1), _ptr(L2), r, A.data_ptr(), M, out.data_ptr(), workspace.data_ptr(),
               workspace.numel(), _stream()), name)
     return out
 
