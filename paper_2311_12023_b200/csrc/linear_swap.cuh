@@ -522,14 +522,14 @@ inline int swap_max_tokens(int b0) {
 }
 
 // The split of a call that costs least by a simple model: waves of clusters, each with a fixed cost, its steps (the
-// slower of dequantization and tensor core) and its reduction.  The constants are those of a sweep over chunks and slices
-// (us with 1, 2, 3, 4 slices): 4096 x 4096 NF3, 64 rows: 24, 17, 15, 26 (16 clusters of eight, of which 15 fit); 8192 x 8192
-// NF4, 17 rows: 53, 32, 45, 56; 11008 x 4096 NF4, 128 rows: 31, 40, 35, 45; 1024 x 1024 NF3, 512 rows in four chunks: 12.3, 12.9,
-// 16, 24, in seven: 11.6, 14, 21, 23; 1024 x 8192 NF3, 1024 rows in four chunks: 47, 32, 39, 55.
+// slower of dequantization and tensor core) and its reduction.  Fitted to 2300 timings of all chunk counts and slices (twelve shapes, 2 to
+// 8 bits, 20 to 1800 rows): the plan that it picks takes 2.5 % longer than the best one on average (4.8 % with the constants before,
+// which had no term for the SMs that the pre-product holds and made a single slice of a long contraction 20 % dearer).  us with 1, 2, 3,
+// 4 slices: 4096 x 4096 NF3, 64 rows: 24, 17, 15, 26 (16 clusters of eight, of which 15 fit); 8192 x 8192 NF4, 17 rows: 53, 32, 45, 56.
 inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
     SwapPlan best{};
     best.us = -1.0;
-    const double dq = b0 == 2 ? 0.22 : b0 == 3 ? 0.26 : b0 == 4 ? 0.35 : 0.40;      // us per step of 128 x 64 weights
+    const double dq = b0 == 2 ? 0.22 : b0 == 3 ? 0.26 : b0 == 4 ? 0.35 : 0.47;      // us per step of 128 x 64 weights
     const long long pairs = (out_cols + 255) / 256;
     int first = static_cast<int>((M + 511) / 512);
     // The search covers eight numbers of chunks.  Where the chunks of all of them are too large for the rings (8-bit codes
@@ -550,18 +550,20 @@ inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q,
             if (!swap_rings(b0, ks, pl)) continue;
             pl.ks = ks;
             pl.ctas = 2 * pairs * pl.chunks * ks;
-            // a rank-r pre-product runs beside this kernel and takes SMs out of the GPCs, which costs large clusters most (a
-            // second wave costs more than a finer split saves)
+            // a rank-r pre-product runs beside this kernel and takes SMs: a CTA per 128 tokens, and out of the GPCs, which costs large
+            // clusters most (a second wave costs more than a finer split saves)
             const int taken[4] = {2, 1, 2, 4};
-            const long long at_once = tc_max_clusters(2 * ks) - (steps_d > 0 ? taken[ks - 1] : 0);
+            long long at_once = tc_max_clusters(2 * ks) - (steps_d > 0 ? taken[ks - 1] : 0);
+            if (ks == 1 && steps_d > 0) {
+                const long long beside = tc_max_clusters(2) - ((M + 127) / 128 + 1) / 2;
+                if (beside < at_once) at_once = beside < 1 ? 1 : beside;
+            }
             const long long waves = (pairs * pl.chunks + at_once - 1) / at_once;
             const double step = dq > tokens * 0.0012 ? dq : tokens * 0.0012;
             const double body = 6.5 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 2.5 + tokens * 0.008 : tokens * 0.006);
             pl.us = waves * body;
-            // A single slice of a long contraction is made 20 % dearer than the model has it.  Both sides (us as a graph, with / without):
-            // 8192 x 8192 at 384 rows 45 / 48 (NF2), 45 / 50 (NF3); but 8192 x 28672 NF3 at 512 rows 198 / 168, 5120 x 5120 NF4 at 512 rows
-            // 49 / 40, 2048 x 2048 NF3 at 1024 rows 20 / 18: right for chunks of fewer than 512 tokens only.
-            if (ks == 1 && steps_q > 16) pl.us *= 1.2;
+            if (ks == 1 && steps_q > 16) pl.us *= 1.1;  // a single slice of a long contraction
+            if (ks > 1 && waves > 1) pl.us *= 1.3;      // clusters of four and more leave GPCs partly empty between waves
             if (best.us < 0 || pl.us < best.us) best = pl;
         }
     }

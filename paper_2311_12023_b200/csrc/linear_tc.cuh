@@ -471,17 +471,6 @@ inline bool make_map(CUtensorMap* map, const void* ptr, uint64_t rows, uint64_t 
 namespace lq {
 namespace tc {
 
-// CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs.  The line was drawn against a kernel with the
-// tokens as rows of its tiles; the transposed tiles that took that kernel's place pad to 16 rows instead of 512 and hold out
-// longer (us as a graph, pair / transposed): 8192 x 8192 NF3 at 512 rows 84 / 54 (transposed by this rule), 600 87 / 61, 800
-// 90 / 77, 1024 93 / 93, 1100 172 / 138, 1536 174 / 144; input gradient 4096 x 4096 NF4 at 1024 rows 49 / 36 (transposed),
-// 1100 50 / 40, 1536 50 / 44, 2048 53 / 56; 28672 x 8192 NF3, blocks of 16, at 300 rows 172 / 122, 600 301 / 263.
-inline bool tc_use_pair(int64_t M, int64_t out_cols, int sms) {
-    if (M <= 256) return false;
-    const long long pair_ctas = 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN);
-    return 2 * pair_ctas > sms;
-}
-
 struct PrePlan {
     int mtiles, nsplit, steps, steps_per_split, rp;
 };
@@ -515,6 +504,24 @@ inline int pair_peel(int64_t M, int64_t out_cols) {
     return peel >= c_tiles ? 0 : peel;
 }
 
+// CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs, unless the transposed tiles, which pad to 16
+// rows instead of 512 and choose their split, are estimated to take less than 0.85 of their time: whole waves of the pair kernel, 6 us
+// and 0.64 us (8-bit codes 0.95) per step each.  From 2048 rows on the two are within 15 % of each other either way and the pairs
+// stay.  us as a graph, pair / transposed: 8192 x 8192 NF3 at 520 rows 87 / 59, 700 88 / 67, 900 91 / 87, 1100 170 / 137, 1400 174 /
+// 131, 1700 180 / 162, 2600 278 / 267, 3300 337 / 343; 5120 x 5120 NF2 at 520 rows 57 / 33, 1100 59 / 47; 11008 x 4096 NF4 input gradient at
+// 1100 rows 112 / 83; 8192 x 8192 NF8 at 520 rows 129 / 87, 1100 253 / 171; 4096 x 4096 NF4 at 1700 rows 54 / 50, 4000 100 / 108.
+inline double pair_estimate(int b0, int64_t M, int64_t out_cols, int steps_q) {
+    const int mt = static_cast<int>((M + 511) / 512), c_tiles = static_cast<int>((out_cols + BN - 1) / BN), peel = pair_peel(M, out_cols);
+    const long long pairs = sm_count() / 2, waves = (static_cast<long long>(mt) * (c_tiles - peel) + pairs - 1) / pairs;
+    return static_cast<double>(waves) * (6.0 + steps_q * (b0 == 8 ? 0.95 : 0.64)) + (peel > 0 ? 20.0 + 0.15 * steps_q : 0.0);
+}
+inline bool tc_use_pair(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+    if (M <= 256) return false;
+    const long long pair_ctas = 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN);
+    if (2 * pair_ctas <= sm_count()) return false;
+    return M >= 2048 || swap_plan(b0, M, out_cols, steps_q, steps_d).us >= 0.85 * pair_estimate(b0, M, out_cols, steps_q);
+}
+
 // The launch on transposed tiles that a call needs: the whole of it, or the output columns from *c_base on that the pair
 // kernel leaves (none where *c_base is not below out_cols).
 inline SwapPlan call_swap_plan(int b0, bool pair, int64_t M, int64_t out_cols, int steps_q, int steps_d, int* c_base) {
@@ -533,7 +540,7 @@ inline PrePlan pre_plan(int b0, int64_t C, int r, int64_t M, int64_t out_cols) {
     // The pre-product runs beside the linear kernel that follows it (programmatic dependent launch):
     // give it the SMs that the last wave of that kernel leaves idle, and at least one CTA per row tile.
     const int sms = sm_count();
-    const long long main_ctas = tc_use_pair(M, out_cols, sms) ? 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN)
+    const long long main_ctas = tc_use_pair(b0, M, out_cols, pl.steps, (r + BK - 1) / BK) ? 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN)
                                                               : swap_plan(b0, M, out_cols, pl.steps, (r + BK - 1) / BK).ctas;
     const int idle = static_cast<int>((sms - main_ctas % sms) % sms);
     int want = idle / pl.mtiles;
@@ -627,7 +634,7 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
     const PrePlan pl = pre_plan(q.b0, C, r, M, backward ? q.K : q.N);
     // workspace: [status word][T bf16]; the status word is cleared by the first kernel of the call (or the caller's memset)
     __nv_bfloat16* T = reinterpret_cast<__nv_bfloat16*>(ws + kStatusBytes);
-    const bool pair = tc_use_pair(M, backward ? q.K : q.N, sm_count());      // CTA pairs (cta_group::2) on [512, 256] tiles; boxes of 128 rows
+    const bool pair = tc_use_pair(q.b0, M, backward ? q.K : q.N, pl.steps, (r + BK - 1) / BK);      // CTA pairs (cta_group::2) on [512, 256] tiles; boxes of 128 rows
     const int out_cols = backward ? q.K : q.N;
     int c_base = 0;
     const SwapPlan sp = call_swap_plan(q.b0, pair, M, out_cols, pl.steps, (r + BK - 1) / BK, &c_base);

@@ -575,7 +575,7 @@ int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, in
     if (tc_supported(v, r, M, bwd)) {
         const int64_t out_cols = bwd ? K : N;
         const int steps_q = static_cast<int>(((bwd ? N : K) + tc::BK - 1) / tc::BK);
-        const bool pair = tc::tc_use_pair(M, out_cols, tc::sm_count());
+        const bool pair = tc::tc_use_pair(v.b0, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK);
         int c_base = 0;
         const tc::SwapPlan sp = tc::call_swap_plan(v.b0, pair, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK, &c_base);
         if (c_base < out_cols && sp.ks < 1) return LQLORA_ERR_INVALID_SHAPE;      // as the call itself
