@@ -10,14 +10,21 @@
 // pairs of the same cluster: each CTA lays its fp32 accumulators down in its own (idle) shared memory and adds up and stores its share of the
 // tokens (rank order: the same bits on every run).
 // Forward reads the weight tile as a K-major operand, the input gradient the same bytes as an MN-major operand.
+// Forward with one token box (at most 256 tokens per pair): the weights go from the registers into tensor memory instead (32 columns
+// per stage), which a row operand may be read from.  Accumulators take at most 256 of the 512 columns there, eight stages the rest; with two
+// boxes the accumulators need them all.  The row operand in tensor memory is K-major only, so the input gradient stays in shared memory.
 // Every wait is bounded (see linear_tc.cuh).
 //
 // What bounds it: the loop of the issuing warp (a dependent chain of about a hundred clocks per wait and commit, so one
 // full and one empty barrier per step, 32-bit descriptors, no divisions), then dequantization (about 500 clocks per 64
-// weights of a row and warp).
+// weights of a row and warp).  A weight tile in shared memory costs its bandwidth twice, when written and when read by the tensor
+// core, and with wide codes or many tokens it takes the room of ring stages.  us as a graph, in shared / in tensor memory: 8192 x 8192
+// NF3 128 rows 28.0 / 26.7 (1.05), 512 rows 52.9 / 50.2, 28672 x 8192 NF3 128 rows 95.2 / 90.8, 8-bit codes 256 rows 62.5 / 60.4; shapes
+// whose grid leaves many SMs idle are even (4096 x 4096 NF4 64 rows 16.6 / 16.7).
 #pragma once
 
 #include <atomic>
+#include <type_traits>
 
 namespace lq {
 namespace tc {
@@ -27,6 +34,7 @@ constexpr int kSwFirstDeq = 4;                                  // warps 0..3: t
 constexpr int kSwThreads = (kSwFirstDeq + kSwDeqWarps) * 32;
 constexpr int kSwWBytes = 128 * 128;                            // this CTA's bf16 weight tile of one step
 constexpr int kSwMaxStages = 8;
+constexpr uint32_t kSwTmemA = 256;                              // first column of the weights in tensor memory (32 per stage)
 constexpr int kSwTail = 512;                                    // barriers, tensor-memory slot, abort flag
 
 struct SwapParams {
@@ -37,8 +45,11 @@ struct SwapParams {
     int out_cols;            // N (forward) or K (backward)
     int steps_q, steps_d;    // contraction steps with dequantized weights / of the rank-r term
     int c_base;              // first output column of this launch
+    const __nv_bfloat16* L1; // forward with the weights in tensor memory: [N][r], read directly
+    int r;
     int nbox, box;           // token boxes (1 or 2) and tokens per box (a multiple of 16, at most 256; half of them per CTA)
     int ss, sp;              // stages of the token + weight ring and of the packed-code ring
+    uint32_t tail_off;       // of the barriers, behind the rings
     uint32_t tmem_cols;
 };
 
@@ -66,6 +77,23 @@ __device__ __forceinline__ void tc_mma2_lo(uint32_t d_tmem, uint32_t a_lo, uint3
         "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n\t}"
         ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(kDescHi), "r"(accumulate) : "memory");
 }
+
+// The same with the weights in tensor memory (a lane per row, two contraction elements per column).
+__device__ __forceinline__ void tc_mma2_ta(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_lo, uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 db;\n\t"
+        "mov.b64 db, {%2, %4};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], db, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "r"(b_lo), "r"(idesc), "r"(kDescHi), "r"(accumulate) : "memory");
+}
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&v)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"
+        ::"r"(taddr), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]) : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // The 64 weights of one row of a step.  words0 / words1: shared-memory addresses of the first word of the two 32-column
 // groups (the others 128 bytes apart); s[h] = scale of the columns 16 h .. 16 h + 15; nsc = distinct scales (1, 2, 4).
@@ -107,6 +135,39 @@ __device__ __forceinline__ void dequant_row64(uint32_t words0, uint32_t words1, 
     }
 }
 
+// The same into 32 columns of tensor memory from `taddr` on (this warp's lanes).
+template <int B>
+__device__ __forceinline__ void dequant_row64_tmem(uint32_t words0, uint32_t words1, const float (&s)[4], int nsc, uint32_t taddr,
+                                                   const float* __restrict__ lut8) {
+    BlockTable<B == 8 ? 2 : B> tab;
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+        uint32_t w[B], o[16];
+#pragma unroll
+        for (int i = 0; i < B; ++i) w[i] = lds_u32((g ? words1 : words0) + i * 128);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const int h = 2 * g + (c >> 1);
+            if constexpr (B == 8) {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const uint32_t ww = w[2 * c + (e >> 1)] >> (16 * (e & 1));
+                    const __nv_bfloat162 hh = __floats2bfloat162_rn(__fmul_rn(lut8[(ww & 255u) << 5], s[h]), __fmul_rn(lut8[((ww >> 8) & 255u) << 5], s[h]));
+                    o[4 * c + e] = *reinterpret_cast<const uint32_t*>(&hh);
+                }
+            } else {
+                if ((c & 1) == 0 && (h == 0 || nsc == 4 || (nsc == 2 && h == 2))) tab.build(s[h]);
+                const uint32_t sel = chunk_selector<B>(w, c);
+                uint32_t selA = sel, selB = 0u;
+                if constexpr (B == 4) { selA = sel & 0x77777777u; selB = ((sel >> 1) & 0x44444444u) | 0x32103210u; }
+                tab.lookup4(selA, selB, o[4 * c], o[4 * c + 1]);
+                tab.lookup4(selA >> 16, selB >> 16, o[4 * c + 2], o[4 * c + 3]);
+            }
+        }
+        tmem_st16(taddr + 16 * g, o);
+    }
+}
+
 __device__ __forceinline__ float4 ld_dsmem_f32x4(uint32_t local_addr, uint32_t rank) {
     uint32_t ra;
     float4 v;
@@ -119,7 +180,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int B, bool BWD>
+template <int B, bool BWD, bool TA>
 __global__ void __launch_bounds__(kSwThreads, 1)
 tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT,
                       const __grid_constant__ CUtensorMap tmF, const SwapParams p) {
@@ -128,9 +189,10 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int half_box = p.box >> 1, half_bytes = half_box * 128;
     const int x_bytes = p.nbox * half_bytes;
-    const int stage_bytes = kSwWBytes + x_bytes;                         // [weight tile][token boxes]
+    constexpr int W_BYTES = TA ? 0 : kSwWBytes;
+    const int stage_bytes = W_BYTES + x_bytes;                           // [weight tile][token boxes]
     uint8_t* p_ring = base + p.ss * stage_bytes;
-    uint8_t* tail = p_ring + p.sp * P_BYTES;
+    uint8_t* tail = base + p.tail_off;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);     // full[8], empty[8], full_p[8], empty_p[8], fbar[2], acc_full, drain
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 36 * 8);
     volatile int* abort_s = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -187,7 +249,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         // ------------------------------------------------------------------ this CTA's half of token box `warp`
         RingAt r(0, p.ss);
         const int row = m0 + warp * p.box + static_cast<int>(rank) * half_box;
-        uint32_t dst0 = ring + kSwWBytes + warp * half_bytes;
+        uint32_t dst0 = ring + W_BYTES + warp * half_bytes;
         int k = q_lo * BK;
         int step = 0;
         for (; step < total; ++step, r.advance(1, p.ss), k += BK) {
@@ -246,7 +308,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         } else {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 15) |
                                    (static_cast<uint32_t>(p.box >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
-            const uint32_t a0 = desc_lo(ring, BWD ? 8192 : 16), b0 = desc_lo(ring + kSwWBytes, 16);
+            const uint32_t a0 = desc_lo(ring, BWD ? 8192 : 16), b0 = desc_lo(ring + W_BYTES, 16);
             const uint32_t stage16 = stage_bytes >> 4, box16 = half_bytes >> 4;
             constexpr uint32_t ka = (BWD ? 2048 : 32) >> 4;            // 16 contraction elements further: rows down, or columns along
             const uint16_t pair_mask = static_cast<uint16_t>(3u << (cluster_rank() & ~1u));
@@ -259,7 +321,16 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                 __syncwarp();
                 tc_fence_after();
                 const uint32_t a = a0 + r.s * stage16, b = b0 + r.s * stage16;
-                if (elect_one()) {
+                if (TA) {
+                    const uint32_t at = tmem + kSwTmemA + r.s * 32;
+                    if (elect_one()) {
+                        tc_mma2_ta(tmem, at, b, idesc, acc);
+                        tc_mma2_ta(tmem, at + 8, b + 2, idesc, 1u);
+                        tc_mma2_ta(tmem, at + 16, b + 4, idesc, 1u);
+                        tc_mma2_ta(tmem, at + 24, b + 6, idesc, 1u);
+                        tc_commit_pair(step + 1 < total ? empty(r.s) : acc_full, pair_mask);
+                    }
+                } else if (elect_one()) {
                     tc_mma2_lo(tmem, a, b, idesc, acc);
                     tc_mma2_lo(tmem, a + ka, b + 2, idesc, 1u);
                     tc_mma2_lo(tmem, a + 2 * ka, b + 4, idesc, 1u);
@@ -340,9 +411,17 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     const uint32_t src = wsrc + rp.s * P_BYTES;
                     ok = wait2(empty(rw.s), rw.ph ^ 1, full_p(rp.s), rp.ph, ctl, 55, 56);
                     if (!ok) break;
-                    dequant_row64<B>(src + slab_row_slot(lane, 0, kt) * 4, src + (B * 32 + slab_row_slot(lane, 1, kt)) * 4, s, nsc,
-                                     dst0 + stage, xr, lut8 + lane);
-                    fence_proxy_async();            // make the generic-proxy stores visible to the tensor core
+                    if constexpr (TA) {
+                        tc_fence_after();               // the tensor core is done with this stage's columns
+                        dequant_row64_tmem<B>(src + slab_row_slot(lane, 0, kt) * 4, src + (B * 32 + slab_row_slot(lane, 1, kt)) * 4, s, nsc,
+                                              tmem + (static_cast<uint32_t>(wi * 32) << 16) + kSwTmemA + rw.s * 32, lut8 + lane);
+                        tmem_st_wait();
+                        tc_fence_before();
+                    } else {
+                        dequant_row64<B>(src + slab_row_slot(lane, 0, kt) * 4, src + (B * 32 + slab_row_slot(lane, 1, kt)) * 4, s, nsc,
+                                         dst0 + stage, xr, lut8 + lane);
+                        fence_proxy_async();            // make the generic-proxy stores visible to the tensor core
+                    }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(empty_p(rp.s));
                     rp.advance(4, p.sp);
@@ -350,7 +429,25 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     // rank-r step: the weight-side operand ([L1] rows or L2 rows) comes by TMA
                     ok = wait(empty(rw.s), rw.ph ^ 1, ctl, 57);
                     if (!ok) break;
-                    if (wi == 0) {
+                    if constexpr (TA) {
+                        // this lane's row of L1, straight from global memory (r is a multiple of 16)
+                        tc_fence_after();
+                        const int n = c0 + row_local, j0 = (step - nq) * BK;
+#pragma unroll
+                        for (int g = 0; g < 2; ++g) {
+                            uint32_t o[16];
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                const int j = j0 + g * 32 + c * 8;
+                                uint4 v = make_uint4(0u, 0u, 0u, 0u);
+                                if (n < q.N && j < p.r) v = __ldg(reinterpret_cast<const uint4*>(p.L1 + static_cast<size_t>(n) * p.r + j));
+                                o[4 * c] = v.x; o[4 * c + 1] = v.y; o[4 * c + 2] = v.z; o[4 * c + 3] = v.w;
+                            }
+                            tmem_st16(tmem + (static_cast<uint32_t>(wi * 32) << 16) + kSwTmemA + rw.s * 32 + 16 * g, o);
+                        }
+                        tmem_st_wait();
+                        tc_fence_before();
+                    } else if (wi == 0) {
                         const int d = step - nq;
                         if (lane == 0) {
                             if (!BWD) {
@@ -464,7 +561,7 @@ inline int tc_max_clusters(int n) {
     if (known >= 0) return known;
     const int fallback[4] = {74, 33, 22, 15};
     int got = 0;
-    auto kern = tc_swap_linear_kernel<3, false>;
+    auto kern = tc_swap_linear_kernel<3, false, false>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2, 1, n / 2);
     cfg.blockDim = dim3(kSwThreads);
@@ -585,10 +682,10 @@ inline const SwapPlan& swap_plan(int b0, int64_t M, int64_t out_cols, int steps_
     return e.plan;
 }
 
-template <int B, bool BWD>
+template <int B, bool BWD, bool TA>
 inline int launch_swap(const CUtensorMap& tX, const CUtensorMap& tT, const CUtensorMap& tF, const SwapParams& p, const SwapPlan& pl,
-                       int pairs, cudaStream_t st, bool after_pre) {
-    auto kern = tc_swap_linear_kernel<B, BWD>;
+                       int smem, int pairs, cudaStream_t st, bool after_pre) {
+    auto kern = tc_swap_linear_kernel<B, BWD, TA>;
     static bool attr_done = false;
     if (!attr_done) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
@@ -600,7 +697,7 @@ inline int launch_swap(const CUtensorMap& tX, const CUtensorMap& tT, const CUten
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * pairs, pl.chunks, pl.ks);
     cfg.blockDim = dim3(kSwThreads);
-    cfg.dynamicSmemBytes = pl.smem;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;      // a pair, and the slices of its contraction
@@ -629,6 +726,23 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     p.steps_d = (r + BK - 1) / BK;
     p.c_base = c_base;
     p.nbox = pl.nbox; p.box = pl.box; p.ss = pl.ss; p.sp = pl.sp; p.tmem_cols = pl.tmem_cols;
+    p.L1 = static_cast<const __nv_bfloat16*>(L1); p.r = r;
+    int smem = pl.smem;
+    p.tail_off = pl.ss * (kSwWBytes + pl.nbox * pl.box * 64) + pl.sp * 1024 * q.b0;
+    const bool ta = !backward && pl.nbox == 1;      // (256 columns of accumulators and eight stages of 32 columns fill tensor memory)
+    if (ta) {
+        // Without weight tiles eight stages of both rings always fit (256 tokens, 8-bit codes: 230,912 of 232,448 bytes, code book
+        // included), so a group's codes of step j - sp are its own (see swap_rings); the token stages alone hold the accumulators
+        // that a sliced contraction lays over them (8 x 64 = 512 bytes per token).
+        const int fixed = 1024 + kSwTail + (q.b0 == 8 ? 32768 : 0), x = pl.box * 64, pk = 1024 * q.b0;
+        p.ss = kSwMaxStages;
+        p.sp = (kSmemLimit - fixed - p.ss * x) / pk;
+        if (p.sp > kSwMaxStages) p.sp = kSwMaxStages;
+        p.tail_off = p.ss * x + p.sp * pk;
+        smem = fixed + p.tail_off;
+        if (smem < 120 * 1024) smem = 120 * 1024;      // no second user of tensor memory on the SM
+        p.tmem_cols = 512;
+    }
     CUtensorMap tX, tT, tF;
     if (!make_map(&tX, A, M, C, pl.box / 2)) return LQLORA_ERR_CUDA;
     if (r > 0) {
@@ -639,11 +753,17 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
         tT = tX; tF = tX;
     }
     const int pairs = (cols + 255) / 256;
+    auto go = [&](auto bits) {
+        constexpr int B = decltype(bits)::value;
+        if (backward) return launch_swap<B, true, false>(tX, tT, tF, p, pl, smem, pairs, st, after_pre);
+        if (ta) return launch_swap<B, false, true>(tX, tT, tF, p, pl, smem, pairs, st, after_pre);
+        return launch_swap<B, false, false>(tX, tT, tF, p, pl, smem, pairs, st, after_pre);
+    };
     switch (q.b0) {
-        case 2: return backward ? launch_swap<2, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<2, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
-        case 3: return backward ? launch_swap<3, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<3, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
-        case 4: return backward ? launch_swap<4, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<4, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
-        default: return backward ? launch_swap<8, true>(tX, tT, tF, p, pl, pairs, st, after_pre) : launch_swap<8, false>(tX, tT, tF, p, pl, pairs, st, after_pre);
+        case 2: return go(std::integral_constant<int, 2>());
+        case 3: return go(std::integral_constant<int, 3>());
+        case 4: return go(std::integral_constant<int, 4>());
+        default: return go(std::integral_constant<int, 8>());
     }
 }
 
