@@ -332,7 +332,7 @@ int lqlora_selftest_bounded_wait(void* workspace_dev, int64_t budget_cycles, voi
  *   LQLORA_PATH_TC_ONE   tcgen05 kernel on transposed output tiles (any number of rows), contraction split over a cluster
  *   LQLORA_PATH_TC_PAIR  tcgen05 kernel, CTA pairs (cta_group::2) on [512, 256] output tiles
  * *splits (may be NULL) receives the number of slices of one output tile's contraction (1 for [512, 256] tiles and the
- * fall-back).  Returns a negative lqlora_status for invalid arguments.  Host only, nothing is enqueued; with a device present the
+ * fall-back; for the weight-streaming kernels the most runs that can share a tile).  Returns a negative lqlora_status for invalid arguments.  Host only, nothing is enqueued; with a device present the
  * first call of a process asks the driver how many thread-block clusters fit on it. */
 enum { LQLORA_PATH_PLAIN = 0, LQLORA_PATH_STREAM = 1, LQLORA_PATH_TC_ONE = 2, LQLORA_PATH_TC_PAIR = 3 };
 int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, int64_t M, int backward, int* splits);

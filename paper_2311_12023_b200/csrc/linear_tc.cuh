@@ -611,11 +611,10 @@ constexpr int kTcMinRowsBwd = 9;  // input gradient of matrices with at least 20
 
 inline bool tc_supported(const QView& q, int r, int64_t M, bool backward) {
     (void)r;
-    // Both lines were drawn against a kernel with the tokens as rows of its tiles, which the transposed tiles replaced; these would win
-    // earlier (us as a graph, streaming / transposed, 2-, 3-, 4- and 8-bit codes of 8192 x 8192): forward 1 row 20 / 25, 22 / 26,
-    // 30 / 32, 44 / 45; 8 rows 26 / 25, 28 / 26, 35 / 32, 50 / 46; 16 rows 34 / 25, 35 / 26, 43 / 32, 62 / 46; input gradient 1 row 27 / 26,
-    // 29 / 27, 40 / 33, 60 / 46; 8 rows 33 / 26, 36 / 27, 46 / 33, 62 / 46.  One row of a larger matrix stays with the streaming kernel:
-    // 28672 x 8192 NF3 forward 70 / 91 (16 rows 104 / 91), 8192 x 28672 NF2 63 / 68 and 81 / 85 (input gradient).
+    // us as a graph, streaming / transposed, 2-, 3-, 4- and 8-bit codes of 8192 x 8192: forward 1 row 17 / 25, 19 / 26, 25 / 32, 30 / 45; 8 rows
+    // 20 / 25, 22 / 26, 28 / 32, 33 / 46; 16 rows 26 / 25, 29 / 26, 35 / 32, 45 / 46; input gradient 1 row 26 / 26, 27 / 27, 30 / 33, 37 / 46; 8 rows
+    // 29 / 26, 30 / 27, 33 / 33, 40 / 46.  Small matrices favour the transposed tiles for more than eight rows of an input gradient: 4096 x 4096 NF3 at
+    // 12 rows 13.8, at 8 rows streaming 18.
     const int min_rows = (backward && q.N >= 2048) ? kTcMinRowsBwd : kTcMinRows;
     if (M < min_rows) return false;
     if (q.N % 8 != 0 || q.K % 8 != 0) return false;
