@@ -115,9 +115,10 @@ __device__ __forceinline__ uint2 ldg_codes(const uint32_t* p) {
 
 // fl(v / levels), levels = 1, 3, 7 or 127: one Newton step on the product with the rounded reciprocal (Markstein 1990; Brisebarre,
 // Muller and Raina 2004, division by a constant).  Equal to the IEEE quotient for every mantissa while the residual does not
-// underflow; smaller v (and 0) take the division.
+// underflow; smaller v (and 0) take the division, and so does infinity (an fp16 second-level scale of block maxima above 65504),
+// whose residual is not a number.
 __device__ __forceinline__ float scale_quotient(float v, float levels) {
-    if (v < 1e-27f) return __fdiv_rn(v, levels);
+    if (v < 1e-27f || v > 3.402823466e38f) return __fdiv_rn(v, levels);
     const float rc = levels == 127.0f ? 1.0f / 127.0f : levels == 7.0f ? 1.0f / 7.0f : levels == 3.0f ? 1.0f / 3.0f : 1.0f;
     const float q0 = __fmul_rn(v, rc);
     return __fmaf_rn(__fmaf_rn(-q0, levels, v), rc, q0);
@@ -241,15 +242,16 @@ __global__ void __maxnreg__(kMaxRegs) stream_fwd_kernel(const Params p) {
         }
         return s;
     };
-    auto build_run = [&](const ScaleRun& s) {
+    auto build_run = [&](const ScaleRun& s, int run) {
         const float sig0 = scale_quotient(s.v0, q.levels);
         float sig1 = sig0;
         if (s.n0 < 8) sig1 = scale_quotient(s.v1, q.levels);
         float* dst = stab + (lane >> 4) * 8 * p.sstr + (lane & 15);
+        const int have = q.KB - run * 16 - (lane >> 4) * 8;    // blocks behind the last column: zero, whatever the group's scale is
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const uint32_t c = ((j < 4 ? s.codes.x : s.codes.y) >> (8 * (j & 3))) & 255u;
-            dst[j * p.sstr] = __fmul_rn(static_cast<float>(c), j < s.n0 ? sig0 : sig1);
+            dst[j * p.sstr] = j < have ? __fmul_rn(static_cast<float>(c), j < s.n0 ? sig0 : sig1) : 0.0f;
         }
     };
 
@@ -330,7 +332,7 @@ __global__ void __maxnreg__(kMaxRegs) stream_fwd_kernel(const Params p) {
         for (int i = a; i < b; ++i) {
             if (fresh) {
                 __syncwarp();
-                build_run(sr);
+                build_run(sr, run);
                 __syncwarp();
                 int ntr = tr, nrun = run + 1;
                 if (nrun * 16 >= q.KB) { ntr = tr + 1; nrun = 0; }

@@ -1,5 +1,7 @@
 """Weight-streaming kernels: edges of units, runs, scale runs, second-level groups and rank-r units."""
+import numpy as np
 import pytest
+import torch
 
 from paper_2311_12023_b200 import binding, inputs
 from test_gpu_linear import C, run_case
@@ -29,3 +31,26 @@ def test_wide_blocks(b0, B0, M):
     A = inputs.student_t(6300 + b0, (N, K), 5.0, 0.02)
     l1b, l2b = inputs.lowrank_factors(6301, N, K, 64, 0.03)
     run_case(A, l1b, l2b, C(b0, B0, 8, 16, 32), M, seed=6400 + M)
+
+
+# block maxima above 65504 with fp16 second-level scales: the group's scale is infinite in lqlora_dequant, and so are its weights;
+# the last unit of 320 columns has blocks behind the last one, which must add nothing
+@pytest.mark.parametrize("K", [512, 320])
+@pytest.mark.parametrize("b0,B0,M", [(2, 16, 1), (2, 64, 16), (3, 64, 3), (4, 32, 1), (8, 64, 9)])
+def test_infinite_second_level_scale(b0, B0, M, K):
+    N = 256
+    cfg = C(b0, B0, 8, 64, 16)
+    A = inputs.gaussian(6500, (N, K), 0.02)
+    whole = 64 * B0 * K // np.gcd(64 * B0, K) // K               # rows that end where a group ends
+    A[:whole] = 7e4
+    q = binding.encode(torch.from_numpy(A).cuda(), cfg)
+    d16 = binding.dequant(q)[1]
+    assert bool(torch.isposinf(d16[:whole]).all()) and bool(torch.isfinite(d16[whole:]).all())
+    assert binding.linear_path(N, K, cfg, 0, M, False) == binding.PATH_STREAM
+    x = torch.ones(M, K, dtype=torch.bfloat16, device="cuda")
+    Y = binding.linear_fwd(q, None, None, x)
+    assert bool(torch.isposinf(Y[:, :whole]).all())
+    want = x.float() @ d16[whole:].float().T
+    assert float((Y[:, whole:].float() - want).norm() / want.norm()) < 5e-3
+    dY = torch.ones(M, N, dtype=torch.bfloat16, device="cuda")
+    assert bool(torch.isposinf(binding.linear_bwd_input(q, None, None, dY)).all())
