@@ -74,9 +74,12 @@ def lib() -> ctypes.CDLL:
         L.lqlora_unpack.argtypes = [ctypes.POINTER(CQMatrix), vp, vp]
         L.lqlora_dequant.argtypes = [ctypes.POINTER(CQMatrix), vp, vp, vp]
         L.lqlora_linear_workspace_bytes.argtypes = [i64, i64, ctypes.POINTER(CConfig), ci, i64, ctypes.POINTER(sz)]
-        # (the quantized matrix as a plain pointer: byref of a CQMatrix, or the bytes of one)
-        L.lqlora_linear_fwd.argtypes = [vp, vp, vp, ci, vp, i64, vp, vp, sz, vp]
-        L.lqlora_linear_bwd_input.argtypes = [vp, vp, vp, ci, vp, i64, vp, vp, sz, vp]
+        L.lqlora_linear_fwd.argtypes = [ctypes.POINTER(CQMatrix), vp, vp, ci, vp, i64, vp, vp, sz, vp]
+        L.lqlora_linear_bwd_input.argtypes = [ctypes.POINTER(CQMatrix), vp, vp, ci, vp, i64, vp, vp, sz, vp]
+        # the same two with the quantized matrix as the bytes of a CQMatrix (indexing gives a function object of its own)
+        L.linear_fwd_packed, L.linear_bwd_input_packed = L["lqlora_linear_fwd"], L["lqlora_linear_bwd_input"]
+        for f in (L.linear_fwd_packed, L.linear_bwd_input_packed):
+            f.argtypes = [ctypes.c_char_p, vp, vp, ci, vp, i64, vp, vp, sz, vp]
         L.lqlora_lora_grads_workspace_bytes.argtypes = [i64, i64, ci, i64, ctypes.POINTER(sz)]
         L.lqlora_lora_grads.argtypes = [vp, vp, ci, i64, i64, vp, vp, i64, vp, vp, vp, sz, vp]
         L.lqlora_linear_intermediate_offset.argtypes = [i64, i64, ctypes.POINTER(CConfig), ci, i64, ci, ctypes.POINTER(sz)]
@@ -301,7 +304,7 @@ def _linear(fn, name, q, L1, L2, A, out_cols, out, workspace):
 def linear_fwd(q: QMatrix, L1, L2, X: torch.Tensor, out=None, workspace=None) -> torch.Tensor:
     """lqlora_linear_fwd: Y = X deq(Q)^T + (X L2^T) L1^T, bf16 [M, N]."""
     assert X.shape[1] == q.K
-    return _linear(lib().lqlora_linear_fwd, "lqlora_linear_fwd", q, L1, L2, X, q.N, out, workspace)
+    return _linear(lib().linear_fwd_packed, "lqlora_linear_fwd", q, L1, L2, X, q.N, out, workspace)
 
 
 def linear_fwd_static(q: QMatrix, L1, L2, X: torch.Tensor, out: Optional[torch.Tensor] = None) -> torch.Tensor:
@@ -330,7 +333,7 @@ def linear_fwd_static(q: QMatrix, L1, L2, X: torch.Tensor, out: Optional[torch.T
 def linear_bwd_input(q: QMatrix, L1, L2, dY: torch.Tensor, out=None, workspace=None) -> torch.Tensor:
     """lqlora_linear_bwd_input: dX = dY deq(Q) + (dY L1) L2, bf16 [M, K]."""
     assert dY.shape[1] == q.N
-    return _linear(lib().lqlora_linear_bwd_input, "lqlora_linear_bwd_input", q, L1, L2, dY, q.K, out, workspace)
+    return _linear(lib().linear_bwd_input_packed, "lqlora_linear_bwd_input", q, L1, L2, dY, q.K, out, workspace)
 
 
 def lora_grads_workspace_bytes(N: int, K: int, r: int, M: int) -> int:

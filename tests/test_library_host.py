@@ -4,6 +4,7 @@ is launched here."""
 import ctypes
 import os
 import re
+import types
 
 import numpy as np
 import pytest
@@ -101,6 +102,24 @@ def test_invalid_arguments_are_rejected_before_any_launch(binding):
     assert L.lqlora_encode(None, ctypes.byref(q), fake, ws, None) == -3
     assert L.lqlora_encode(fake, ctypes.byref(q), fake, 8, None) == -5
     assert binding.status_string(-7) == "device-side wait timed out"
+
+
+def test_linear_entry_points_take_a_matrix_and_nothing_else_for_one(binding):
+    """The typed prototypes: a CQMatrix by value or by reference is taken, an address or bytes in its place refused before the call."""
+    L = binding.lib()
+    fake = 0x10000      # never dereferenced: validation fails first
+    q = binding.CQMatrix(fake, fake, fake, 128, 128, binding._cfg(inputs.QuantConfig(3, 64, 8, 256, 32)))
+    for fn in (L.lqlora_linear_fwd, L.lqlora_linear_bwd_input):
+        for arg in (q, ctypes.byref(q), ctypes.pointer(q)):
+            assert fn(arg, fake, fake, 64, fake, 0, fake, fake, 1 << 30, None) == -2      # M
+        for arg in (fake, bytes(q)):
+            with pytest.raises(ctypes.ArgumentError):
+                fn(arg, fake, fake, 64, fake, 0, fake, fake, 1 << 30, None)
+    # what the binding's own calls pass
+    packed = binding.QMatrix(*(types.SimpleNamespace(data_ptr=lambda: fake) for _ in range(3)), 128, 128, inputs.QuantConfig(3, 64, 8, 256, 32)).cbytes()
+    assert packed == bytes(q)
+    for fn in (L.linear_fwd_packed, L.linear_bwd_input_packed):
+        assert fn(packed, fake, fake, 64, fake, 0, fake, fake, 1 << 30, None) == -2
 
 
 def test_no_fallback_without_a_device(binding):
