@@ -293,7 +293,8 @@ def _linear(fn, name, q, L1, L2, A, out_cols, out, workspace):
         assert L1.dtype == torch.bfloat16 and L2.dtype == torch.bfloat16 and L1.is_contiguous() and L2.is_contiguous()
         assert L1.shape == (q.N, r) and L2.shape == (r, q.K)
     if out is None:
-        out = A.new_empty((M, out_cols))
+        # (new_empty takes 1.6 us instead of 2.5, but would hand the class of a tensor subclass on to the result)
+        out = A.new_empty((M, out_cols)) if type(A) is torch.Tensor else torch.empty((M, out_cols), dtype=torch.bfloat16, device=A.device)
     if workspace is None:
         workspace = alloc_workspace(q, r, M)
     _check(fn(q.cbytes(), _ptr(L1), _ptr(L2), r, A.data_ptr(), M, out.data_ptr(), workspace.data_ptr(),

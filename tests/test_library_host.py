@@ -122,6 +122,20 @@ def test_linear_entry_points_take_a_matrix_and_nothing_else_for_one(binding):
         assert fn(packed, fake, fake, 64, fake, 0, fake, fake, 1 << 30, None) == -2
 
 
+def test_result_of_a_tensor_subclass_is_a_plain_tensor(binding, monkeypatch):
+    import torch
+
+    class Tagged(torch.Tensor):
+        is_cuda = True                        # host tensors in place of device ones: the call itself is replaced
+
+    monkeypatch.setattr(binding, "_stream", lambda: None)
+    cfg = inputs.QuantConfig(3, 64, 8, 256, 32)
+    q = binding.QMatrix(*(torch.zeros(n, dtype=torch.uint8) for n in binding.packed_sizes(128, 64, cfg)[:3]), 128, 64, cfg)
+    X = torch.zeros(4, 64, dtype=torch.bfloat16).as_subclass(Tagged)
+    out = binding._linear(lambda *a: 0, "", q, None, None, X, 128, None, torch.zeros(512, dtype=torch.uint8))
+    assert type(out) is torch.Tensor and out.dtype == torch.bfloat16 and out.shape == (4, 128) and not out.requires_grad
+
+
 def test_no_fallback_without_a_device(binding):
     import torch
     if torch.cuda.is_available():
