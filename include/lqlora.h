@@ -339,11 +339,18 @@ int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, in
 
 /* lqlora_encode finds the nearest 8-bit code (Sec. 2.2: c_j = argmin_k |q~_k - u_j / s_i|) with a bin table over [-1, 1]:
  * every bin holds at most one decision threshold (the midpoint of two neighbouring code-book entries), and inputs
- * closer than 1e-6 to a threshold are decided with the exact IEEE quotient.  (2-, 3- and 4-bit codes are found on a curve through
- * the thresholds, with the same exact decision next to them.)  This returns the smallest distance
+ * closer than 1e-6 to a threshold are decided with the exact IEEE quotient.  This returns the smallest distance
  * between a threshold and a bin edge for the b0-bit table; it must exceed that 1e-6 by a wide margin for the
- * fast and the exact route to agree (checked by the host tests).  Negative for an invalid b0.  Host only. */
+ * fast and the exact route to agree (checked by the host tests).  Only the 8-bit table is in use (for 2, 3 and 4 bits the
+ * figure is that of the table such codes would have).  Negative for an invalid b0.  Host only. */
 double lqlora_encode_search_clearance(int b0);
+
+/* 2-, 3- and 4-bit codes are the integer part of a curve through the thresholds, whose fraction says which inputs are too close to
+ * one and are decided with the exact quotient.  This evaluates the curve on the host, in fp32 as the kernel does, for all floats around
+ * the thresholds and every 61st one elsewhere in [-1 - 4 ulp, 1 + 4 ulp], and returns the smallest distance to a threshold of a
+ * float that is taken from the curve; -2 if one of them gets a wrong code, -1 for another b0.  It must exceed the 2.4e-7 that the kernel's
+ * quotient can be off by.  Host only; takes a fraction of a second. */
+double lqlora_encode_curve_clearance(int b0);
 
 /* Number of kernel launches the library has enqueued since it was loaded (for launch accounting). */
 int64_t lqlora_launch_count(void);

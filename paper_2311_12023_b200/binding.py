@@ -24,7 +24,7 @@ EXPORTS = [
     "lqlora_linear_bwd_input", "lqlora_workspace_status", "lqlora_linear_path", "lqlora_launch_count",
     "lqlora_status_string", "lqlora_encode_host", "lqlora_linear_fwd_host", "lqlora_linear_bwd_input_host",
     "lqlora_static_scratch_bytes", "lqlora_linear_fwd_static", "lqlora_static_scratch_status",
-    "lqlora_encode_search_clearance",
+    "lqlora_encode_search_clearance", "lqlora_encode_curve_clearance",
     "lqlora_lora_grads_workspace_bytes", "lqlora_lora_grads",
     "lqlora_lq_workspace_bytes", "lqlora_lq_decompose", "lqlora_to_bf16", "lqlora_assign_configs",
     "lqlora_unpack_scales", "lqlora_linear_qfactors_workspace_bytes", "lqlora_linear_fwd_qfactors",
@@ -91,6 +91,8 @@ def lib() -> ctypes.CDLL:
         L.lqlora_static_scratch_bytes.restype = sz
         L.lqlora_encode_search_clearance.argtypes = [ci]
         L.lqlora_encode_search_clearance.restype = ctypes.c_double
+        L.lqlora_encode_curve_clearance.argtypes = [ci]
+        L.lqlora_encode_curve_clearance.restype = ctypes.c_double
         L.lqlora_linear_fwd_static.argtypes = [ctypes.POINTER(CQMatrix), vp, vp, ci, vp, i64, vp, vp]
         L.lqlora_static_scratch_status.argtypes = [vp]
         L.lqlora_selftest_bounded_wait.argtypes = [vp, i64, vp]

@@ -36,14 +36,15 @@ __device__ __forceinline__ uint32_t nearest_code(float x, const float* __restric
 // coefficients come from HostTables; 2^B is added to E, so the integer part stands in the top B mantissa bits, and half of kLim units in
 // the last place are added too, so that the fraction bits below kLim mean "within about 1e-6 of a threshold": those elements are decided
 // exactly.  Evaluated in fp32 for every float in [-1 - 4 ulp, 1 + 4 ulp]: every other x gives the right code, and lies at least 8.2e-7
-// from any threshold (x^ below differs from the quotient by at most 2.4e-7).  Two elements per instruction (fma.f32x2).
+// from any threshold (x^ below differs from the quotient by at most 2.4e-7); lqlora_encode_curve_clearance repeats that on a sample.
+// Two elements per instruction (fma.f32x2).
 //
 // What bounds the kernel: loads in flight (a CTA loads, then computes, then stores) and instruction issue, 18 instructions per 3-bit weight
 // (25.6 before, with a saturating sum over the thresholds; 4-bit codes looked a bin table up in shared memory).  us per call with the
 // scale kernel, before / now: 8192 x 8192 2 bits 61 / 59, 3 bits 75 / 70, blocks of 16 82 / 75, 4 bits 91 / 81; 11008 x 4096 4 bits
 // 65.5 / 58.  The scalar form of the same polynomials: 4 bits 88 and 63.
 template <int B> struct Curve {
-    static constexpr int NE = B == 2 ? 2 : B == 3 ? 4 : 8, NO = B == 2 ? 1 : B == 3 ? 4 : 7;
+    static constexpr int NE = curve_even(B), NO = curve_odd(B);
     static constexpr uint32_t kMask = (1u << (23 - B)) - 1u;               // fraction bits
     static constexpr uint32_t kLim = curve_limit(B);
 };
@@ -159,10 +160,10 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
     }
     // 8-bit codes (255 thresholds) find their code through a bin table, the others on a curve through the thresholds
     constexpr bool kUseBins = (B == 8);
-    const int nb = kUseBins ? c_nbins[bits_index(B)] : 0;
+    const int nb = kUseBins ? c_nbins : 0;
     if constexpr (kUseBins) {
         for (int i = threadIdx.x; i <= nb; i += 256) {
-            const BinEntry e = g_bins[bits_index(B)][i];       // global memory: coalesced (the constant bank would serialize the lanes)
+            const BinEntry e = g_bins[i];       // global memory: coalesced (the constant bank would serialize the lanes)
             bins[i] = make_float2(e.thr, __int_as_float(e.base));
         }
     }

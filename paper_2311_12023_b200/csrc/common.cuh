@@ -148,6 +148,8 @@ __constant__ float c_threshold[4][256];
 // 2-, 3- and 4-bit encoder: coefficients of the curve through the thresholds (E, then O; each twice, for two elements per
 // instruction), and the fraction (in units of the last place) below which a value counts as close to a threshold.
 constexpr int kCurveCoefs = 15;
+__host__ __device__ constexpr int curve_even(int b0) { return b0 == 2 ? 2 : b0 == 3 ? 4 : 8; }      // coefficients of E, of O
+__host__ __device__ constexpr int curve_odd(int b0) { return b0 == 2 ? 1 : b0 == 3 ? 4 : 7; }
 __host__ __device__ constexpr uint32_t curve_limit(int b0) { return b0 == 2 ? 10u : b0 == 3 ? 16u : 12u; }
 __constant__ float2 c_curve[3][kCurveCoefs + 1];
 
@@ -156,8 +158,8 @@ __constant__ float2 c_curve[3][kCurveCoefs + 1];
 // number of thresholds below the bin); entry nb serves x slightly above 1.
 constexpr int kMaxBins = 1280;
 struct BinEntry { float thr; int base; };
-__device__ BinEntry g_bins[4][kMaxBins + 1];
-__constant__ int c_nbins[4];
+__device__ BinEntry g_bins[kMaxBins + 1];
+__constant__ int c_nbins;
 
 int ensure_tables();                 // uploads the tables to the current device once; LQLORA_OK or error
 const float* host_codebook(int b0);  // 2^b0 floats

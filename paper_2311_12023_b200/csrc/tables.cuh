@@ -4,6 +4,7 @@
 
 #include <atomic>
 #include <cmath>
+#include <cstring>
 #include <mutex>
 #include <utility>
 
@@ -34,12 +35,12 @@ inline double gauss_quantile(double p) {
 struct HostTables {
     float codebook[4][256];
     float threshold[4][256];
-    BinEntry bins[4][kMaxBins + 1];
-    int nbins[4];
+    BinEntry bins[kMaxBins + 1];              // 8-bit codes
+    int nbins;
     float2 curve[3][kCurveCoefs + 1];
     // Bin count for `n - 1` thresholds: the candidate with the largest distance between any threshold and any
     // bin edge among those with at most one threshold per bin.
-    void build_bins(int t, int n) {
+    double best_bins(int t, int n, int* nb_out) const {
         const int lo = (n <= 16) ? 48 : 1000, hi = (n <= 16) ? 96 : kMaxBins;
         int best_nb = 0;
         double best_clear = -1.0;
@@ -57,26 +58,30 @@ struct HostTables {
             }
             if (ok && clear > best_clear) { best_clear = clear; best_nb = nb; }
         }
-        nbins[t] = best_nb;
-        for (int k = 0; k <= kMaxBins; ++k) { bins[t][k].thr = INFINITY; bins[t][k].base = n - 1; }
+        *nb_out = best_nb;
+        return best_clear;
+    }
+    void build_bins() {
+        constexpr int t = 3, n = 256;
+        best_bins(t, n, &nbins);
+        for (int k = 0; k <= kMaxBins; ++k) { bins[k].thr = INFINITY; bins[k].base = n - 1; }
         int below = 0;
-        for (int k = 0; k < best_nb; ++k) {
-            bins[t][k].base = below;
-            bins[t][k].thr = INFINITY;
+        for (int k = 0; k < nbins; ++k) {
+            bins[k].base = below;
+            bins[k].thr = INFINITY;
             while (below + 1 < n) {
-                const double pos = (static_cast<double>(threshold[t][below]) + 1.0) * 0.5 * best_nb;
+                const double pos = (static_cast<double>(threshold[t][below]) + 1.0) * 0.5 * nbins;
                 if (static_cast<int>(std::floor(pos)) != k) break;
-                bins[t][k].thr = threshold[t][below];
+                bins[k].thr = threshold[t][below];
                 ++below;
             }
         }
-        bin_clearance[t] = best_clear;
     }
     // Coefficients of P(x) = E(|x|) + x O(|x|), P(T_k) = k at the thresholds (3-bit codes: and P(1) = 7.55), by Gaussian
     // elimination with row pivoting; 2^b0 and half of the "close to a threshold" range are added to the constant term.
     void build_curve(int b0) {
         const int t = bits_index(b0), n = 1 << b0;
-        const int ne = b0 == 2 ? 2 : b0 == 3 ? 4 : 8, no = b0 == 2 ? 1 : b0 == 3 ? 4 : 7, m = ne + no;
+        const int ne = curve_even(b0), no = curve_odd(b0), m = ne + no;
         double A[kCurveCoefs][kCurveCoefs + 1];
         for (int i = 0; i < m; ++i) {
             const double x = i + 1 < n ? 0.5 * (static_cast<double>(codebook[t][i]) + static_cast<double>(codebook[t][i + 1])) : 1.0;
@@ -104,7 +109,42 @@ struct HostTables {
         }
         for (int j = m; j <= kCurveCoefs; ++j) curve[t][j] = make_float2(0.0f, 0.0f);
     }
-    double bin_clearance[4];
+    // What the encoder takes from the curve, evaluated as the kernel does: every float within 32768 of its neighbours around each threshold,
+    // and every 61st float of [2^-24, 1 + 4 ulp] with both signs.  Smallest distance between a threshold and a float whose fraction does
+    // not call it close to one; -2 if such a float gets a wrong code.
+    double curve_clearance(int b0) const {
+        const int t = bits_index(b0), n = 1 << b0, ne = curve_even(b0), no = curve_odd(b0);
+        double least = 1.0;
+        bool right = true;
+        auto check = [&](uint32_t bits_of_x) {
+            float x;
+            std::memcpy(&x, &bits_of_x, 4);
+            const float y = std::fabs(x);
+            float e = curve[t][ne - 1].x, o = curve[t][ne + no - 1].x;
+            for (int i = ne - 2; i >= 0; --i) e = std::fmaf(e, y, curve[t][i].x);
+            for (int i = no - 2; i >= 0; --i) o = std::fmaf(o, y, curve[t][ne + i].x);
+            const float p = std::fmaf(x, o, e);
+            uint32_t bits;
+            std::memcpy(&bits, &p, 4);
+            if ((bits & ((1u << (23 - b0)) - 1u)) < curve_limit(b0)) return;
+            int below = 0;
+            while (below + 1 < n && x > threshold[t][below]) ++below;
+            right = right && static_cast<int>((bits >> (23 - b0)) & (n - 1)) == below;
+            for (int k = below > 0 ? below - 1 : 0; k <= below && k + 1 < n; ++k)
+                least = std::fmin(least, std::fabs(static_cast<double>(x) - 0.5 * (static_cast<double>(codebook[t][k]) + static_cast<double>(codebook[t][k + 1]))));
+        };
+        constexpr uint32_t kSign = 0x80000000u, kOne = 0x3F800000u + 4u;      // 1 + 4 ulp
+        check(0u);
+        check(kSign);
+        for (uint32_t x = 0x33800000u; x <= kOne; x += 61) { check(x); check(x | kSign); }
+        for (int k = 0; k + 1 < n; ++k) {
+            uint32_t at;
+            std::memcpy(&at, &threshold[t][k], 4);
+            for (uint32_t x = at - 32768u; x != at + 32768u; ++x)
+                if ((x & ~kSign) <= kOne) check(x);
+        }
+        return right ? least : -2.0;
+    }
     HostTables() {
         const int bits[4] = {2, 3, 4, 8};
         const double delta = 0.5 * (1.0 / 30.0 + 1.0 / 32.0);
@@ -127,8 +167,8 @@ struct HostTables {
                 if (static_cast<double>(th) > mid) th = std::nextafterf(th, -INFINITY);
                 threshold[t][i] = th;                       // largest fp32 <= midpoint
             }
-            build_bins(t, n);
         }
+        build_bins();
         for (int b0 = 2; b0 <= 4; ++b0) build_curve(b0);
     }
 };
@@ -154,7 +194,7 @@ int ensure_tables() {
         cudaMemcpyToSymbol(c_threshold, t.threshold, sizeof(t.threshold)) != cudaSuccess ||
         cudaMemcpyToSymbol(c_curve, t.curve, sizeof(t.curve)) != cudaSuccess ||
         cudaMemcpyToSymbol(g_bins, t.bins, sizeof(t.bins)) != cudaSuccess ||
-        cudaMemcpyToSymbol(c_nbins, t.nbins, sizeof(t.nbins)) != cudaSuccess) {
+        cudaMemcpyToSymbol(c_nbins, &t.nbins, sizeof(t.nbins)) != cudaSuccess) {
         cudaGetLastError();
         return LQLORA_ERR_CUDA;
     }
@@ -206,7 +246,13 @@ int lqlora_nf_codebook(int b0, float* out_host) {
 
 double lqlora_encode_search_clearance(int b0) {
     if (!(b0 == 2 || b0 == 3 || b0 == 4 || b0 == 8)) return -1.0;
-    return lq::detail::host_tables().bin_clearance[lq::bits_index(b0)];
+    int nb = 0;
+    return lq::detail::host_tables().best_bins(lq::bits_index(b0), 1 << b0, &nb);
+}
+
+double lqlora_encode_curve_clearance(int b0) {
+    if (!(b0 == 2 || b0 == 3 || b0 == 4)) return -1.0;
+    return lq::detail::host_tables().curve_clearance(b0);
 }
 
 int64_t lqlora_launch_count(void) { return lq::g_launches.load(std::memory_order_relaxed); }

@@ -48,6 +48,14 @@ def test_encoder_bin_table_keeps_thresholds_away_from_bin_edges(binding, b):
     assert binding.lib().lqlora_encode_search_clearance(b) >= 1e-5
 
 
+@pytest.mark.parametrize("b", [2, 3, 4])
+def test_encoder_curve_gives_the_right_code_wherever_it_is_trusted(binding, b):
+    # inputs that the curve does not call close to a threshold: right code, and further from any threshold than the 2 ulp (2.4e-7) by
+    # which the kernel's quotient can differ from the exact one
+    assert binding.lib().lqlora_encode_curve_clearance(b) >= 4.8e-7
+    assert binding.lib().lqlora_encode_curve_clearance(8) == -1.0
+
+
 def test_storage_formula_and_packed_sizes(binding):
     for b0 in (2, 3, 4, 8):
         for B0 in (16, 32, 64, 128, 256):
