@@ -187,6 +187,24 @@ __device__ __forceinline__ Share share_of(const Runs& runs, int piece, int tile)
     return Share{piece - f, runs.of_unit(tile * runs.L + runs.L - 1) - f + 1};
 }
 
+// Four neighbouring sums over the slots, in slot order, eight slots in flight at a time.  The CTA that arrives last at a tile adds them
+// alone; one number and four slots at a time, the round trips to L2 took longer than all else in a call on a small matrix.  us per call in a
+// graph, the ring kernels before these / that / this (3-bit codes, rank 64): input gradient 4096 x 1024, 8 rows, 20 slots 18.5 / 25.9 / 13.7;
+// 768 x 768, 8 rows, 26 slots 16.4 / 20.2 / 10.8; forward 1024 x 4096, 16 rows, 16 slots 15.4 / 21.1 / 10.9; 568 x 11520, 14 rows, no
+// rank-r term, 45 slots 22.6 / 32.9 / 16.7.
+__device__ __forceinline__ float4 sum_slots(const float* src, size_t stride, int slots) {
+    float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int s0 = 0; s0 < slots; s0 += 8) {
+        float4 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = __ldcg(reinterpret_cast<const float4*>(src + min(s0 + u, slots - 1) * stride));
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (s0 + u < slots) { sum.x += v[u].x; sum.y += v[u].y; sum.z += v[u].z; sum.w += v[u].w; }
+    }
+    return sum;
+}
+
 // The scales of a warp's 16 rows and 16 blocks: lane = (row, half of the blocks), eight codes and the (at most two, since
 // B1 >= 16) second-level scales of their groups.
 struct ScaleRun {
@@ -441,12 +459,13 @@ __global__ void __maxnreg__(kMaxRegs) stream_fwd_kernel(const Params p) {
         for (int seg = 0; seg < nseg; ++seg) {
             const int slots = last_s[seg];
             if (slots == 0) continue;
-            for (int e = threadIdx.x; e < 128 * M; e += nthr) {
-                const float* src = p.partial + static_cast<size_t>(e >> 7) * npad + (tr0 + seg) * 128 + (e & 127);
-                float sum = 0.0f;
-#pragma unroll 4
-                for (int sl = 0; sl < slots; ++sl) sum += __ldcg(src + static_cast<size_t>(sl) * M * npad);
-                put_out(e >> 7, (tr0 + seg) * 128 + (e & 127), sum);
+            for (int e = threadIdx.x; e < 32 * M; e += nthr) {
+                const int m = e >> 5, row = (tr0 + seg) * 128 + (e & 31) * 4;
+                const float4 sum = sum_slots(p.partial + static_cast<size_t>(m) * npad + row, static_cast<size_t>(M) * npad, slots);
+                put_out(m, row, sum.x);
+                put_out(m, row + 1, sum.y);
+                put_out(m, row + 2, sum.z);
+                put_out(m, row + 3, sum.w);
             }
         }
     }
@@ -751,12 +770,13 @@ __global__ void __maxnreg__(NT == 1 ? kMaxRegs : 128) stream_bwd_kernel(const Bw
         for (int seg = 0; seg < nseg; ++seg) {
             const int slots = last_s[seg];
             if (slots == 0) continue;
-            for (int e = threadIdx.x; e < 128 * M; e += nthr) {
-                const float* src = p.partial + static_cast<size_t>(e >> 7) * kpad + (w0 + seg) * 128 + (e & 127);
-                float sum = 0.0f;
-#pragma unroll 4
-                for (int sl = 0; sl < slots; ++sl) sum += __ldcg(src + static_cast<size_t>(sl) * M * kpad);
-                put_out(e >> 7, (w0 + seg) * 128 + (e & 127), sum);
+            for (int e = threadIdx.x; e < 32 * M; e += nthr) {
+                const int m = e >> 5, col = (w0 + seg) * 128 + (e & 31) * 4;
+                const float4 sum = sum_slots(p.partial + static_cast<size_t>(m) * kpad + col, static_cast<size_t>(M) * kpad, slots);
+                put_out(m, col, sum.x);
+                put_out(m, col + 1, sum.y);
+                put_out(m, col + 2, sum.z);
+                put_out(m, col + 3, sum.w);
             }
         }
     }

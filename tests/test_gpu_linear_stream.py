@@ -33,6 +33,24 @@ def test_wide_blocks(b0, B0, M):
     run_case(A, l1b, l2b, C(b0, B0, 8, 16, 32), M, seed=6400 + M)
 
 
+# one tile row / a few windows shared by many runs: slots on both sides of the eight that are summed at a time, last columns of a tile
+@pytest.mark.parametrize("M", [1, 5, 16])
+@pytest.mark.parametrize("slots", [2, 7, 8, 9, 17])
+def test_slots_of_a_shared_tile(slots, M):
+    N, K, r = 120, 256 * slots, 32
+    cfg = C(3, 64, 8, 64, 32)
+    assert binding.linear_route(N, K, cfg, r, M, False) == (binding.PATH_STREAM, slots)
+    A = inputs.gaussian(6600 + slots, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(6601, N, K, r, 0.05)
+    run_case(A, l1b, l2b, cfg, M, seed=6700 + M, passes=("fwd",))
+    # input gradient of the transposed shape: 32 rows per unit, one of them the rank-r term
+    N, K = 32 * (slots - 1), 128
+    assert binding.linear_route(N, K, cfg, r, M, True) == (binding.PATH_STREAM, slots)
+    A = inputs.gaussian(6602 + slots, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(6603, N, K, r, 0.05)
+    run_case(A, l1b, l2b, cfg, M, seed=6800 + M, passes=("bwd",))
+
+
 # block maxima above 65504 with fp16 second-level scales: the group's scale is infinite in lqlora_dequant, and so are its weights;
 # the last unit of 320 columns has blocks behind the last one, which must add nothing
 @pytest.mark.parametrize("K", [512, 320])
