@@ -145,6 +145,7 @@ __device__ __forceinline__ float bf16_bits_to_float(uint16_t b) { return __uint_
 // neighbouring code-book entries (x > midpoint  <=>  x > threshold for fp32 x).
 __constant__ float c_codebook[4][256];
 __constant__ float c_threshold[4][256];
+__device__ float g_codebook8[256];     // the 8-bit code book for lanes that read different entries
 // 2-, 3- and 4-bit encoder: coefficients of the curve through the thresholds (E, then O; each twice, for two elements per
 // instruction), and the fraction (in units of the last place) below which a value counts as close to a threshold.
 constexpr int kCurveCoefs = 15;

@@ -172,6 +172,19 @@ __device__ __forceinline__ float lut8_at(uint32_t lut, uint32_t byte_offset) {
     asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(lut + byte_offset));
     return v;
 }
+// Fills it (256, 384 or 512 threads): a warp reads 32 entries with one load and hands them round.  (Read from constant memory, 16 entries per
+// warp one after the other in front of the first codes, 8-bit calls on small matrices were slower than the kernels before; us in a graph, those /
+// that / this, one row: 1024 x 1024 rank 64 8.6 / 9.4 / 8.4, without a rank-r term 10.4 / 11.2 / 10.4.)
+__device__ __forceinline__ void fill_lut8(uint8_t* lut) {
+    const int lane = threadIdx.x & 31;
+    for (int w = threadIdx.x >> 5; w < 16; w += blockDim.x >> 5) {
+        const int first = (w & 7) * 32, half = (w >> 3) * 16;
+        const float mine = g_codebook8[first + lane];
+#pragma unroll
+        for (int j = 0; j < 16; ++j)
+            reinterpret_cast<float*>(lut)[(first + half + j) * 32 + lane] = __shfl_sync(0xffffffffu, mine, half + j);
+    }
+}
 __device__ __forceinline__ void dequant8_lut(const uint32_t (&w)[8], int c, uint32_t lut, float s, uint32_t (&o)[4]) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
@@ -233,11 +246,6 @@ __global__ void __maxnreg__(kMaxRegs) stream_fwd_kernel(const Params p) {
     const int off1 = (hs >> 1) * (64 * B) + B * 32 + slab_row_slot(row_in_slab, 1, t);
     const int wrap_words = (kUnitTiles * L - q.ktiles) * (256 * B);      // from the end of a ragged tile row to the next one
     const int run_shift = q.logB0 - 4;                                    // units per run of 16 blocks = 1 << run_shift
-
-    if constexpr (B == 8) {
-        float* lut = reinterpret_cast<float*>(smem + p.lut_off);
-        for (int i = threadIdx.x; i < 256 * 32; i += nthr) lut[i] = c_codebook[3][i >> 5];     // one copy per bank
-    }
 
     auto load_run = [&](int tr, int run) {
         ScaleRun s;
@@ -305,6 +313,9 @@ __global__ void __maxnreg__(kMaxRegs) stream_fwd_kernel(const Params p) {
             sr = load_run(tr, run);
         }
         if (r0 > i0) __syncthreads();                         // everybody has left the staged activations
+        if constexpr (B == 8) {
+            if (pc == 0 && r0 == i0) fill_lut8(smem + p.lut_off);      // while the first codes are on their way
+        }
         for (int e = threadIdx.x; e < staged * M * 16; e += nthr) {
             const int v = e & 15, pm = e >> 4;                 // 16 columns of one token
             const int pos = p.by_M(pm), m = pm - pos * M;
@@ -531,8 +542,7 @@ __global__ void __maxnreg__(NT == 1 ? kMaxRegs : 128) stream_bwd_kernel(const Bw
     const int mrow = (lane & 7) + ((lane >> 4) << 3), mchunk = (lane >> 3) & 1;
 
     if constexpr (B == 8) {
-        float* lut = reinterpret_cast<float*>(smem + p.lut_off);
-        for (int i = threadIdx.x; i < 256 * 32; i += nthr) lut[i] = c_codebook[3][i >> 5];     // one copy per bank
+        fill_lut8(smem + p.lut_off);
         __syncthreads();
     }
 

@@ -192,6 +192,7 @@ int ensure_tables() {
     const detail::HostTables& t = detail::host_tables();
     if (cudaMemcpyToSymbol(c_codebook, t.codebook, sizeof(t.codebook)) != cudaSuccess ||
         cudaMemcpyToSymbol(c_threshold, t.threshold, sizeof(t.threshold)) != cudaSuccess ||
+        cudaMemcpyToSymbol(g_codebook8, t.codebook[3], sizeof(t.codebook[3])) != cudaSuccess ||
         cudaMemcpyToSymbol(c_curve, t.curve, sizeof(t.curve)) != cudaSuccess ||
         cudaMemcpyToSymbol(g_bins, t.bins, sizeof(t.bins)) != cudaSuccess ||
         cudaMemcpyToSymbol(c_nbins, &t.nbins, sizeof(t.nbins)) != cudaSuccess) {

@@ -33,6 +33,15 @@ def test_wide_blocks(b0, B0, M):
     run_case(A, l1b, l2b, C(b0, B0, 8, 16, 32), M, seed=6400 + M)
 
 
+# 8-bit codes: the code book is laid out by CTAs of 8 warps (192 rows: one unit per run; input gradient: up to eight), 12 and 16
+@pytest.mark.parametrize("N", [192, 2600, 4096])
+def test_code_book_of_eight_bit_codes(N):
+    K = 2304
+    A = inputs.gaussian(6550, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(6551, N, K, 16, 0.03)
+    run_case(A, l1b, l2b, C(8, 64, 8, 64, 32), 3, seed=6552)
+
+
 # one tile row / a few windows shared by many runs: slots on both sides of the eight that are summed at a time, last columns of a tile
 @pytest.mark.parametrize("M", [1, 5, 16])
 @pytest.mark.parametrize("slots", [2, 7, 8, 9, 17])
