@@ -660,7 +660,10 @@ inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q,
             const double body = 6.5 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 2.5 + tokens * 0.008 : tokens * 0.006);
             pl.us = waves * body;
             if (ks == 1 && steps_q > 16) pl.us *= 1.1;  // a single slice of a long contraction
-            if (ks > 1 && waves > 1) pl.us *= 1.3;      // clusters of four and more leave GPCs partly empty between waves
+            // clusters of four and more leave GPCs partly empty between waves; 1.3 with one chunk of few tokens too had made long contractions
+            // run unsliced (us in a graph, one slice / as picked now: 9472 x 16640 NF3, 30 rows 88 / 70; 9088 x 16896 NF2, 19 rows 74 / 59;
+            // 8320 x 22272 NF8 input gradient, 24 rows 153 / 130; 9856 x 17408 NF8, 1384 rows in four chunks and two waves 484, pairs 469)
+            if (ks > 1 && waves > 1) pl.us *= pl.chunks > 1 ? 1.3 : 1.1;
             if (best.us < 0 || pl.us < best.us) best = pl;
         }
     }

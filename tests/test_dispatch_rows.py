@@ -15,6 +15,14 @@ def test_route_between_256_and_2048_rows(N, K, b0, M, want):
     assert binding.linear_path(N, K, C(b0, 64, 8, 256, 32), 64, M, False) == want
 
 
+# few rows against a long contraction: sliced over clusters although these need a second wave
+@pytest.mark.parametrize("N,K,b0,B0,M,r,backward", [(9472, 16640, 3, 16, 30, 0, False), (9088, 16896, 2, 64, 19, 64, False), (8264, 10752, 3, 256, 17, 64, False),
+                                                    (8320, 22272, 8, 64, 24, 64, True)])
+def test_long_contractions_of_few_rows_are_sliced(N, K, b0, B0, M, r, backward):
+    kernel, splits = binding.linear_route(N, K, C(b0, B0, 8, 256, 32), r, M, backward)
+    assert kernel == ONE and splits > 1
+
+
 # many chunks of transposed tiles where the pairs ran before: a last chunk that is not full, both passes, rank below and above 64
 @pytest.mark.gpu
 @pytest.mark.parametrize("N,K,b0,M,r", [(8192, 2048, 3, 1100, 64), (5120, 1024, 2, 700, 128), (8200, 1024, 8, 1101, 16)])
