@@ -174,7 +174,7 @@ __device__ __forceinline__ float lut8_at(uint32_t lut, uint32_t byte_offset) {
 }
 // Fills it (256, 384 or 512 threads): a warp reads 32 entries with one load and hands them round.  (Read from constant memory, 16 entries per
 // warp one after the other in front of the first codes, 8-bit calls on small matrices were slower than the kernels before; us in a graph, those /
-// that / this, one row: 1024 x 1024 rank 64 8.6 / 9.4 / 8.4, without a rank-r term 10.4 / 11.2 / 10.4.)
+// that / this, rank 64: 1024 x 1024, one row 8.6 / 9.1 / 8.4; 4096 x 1024, one row 8.8 / 9.4 / 8.6, eight rows 11.0 / 13.6 / 11.5.)
 __device__ __forceinline__ void fill_lut8(uint8_t* lut) {
     const int lane = threadIdx.x & 31;
     for (int w = threadIdx.x >> 5; w < 16; w += blockDim.x >> 5) {

@@ -129,3 +129,61 @@ def test_chained_calls_give_the_bits_of_synchronised_ones():
         graph.replay()
         got = chain.take()
         assert [i for i in written if not same_bits(want[i], got[i])] == []
+
+
+class EncodeChain:
+    """Matrices quantized between other calls: each call reads what the one in front writes, or overwrites what it reads."""
+
+    def __init__(self):
+        N, K, rows = 384, 512, 600
+        cfgs = [C(3, 64, 8, 256, 32), C(4, 32, 8, 512, 32), C(8, 64, 8, 64, 32), C(2, 16, 4, 64, 16)]      # groups above 256 blocks; packed scales
+        W = [torch.from_numpy(inputs.gaussian(9200 + i, (N, K), 0.04)).cuda() for i in range(2)]
+        q = [binding.alloc_qmatrix(N, K, c, torch.device("cuda")) for c in cfgs]
+        l1b, l2b = inputs.lowrank_factors(9210, N, K, R, 0.02)
+        L1, L2 = binding.bf16_from_bits(l1b), binding.bf16_from_bits(l2b)
+        X, dY = (binding.bf16_from_bits(inputs.activations(9220 + i, rows, n)) for i, n in enumerate((K, N)))
+        ws = torch.empty(max([binding.linear_workspace_bytes(N, K, c, R, m) for c in cfgs for m in (8, rows)] + [binding.packed_sizes(N, K, c)[3] for c in cfgs] +
+                             [binding.lora_grads_workspace_bytes(N, K, R, rows)]), dtype=torch.uint8, device="cuda")      # one scratch for all
+        g1, g2 = torch.empty(N, R, device="cuda"), torch.empty(R, K, device="cuda")
+        qg = binding.alloc_qmatrix(N, R, cfgs[0], torch.device("cuda"))
+        Y, Z = (torch.empty(8, rows, N, dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        self.results = [Y, Z, g1, g2, qg.codes, qg.scale_codes, qg.scale2.view(torch.uint8)]
+        self.codes = torch.empty(4, max(x.codes.numel() for x in q), dtype=torch.uint8, device="cuda")
+        self.results.append(self.codes)
+
+        def run():
+            for i in range(4):
+                binding.encode(W[0], cfgs[i], out=q[i], workspace=ws)
+                binding.linear_fwd(q[i], L1, L2, X[:8], out=Y[i, :8], workspace=ws)
+                binding.encode(W[1], cfgs[i], out=q[i], workspace=ws)                 # overwrites what the call in front reads
+                binding.linear_fwd(q[i], L1, L2, X, out=Y[4 + i], workspace=ws)
+                binding.encode(W[0], cfgs[3 - i], out=q[3 - i], workspace=ws)         # two in a row, one scratch
+                binding.encode(W[1], cfgs[i], out=q[i], workspace=ws)
+                binding.linear_bwd_input(q[i], L1, L2, dY[:4], out=Z[i].view(-1)[:4 * K].view(4, K), workspace=ws)
+                binding.lora_grads(L1, L2, X, dY, out=(g1, g2), workspace=ws)
+                binding.encode(g1, cfgs[0], out=qg, workspace=ws)                     # a gradient, straight from its kernel
+                binding.encode(W[i & 1], cfgs[i], out=q[i], workspace=ws)
+                self.codes[i, :q[i].codes.numel()].copy_(q[i].codes)
+        self.run = run
+
+    def take(self, run):
+        for t in self.results:
+            t.view(torch.uint8).fill_(0x5A)
+        run()
+        torch.cuda.synchronize()
+        return [t.view(torch.uint8).clone() for t in self.results]
+
+
+def test_encodes_between_calls_give_the_bits_of_synchronised_ones(monkeypatch):
+    chain = EncodeChain()
+    with monkeypatch.context() as m:                  # a synchronisation behind every call of the library
+        check = binding._check
+        m.setattr(binding, "_check", lambda status, where: (check(status, where), torch.cuda.synchronize()))
+        want = chain.take(chain.run)
+    for _ in range(20):
+        assert [i for i, (a, b) in enumerate(zip(want, chain.take(chain.run))) if not torch.equal(a, b)] == []
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain.run()
+    for _ in range(10):
+        assert [i for i, (a, b) in enumerate(zip(want, chain.take(graph.replay))) if not torch.equal(a, b)] == []

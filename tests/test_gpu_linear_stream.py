@@ -33,6 +33,29 @@ def test_wide_blocks(b0, B0, M):
     run_case(A, l1b, l2b, C(b0, B0, 8, 16, 32), M, seed=6400 + M)
 
 
+# more units than the SMs can take in one run each (two and more runs per CTA, with buffers used again), and tiles that are given to a run
+# whole because the slots would exceed their room (one slot), in both directions, with and without a rank-r term
+@pytest.mark.parametrize("N,K,M,backward,whole", [(60000, 320, 1, False, False), (60000, 320, 5, False, False), (60000, 320, 16, False, True),
+                                                  (64, 53248, 8, True, False), (64, 53248, 16, True, True)])
+@pytest.mark.parametrize("r", [0, 32])
+def test_several_runs_per_cta_and_whole_tiles(N, K, M, backward, whole, r):
+    cfg = C(3, 64, 8, 64, 32)
+    kernel, slots = binding.linear_route(N, K, cfg, r, M, backward)
+    assert kernel == binding.PATH_STREAM and (slots == 1) == whole
+    A = inputs.gaussian(6560 + M, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(6561, N, K, r, 0.05) if r else (None, None)
+    run_case(A, l1b, l2b, cfg, M, seed=6562, passes=("bwd",) if backward else ("fwd",))
+
+
+# sixteen rows of a long contraction: a run has more units than there is room for activations, which are staged in turns
+@pytest.mark.parametrize("b0", [3, 8])
+def test_activations_staged_in_turns(b0):
+    N, K, M = 3200, 28672, 16
+    A = inputs.gaussian(6570, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(6571, N, K, 64, 0.02)
+    run_case(A, l1b, l2b, C(b0, 64, 8, 256, 32), M, seed=6572, passes=("fwd",), route=binding.PATH_STREAM)
+
+
 # 8-bit codes: the code book is laid out by CTAs of 8 warps (192 rows: one unit per run; input gradient: up to eight), 12 and 16
 @pytest.mark.parametrize("N", [192, 2600, 4096])
 def test_code_book_of_eight_bit_codes(N):
