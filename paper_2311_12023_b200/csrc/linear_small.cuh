@@ -261,7 +261,7 @@ inline cudaError_t launch_small(const QView& q, const void* L1, const void* L2, 
         launches += 2;
     } else {
         if (r > 0) {
-            if (M <= 16 && q.N % 8 == 0 && q.N <= 40960) {
+            if (M <= 16 && q.N % 8 == 0 && q.N <= 40960) {      // (the bound of the weight-streaming kernels, for the same reason)
                 const cudaError_t e = dec::launch_pre<true>(a, l1, T, reinterpret_cast<int*>(ws), nullptr, 0, M, q.N, r, 0, st);
                 if (e != cudaSuccess) return e;
             } else {

@@ -509,8 +509,8 @@ struct BwdParams {
     uint32_t mid_off, lut_off; // shared-memory offsets
 };
 
-// Sixteen warps.  (24 or 20 with 80 or 96 registers spill: 8192 x 28672 NF2, one row, 81 us instead of 57; 8192 x 8192 NF4 37.4
-// instead of 31.8.)
+// Sixteen warps.  (24 or 20 with 80 or 96 registers: 8192 x 28672 NF2, one row, 81 us instead of 57; 8192 x 8192 NF4 37.4 instead of 31.8, from
+// spills.  These spill as well, less: 16 to 60 bytes of stores a thread at up to eight rows with 104 registers, 64 to 232 above with 128.)
 constexpr int kBwdWarps = 16;
 template <int NT> __host__ __device__ constexpr int bwd_warp_bytes() { return 4096 + 8 * NT * 80; }      // weight tile, 32 output gradients of each token
 
@@ -964,12 +964,14 @@ inline cudaError_t launch_bwd(const QView& q, const void* L1, const void* L2, in
 }
 
 inline bool supported(const QView& q, int64_t M) {
-    if (M > 16 || q.K % 8 != 0 || q.K > 40960) return false;   // the pre-product stages K / 8 columns of X per CTA
+    // 40960: as for the kernels before these, which staged a contraction in shared memory.  Nothing here depends on it; longer contractions
+    // have been neither timed nor tested on these kernels and take the plain one.
+    if (M > 16 || q.K % 8 != 0 || q.K > 40960) return false;
     if (static_cast<long long>(q.N) * q.KB >= (1LL << 31)) return false;
     return make_plan(q, static_cast<int>(M)).ok;
 }
 inline bool bwd_supported(const QView& q, int r, int64_t M) {
-    if (M > 16 || q.N % 8 != 0 || q.K % 8 != 0 || q.N > 40960) return false;
+    if (M > 16 || q.N % 8 != 0 || q.K % 8 != 0 || q.N > 40960) return false;      // (see above)
     if (static_cast<long long>(q.N) * q.KB >= (1LL << 31)) return false;
     return make_bwd_plan(q, static_cast<int>(M), r).ok;
 }

@@ -426,7 +426,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     if (lane == 0) mbar_arrive(empty_p(rp.s));
                     rp.advance(4, p.sp);
                 } else {
-                    // rank-r step: the weight-side operand ([L1] rows or L2 rows) comes by TMA
+                    // rank-r step: the weight-side operand is rows of L1 (forward) or L2; by TMA where it goes to shared memory
                     ok = wait(empty(rw.s), rw.ph ^ 1, ctl, 57);
                     if (!ok) break;
                     if constexpr (TA) {
@@ -748,7 +748,7 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     }
     CUtensorMap tX, tT, tF;
     if (!make_map(&tX, A, M, C, pl.box / 2)) return LQLORA_ERR_CUDA;
-    if (r > 0) {
+    if (r > 0) {                          // (tF is not read where the weights go to tensor memory; its map comes from the cache)
         if (!make_map(&tT, T, M, r, pl.box / 2)) return LQLORA_ERR_CUDA;
         const bool ok = backward ? make_map(&tF, L2, r, q.K, 64) : make_map(&tF, L1, q.N, r, 128);
         if (!ok) return LQLORA_ERR_CUDA;

@@ -504,12 +504,16 @@ inline int pair_peel(int64_t M, int64_t out_cols) {
     return peel >= c_tiles ? 0 : peel;
 }
 
-// CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs, unless the transposed tiles, which pad to 16
-// rows instead of 512 and choose their split, are estimated to take less than 0.85 of their time: whole waves of the pair kernel, 6 us
-// and 0.64 us (8-bit codes 0.95) per step each.  From 2048 rows on the two are within 15 % of each other either way and the pairs
-// stay.  us as a graph, pair / transposed: 8192 x 8192 NF3 at 520 rows 87 / 59, 700 88 / 67, 900 91 / 87, 1100 170 / 137, 1400 174 /
-// 131, 1700 180 / 162, 2600 278 / 267, 3300 337 / 343; 5120 x 5120 NF2 at 520 rows 57 / 33, 1100 59 / 47; 11008 x 4096 NF4 input gradient at
-// 1100 rows 112 / 83; 8192 x 8192 NF8 at 520 rows 129 / 87, 1100 253 / 171; 4096 x 4096 NF4 at 1700 rows 54 / 50, 4000 100 / 108.
+// CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs, and below 2048 rows unless the transposed tiles,
+// which pad to 16 rows instead of 512 and choose their split, are estimated to take less than 0.85 of their time: whole waves of the pair
+// kernel, 6 us and 0.64 us (8-bit codes 0.95) per step each.  us as a graph, pair / transposed: 8192 x 8192 NF3 at 520 rows 87 / 59, 700 88 /
+// 67, 900 91 / 87, 1100 170 / 137, 1400 174 / 131, 1700 180 / 162; 5120 x 5120 NF2 at 520 rows 57 / 33, 1100 59 / 47; 11008 x 4096 NF4 input
+// gradient at 1100 rows 112 / 83; 8192 x 8192 NF8 at 520 rows 129 / 87, 1100 253 / 171; 4096 x 4096 NF4 at 1700 rows 54 / 50.
+// From 2048 rows on the pairs stay whatever the estimates say.  That line is drawn by hand.  Both sides measured on nine shapes, both passes,
+// 3-, 4- and 8-bit codes, 2048 to 4096 rows: where the last wave of pair tiles is well filled the pairs are up to a fifth faster (4096 x 4096 NF3
+// at 4096 rows 97 / 120, 28672 x 8192 NF8 at 2048 902 / 1064, 8192 x 8192 NF8 at 2048 273 / 306); where it is between a quarter and a half
+// full the transposed tiles would be, by up to a third and on narrow outputs by more (4096 x 11008 NF3 at 2600 rows 240 / 186, NF8 299 / 226; 4392 x
+// 26688 NF8 at 2600 726 / 557; 5120 x 5120 NF8 at 2304 148 / 116; 2040 x 27008 NF3 at 2048 274 / 156).
 inline double pair_estimate(int b0, int64_t M, int64_t out_cols, int steps_q) {
     const int mt = static_cast<int>((M + 511) / 512), c_tiles = static_cast<int>((out_cols + BN - 1) / BN), peel = pair_peel(M, out_cols);
     const long long pairs = sm_count() / 2, waves = (static_cast<long long>(mt) * (c_tiles - peel) + pairs - 1) / pairs;
@@ -611,10 +615,12 @@ constexpr int kTcMinRowsBwd = 9;  // input gradient of matrices with at least 20
 
 inline bool tc_supported(const QView& q, int r, int64_t M, bool backward) {
     (void)r;
-    // us as a graph, streaming / transposed, 2-, 3-, 4- and 8-bit codes of 8192 x 8192: forward 1 row 17 / 25, 19 / 26, 25 / 32, 30 / 45; 8 rows
-    // 20 / 25, 22 / 26, 28 / 32, 33 / 46; 16 rows 26 / 25, 29 / 26, 35 / 32, 45 / 46; input gradient 1 row 26 / 26, 27 / 27, 30 / 33, 37 / 46; 8 rows
-    // 29 / 26, 30 / 27, 33 / 33, 40 / 46.  Small matrices favour the transposed tiles for more than eight rows of an input gradient: 4096 x 4096 NF3 at
-    // 12 rows 13.8, at 8 rows streaming 18.
+    // us as a graph, streaming / transposed, 2-, 3-, 4- and 8-bit codes of 8192 x 8192, rank 64: forward 1 row 17 / 24, 18 / 24, 25 / 30, 29 / 42; 8 rows
+    // 19 / 24, 20 / 24, 27 / 31, 32 / 42; 16 rows 24 / 24, 25 / 25, 31 / 31, 42 / 42 (other shapes: streaming at most 3 % behind at 16 rows, up to a
+    // quarter ahead on 28672 x 8192).  Input gradient 1 row 25 / 25, 26 / 26, 29 / 32, 36 / 44; 8 rows 27 / 25, 28 / 26, 31 / 32, 38 / 44; 9 rows (two
+    // token groups) 36 / 26, 40 / 26, 47 / 32, 58 / 44.  One line for all widths and shapes: 2- and 3-bit input gradients of 1 to 8 rows stay with the
+    // streaming kernels although the transposed tiles would be faster on few rows of weights (2048 x 8192 1 row 13 / 12, 8 rows 15 / 12; 4096 x
+    // 4096 8 rows 14.6 / 13; even on 11008 x 4096 and behind on 28672 x 8192, 70 / 72).
     const int min_rows = (backward && q.N >= 2048) ? kTcMinRowsBwd : kTcMinRows;
     if (M < min_rows) return false;
     if (q.N % 8 != 0 || q.K % 8 != 0) return false;
