@@ -19,12 +19,14 @@
 //     that kernel, or by the caller's memset when there is no rank-r term.
 //
 // What bounds it: the pipe of byte permutes and logic (64 lanes per clock and SM): about two operations per weight of 3 bits, 2.6 of 4
-// bits, 1.2 of 2 bits; it is busy 75-80 % of the main loop, which runs at 21 weights per clock and SM (3 bits).  Around the loop a call
-// takes 6 us: 2.5 from the end of the kernel in front to the first unit, 3 for sums, counter and output.  The kernel before this
-// one (tiles and scale tables staged through a ring in shared memory, short CTAs in waves) held the pipe at 50 % of its active cycles.
-// us per call in a graph, before / now (one row, rank 64): 8192 x 8192 2 bits 20.1 / 16.7, 3 bits 22.1 / 18.6, 4 bits 29.7 / 25.1, 8 bits
-// 43.7 / 29.7; 28672 x 8192 3 bits in blocks of 16 68.6 / 58.4; 8192 x 28672 2 bits 62.5 / 36.9; sixteen rows of 8192 x 8192 4 bits
-// 43.0 / 34.6.  Input gradient: 8192 x 8192 3 bits 29.3 / 26.6, 4 bits 40.2 / 30.2; 8192 x 28672 2 bits 80.9 / 58.0.
+// bits, 1.2 of 2 bits; busy 53 % of the active cycles of the whole kernel (8192 x 8192 NF3, one row; input gradient 47 %), of which the main
+// loop, at 21 weights per clock and SM, is about two thirds.  Around the loop a call takes 6 us: 2.5 from the end of the kernel in front to
+// the first unit, 3 for sums, counter and output.  The kernel before this one (tiles and scale tables staged through a ring in shared memory,
+// short CTAs in waves) held the pipe at 50 % of its active cycles.
+// us per call in a graph, kernels before / these (rank 64): one row of 8192 x 8192 2 bits 19.6 / 16.0, 3 bits 21.2 / 17.7, 4 bits 28.6 / 24.0,
+// 8 bits 43.1 / 28.5; 28672 x 8192 3 bits in blocks of 16 68.3 / 57.9; 8192 x 28672 2 bits in blocks of 128 61.5 / 36.0; sixteen rows of 8192 x 8192
+// 32.9 / 23.2, 34.1 / 24.6, 41.9 / 30.9, 60.6 / 42.0.  Input gradient, one row: 8192 x 8192 2 bits 26.4 / 24.7, 3 bits 28.6 / 25.4, 4 bits 39.3 / 28.8,
+// 8 bits 58.4 / 35.7; 8192 x 28672 2 bits in blocks of 128 80.5 / 57.0.
 #pragma once
 
 #include "common.cuh"
