@@ -15,6 +15,12 @@ def test_route_between_256_and_2048_rows(N, K, b0, M, want):
     assert binding.linear_path(N, K, C(b0, 64, 8, 256, 32), 64, M, False) == want
 
 
+# from 2048 rows on the pairs, also where their last wave is between a quarter and a half full
+@pytest.mark.parametrize("N,K,b0,M", [(4392, 26688, 8, 2579), (2040, 27008, 3, 2251), (8192, 28672, 8, 2300), (5120, 5120, 8, 2100), (4096, 11008, 8, 2600)])
+def test_pairs_from_2048_rows(N, K, b0, M):
+    assert binding.linear_path(N, K, C(b0, 64, 8, 256, 32), 64, M, False) == PAIR
+
+
 # few rows against a long contraction: sliced over clusters although these need a second wave
 @pytest.mark.parametrize("N,K,b0,B0,M,r,backward", [(9472, 16640, 3, 16, 30, 0, False), (9088, 16896, 2, 64, 19, 64, False), (8264, 10752, 3, 256, 17, 64, False),
                                                     (8320, 22272, 8, 64, 24, 64, True)])

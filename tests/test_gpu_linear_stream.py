@@ -65,6 +65,27 @@ def test_code_book_of_eight_bit_codes(N):
     run_case(A, l1b, l2b, C(8, 64, 8, 64, 32), 3, seed=6552)
 
 
+# rows of the identity: the weights of the streaming kernels are the bits of lqlora_dequant, which forms the second-level scale v / levels by a
+# division.  Many groups, because one unit in the last place of a scale shows in few of the rounded products
+@pytest.mark.parametrize("b1", [8, 4])
+@pytest.mark.parametrize("b0,B0", [(2, 16), (3, 64), (4, 32), (8, 64)])
+def test_identity_rows_return_the_dequantized_weights(b0, B0, b1):
+    cfg = C(b0, B0, b1, 16, 32)
+    for N, K, backward in ((40000, 64, False), (64, 16384, True)):
+        A = inputs.student_t(6590 + b0, (N, K), 5.0, 0.02)
+        q = binding.encode(torch.from_numpy(A).cuda(), cfg)
+        d16 = binding.dequant(q)[1]
+        at = torch.arange(3, 3 + 4 * 16, 4, device="cuda")
+        x = torch.zeros(16, N if backward else K, dtype=torch.bfloat16, device="cuda")
+        x[torch.arange(16, device="cuda"), at] = 1.0
+        assert binding.linear_path(N, K, cfg, 0, 16, backward) == binding.PATH_STREAM
+        if backward:
+            got, want = binding.linear_bwd_input(q, None, None, x), d16[at]
+        else:
+            got, want = binding.linear_fwd(q, None, None, x), d16[:, at].T
+        assert torch.equal(got, want)
+
+
 # one tile row / a few windows shared by many runs: slots on both sides of the eight that are summed at a time, last columns of a tile
 @pytest.mark.parametrize("M", [1, 5, 16])
 @pytest.mark.parametrize("slots", [2, 7, 8, 9, 17])
