@@ -15,8 +15,13 @@
 // boxes the accumulators need them all.  The row operand in tensor memory is K-major only, so the input gradient stays in shared memory.
 // Every wait is bounded (see linear_tc.cuh).
 //
-// What bounds it: the loop of the issuing warp (a dependent chain of about a hundred clocks per wait and commit, so one
-// full and one empty barrier per step, 32-bit descriptors, no divisions), then dequantization (about 500 clocks per 64
+// With one token box a stage is two steps, with one wait and one commit for both: without loads and dequantization a step still took 370 clocks, of which
+// the issuing warp spent 140 in a wait that was satisfied and 170 to 210 issuing.  What every step needs is requested before tensor memory, the
+// code book and the cluster barrier are set up, and arrivals on that barrier are relaxed (the initialisation of the mbarriers has a fence of its own): a
+// releasing arrival waited for the scale loads in front of it.  us as a graph, one step per stage and a set-up in front of the loads / this: 8192 x 8192 NF3,
+// 128 rows 27.6 / 24.6, without a rank-r term (a memset in front of the kernel before) 30.9 / 23.2, 28672 x 8192 83.5 / 73.4, input gradient 30.9 / 29.2.
+// What bounds it: the loop of the issuing warp (32-bit descriptors, no divisions), then dequantization (about 450 clocks per step of an SM, of which
+// the pipe of byte permutes and logic is busy 275; warps started out of step, 24 of them with 72 registers, changed nothing or cost time): about 500 clocks per 64
 // weights of a row and warp).  A weight tile in shared memory costs its bandwidth twice, when written and when read by the tensor
 // core, and with wide codes or many tokens it takes the room of ring stages.  us as a graph, in shared / in tensor memory: 8192 x 8192
 // NF3 128 rows 28.0 / 26.7 (1.05), 512 rows 52.9 / 50.2, 28672 x 8192 NF3 128 rows 95.2 / 90.8, 8-bit codes 256 rows 62.5 / 60.4; shapes
@@ -24,6 +29,7 @@
 #pragma once
 
 #include <atomic>
+#include <cmath>
 #include <type_traits>
 
 namespace lq {
@@ -36,19 +42,22 @@ constexpr int kSwWBytes = 128 * 128;                            // this CTA's bf
 constexpr int kSwMaxStages = 8;
 constexpr uint32_t kSwTmemA = 256;                              // first column of the weights in tensor memory (32 per stage)
 constexpr int kSwTail = 512;                                    // barriers, tensor-memory slot, abort flag
+// Steps of 64 contraction elements per stage, i.e. per round of waits and commits: two with one token box, one with two.
+constexpr int swap_stage_steps(int nbox) { return nbox == 1 ? 2 : 1; }
 
 struct SwapParams {
     QView q;
     __nv_bfloat16* out;
     int* status;
     int M;
+    int clear_status;        // without a rank-r term: 1 = this kernel is the first of its call and clears the status word
     int out_cols;            // N (forward) or K (backward)
     int steps_q, steps_d;    // contraction steps with dequantized weights / of the rank-r term
     int c_base;              // first output column of this launch
     const __nv_bfloat16* L1; // forward with the weights in tensor memory: [N][r], read directly
     int r;
     int nbox, box;           // token boxes (1 or 2) and tokens per box (a multiple of 16, at most 256; half of them per CTA)
-    int ss, sp;              // stages of the token + weight ring and of the packed-code ring
+    int ss, sp;              // stages (of swap_stage_steps steps) of the token + weight ring and of the packed-code ring
     uint32_t tail_off;       // of the barriers, behind the rings
     uint32_t tmem_cols;
 };
@@ -168,6 +177,73 @@ __device__ __forceinline__ void dequant_row64_tmem(uint32_t words0, uint32_t wor
     }
 }
 
+// The scales of a lane's row of 64 weights for the steps of its warp (every fourth one), requested ahead.
+// Input gradient: the row changes with the step, so each step loads its own, two steps ahead.
+// Forward: the codes of a row are consecutive bytes.  The lane keeps the aligned 16 bytes that hold its current ones, and the 16 behind them; 16 aligned
+// blocks share their second-level scale (B1 >= 16).  (A load per step and lane touches 32 lines each time: without any scale loads 8192 x 8192
+// NF3 at 128 rows took 1.4 us less.)
+template <bool BWD> struct SwapScales {
+    const QView& q;
+    uint32_t blk, nblk;              // current block, blocks of the matrix
+    int st, st_end;                  // BWD: next step to be requested
+    int row;
+    bool live;
+    RawScale slot[2];                // BWD
+    uint4 w0, w1;                    // forward
+    float v0, v1;
+    __device__ __forceinline__ SwapScales(const QView& q_, int row_, int col, int st_, int st_end_) : q(q_), st(st_), st_end(st_end_), row(row_) {
+        live = BWD ? col < q.K : row < q.N;
+        nblk = static_cast<uint32_t>(q.N) * q.KB;
+        blk = BWD ? static_cast<uint32_t>(col >> q.logB0) : static_cast<uint32_t>(row) * q.KB + (col >> q.logB0);
+    }
+    __device__ __forceinline__ RawScale fetch() {
+        RawScale r{0u, 0.0f};
+        const int n = st * BK + row;
+        if (live && st < st_end && n < q.N) {
+            const uint32_t b = static_cast<uint32_t>(n) * q.KB + blk;
+            if (q.logB0 == 4) r.sc = __ldg(reinterpret_cast<const uint32_t*>(q.sc + b));
+            else if (q.logB0 == 5) r.sc = __ldg(reinterpret_cast<const uint16_t*>(q.sc + b));
+            else r.sc = __ldg(q.sc + b);
+            r.v = __ldg(q.v + (b >> q.logB1));
+        }
+        st += 4;
+        return r;
+    }
+    __device__ __forceinline__ void window(uint32_t b, uint4& w, float& v) {
+        w = make_uint4(0u, 0u, 0u, 0u); v = 0.0f;
+        b &= ~15u;
+        if (!live || b >= nblk) return;
+        v = __ldg(q.v + (b >> q.logB1));
+        if (b + 16 <= nblk) { w = __ldg(reinterpret_cast<const uint4*>(q.sc + b)); return; }
+        uint32_t t[4] = {0u, 0u, 0u, 0u};                // the last blocks of the matrix
+#pragma unroll
+        for (int i = 0; i < 15; ++i)
+            if (b + i < nblk) t[i >> 2] |= static_cast<uint32_t>(__ldg(q.sc + b + i)) << (8 * (i & 3));
+        w = make_uint4(t[0], t[1], t[2], t[3]);
+    }
+    __device__ __forceinline__ void start() {
+        if constexpr (BWD) { slot[0] = fetch(); slot[1] = fetch(); }
+        else { window(blk, w0, v0); window(blk + 16, w1, v1); }
+    }
+    // The scale codes of the current step (a byte each, from the lowest on), and on to the next one; u = parity of the step's number.
+    __device__ __forceinline__ RawScale next(int u) {
+        if constexpr (BWD) {
+            const RawScale r = slot[u];
+            slot[u] = fetch();
+            return r;
+        } else {
+            const uint32_t word = (blk & 8u) ? ((blk & 4u) ? w0.w : w0.z) : ((blk & 4u) ? w0.y : w0.x);
+            const RawScale r{word >> (8 * (blk & 3u)), v0};
+            const uint32_t to = blk + (256u >> q.logB0);
+            if ((to ^ blk) & ~15u) { w0 = w1; v0 = v1; window(to + 16, w1, v1); }
+            blk = to;
+            return r;
+        }
+    }
+};
+
+__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 __device__ __forceinline__ float4 ld_dsmem_f32x4(uint32_t local_addr, uint32_t rank) {
     uint32_t ra;
     float4 v;
@@ -180,7 +256,7 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int B, bool BWD, bool TA>
+template <int B, bool BWD, bool TA, int PS>
 __global__ void __launch_bounds__(kSwThreads, 1)
 tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT,
                       const __grid_constant__ CUtensorMap tmF, const SwapParams p) {
@@ -188,25 +264,27 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int half_box = p.box >> 1, half_bytes = half_box * 128;
-    const int x_bytes = p.nbox * half_bytes;
+    const int nbox = PS == 2 ? 1 : 2;
+    const int x_bytes = nbox * half_bytes;
     constexpr int W_BYTES = TA ? 0 : kSwWBytes;
-    const int stage_bytes = W_BYTES + x_bytes;                           // [weight tile][token boxes]
-    uint8_t* p_ring = base + p.ss * stage_bytes;
+    const int step_bytes = W_BYTES + x_bytes;                            // [weight tile][token boxes] of a step; a stage is PS of them
+    uint8_t* p_ring = base + p.ss * PS * step_bytes;
     uint8_t* tail = base + p.tail_off;
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);     // full[8], empty[8], full_p[8], empty_p[8], fbar[2], acc_full, drain
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 36 * 8);
     volatile int* abort_s = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    int* reached = reinterpret_cast<int*>(tmem_slot + 2);    // [20] per warp: the first step that it has not (issued or) arrived at
+    int* reached = reinterpret_cast<int*>(tmem_slot + 2);    // [20] per warp: the first stage (from 0 on, ring passes counted) that it has not (issued or) arrived at
     float* lut8 = reinterpret_cast<float*>(tail + kSwTail);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank() & 1u;                           // CTA of the pair; 0 = leader
     const int c0 = p.c_base + blockIdx.x * 128;                          // first output column of this CTA
-    const int m0 = blockIdx.y * (p.nbox * p.box);                        // first token
+    const int m0 = blockIdx.y * (nbox * p.box);                          // first token
     const int nsplit = gridDim.z, split = blockIdx.z;
     const int q_lo = static_cast<int>(static_cast<long long>(p.steps_q) * split / nsplit);
     const int nq = static_cast<int>(static_cast<long long>(p.steps_q) * (split + 1) / nsplit) - q_lo;
     const int total = nq + (split == 0 ? p.steps_d : 0);                 // the rank-r steps go to the first slice
+    const int rounds = (total + PS - 1) / PS;                            // stages of the slice; the last one may hold one step of two
     const int have = min(2, max(0, (p.out_cols - c0 + 63) >> 6));        // 64-column tiles of this CTA that exist
     const Ctl ctl{abort_s, p.status};
 
@@ -218,131 +296,197 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     auto fbar = [&](int d) { return bar0 + 256 + 8 * d; };
     const uint32_t acc_full = bar0 + 272, drain = bar0 + 280;
 
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kSwMaxStages; ++s) {
-            // token boxes and four dequantization warps; leader: also the word of the second CTA that its step is complete
-            mbar_init(full(s), p.nbox + 4 + (rank == 0 ? 1 : 0));
-            mbar_init(empty(s), 1);
-            mbar_init(full_p(s), 1);
-            mbar_init(empty_p(s), 4);
+    // This CTA's half of token box w of a stage (PS = 1), or of the token box of its step w.  By one lane.
+    auto issue_box = [&](int w, int round, int stage) {
+        const int step = PS == 1 ? round : 2 * round + w;
+        const int row = m0 + (PS == 1 ? w * p.box : 0) + static_cast<int>(rank) * half_box;
+        const uint32_t dst = ring + W_BYTES + w * (PS == 1 ? half_bytes : step_bytes) + stage * (PS * step_bytes);
+        if (step >= total) {
+            mbar_arrive(full(stage));                     // the second step of the last stage does not exist
+        } else {
+            mbar_expect_tx(full(stage), half_bytes);
+            if (step < nq) tma_load_2d(dst, &tmX, (q_lo + step) * BK, row, full(stage));
+            else tma_load_2d(dst, &tmT, (step - nq) * BK, row, full(stage));
         }
-        mbar_init(fbar(0), 1);
-        mbar_init(fbar(1), 1);
-        mbar_init(acc_full, 1);
-        mbar_init(drain, 1);
-        *abort_s = 0;
-        fence_barrier_init();
+    };
+    // The packed codes of a stage.
+    auto issue_codes = [&](int round, int stage) {
+        const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
+        const uint32_t dst = smem_u32(p_ring) + stage * (PS * P_BYTES), bar = full_p(stage);
+        const int qs = q_lo + round * PS;
+        const bool two = PS == 2 && round * PS + 1 < nq;
+        if (have == 0) {
+            mbar_arrive(bar);                             // nothing behind the last column: the scales are zero
+        } else if (!BWD) {
+            // one tile, or two neighbouring ones
+            const uint32_t bytes = two ? 2 * P_BYTES : P_BYTES;
+            mbar_expect_tx(bar, bytes);
+            bulk_load(dst, codes + (static_cast<size_t>(c0 >> 7) * p.q.ktiles + qs) * P_BYTES, bytes, bar);
+        } else {
+            // 64 rows (half a tile) of the two 64-column tiles of this CTA, for each step
+            mbar_expect_tx(bar, (two ? 2 : 1) * have * (P_BYTES / 2));
+#pragma unroll
+            for (int h = 0; h < PS; ++h) {
+                if (h == 1 && !two) break;
+                const uint8_t* src = codes + (static_cast<size_t>((qs + h) >> 1) * p.q.ktiles + (c0 >> 6)) * P_BYTES + ((qs + h) & 1) * (P_BYTES / 2);
+                for (int t = 0; t < have; ++t) bulk_load(dst + h * P_BYTES + t * (P_BYTES / 2), src + t * P_BYTES, P_BYTES / 2, bar);
+            }
+        }
+    };
+
+    // Dequantization warps: four per step, warp = steps grp, grp + 4, ...  Forward: row c0 + 32 wi + lane of the tile; backward: contraction row
+    // 32 (wi & 1) + lane, 64-column tile wi >> 1.
+    const int dw = warp - kSwFirstDeq, grp = (dw >> 2) & 3, wi = dw & 3;
+    const int half = PS == 2 ? grp & 1 : 0;               // which step of its stage
+    const int row_local = BWD ? (wi & 1) * 32 + lane : wi * 32 + lane;
+    SwapScales<BWD> scales(p.q, BWD ? row_local : c0 + row_local, BWD ? c0 + (wi >> 1) * 64 : (q_lo + grp) * BK, BWD ? q_lo + grp : 0, q_lo + nq);
+
+    // Everything that a step needs is requested first; what follows (tensor memory, the code book, the barrier of the cluster) takes about
+    // as long as those requests.  Only arrivals on the other CTA's barriers have to wait for the cluster.
+    // (Without a rank-r term this is the first kernel of its call, launched while the one in front ends: it waits for that one before it reads.)
+    const bool lead = p.steps_d == 0;
+    const int early_x = min(p.ss, nq / PS), early_p = min(p.sp, (nq + PS - 1) / PS);
+    if (warp < 2) {
+        if (warp == 0 && elect_one()) {
+            for (int s = 0; s < kSwMaxStages; ++s) {
+                // two token boxes (of a step, or of two) and four dequantization warps per step; leader: also the word of the second
+                // CTA that its stage is complete
+                mbar_init(full(s), 2 + 4 * PS + (rank == 0 ? 1 : 0));
+                mbar_init(empty(s), 1);
+            }
+            mbar_init(fbar(0), 1);
+            mbar_init(fbar(1), 1);
+            mbar_init(acc_full, 1);
+            mbar_init(drain, 1);
+            *abort_s = 0;
+            fence_barrier_init();
+            fence_proxy_async();
+        }
+        __syncwarp();
+        asm volatile("bar.sync 1, 64;" ::: "memory");
+        if (lead) pdl_wait();
+        if (elect_one()) {
+            for (int i = 0; i < early_x; ++i) issue_box(warp, i, i);
+        }
+        __syncwarp();
+    } else if (warp == 2) {
+        if (elect_one()) {
+            for (int s = 0; s < kSwMaxStages; ++s) {
+                mbar_init(full_p(s), 1);
+                mbar_init(empty_p(s), 4 * PS);
+            }
+            fence_barrier_init();
+            fence_proxy_async();
+            if (lead) pdl_wait();
+            for (int i = 0; i < early_p; ++i) issue_codes(i, i);
+        }
+        __syncwarp();
+    } else if (warp == 3) {
+        tmem_alloc2(smem_u32(tmem_slot), p.tmem_cols);
+        tmem_relinquish2();
+    } else if (warp >= kSwFirstDeq) {
+        if (lead) {
+            pdl_wait();
+            if (p.clear_status && dw == 0 && lane == 0 && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) *p.status = 0;
+        }
+        scales.start();
+        if constexpr (B == 8) {
+            for (int i = threadIdx.x - kSwFirstDeq * 32; i < 256 * 32; i += kSwDeqWarps * 32) lut8[i] = c_codebook[3][i >> 5];     // one copy per bank
+        }
     }
-    if constexpr (B == 8) {
-        for (int i = threadIdx.x; i < 256 * 32; i += kSwThreads) lut8[i] = c_codebook[3][i >> 5];     // one copy per bank
-    }
-    if (warp == 3) { tmem_alloc2(smem_u32(tmem_slot), p.tmem_cols); tmem_relinquish2(); }
     tc_fence_before();
     __syncthreads();
-    cluster_barrier();                                    // barriers of both CTAs are initialised before any remote arrive
+    // The barriers and tensor memory of this CTA are ready.  The threads that initialised the barriers have passed fence.mbarrier_init; a
+    // releasing arrival would make every warp wait for its scales here first (1700 clocks when they come from DRAM).
+    dec::cluster_arrive_relaxed();
+    if (warp == 3) cluster_wait_acquire();                // (the others wait behind their loops)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
     bool acc_ok = false;
-    int issued = 0;               // steps whose codes have been requested (warp 2)
+    int issued = early_p;         // stages whose codes have been requested (warp 2)
 
-    if (warp < p.nbox) {
-        // ------------------------------------------------------------------ this CTA's half of token box `warp`
-        RingAt r(0, p.ss);
-        const int row = m0 + warp * p.box + static_cast<int>(rank) * half_box;
-        uint32_t dst0 = ring + W_BYTES + warp * half_bytes;
-        int k = q_lo * BK;
-        int step = 0;
-        for (; step < total; ++step, r.advance(1, p.ss), k += BK) {
+    if (warp < 2) {
+        // ------------------------------------------------------------------ token boxes
+        RingAt r(early_x, p.ss);
+        int round = early_x;
+        for (; round < rounds; ++round, r.advance(1, p.ss)) {
             if (!wait(empty(r.s), r.ph ^ 1, ctl, 51)) break;
-            if (step == nq) {
+            const int step = PS == 1 ? round : 2 * round + warp;
+            if (step >= nq && step < nq + PS && step < total) {
                 // the rank-r intermediate comes from the kernel in front (programmatic dependent launch)
                 pdl_wait();
                 fence_proxy_async_all();
             }
             __syncwarp();
-            if (elect_one()) {
-                mbar_expect_tx(full(r.s), half_bytes);
-                if (step < nq) tma_load_2d(dst0 + r.s * stage_bytes, &tmX, k, row, full(r.s));
-                else tma_load_2d(dst0 + r.s * stage_bytes, &tmT, (step - nq) * BK, row, full(r.s));
-            }
+            if (elect_one()) issue_box(warp, round, r.s);
             __syncwarp();
         }
-        if (lane == 0) reached[warp] = step;
+        if (lane == 0) reached[warp] = round;
     } else if (warp == 2) {
         // ------------------------------------------------------------------ packed codes
-        const uint8_t* codes = reinterpret_cast<const uint8_t*>(p.q.codes);
-        RingAt r(0, p.sp);
-        for (int step = 0; step < nq; ++step, r.advance(1, p.sp)) {
+        RingAt r(early_p, p.sp);
+        for (int round = early_p; round * PS < nq; ++round, r.advance(1, p.sp)) {
             if (!wait(empty_p(r.s), r.ph ^ 1, ctl, 52)) break;
             __syncwarp();
-            if (elect_one()) {
-                const uint32_t dst = smem_u32(p_ring) + r.s * P_BYTES;
-                const int qs = q_lo + step;
-                if (have == 0) {
-                    mbar_arrive(full_p(r.s));             // nothing behind the last column: the scales below are zero
-                } else if (!BWD) {
-                    mbar_expect_tx(full_p(r.s), P_BYTES);
-                    bulk_load(dst, codes + (static_cast<size_t>(c0 >> 7) * p.q.ktiles + qs) * P_BYTES, P_BYTES, full_p(r.s));
-                } else {
-                    // 64 rows (half a tile) of the two 64-column tiles of this CTA
-                    const uint8_t* src = codes + (static_cast<size_t>(qs >> 1) * p.q.ktiles + (c0 >> 6)) * P_BYTES + (qs & 1) * (P_BYTES / 2);
-                    mbar_expect_tx(full_p(r.s), have * (P_BYTES / 2));
-                    for (int t = 0; t < have; ++t) bulk_load(dst + t * (P_BYTES / 2), src + t * P_BYTES, P_BYTES / 2, full_p(r.s));
-                }
-            }
+            if (elect_one()) issue_codes(round, r.s);
             __syncwarp();
-            issued = step + 1;
+            issued = round + 1;
         }
     } else if (warp == 3) {
         // ------------------------------------------------------------------ MMA issuer (leader), messenger (second CTA)
         if (rank == 1) {
-            // tells the leader that this CTA's half of a step is complete
+            // tells the leader that this CTA's half of a stage is complete
             RingAt r(0, p.ss);
-            int step = 0;
-            for (; step < total; ++step, r.advance(1, p.ss)) {
+            int round = 0;
+            for (; round < rounds; ++round, r.advance(1, p.ss)) {
                 if (!wait(full(r.s), r.ph, ctl, 60)) break;
                 __syncwarp();
                 if (elect_one()) mbar_arrive_cluster(full(r.s), cluster_rank() & ~1u);
             }
-            if (lane == 0) dec::st_dsmem_f32(smem_u32(reached + 3), cluster_rank() & ~1u, __int_as_float(step));     // to the leader
+            if (lane == 0) dec::st_dsmem_f32(smem_u32(reached + 3), cluster_rank() & ~1u, __int_as_float(round));    // to the leader
         } else {
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((BWD ? 1u : 0u) << 15) |
                                    (static_cast<uint32_t>(p.box >> 3) << 17) | (static_cast<uint32_t>(256 >> 4) << 24);
             const uint32_t a0 = desc_lo(ring, BWD ? 8192 : 16), b0 = desc_lo(ring + W_BYTES, 16);
-            const uint32_t stage16 = stage_bytes >> 4, box16 = half_bytes >> 4;
+            const uint32_t step16 = step_bytes >> 4, box16 = half_bytes >> 4;
             constexpr uint32_t ka = (BWD ? 2048 : 32) >> 4;            // 16 contraction elements further: rows down, or columns along
             const uint16_t pair_mask = static_cast<uint16_t>(3u << (cluster_rank() & ~1u));
             bool ok = true;
             uint32_t acc = 0;
             RingAt r(0, p.ss);
-            for (int step = 0; step < total; ++step, r.advance(1, p.ss)) {
+            for (int round = 0; round < rounds; ++round, r.advance(1, p.ss)) {
                 ok = wait_cluster(full(r.s), r.ph, ctl, 53);
                 if (!ok) break;
                 __syncwarp();
                 tc_fence_after();
-                const uint32_t a = a0 + r.s * stage16, b = b0 + r.s * stage16;
-                if (TA) {
-                    const uint32_t at = tmem + kSwTmemA + r.s * 32;
-                    if (elect_one()) {
-                        tc_mma2_ta(tmem, at, b, idesc, acc);
-                        tc_mma2_ta(tmem, at + 8, b + 2, idesc, 1u);
-                        tc_mma2_ta(tmem, at + 16, b + 4, idesc, 1u);
-                        tc_mma2_ta(tmem, at + 24, b + 6, idesc, 1u);
-                        tc_commit_pair(step + 1 < total ? empty(r.s) : acc_full, pair_mask);
+                const bool two = PS == 2 && 2 * round + 1 < total;
+                if (elect_one()) {
+#pragma unroll
+                    for (int h = 0; h < PS; ++h) {
+                        if (h == 1 && !two) break;
+                        const uint32_t slot = r.s * PS + h, b = b0 + slot * step16, keep = h == 0 ? acc : 1u;
+                        if (TA) {
+                            const uint32_t at = tmem + kSwTmemA + slot * 32;
+                            tc_mma2_ta(tmem, at, b, idesc, keep);
+                            tc_mma2_ta(tmem, at + 8, b + 2, idesc, 1u);
+                            tc_mma2_ta(tmem, at + 16, b + 4, idesc, 1u);
+                            tc_mma2_ta(tmem, at + 24, b + 6, idesc, 1u);
+                        } else {
+                            const uint32_t a = a0 + slot * step16;
+                            tc_mma2_lo(tmem, a, b, idesc, keep);
+                            tc_mma2_lo(tmem, a + ka, b + 2, idesc, 1u);
+                            tc_mma2_lo(tmem, a + 2 * ka, b + 4, idesc, 1u);
+                            tc_mma2_lo(tmem, a + 3 * ka, b + 6, idesc, 1u);
+                            if (PS == 1) {
+                                const uint32_t b2 = b + box16;
+                                tc_mma2_lo(tmem + 256, a, b2, idesc, keep);
+                                tc_mma2_lo(tmem + 256, a + ka, b2 + 2, idesc, 1u);
+                                tc_mma2_lo(tmem + 256, a + 2 * ka, b2 + 4, idesc, 1u);
+                                tc_mma2_lo(tmem + 256, a + 3 * ka, b2 + 6, idesc, 1u);
+                            }
+                        }
                     }
-                } else if (elect_one()) {
-                    tc_mma2_lo(tmem, a, b, idesc, acc);
-                    tc_mma2_lo(tmem, a + ka, b + 2, idesc, 1u);
-                    tc_mma2_lo(tmem, a + 2 * ka, b + 4, idesc, 1u);
-                    tc_mma2_lo(tmem, a + 3 * ka, b + 6, idesc, 1u);
-                    if (p.nbox == 2) {
-                        const uint32_t b2 = b + box16;
-                        tc_mma2_lo(tmem + 256, a, b2, idesc, acc);
-                        tc_mma2_lo(tmem + 256, a + ka, b2 + 2, idesc, 1u);
-                        tc_mma2_lo(tmem + 256, a + 2 * ka, b2 + 4, idesc, 1u);
-                        tc_mma2_lo(tmem + 256, a + 3 * ka, b2 + 6, idesc, 1u);
-                    }
-                    tc_commit_pair(step + 1 < total ? empty(r.s) : acc_full, pair_mask);
+                    tc_commit_pair(round + 1 < rounds ? empty(r.s) : acc_full, pair_mask);
                 }
                 acc = 1u;
                 __syncwarp();
@@ -356,65 +500,43 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         }
         __syncwarp();
     } else if (warp >= kSwFirstDeq) {
-        // ------------------------------------------------------------------ dequantization: four warps per step
-        const int dw = warp - kSwFirstDeq;
-        const int grp = dw >> 2, wi = dw & 3;
+        // ------------------------------------------------------------------ dequantization
         const QView& q = p.q;
-        // forward: row c0 + 32 wi + lane of the tile; backward: contraction row 32 (wi & 1) + lane, 64-column tile wi >> 1
-        const int row_local = BWD ? (wi & 1) * 32 + lane : wi * 32 + lane;
         const int my_col = BWD ? c0 + (wi >> 1) * 64 : 0;
-        const bool live = BWD ? my_col < q.K : c0 + row_local < q.N;
-        const uint32_t dst0 = ring + (BWD ? (wi >> 1) * 8192 : 0) + row_local * 128;
+        const uint32_t dst0 = ring + half * step_bytes + (BWD ? (wi >> 1) * 8192 : 0) + row_local * 128;
         const uint32_t xr = (row_local & 7) << 4;
-        const uint32_t wsrc = smem_u32(p_ring) + (BWD ? (wi >> 1) * (128 * B) + (wi & 1) * (64 * B) : wi * (64 * B)) * 4;
+        const uint32_t wsrc = smem_u32(p_ring) + half * P_BYTES + (BWD ? (wi >> 1) * (128 * B) + (wi & 1) * (64 * B) : wi * (64 * B)) * 4;
         const int nsc = q.B0 == 16 ? 4 : q.B0 == 32 ? 2 : 1;
-        // scale codes of the row's 64 columns (aligned, at most four, one second-level group: B1 >= 16)
-        auto fetch = [&](int st) {
-            RawScale r{0u, 0.0f};
-            const int row = BWD ? st * BK + row_local : c0 + row_local;
-            if (live && row < q.N) {
-                const uint32_t blk = static_cast<uint32_t>(row) * q.KB + ((BWD ? my_col : st * BK) >> q.logB0);
-                if (nsc == 4) r.sc = __ldg(reinterpret_cast<const uint32_t*>(q.sc + blk));
-                else if (nsc == 2) r.sc = __ldg(reinterpret_cast<const uint16_t*>(q.sc + blk));
-                else r.sc = __ldg(q.sc + blk);
-                r.v = __ldg(q.v + (blk >> q.logB1));
-            }
-            return r;
-        };
         float v_cached = -1.0f, sigma = 0.0f;
-        RawScale slot[2];
-        slot[0] = (grp < nq) ? fetch(q_lo + grp) : RawScale{0u, 0.0f};
-        slot[1] = (grp + 4 < nq) ? fetch(q_lo + grp + 4) : RawScale{0u, 0.0f};
-        RingAt rw(grp, p.ss), rp(grp, p.sp);
+        RingAt rw(grp / PS, p.ss), rp(grp / PS, p.sp);
         bool ok = true;
-        int next = grp;
-        for (int step8 = grp; step8 < total && ok; step8 += 8) {
+        int next = grp / PS;
+        for (int step8 = grp; step8 < rounds * PS && ok; step8 += 8) {
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
                 const int step = step8 + 4 * u;
-                if (step >= total || !ok) break;
-                const uint32_t stage = rw.s * stage_bytes;
+                if (step >= rounds * PS || !ok) break;
+                const uint32_t stage = rw.s * (PS * step_bytes);
                 if (step < nq) {
-                    const RawScale rs = slot[u];
-                    if (step + 8 < nq) slot[u] = fetch(q_lo + step + 8);
+                    const RawScale rs = scales.next(u);
                     if (rs.v != v_cached) { v_cached = rs.v; sigma = __fdiv_rn(rs.v, q.levels); }
                     float s[4];
                     s[0] = __fmul_rn(static_cast<float>(rs.sc & 255u), sigma);
                     s[1] = s[0]; s[2] = s[0]; s[3] = s[0];
-                    if (nsc == 2) { s[2] = __fmul_rn(static_cast<float>(rs.sc >> 8), sigma); s[3] = s[2]; }
+                    if (nsc == 2) { s[2] = __fmul_rn(static_cast<float>((rs.sc >> 8) & 255u), sigma); s[3] = s[2]; }
                     if (nsc == 4) {
                         s[1] = __fmul_rn(static_cast<float>((rs.sc >> 8) & 255u), sigma);
                         s[2] = __fmul_rn(static_cast<float>((rs.sc >> 16) & 255u), sigma);
                         s[3] = __fmul_rn(static_cast<float>(rs.sc >> 24), sigma);
                     }
                     const int kt = BWD ? (my_col >> 6) : q_lo + step;
-                    const uint32_t src = wsrc + rp.s * P_BYTES;
+                    const uint32_t src = wsrc + rp.s * (PS * P_BYTES);
                     ok = wait2(empty(rw.s), rw.ph ^ 1, full_p(rp.s), rp.ph, ctl, 55, 56);
                     if (!ok) break;
                     if constexpr (TA) {
                         tc_fence_after();               // the tensor core is done with this stage's columns
                         dequant_row64_tmem<B>(src + slab_row_slot(lane, 0, kt) * 4, src + (B * 32 + slab_row_slot(lane, 1, kt)) * 4, s, nsc,
-                                              tmem + (static_cast<uint32_t>(wi * 32) << 16) + kSwTmemA + rw.s * 32, lut8 + lane);
+                                              tmem + (static_cast<uint32_t>(wi * 32) << 16) + kSwTmemA + (rw.s * PS + half) * 32, lut8 + lane);
                         tmem_st_wait();
                         tc_fence_before();
                     } else {
@@ -424,7 +546,10 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(empty_p(rp.s));
-                    rp.advance(4, p.sp);
+                    rp.advance(4 / PS, p.sp);
+                } else if (step >= total) {
+                    ok = wait(empty(rw.s), rw.ph ^ 1, ctl, 57);      // the second step of the last stage does not exist
+                    if (!ok) break;
                 } else {
                     // rank-r step: the weight-side operand is rows of L1 (forward) or L2; by TMA where it goes to shared memory
                     ok = wait(empty(rw.s), rw.ph ^ 1, ctl, 57);
@@ -443,7 +568,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                                 if (n < q.N && j < p.r) v = __ldg(reinterpret_cast<const uint4*>(p.L1 + static_cast<size_t>(n) * p.r + j));
                                 o[4 * c] = v.x; o[4 * c + 1] = v.y; o[4 * c + 2] = v.z; o[4 * c + 3] = v.w;
                             }
-                            tmem_st16(tmem + (static_cast<uint32_t>(wi * 32) << 16) + kSwTmemA + rw.s * 32 + 16 * g, o);
+                            tmem_st16(tmem + (static_cast<uint32_t>(wi * 32) << 16) + kSwTmemA + (rw.s * PS + half) * 32 + 16 * g, o);
                         }
                         tmem_st_wait();
                         tc_fence_before();
@@ -452,10 +577,10 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                         if (lane == 0) {
                             if (!BWD) {
                                 mbar_expect_tx(fbar(d), kSwWBytes);
-                                tma_load_2d(ring + stage, &tmF, d * BK, c0, fbar(d));
+                                tma_load_2d(ring + half * step_bytes + stage, &tmF, d * BK, c0, fbar(d));
                             } else {
                                 mbar_expect_tx(fbar(d), have * 8192);
-                                for (int t = 0; t < have; ++t) tma_load_2d(ring + stage + t * 8192, &tmF, c0 + t * 64, d * BK, fbar(d));
+                                for (int t = 0; t < have; ++t) tma_load_2d(ring + half * step_bytes + stage + t * 8192, &tmF, c0 + t * 64, d * BK, fbar(d));
                             }
                         }
                         ok = wait(fbar(d), 0, ctl, 59);
@@ -464,8 +589,8 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                     __syncwarp();
                 }
                 if (lane == 0) mbar_arrive(full(rw.s));
-                next = step + 4;
-                rw.advance(4, p.ss);
+                next = step / PS + 4 / PS;
+                rw.advance(4 / PS, p.ss);
             }
         }
         if (lane == 0) reached[warp] = next;
@@ -476,7 +601,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             tc_fence_after();
             const int quarter = warp & 3, chunks = (p.box + 31) >> 5;
             float* accbuf = reinterpret_cast<float*>(base);           // [token][128 columns], over the idle rings
-            for (int ch = dw >> 2; ch < p.nbox * chunks; ch += 4) {
+            for (int ch = dw >> 2; ch < nbox * chunks; ch += 4) {
                 const int h = ch / chunks, t0 = (ch - h * chunks) * 32;
                 uint32_t v[32];
                 tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + h * 256 + t0, v);
@@ -503,43 +628,52 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             }
         }
     }
+    if (warp != 3) { __syncwarp(); cluster_wait_acquire(); }
     if (nsplit > 1) {
         // every CTA adds up and stores its share of the tokens from the CTAs with the same columns; the barriers are executed
         // by all threads of all CTAs, whatever happened before
         const uint32_t acc_addr = ring;
-        const int tokens = p.nbox * p.box;
+        const int tokens = nbox * p.box;
         const int t_lo = tokens * split / nsplit, t_hi = tokens * (split + 1) / nsplit;
         __syncthreads();
         cluster_barrier();
-        for (int item = threadIdx.x; item < (t_hi - t_lo) * 32; item += kSwThreads) {
-            const int t = t_lo + (item >> 5), cg = (item & 31) * 4;
-            const int m = m0 + t;
-            if (m >= p.M) break;                                   // tokens rise with the item
-            float4 part[4];
+        // four items of four columns at a time: one round trip through the cluster for most calls
+        const int items = (min(t_hi, p.M - m0) - t_lo) * 32;
+        for (int item0 = threadIdx.x; item0 < items; item0 += 4 * kSwThreads) {
+            float4 part[4][4];
 #pragma unroll
-            for (int z = 0; z < 4; ++z)
-                if (z < nsplit) part[z] = ld_dsmem_f32x4(acc_addr + static_cast<uint32_t>(t * 128 + cg) * 4u, rank + 2 * z);
-            float4 sum = part[0];
+            for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int z = 1; z < 4; ++z)
-                if (z < nsplit) { sum.x += part[z].x; sum.y += part[z].y; sum.z += part[z].z; sum.w += part[z].w; }
-            if (c0 + cg < p.out_cols)
-                *reinterpret_cast<uint2*>(p.out + static_cast<size_t>(m) * p.out_cols + c0 + cg) = make_uint2(pack_bf16(sum.x, sum.y), pack_bf16(sum.z, sum.w));
+                for (int z = 0; z < 4; ++z) {
+                    const int item = item0 + u * kSwThreads;
+                    if (z < nsplit && item < items)
+                        part[u][z] = ld_dsmem_f32x4(acc_addr + static_cast<uint32_t>((t_lo + (item >> 5)) * 128 + (item & 31) * 4) * 4u, rank + 2 * z);
+                }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int item = item0 + u * kSwThreads, cg = (item & 31) * 4;
+                if (item >= items || c0 + cg >= p.out_cols) continue;
+                float4 sum = part[u][0];
+#pragma unroll
+                for (int z = 1; z < 4; ++z)
+                    if (z < nsplit) { sum.x += part[u][z].x; sum.y += part[u][z].y; sum.z += part[u][z].z; sum.w += part[u][z].w; }
+                *reinterpret_cast<uint2*>(p.out + static_cast<size_t>(m0 + t_lo + (item >> 5)) * p.out_cols + c0 + cg) = make_uint2(pack_bf16(sum.x, sum.y), pack_bf16(sum.z, sum.w));
+            }
         }
     }
     tc_fence_before();
     __syncthreads();
     cluster_barrier();            // tensor and shared memory are released only when no CTA of the cluster uses them any more
     if (*abort_s) {
-        // copies in flight land before the CTA exits.  The barrier of a step counts its token boxes, the warps of its weights and
+        // copies in flight land before the CTA exits.  The barrier of a stage counts its token boxes, the warps of its weights and
         // the second CTA's word: those that have not come will not (everybody has left the loops), so they are made up for here, and
-        // the phase then waits for the boxes alone.  A box of step j is issued behind the end of step j - ss, so the last ss steps
-        // that any box was issued for are the ones that can be open, each in the phase j / ss of its stage.
+        // the phase then waits for the boxes alone.  A box of stage j is issued behind the end of stage j - ss, so the last ss stages
+        // that any box was issued for are the ones that can be open, each in the phase j / ss of its place in the ring.
         if (warp == 0) {
-            const int top = p.nbox == 2 ? max(reached[0], reached[1]) : reached[0];
+            const int top = max(reached[0], reached[1]);
             for (int j = max(0, top - p.ss); j < top; ++j) {
-                int missing = (j >= reached[0] ? 1 : 0) + (p.nbox == 2 && j >= reached[1] ? 1 : 0) + (rank == 0 && j >= reached[3] ? 1 : 0);
-                for (int w = 0; w < 4; ++w) missing += (j >= reached[kSwFirstDeq + 4 * (j & 3) + w] ? 1 : 0);
+                int missing = (j >= reached[0] ? 1 : 0) + (j >= reached[1] ? 1 : 0) + (rank == 0 && j >= reached[3] ? 1 : 0);
+                for (int w = 0; w < 4 * PS; ++w) missing += (j >= reached[kSwFirstDeq + 4 * PS * (j & (4 / PS - 1)) + w] ? 1 : 0);
                 if (lane < missing) mbar_arrive(full(j % p.ss));
                 let_land(full(j % p.ss), (j / p.ss) & 1);
             }
@@ -561,7 +695,7 @@ inline int tc_max_clusters(int n) {
     if (known >= 0) return known;
     const int fallback[4] = {74, 33, 22, 15};
     int got = 0;
-    auto kern = tc_swap_linear_kernel<3, false, false>;
+    auto kern = tc_swap_linear_kernel<3, false, false, 1>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2, 1, n / 2);
     cfg.blockDim = dim3(kSwThreads);
@@ -588,22 +722,25 @@ struct SwapPlan {
     double us;                       // estimated time
 };
 
-// Ring depths; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase
-// while the one before it can be incomplete.  A dequantization warp works on every fourth step:
-//   - it may wait for stage j % ss to be free (the tensor core is done with step j - ss) once step j - 2 ss is known to be
-//     done; its own step j - 4 waited for j - 4 - ss, hence ss >= 4;
-//   - it may wait for the codes of step j once those of step j - sp are known to have landed: they have where its own
-//     group used them (sp = 4, 8) or where the tensor core is done with that step (sp >= ss).
+// Ring depths in stages; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase
+// while the one before it can be incomplete.  A dequantization warp works on every fourth step, i.e. on every fourth (one step per
+// stage) or second stage; with g for that number:
+//   - it may wait for stage j % ss to be free (the tensor core is done with stage j - ss) once stage j - 2 ss is known to be
+//     done; its own stage j - g waited for j - g - ss, hence ss >= g;
+//   - it may wait for the codes of stage j once those of stage j - sp are known to have landed: they have where its own
+//     group used them (sp a multiple of g) or where the tensor core is done with that stage (sp >= ss).
 inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
-    const int stage = kSwWBytes + pl.nbox * pl.box * 64, pk = 1024 * b0;
+    const int steps = swap_stage_steps(pl.nbox), g = 4 / steps;
+    const int stage = steps * (kSwWBytes + pl.nbox * pl.box * 64), pk = steps * 1024 * b0;
     const int fixed = 1024 + kSwTail + (b0 == 8 ? 32768 : 0);
     const int room = kSmemLimit - fixed;
-    pl.ss = (room - 4 * pk) / stage;
-    if (pl.ss > kSwMaxStages) pl.ss = kSwMaxStages;
-    if (pl.ss < 4) return false;
+    pl.ss = (room - g * pk) / stage;
+    if (pl.ss > kSwMaxStages / steps) pl.ss = kSwMaxStages / steps;
+    if (pl.ss < g) return false;
+    while (pl.ss > g && (room - pl.ss * stage) / pk < pl.ss) --pl.ss;      // (wide codes: no fewer stages of codes than of weights)
     pl.sp = (room - pl.ss * stage) / pk;
     if (pl.sp > kSwMaxStages) pl.sp = kSwMaxStages;
-    if (pl.sp < pl.ss) pl.sp = 4;
+    if (pl.sp < pl.ss) pl.sp = g;
     const int bytes = pl.ss * stage + pl.sp * pk;
     if (ks > 1 && pl.nbox * pl.box * 512 > bytes) return false;      // the accumulators are laid over the rings
     pl.smem = fixed + bytes;
@@ -618,15 +755,38 @@ inline int swap_max_tokens(int b0) {
     return 2 * pl.box;
 }
 
+// Splits of the contraction of a rank-r pre-product with `mtiles` row tiles and `steps` steps of 64 that runs beside a linear kernel of
+// `main_ctas` CTAs (programmatic dependent launch): it gets the SMs that the last wave of that kernel leaves idle, and at least one CTA per row
+// tile.  A power of two: it divides the 64 columns of the accumulator.
+inline int pre_splits(int mtiles, int steps, long long main_ctas) {
+    const int sms = dec::sm_count_cached(), idle = static_cast<int>((sms - main_ctas % sms) % sms);
+    int want = idle / mtiles;
+    if (main_ctas < sms) want = idle / 2 / mtiles;      // beside a single wave of clusters: half of what it leaves (clusters need room)
+    if (want > steps / 4) want = steps / 4;
+    if (want > 8) want = 8;          // splits of a tile form a cluster (and more than eight made the sum the critical path)
+    if (idle < 48) {
+        // beside a nearly full linear kernel (itself made of clusters) large pre-product clusters took a cluster's place from it
+        const int cap = (idle / mtiles < 4) ? (idle / mtiles > 1 ? idle / mtiles : 1) : 4;
+        if (want > cap) want = cap;
+    }
+    if (want < 1) want = 1;
+    while (want & (want - 1)) want &= want - 1;
+    return want;
+}
+
 // The split of a call that costs least by a simple model: waves of clusters, each with a fixed cost, its steps (the
-// slower of dequantization and tensor core) and its reduction.  Fitted to 2300 timings of all chunk counts and slices (twelve shapes, 2 to
-// 8 bits, 20 to 1800 rows): the plan that it picks takes 2.5 % longer than the best one on average (4.8 % with the constants before,
-// which had no term for the SMs that the pre-product holds and made a single slice of a long contraction 20 % dearer).  us with 1, 2, 3,
-// 4 slices: 4096 x 4096 NF3, 64 rows: 24, 17, 15, 26 (16 clusters of eight, of which 15 fit); 8192 x 8192 NF4, 17 rows: 53, 32, 45, 56.
-inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+// slower of dequantization and tensor core, softened) and its reduction, or the pre-product that runs beside it where that takes longer.  Fitted to
+// the timings of all chunk counts and slices of 1400 drawn shapes (2 to 8 bits, 9 to 2000 rows, with and without a rank-r term): the plan that it
+// picks takes 1.8 % longer than the best one on average (3.4 % with the constants before, which did not count the clusters that the
+// pre-product displaces).  us as a
+// graph, plans and kernel before / now: 4096 x 4096 NF4, 64 rows 16.1 / 15.4; 28672 x 8192 NF3, 128 rows 83 / 73; 4008 x 15616 NF3, 517 rows 61.4 / 61.5;
+// 1024 x 1024 NF3, 512 rows 11.8 / 10.3.  Left slower: 1664 x 11776 NF3 input gradient, 778 rows 38 / 45; 2904 x 4288 NF3, 309 rows 18.6 / 21.3.
+inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
     SwapPlan best{};
     best.us = -1.0;
-    const double dq = b0 == 2 ? 0.22 : b0 == 3 ? 0.26 : b0 == 4 ? 0.35 : 0.47;      // us per step of 128 x 64 weights
+    // us per step of 128 x 64 weights: through tensor memory, through shared memory; small blocks cost more tables
+    static const double dq_ta[4] = {0.22, 0.245, 0.355, 0.50}, dq_smem[4] = {0.245, 0.27, 0.355, 0.525};
+    const double dq_block = B0 == 16 ? 1.15 : B0 == 32 ? 1.06 : 1.0;
     const long long pairs = (out_cols + 255) / 256;
     int first = static_cast<int>((M + 511) / 512);
     // The search covers eight numbers of chunks.  Where the chunks of all of them are too large for the rings (8-bit codes
@@ -647,23 +807,26 @@ inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q,
             if (!swap_rings(b0, ks, pl)) continue;
             pl.ks = ks;
             pl.ctas = 2 * pairs * pl.chunks * ks;
-            // a rank-r pre-product runs beside this kernel and takes SMs: a CTA per 128 tokens, and out of the GPCs, which costs large
-            // clusters most (a second wave costs more than a finer split saves)
-            const int taken[4] = {2, 1, 2, 4};
-            long long at_once = tc_max_clusters(2 * ks) - (steps_d > 0 ? taken[ks - 1] : 0);
-            if (ks == 1 && steps_d > 0) {
-                const long long beside = tc_max_clusters(2) - ((M + 127) / 128 + 1) / 2;
-                if (beside < at_once) at_once = beside < 1 ? 1 : beside;
+            const double dq = dq_block * (!backward && pl.nbox == 1 ? dq_ta : dq_smem)[bits_index(b0)], mma = 0.001 * tokens;
+            const double step = std::pow(dq * dq * dq * dq + mma * mma * mma * mma, 0.25);
+            // a rank-r pre-product runs beside this kernel and takes SMs out of the GPCs, which costs large clusters most
+            long long at_once = tc_max_clusters(2 * ks);
+            double pre = 0.0;
+            if (steps_d > 0) {
+                const int mtiles = static_cast<int>((M + 127) / 128), w = pre_splits(mtiles, steps_q, pl.ctas);
+                // Single CTAs fill a TPC together; an odd number of one-split tiles is launched one by one and holds a TPC each.  Beside clusters of
+                // four and six a GPC has a TPC or two to spare, which small pre-product clusters take first.
+                const int tpcs = w == 1 ? (mtiles % 2 && ks == 1 ? mtiles : (mtiles + 1) / 2) : mtiles * w / 2;
+                at_once -= ks == 1 ? tpcs : ks == 2 ? (w >= 4 ? (tpcs > 2 ? mtiles * (w / 4) : 0) : tpcs > 5 ? (tpcs - 4) / 2 : 0) : ks == 3 ? (tpcs > 4 ? (tpcs - 2) / 3 : 0) : mtiles;
+                if (at_once < 1) at_once = 1;
+                pre = 8.9 + 0.3 * ((steps_q + w - 1) / w);
             }
             const long long waves = (pairs * pl.chunks + at_once - 1) / at_once;
-            const double step = dq > tokens * 0.0012 ? dq : tokens * 0.0012;
-            const double body = 6.5 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 2.5 + tokens * 0.008 : tokens * 0.006);
-            pl.us = waves * body;
-            if (ks == 1 && steps_q > 16) pl.us *= 1.1;  // a single slice of a long contraction
-            // clusters of four and more leave GPCs partly empty between waves; 1.3 with one chunk of few tokens too had made long contractions
-            // run unsliced (us in a graph, one slice / as picked now: 9472 x 16640 NF3, 30 rows 88 / 70; 9088 x 16896 NF2, 19 rows 74 / 59;
-            // 8320 x 22272 NF8 input gradient, 24 rows 153 / 130; 9856 x 17408 NF8, 1384 rows in four chunks and two waves 484, pairs 469)
-            if (ks > 1 && waves > 1) pl.us *= pl.chunks > 1 ? 1.3 : 1.1;
+            const double body = 5.4 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 1.4 + 0.04 * tokens / ks : 0.0115 * tokens);
+            // clusters of four and more leave GPCs partly empty between waves
+            pl.us = body * (1.0 + (ks == 1 ? 0.8 : ks == 2 ? 0.85 : 1.2) * (waves - 1) + (waves > 1 ? (ks == 1 ? 0.0 : ks == 2 ? 0.1 : 0.3) : 0.0));
+            if (ks == 1 && steps_q > 16) pl.us *= 1.1;      // a single slice of a long contraction
+            if (pre > 0.0) pl.us = std::pow(std::pow(pl.us, 6.0) + std::pow(pre, 6.0), 1.0 / 6.0);
             if (best.us < 0 || pl.us < best.us) best = pl;
         }
     }
@@ -671,24 +834,24 @@ inline SwapPlan make_swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q,
 }
 
 // The same, with the plans of the last few shapes kept by the calling thread (pure arithmetic, about 3 us).
-inline const SwapPlan& swap_plan(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
-    struct Entry { int b0 = 0, steps_q = 0, steps_d = 0; int64_t M = 0, out_cols = 0; SwapPlan plan; };
+inline const SwapPlan& swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+    struct Entry { int b0 = 0, B0 = 0, steps_q = 0, steps_d = 0; bool backward = false; int64_t M = 0, out_cols = 0; SwapPlan plan; };
     constexpr int kEntries = 32;
     thread_local Entry cache[kEntries];
     const uint64_t h = (static_cast<uint64_t>(M) * 0x9E3779B97F4A7C15ull) ^ (static_cast<uint64_t>(out_cols) * 0xC2B2AE3D27D4EB4Full) ^
-                       (static_cast<uint64_t>(steps_q * 8 + steps_d * 64 + b0) * 0x165667B19E3779F9ull);
+                       (static_cast<uint64_t>(steps_q * 8 + steps_d * 64 + b0 + B0 * 4096 + (backward ? 16 : 0)) * 0x165667B19E3779F9ull);
     Entry& e = cache[(h >> 40) % kEntries];
-    if (e.b0 != b0 || e.M != M || e.out_cols != out_cols || e.steps_q != steps_q || e.steps_d != steps_d) {
-        e.plan = make_swap_plan(b0, M, out_cols, steps_q, steps_d);
-        e.b0 = b0; e.M = M; e.out_cols = out_cols; e.steps_q = steps_q; e.steps_d = steps_d;
+    if (e.b0 != b0 || e.B0 != B0 || e.backward != backward || e.M != M || e.out_cols != out_cols || e.steps_q != steps_q || e.steps_d != steps_d) {
+        e.plan = make_swap_plan(b0, B0, backward, M, out_cols, steps_q, steps_d);
+        e.b0 = b0; e.B0 = B0; e.backward = backward; e.M = M; e.out_cols = out_cols; e.steps_q = steps_q; e.steps_d = steps_d;
     }
     return e.plan;
 }
 
-template <int B, bool BWD, bool TA>
+template <int B, bool BWD, bool TA, int PS>
 inline int launch_swap(const CUtensorMap& tX, const CUtensorMap& tT, const CUtensorMap& tF, const SwapParams& p, const SwapPlan& pl,
-                       int smem, int pairs, cudaStream_t st, bool after_pre) {
-    auto kern = tc_swap_linear_kernel<B, BWD, TA>;
+                       int smem, int pairs, cudaStream_t st, bool first) {
+    auto kern = tc_swap_linear_kernel<B, BWD, TA, PS>;
     static bool attr_done = false;
     if (!attr_done) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
@@ -708,16 +871,17 @@ inline int launch_swap(const CUtensorMap& tX, const CUtensorMap& tT, const CUten
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = (p.steps_d > 0 && after_pre) ? 2 : 1;      // overlap with the rank-r pre-product kernel in front of it
+    cfg.numAttrs = first ? 2 : 1;      // overlap with the rank-r pre-product, or with the call in front
     const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tX, tT, tF, p);
     count_launch(1);
     if (e != cudaSuccess) { cudaGetLastError(); return LQLORA_ERR_CUDA; }
     return LQLORA_OK;
 }
 
-// Output columns [c_base, c_base + cols) of a call with the plan `pl`; T: the rank-r intermediate [M][r] (r > 0).
+// Output columns [c_base, c_base + cols) of a call with the plan `pl`; T: the rank-r intermediate [M][r] (r > 0).  first: nothing but the
+// pre-product of the call runs in front of it.
 inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const void* A, int M, void* out, const void* T, int* status,
-                    bool backward, const SwapPlan& pl, int c_base, int cols, cudaStream_t st, bool after_pre) {
+                    bool backward, const SwapPlan& pl, int c_base, int cols, cudaStream_t st, bool first) {
     const int C = backward ? q.N : q.K;
     SwapParams p;
     p.q = q;
@@ -730,15 +894,16 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     p.c_base = c_base;
     p.nbox = pl.nbox; p.box = pl.box; p.ss = pl.ss; p.sp = pl.sp; p.tmem_cols = pl.tmem_cols;
     p.L1 = static_cast<const __nv_bfloat16*>(L1); p.r = r;
+    p.clear_status = first ? 1 : 0;
     int smem = pl.smem;
-    p.tail_off = pl.ss * (kSwWBytes + pl.nbox * pl.box * 64) + pl.sp * 1024 * q.b0;
+    p.tail_off = swap_stage_steps(pl.nbox) * (pl.ss * (kSwWBytes + pl.nbox * pl.box * 64) + pl.sp * 1024 * q.b0);
     const bool ta = !backward && pl.nbox == 1;      // (256 columns of accumulators and eight stages of 32 columns fill tensor memory)
     if (ta) {
-        // Without weight tiles eight stages of both rings always fit (256 tokens, 8-bit codes: 230,912 of 232,448 bytes, code book
-        // included), so a group's codes of step j - sp are its own (see swap_rings); the token stages alone hold the accumulators
-        // that a sliced contraction lays over them (8 x 64 = 512 bytes per token).
-        const int fixed = 1024 + kSwTail + (q.b0 == 8 ? 32768 : 0), x = pl.box * 64, pk = 1024 * q.b0;
-        p.ss = kSwMaxStages;
+        // Without weight tiles four stages of two steps of both rings always fit (256 tokens, 8-bit codes: 230,912 of 232,448 bytes, code
+        // book included), so the tensor core is done with the codes of stage j - sp (see swap_rings); the token stages alone hold the
+        // accumulators that a sliced contraction lays over them (8 x 64 = 512 bytes per token).
+        const int fixed = 1024 + kSwTail + (q.b0 == 8 ? 32768 : 0), x = 2 * pl.box * 64, pk = 2 * 1024 * q.b0;
+        p.ss = kSwMaxStages / 2;
         p.sp = (kSmemLimit - fixed - p.ss * x) / pk;
         if (p.sp > kSwMaxStages) p.sp = kSwMaxStages;
         p.tail_off = p.ss * x + p.sp * pk;
@@ -758,9 +923,10 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     const int pairs = (cols + 255) / 256;
     auto go = [&](auto bits) {
         constexpr int B = decltype(bits)::value;
-        if (backward) return launch_swap<B, true, false>(tX, tT, tF, p, pl, smem, pairs, st, after_pre);
-        if (ta) return launch_swap<B, false, true>(tX, tT, tF, p, pl, smem, pairs, st, after_pre);
-        return launch_swap<B, false, false>(tX, tT, tF, p, pl, smem, pairs, st, after_pre);
+        if (ta) return launch_swap<B, false, true, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (!backward) return launch_swap<B, false, false, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (pl.nbox == 1) return launch_swap<B, true, false, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        return launch_swap<B, true, false, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
     };
     switch (q.b0) {
         case 2: return go(std::integral_constant<int, 2>());

@@ -348,8 +348,10 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
         // all threads of all CTAs of the cluster pass here, whatever happened before
         __syncthreads();
         if (nsplit > 1) dec::cluster_wait();           // every CTA of the cluster has started
-        const uint32_t recv_addr = smem_u32(recv);
-        const int cols_share = p.rp / nsplit;
+        // Four columns at a time: a thread's scalar stores, with a division each to find the column's owner, took longer than the four
+        // steps of a short contraction (1024 x 1024 NF3 at 512 rows, whole call: 12.0 us, with this 10.3).  The shares are powers of two from eight columns on.
+        const uint32_t recv_addr = smem_u32(recv);         // [split][column / 4 of the share][row] of float4
+        const int cols_share = p.rp / nsplit, log_share = 31 - __clz(cols_share);
         if (warp > kLrProducers && cl_ok) {
             tc_fence_after();
             const int quarter = warp & 3;
@@ -362,23 +364,28 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
                     for (int i = 0; i < 32; ++i) v[i] = 0u;
                 }
 #pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    const int c = col + i;
-                    const int owner = c / cols_share, cl = c - owner * cols_share;
-                    const uint32_t off = static_cast<uint32_t>((split * cols_share + cl) * 128 + row) * 4u;
-                    if (nsplit > 1) dec::st_dsmem_f32(recv_addr + off, static_cast<uint32_t>(owner), __uint_as_float(v[i]));
-                    else recv[cl * 128 + row] = __uint_as_float(v[i]);
+                for (int i = 0; i < 32; i += 4) {
+                    const int c = col + i, owner = c >> log_share, c4 = (c & (cols_share - 1)) >> 2;
+                    dec::st_dsmem_v4(recv_addr + static_cast<uint32_t>((split * (cols_share >> 2) + c4) * 128 + row) * 16u, static_cast<uint32_t>(owner),
+                                     v[i], v[i + 1], v[i + 2], v[i + 3]);
                 }
             }
         }
         __syncthreads();
         if (nsplit > 1) dec::cluster_sync_all();
-        for (int item = threadIdx.x; item < 128 * cols_share; item += kLrThreads) {
-            const int row = item & 127, cl = item >> 7;
-            float sum = 0.0f;
-            for (int src = 0; src < nsplit; ++src) sum += recv[(src * cols_share + cl) * 128 + row];
-            const int m = m0 + row, col = split * cols_share + cl;
-            if (m < p.M && col < p.r) p.T[static_cast<size_t>(m) * p.r + col] = __float2bfloat16_rn(sum);
+        for (int item = threadIdx.x; item < 32 * cols_share; item += kLrThreads) {
+            const int row = item & 127, c4 = item >> 7;
+            float4 sum = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            for (int src = 0; src < nsplit; ++src) {
+                const float4 x = reinterpret_cast<const float4*>(recv)[(src * (cols_share >> 2) + c4) * 128 + row];
+                sum.x += x.x; sum.y += x.y; sum.z += x.z; sum.w += x.w;
+            }
+            const int m = m0 + row, col = split * cols_share + c4 * 4;
+            if (m < p.M && col < p.r) {
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(sum.x, sum.y), hi = __floats2bfloat162_rn(sum.z, sum.w);
+                *reinterpret_cast<uint2*>(p.T + static_cast<size_t>(m) * p.r + col) =
+                    make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+            }
         }
     }
     tc_fence_before();
@@ -505,10 +512,11 @@ inline int pair_peel(int64_t M, int64_t out_cols) {
 }
 
 // CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs, and below 2048 rows unless the transposed tiles,
-// which pad to 16 rows instead of 512 and choose their split, are estimated to take less than 0.85 of their time: whole waves of the pair
-// kernel, 6 us and 0.64 us (8-bit codes 0.95) per step each.  us as a graph, pair / transposed: 8192 x 8192 NF3 at 520 rows 87 / 59, 700 88 /
-// 67, 900 91 / 87, 1100 170 / 137, 1400 174 / 131, 1700 180 / 162; 5120 x 5120 NF2 at 520 rows 57 / 33, 1100 59 / 47; 11008 x 4096 NF4 input
-// gradient at 1100 rows 112 / 83; 8192 x 8192 NF8 at 520 rows 129 / 87, 1100 253 / 171; 4096 x 4096 NF4 at 1700 rows 54 / 50.
+// which pad to 16 rows instead of 512 and choose their split, are estimated faster: whole waves of the pair kernel are taken as 6 us and 0.64 us
+// (8-bit codes 0.95) per step each, 7 % less than they last on average, hence the 1.1.  Over 260 drawn calls of 257 to 2000 rows the side taken is 2.6 %
+// behind the faster one (7.8 % with 0.85, the line of the transposed tiles with one step per stage).  One wave that is at least four
+// fifths full, and more than four waves of rows without padding, stay with the pairs up to 0.88.  us as a graph, pair / transposed: 8192 x 8192 NF3 at 520 rows 87 / 50,
+// 11904 x 8448 NF3 at 546 rows 123 / 80, 4352 x 11008 NF3 at 688 rows 78 / 60, 7552 x 2176 NF2 at 1285 rows 50 / 44; 8320 x 4992 NF8 at 825 rows 79 / 100.
 // From 2048 rows on the pairs stay whatever the estimates say.  That line is drawn by hand.  Both sides measured on nine shapes, both passes,
 // 3-, 4- and 8-bit codes, 2048 to 4096 rows: where the last wave of pair tiles is well filled the pairs are up to a fifth faster (4096 x 4096 NF3
 // at 4096 rows 97 / 120, 28672 x 8192 NF8 at 2048 902 / 1064, 8192 x 8192 NF8 at 2048 273 / 306); where it is between a quarter and a half
@@ -519,48 +527,36 @@ inline double pair_estimate(int b0, int64_t M, int64_t out_cols, int steps_q) {
     const long long pairs = sm_count() / 2, waves = (static_cast<long long>(mt) * (c_tiles - peel) + pairs - 1) / pairs;
     return static_cast<double>(waves) * (6.0 + steps_q * (b0 == 8 ? 0.95 : 0.64)) + (peel > 0 ? 20.0 + 0.15 * steps_q : 0.0);
 }
-inline bool tc_use_pair(int b0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+inline bool tc_use_pair(const QView& q, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
     if (M <= 256) return false;
     const long long pair_ctas = 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN);
     if (2 * pair_ctas <= sm_count()) return false;
-    return M >= 2048 || swap_plan(b0, M, out_cols, steps_q, steps_d).us >= 0.85 * pair_estimate(b0, M, out_cols, steps_q);
+    if (M >= 2048) return true;
+    const int64_t rows = (M + 511) / 512 * 512;
+    const bool full = pair_ctas <= sm_count() ? 5 * pair_ctas >= 4 * sm_count() : 16 * M >= 15 * rows && pair_ctas > 4 * sm_count();
+    return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d).us >= (full ? 0.88 : 1.1) * pair_estimate(q.b0, M, out_cols, steps_q);
 }
 
 // The launch on transposed tiles that a call needs: the whole of it, or the output columns from *c_base on that the pair
 // kernel leaves (none where *c_base is not below out_cols).
-inline SwapPlan call_swap_plan(int b0, bool pair, int64_t M, int64_t out_cols, int steps_q, int steps_d, int* c_base) {
+inline SwapPlan call_swap_plan(const QView& q, bool backward, bool pair, int64_t M, int64_t out_cols, int steps_q, int steps_d, int* c_base) {
     *c_base = 0;
-    if (!pair) return swap_plan(b0, M, out_cols, steps_q, steps_d);
+    if (!pair) return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d);
     const int peel = pair_peel(M, out_cols);
     *c_base = (static_cast<int>((out_cols + BN - 1) / BN) - peel) * BN;
-    return peel > 0 ? swap_plan(b0, M, out_cols - *c_base, steps_q, steps_d) : SwapPlan{};
+    return peel > 0 ? swap_plan(q.b0, q.B0, backward, M, out_cols - *c_base, steps_q, steps_d) : SwapPlan{};
 }
 
 // C = contraction length, out_cols = width of the output of the linear kernel that follows.
-inline PrePlan pre_plan(int b0, int64_t C, int r, int64_t M, int64_t out_cols) {
+inline PrePlan pre_plan(const QView& q, bool backward, int64_t C, int r, int64_t M, int64_t out_cols) {
     PrePlan pl;
     pl.mtiles = static_cast<int>((M + 127) / 128);
     pl.steps = static_cast<int>((C + BK - 1) / BK);
-    // The pre-product runs beside the linear kernel that follows it (programmatic dependent launch):
-    // give it the SMs that the last wave of that kernel leaves idle, and at least one CTA per row tile.
-    const int sms = sm_count();
-    const long long main_ctas = tc_use_pair(b0, M, out_cols, pl.steps, (r + BK - 1) / BK) ? 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN)
-                                                              : swap_plan(b0, M, out_cols, pl.steps, (r + BK - 1) / BK).ctas;
-    const int idle = static_cast<int>((sms - main_ctas % sms) % sms);
-    int want = idle / pl.mtiles;
-    if (main_ctas < sms) want = idle / 2 / pl.mtiles;      // beside a single wave of clusters: half of what it leaves (clusters need room)
-    if (want > pl.steps / 4) want = pl.steps / 4;
-    if (want > 8) want = 8;          // splits of a tile form a cluster (and more than eight made the sum the critical path)
-    if (idle < 48) {
-        // beside a nearly full linear kernel (itself made of clusters) large pre-product clusters took a cluster's place
-        // from it: at most four pre-product CTAs in all
-        const int cap = (idle / pl.mtiles < 4) ? (idle / pl.mtiles > 1 ? idle / pl.mtiles : 1) : 4;
-        if (want > cap) want = cap;
-    }
-    if (want < 1) want = 1;
-    while (want & (want - 1)) want &= want - 1;          // a power of two: it divides the 64 columns of the accumulator
-    pl.steps_per_split = (pl.steps + want - 1) / want;
-    pl.nsplit = want;
+    const int steps_d = (r + BK - 1) / BK;
+    const long long main_ctas = tc_use_pair(q, backward, M, out_cols, pl.steps, steps_d) ? 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN)
+                                                                                        : swap_plan(q.b0, q.B0, backward, M, out_cols, pl.steps, steps_d).ctas;
+    pl.nsplit = pre_splits(pl.mtiles, pl.steps, main_ctas);
+    pl.steps_per_split = (pl.steps + pl.nsplit - 1) / pl.nsplit;
     pl.rp = (r <= 64) ? 64 : 128;
     return pl;
 }
@@ -636,14 +632,15 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
                      bool backward, cudaStream_t st) {
     using namespace tc;
     const int C = backward ? q.N : q.K;              // contraction length
-    const PrePlan pl = pre_plan(q.b0, C, r, M, backward ? q.K : q.N);
-    // workspace: [status word][T bf16]; the status word is cleared by the first kernel of the call (or the caller's memset)
+    const PrePlan pl = pre_plan(q, backward, C, r, M, backward ? q.K : q.N);
+    // workspace: [status word][T bf16]; the status word is cleared by the first kernel of the call (CTA pairs without a rank-r term: by a memset)
     __nv_bfloat16* T = reinterpret_cast<__nv_bfloat16*>(ws + kStatusBytes);
-    const bool pair = tc_use_pair(q.b0, M, backward ? q.K : q.N, pl.steps, (r + BK - 1) / BK);      // CTA pairs (cta_group::2) on [512, 256] tiles; boxes of 128 rows
+    const bool pair = tc_use_pair(q, backward, M, backward ? q.K : q.N, pl.steps, (r + BK - 1) / BK);      // CTA pairs (cta_group::2) on [512, 256] tiles; boxes of 128 rows
     const int out_cols = backward ? q.K : q.N;
     int c_base = 0;
-    const SwapPlan sp = call_swap_plan(q.b0, pair, M, out_cols, pl.steps, (r + BK - 1) / BK, &c_base);
+    const SwapPlan sp = call_swap_plan(q, backward, pair, M, out_cols, pl.steps, (r + BK - 1) / BK, &c_base);
     if (c_base < out_cols && sp.ks < 1) return LQLORA_ERR_INVALID_SHAPE;      // (never: a plan exists for every shape) before any launch
+    if (pair && r == 0 && cudaMemsetAsync(ws, 0, kStatusBytes, st) != cudaSuccess) { cudaGetLastError(); return LQLORA_ERR_CUDA; }
     CUtensorMap tA, tA2, tB2;
     if (pair && !make_map(&tA, A, M, C, 128)) return LQLORA_ERR_CUDA;
     if (r > 0) {

@@ -77,9 +77,9 @@ static int run_linear(const lqlora_qmatrix* q, const void* L1, const void* L2, i
     }
     const bool use_tc = tc_supported(v, r, M, backward);
     const bool use_decode = !use_tc && stream_supported(v, r, M, backward);
-    // With a rank-r term the first kernel of the call (the pre-product) clears what has to start at zero (the status
-    // word, and the arrival counters of the weight-streaming kernels); otherwise a memset does.
-    const bool first_kernel_clears = r > 0 && (use_decode || use_tc);
+    // The first kernel of a tensor-core call, and of a decode-sized one with a rank-r term (the pre-product), clears what has to start
+    // at zero (the status word, and the arrival counters of the weight-streaming kernels); otherwise a memset does.
+    const bool first_kernel_clears = use_tc || (r > 0 && use_decode);
     if (!first_kernel_clears) {
         const size_t n = use_decode ? stream::clear_bytes(v, backward) : static_cast<size_t>(kStatusBytes);
         if (cudaMemsetAsync(ws, 0, n, st) != cudaSuccess) return cuda_rc(cudaGetLastError());
@@ -575,9 +575,9 @@ int lqlora_linear_path(int64_t N, int64_t K, const lqlora_config* cfg, int r, in
     if (tc_supported(v, r, M, bwd)) {
         const int64_t out_cols = bwd ? K : N;
         const int steps_q = static_cast<int>(((bwd ? N : K) + tc::BK - 1) / tc::BK);
-        const bool pair = tc::tc_use_pair(v.b0, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK);
+        const bool pair = tc::tc_use_pair(v, backward != 0, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK);
         int c_base = 0;
-        const tc::SwapPlan sp = tc::call_swap_plan(v.b0, pair, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK, &c_base);
+        const tc::SwapPlan sp = tc::call_swap_plan(v, backward != 0, pair, M, out_cols, steps_q, (r + tc::BK - 1) / tc::BK, &c_base);
         if (c_base < out_cols && sp.ks < 1) return LQLORA_ERR_INVALID_SHAPE;      // as the call itself
         kernel = pair ? LQLORA_PATH_TC_PAIR : LQLORA_PATH_TC_ONE;
         if (!pair) ks = sp.ks;
