@@ -784,6 +784,7 @@ inline int pre_splits(int mtiles, int steps, long long main_ctas) {
 inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
     SwapPlan best{};
     best.us = -1.0;
+    double best_score = 0.0;
     // us per step of 128 x 64 weights: through tensor memory, through shared memory; small blocks cost more tables
     static const double dq_ta[4] = {0.22, 0.245, 0.355, 0.50}, dq_smem[4] = {0.245, 0.27, 0.355, 0.525};
     const double dq_block = B0 == 16 ? 1.15 : B0 == 32 ? 1.06 : 1.0;
@@ -822,12 +823,13 @@ inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t
                 pre = 8.9 + 0.3 * ((steps_q + w - 1) / w);
             }
             const long long waves = (pairs * pl.chunks + at_once - 1) / at_once;
-            const double body = 5.4 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? 1.4 + 0.04 * tokens / ks : 0.0115 * tokens);
+            const double body = 5.4 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? (ks > 2 ? 2.4 : 1.8) + 0.04 * tokens / ks : 0.0115 * tokens);
             // clusters of four and more leave GPCs partly empty between waves
             pl.us = body * (1.0 + (ks == 1 ? 0.8 : ks == 2 ? 0.85 : 1.2) * (waves - 1) + (waves > 1 ? (ks == 1 ? 0.0 : ks == 2 ? 0.1 : 0.3) : 0.0));
-            if (ks == 1 && steps_q > 16) pl.us *= 1.1;      // a single slice of a long contraction
             if (pre > 0.0) pl.us = std::pow(std::pow(pl.us, 6.0) + std::pow(pre, 6.0), 1.0 / 6.0);
-            if (best.us < 0 || pl.us < best.us) best = pl;
+            // of plans that are estimated alike, slices rather than one long contraction
+            const double score = pl.us * (ks == 1 && steps_q > 16 ? 1.15 : 1.0);
+            if (best.us < 0 || score < best_score) { best = pl; best_score = score; }
         }
     }
     return best;
