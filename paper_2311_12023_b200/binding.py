@@ -226,8 +226,32 @@ def alloc_qmatrix(N: int, K: int, cfg, device="cuda") -> QMatrix:
                    torch.empty(sb, dtype=torch.uint8, device=device), s2, N, K, cfg)
 
 
+# The native part of the binding (csrc/fast_binding.cpp): marshals an ordinary call and returns its result, the status number of a call that
+# failed, or None for a call that the Python code below has to look at.
+_fast = None
+
+
+def _fast_part():
+    global _fast
+    L = lib()
+    try:
+        from . import _fast as module
+    except ImportError as e:
+        raise FileNotFoundError(f"native part of the binding: {e}; build it with `python -m paper_2311_12023_b200.build`") from e
+    module.setup(*[ctypes.cast(f, ctypes.c_void_p).value for f in (L.lqlora_linear_fwd, L.lqlora_linear_bwd_input, L.lqlora_packed_sizes, L.lqlora_encode)],
+                 torch.nn.Parameter, QMatrix)
+    _fast = module
+    return module
+
+
 def encode(W: torch.Tensor, cfg, out: Optional[QMatrix] = None, workspace: Optional[torch.Tensor] = None) -> QMatrix:
     """lqlora_encode: W fp32 [N, K] on the device -> packed codes, scale codes, second-level scales."""
+    if out is None:
+        parts = (_fast or _fast_part()).encode(W, cfg, workspace)
+        if type(parts) is tuple:
+            return QMatrix(*parts, *W.shape, cfg)
+        if parts is not None:
+            raise LqloraError(parts, "lqlora_encode")
     assert W.is_cuda and W.dtype == torch.float32 and W.is_contiguous() and W.dim() == 2
     N, K = W.shape
     q = out if out is not None else alloc_qmatrix(N, K, cfg, W.device)
@@ -306,6 +330,11 @@ def _linear(fn, name, q, L1, L2, A, out_cols, out, workspace):
 
 def linear_fwd(q: QMatrix, L1, L2, X: torch.Tensor, out=None, workspace=None) -> torch.Tensor:
     """lqlora_linear_fwd: Y = X deq(Q)^T + (X L2^T) L1^T, bf16 [M, N]."""
+    y = (_fast or _fast_part()).linear(False, q, L1, L2, X, out, workspace)
+    if y is not None:
+        if type(y) is int:
+            raise LqloraError(y, "lqlora_linear_fwd")
+        return y
     assert X.shape[1] == q.K
     return _linear(lib().linear_fwd_packed, "lqlora_linear_fwd", q, L1, L2, X, q.N, out, workspace)
 
@@ -335,6 +364,11 @@ def linear_fwd_static(q: QMatrix, L1, L2, X: torch.Tensor, out: Optional[torch.T
 
 def linear_bwd_input(q: QMatrix, L1, L2, dY: torch.Tensor, out=None, workspace=None) -> torch.Tensor:
     """lqlora_linear_bwd_input: dX = dY deq(Q) + (dY L1) L2, bf16 [M, K]."""
+    y = (_fast or _fast_part()).linear(True, q, L1, L2, dY, out, workspace)
+    if y is not None:
+        if type(y) is int:
+            raise LqloraError(y, "lqlora_linear_bwd_input")
+        return y
     assert dY.shape[1] == q.N
     return _linear(lib().linear_bwd_input_packed, "lqlora_linear_bwd_input", q, L1, L2, dY, q.K, out, workspace)
 
