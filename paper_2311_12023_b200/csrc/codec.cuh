@@ -113,27 +113,38 @@ __device__ __forceinline__ void curve_encode(const float (&u)[32], float r_lo, f
         words[2] |= (word[3] & 0x44444444u) << 1;
     }
 }
-// The same for a thread with an element close to a threshold, or a reciprocal that is not a normal number: element by element (a
-// loop over the thread's row in shared memory, `at(j)`), the close ones with the IEEE quotient and the full search.
-template <int B, typename F>
-__device__ __forceinline__ void curve_encode_exact(F at, float s_lo, float s_hi, float r_lo, float r_hi, uint32_t (&words)[B]) {
-    constexpr uint32_t zero_code = (1u << (B - 1)) - 1u;
+// Code j of a group's words becomes c.
+template <int B>
+__device__ __forceinline__ void replace_code(uint32_t (&words)[B], int j, uint32_t c) {
+    uint32_t field[B] = {}, code[B] = {};
+    deposit_code<B>(field, j, (1u << B) - 1u);
+    deposit_code<B>(code, j, c);
 #pragma unroll
-    for (int w = 0; w < B; ++w) words[w] = 0u;
-#pragma unroll 1
-    for (int j = 0; j < 32; ++j) {
-        const float u = at(j), s = j < 16 ? s_lo : s_hi, r = j < 16 ? r_lo : r_hi;
-        uint32_t b0, b1;
-        curve_bits<B>(pack2(__fmul_rn(u, r), 0.0f), b0, b1);
-        uint32_t c = (b0 >> (23 - B)) & ((1u << B) - 1u);
-        if ((b0 & Curve<B>::kMask) < Curve<B>::kLim || !(r == r)) {
-            c = zero_code;
-            if (s != 0.0f) c = nearest_code<B>(__fdiv_rn(u, s), nullptr);
+    for (int w = 0; w < B; ++w) words[w] = (words[w] & ~field[w]) | code[w];
+}
+// Elements close to a threshold, and rows whose reciprocal is not a normal number, are decided with the IEEE quotient and the full search: the
+// warp goes through its marked rows (`marked`: this lane's), a lane per element.  at(row, j) reads the warp's tile, close(x^) and
+// exact(quotient) are the search's.  With 3-bit codes 3 to 5 % of the warps have such a row, with 8-bit codes every third: one lane going through its 32
+// elements alone held the other 31 for up to 2500 instructions.  us per call in a graph, that / this: 8192 x 8192 3 bits 69.3 / 60.7, 4 bits in blocks
+// of 32 77.5 / 69.5, 8 bits 143.7 / 116.0; 11008 x 4096 4 bits 57.1 / 51.1; 1024 x 1024 3 bits 9.0 / 6.4.
+template <int B, typename F, typename G, typename H>
+__device__ __forceinline__ void encode_exact(F at, G close, H exact, bool marked, float s_lo, float s_hi, float r_lo, float r_hi, uint32_t (&words)[B]) {
+    const int lane = threadIdx.x & 31;
+    uint32_t rows = __ballot_sync(0xffffffffu, marked);
+    while (rows) {
+        const int row = __ffs(rows) - 1;
+        rows &= rows - 1;
+        const float sl = __shfl_sync(0xffffffffu, s_lo, row), sh = __shfl_sync(0xffffffffu, s_hi, row);
+        const float rl = __shfl_sync(0xffffffffu, r_lo, row), rh = __shfl_sync(0xffffffffu, r_hi, row);
+        const float u = at(row, lane), s = lane < 16 ? sl : sh, r = lane < 16 ? rl : rh;
+        const bool again = !(rl == rl) || !(rh == rh) || close(__fmul_rn(u, r));
+        uint32_t c = (1u << (B - 1)) - 1u;                    // the code of zero
+        if (again && s != 0.0f) c = exact(__fdiv_rn(u, s));
+        for (uint32_t m = __ballot_sync(0xffffffffu, again); m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            const uint32_t cj = __shfl_sync(0xffffffffu, c, j);
+            if (lane == row) replace_code<B>(words, j, cj);
         }
-        uint32_t one[B] = {};
-        deposit_code<B>(one, j, c);
-#pragma unroll
-        for (int w = 0; w < B; ++w) words[w] |= one[w];
     }
 }
 
@@ -236,7 +247,6 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
     }
     if (!live) return;
 
-    constexpr uint32_t zero_code = (1u << (B - 1)) - 1u;
     uint32_t words[B];
 #pragma unroll
     for (int i = 0; i < B; ++i) words[i] = 0u;
@@ -245,19 +255,21 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
     // IEEE quotient and the full search.
     const float r_lo = search_reciprocal(s_lo);
     const float r_hi = search_reciprocal(s_hi);
+    const float* mine = reinterpret_cast<const float*>(tile[grp]);
+    auto in_tile = [&](int r, int j) { return mine[r * 32 + ((((j >> 2) ^ (r & 7)) << 2) + (j & 3))]; };
     if constexpr (B <= 4) {
         uint32_t closest = (r_lo == r_lo && r_hi == r_hi) ? Curve<B>::kMask : 0u;
         curve_encode<B>(u, r_lo, r_hi, words, closest);
-        if (closest < Curve<B>::kLim) {
-            const float* mine = reinterpret_cast<const float*>(tile[grp] + rl * 8);
-            curve_encode_exact<B>([&](int j) { return mine[(((j >> 2) ^ (rl & 7)) << 2) + (j & 3)]; }, s_lo, s_hi, r_lo, r_hi, words);
-        }
+        encode_exact<B>(in_tile, [&](float x) {
+            uint32_t b0, b1;
+            curve_bits<B>(pack2(x, 0.0f), b0, b1);
+            return (b0 & Curve<B>::kMask) < Curve<B>::kLim;
+        }, [&](float x) { return nearest_code<B>(x, nullptr); }, closest < Curve<B>::kLim, s_lo, s_hi, r_lo, r_hi, words);
     } else {
         // Bin table: the bin of x^ holds at most one threshold, and none lies close to a bin edge (the bin count is chosen on the
         // host for the largest clearance); code = thresholds below the bin plus (x^ > threshold).
-        // First all 32 codes without a branch (32 independent chains for the scheduler), keeping the smallest distance
-        // between an x^ and the threshold it was compared with; only a thread where that distance is within 1e-6 (or a
-        // reciprocal is not a normal number) goes through its elements again and decides the close ones exactly.
+        // All 32 codes without a branch (32 independent chains for the scheduler), keeping the smallest distance between an x^ and the
+        // threshold it was compared with; rows where that distance is within 1e-6 (or a reciprocal is not a normal number) are gone through again.
         float margin = (r_lo == r_lo && r_hi == r_hi) ? 1.0f : 0.0f;
         if (margin != 0.0f) {
 #pragma unroll
@@ -269,23 +281,10 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
                 margin = fminf(margin, fabsf(xh - e.x));
             }
         }
-        if (!(margin > 1e-6f)) {
-#pragma unroll
-            for (int i = 0; i < B; ++i) words[i] = 0u;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float s = (j < 16) ? s_lo : s_hi, r = (j < 16) ? r_lo : r_hi;
-                const float xh = u[j] * r;
-                const uint32_t k = min(__float2uint_rd(fmaf(xh, bin_scale, bin_scale)), static_cast<uint32_t>(nb));
-                const float2 e = bins[k];
-                uint32_t c = static_cast<uint32_t>(__float_as_int(e.y)) + ((xh > e.x) ? 1u : 0u);
-                if (!(fabsf(xh - e.x) > 1e-6f) || !(r == r)) {
-                    c = zero_code;
-                    if (s != 0.0f) c = nearest_code<B>(__fdiv_rn(u[j], s), th8);
-                }
-                deposit_code<B>(words, j, c);
-            }
-        }
+        encode_exact<B>(in_tile, [&](float x) {
+            const uint32_t k = min(__float2uint_rd(fmaf(x, bin_scale, bin_scale)), static_cast<uint32_t>(nb));
+            return !(fabsf(x - bins[k].x) > 1e-6f);
+        }, [&](float x) { return nearest_code<B>(x, th8); }, !(margin > 1e-6f), s_lo, s_hi, r_lo, r_hi, words);
     }
     dev::pdl_launch_dependents();                // the scale kernel may take its place (it waits for this one)
     uint32_t* dst = codes + slab_word_base(row, k0 >> 6, K >> 6, B);
