@@ -16,7 +16,7 @@
 //     last one adds the slots in order (the same bits on every run) and writes the bf16 output.
 //   - The rank-r intermediate T = X L2^T comes from a small kernel launched in front; the two overlap (programmatic dependent
 //     launch), and the warps that work on the last unit of a tile row add T L1^T to their accumulators.  The counters are cleared by
-//     that kernel, or by the caller's memset when there is no rank-r term.
+//     that kernel, or by one that does nothing else when there is no rank-r term.
 //
 // What bounds it: the pipe of byte permutes and logic (64 lanes per clock and SM): about two operations per weight of 3 bits, 2.6 of 4
 // bits, 1.2 of 2 bits; busy 53 % of the active cycles of the whole kernel (8192 x 8192 NF3, one row; input gradient 47 %), of which the main
@@ -441,7 +441,7 @@ __global__ void __maxnreg__(kMaxRegs) stream_fwd_kernel(const Params p) {
         if (threadIdx.x < nseg) share_s[threadIdx.x] = share_of(runs, piece, tr0 + threadIdx.x);
         if (pc + 1 == runs.per_cta || piece + 1 == runs.pieces) pdl_launch_dependents();    // the next call's pre-product may take its place (it waits for this kernel)
         __syncthreads();
-        if (p.r > 0) pdl_wait();                              // the kernel in front has cleared the counters
+        pdl_wait();                                           // the kernel in front has cleared the counters
         auto put_out = [&](int m, int row, float v) {
             if (row < q.N) p.Y[static_cast<size_t>(m) * q.N + row] = __float2bfloat16_rn(v);
         };
@@ -744,7 +744,7 @@ __global__ void __maxnreg__(NT == 1 ? kMaxRegs : 128) stream_bwd_kernel(const Bw
         if (pc + 1 == runs.per_cta || piece + 1 == runs.pieces) pdl_launch_dependents();    // the next call's pre-product may take its place (it waits for this kernel)
         __syncthreads();                                      // the warps' tiles are idle
         if (a < b) flush(fin + static_cast<size_t>(warp) * M * 128);
-        if (p.r > 0) pdl_wait();                              // the kernel in front has cleared the counters
+        pdl_wait();                                           // the kernel in front has cleared the counters
         __syncthreads();
         auto put_out = [&](int m, int col, float v) {
             if (col < q.K) p.dX[static_cast<size_t>(m) * q.K + col] = __float2bfloat16_rn(v);
@@ -848,7 +848,7 @@ inline Plan compute_plan(const QView& q, int M) {
 inline Plan make_plan(const QView& q, int M) { return dec::cached_plan<Plan>(q, M, 0, [&] { return compute_plan(q, M); }); }
 
 template <int B, int NT>
-inline cudaError_t launch_nt(const Params& p, const Plan& pl, bool after_pre, cudaStream_t st) {
+inline cudaError_t launch_nt(const Params& p, const Plan& pl, cudaStream_t st) {
     auto kern = stream_fwd_kernel<B, NT>;
     static bool attr_done = false;
     if (!attr_done) {
@@ -856,11 +856,10 @@ inline cudaError_t launch_nt(const Params& p, const Plan& pl, bool after_pre, cu
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
-    return dec::launch_stream_kernel(kern, p, dim3(pl.ctas), pl.phases * 256, pl.smem, after_pre, st);
+    return dec::launch_stream_kernel(kern, p, dim3(pl.ctas), pl.phases * 256, pl.smem, st);
 }
 
-// Forward for M <= 16.  When r > 0 the pre-product kernel clears the status word and the arrival counters; otherwise the caller has
-// cleared them (clear_bytes of the workspace).
+// Forward for M <= 16.  The kernel in front (the pre-product, or one that does nothing else) clears the status word and the arrival counters.
 template <int B>
 inline cudaError_t launch_fwd(const QView& q, const void* L1, const void* L2, int r, const void* X, int M, void* Y, char* ws,
                               cudaStream_t st) {
@@ -883,8 +882,11 @@ inline cudaError_t launch_fwd(const QView& q, const void* L1, const void* L2, in
         const cudaError_t e = dec::launch_pre<false>(p.X, static_cast<const __nv_bfloat16*>(L2), reinterpret_cast<__nv_bfloat16*>(ws + w.t_off),
                                                      reinterpret_cast<int*>(ws), p.counters, q.ntiles, M, q.K, r, pl.smem, st);
         if (e != cudaSuccess) return e;
+    } else {
+        const cudaError_t e = dec::launch_clear(reinterpret_cast<int*>(ws), p.counters, q.ntiles, st);
+        if (e != cudaSuccess) return e;
     }
-    return pl.NT == 1 ? launch_nt<B, 1>(p, pl, r > 0, st) : launch_nt<B, 2>(p, pl, r > 0, st);
+    return pl.NT == 1 ? launch_nt<B, 1>(p, pl, st) : launch_nt<B, 2>(p, pl, st);
 }
 
 
@@ -928,7 +930,7 @@ inline BwdPlan compute_bwd_plan(const QView& q, int M, int r) {
 inline BwdPlan make_bwd_plan(const QView& q, int M, int r) { return dec::cached_plan<BwdPlan>(q, M, r, [&] { return compute_bwd_plan(q, M, r); }); }
 
 template <int B, int NT>
-inline cudaError_t launch_bwd_nt(const BwdParams& p, const BwdPlan& pl, bool after_pre, cudaStream_t st) {
+inline cudaError_t launch_bwd_nt(const BwdParams& p, const BwdPlan& pl, cudaStream_t st) {
     auto kern = stream_bwd_kernel<B, NT>;
     static bool attr_done = false;
     if (!attr_done) {
@@ -936,7 +938,7 @@ inline cudaError_t launch_bwd_nt(const BwdParams& p, const BwdPlan& pl, bool aft
         if (e != cudaSuccess) return e;
         attr_done = true;
     }
-    return dec::launch_stream_kernel(kern, p, dim3(pl.ctas), pl.threads, pl.smem, after_pre, st);
+    return dec::launch_stream_kernel(kern, p, dim3(pl.ctas), pl.threads, pl.smem, st);
 }
 
 // Input gradient for M <= 16; same conventions as launch_fwd.
@@ -961,8 +963,11 @@ inline cudaError_t launch_bwd(const QView& q, const void* L1, const void* L2, in
         const cudaError_t e = dec::launch_pre<true>(p.dY, static_cast<const __nv_bfloat16*>(L1), reinterpret_cast<__nv_bfloat16*>(ws + w.t_off),
                                                     reinterpret_cast<int*>(ws), p.counters, pl.windows, M, q.N, r, pl.smem, st);
         if (e != cudaSuccess) return e;
+    } else {
+        const cudaError_t e = dec::launch_clear(reinterpret_cast<int*>(ws), p.counters, pl.windows, st);
+        if (e != cudaSuccess) return e;
     }
-    return pl.NT == 1 ? launch_bwd_nt<B, 1>(p, pl, r > 0, st) : launch_bwd_nt<B, 2>(p, pl, r > 0, st);
+    return pl.NT == 1 ? launch_bwd_nt<B, 1>(p, pl, st) : launch_bwd_nt<B, 2>(p, pl, st);
 }
 
 inline bool supported(const QView& q, int64_t M) {

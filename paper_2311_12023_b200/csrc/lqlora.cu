@@ -77,13 +77,9 @@ static int run_linear(const lqlora_qmatrix* q, const void* L1, const void* L2, i
     }
     const bool use_tc = tc_supported(v, r, M, backward);
     const bool use_decode = !use_tc && stream_supported(v, r, M, backward);
-    // The first kernel of a tensor-core call, and of a decode-sized one with a rank-r term (the pre-product), clears what has to start
-    // at zero (the status word, and the arrival counters of the weight-streaming kernels); otherwise a memset does.
-    const bool first_kernel_clears = use_tc || (r > 0 && use_decode);
-    if (!first_kernel_clears) {
-        const size_t n = use_decode ? stream::clear_bytes(v, backward) : static_cast<size_t>(kStatusBytes);
-        if (cudaMemsetAsync(ws, 0, n, st) != cudaSuccess) return cuda_rc(cudaGetLastError());
-    }
+    // The first kernel of a tensor-core or decode-sized call clears what has to start at zero (the status word, and the arrival counters
+    // of the weight-streaming kernels); for the plain kernels a memset does.
+    if (!use_tc && !use_decode && cudaMemsetAsync(ws, 0, kStatusBytes, st) != cudaSuccess) return cuda_rc(cudaGetLastError());
     cudaError_t e = cudaSuccess;
     if (use_tc) {
         return tc_launch(v, L1, L2, r, A, static_cast<int>(M), out, static_cast<char*>(ws), backward, st);
