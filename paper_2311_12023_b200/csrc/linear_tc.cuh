@@ -611,6 +611,9 @@ constexpr int kTcMinRowsBwd = 9;  // input gradient of matrices with at least 20
 
 inline bool tc_supported(const QView& q, int r, int64_t M, bool backward) {
     (void)r;
+    // With two steps per stage of the transposed tiles, over some 75 drawn calls each (512 .. 28672 rows and columns, with and without a rank-r term), transposed /
+    // streaming: forward 1 row 1.34, 4 rows 1.24, 8 rows 1.12, 12 rows 1.05, 16 rows 0.98; input gradient 1 to 4 rows 1.05, 8 rows 0.95, 9 rows 0.76, 16 rows 0.66 (matrices
+    // of fewer than 2048 rows among them, which stay with the streaming kernels up to 16 rows all the same).  One step per stage:
     // us as a graph, streaming / transposed, 2-, 3-, 4- and 8-bit codes of 8192 x 8192, rank 64: forward 1 row 17 / 24, 18 / 24, 25 / 30, 29 / 42; 8 rows
     // 19 / 24, 20 / 24, 27 / 31, 32 / 42; 16 rows 24 / 24, 25 / 25, 31 / 31, 42 / 42 (other shapes: streaming at most 3 % behind at 16 rows, up to a
     // quarter ahead on 28672 x 8192).  Input gradient 1 row 25 / 25, 26 / 26, 29 / 32, 36 / 44; 8 rows 27 / 25, 28 / 26, 31 / 32, 38 / 44; 9 rows (two
