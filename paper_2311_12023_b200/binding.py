@@ -9,11 +9,14 @@ from __future__ import annotations
 import ctypes
 import os
 import struct
+import warnings
 from dataclasses import dataclass
 from typing import Optional, Tuple
 
 import numpy as np
 import torch
+
+from .build import built_for
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "liblqlora.so")
@@ -227,8 +230,16 @@ def alloc_qmatrix(N: int, K: int, cfg, device="cuda") -> QMatrix:
 
 
 # The native part of the binding (csrc/fast_binding.cpp): marshals an ordinary call and returns its result, the status number of a call that
-# failed, or None for a call that the Python code below has to look at.
+# failed, or None for a call that the Python code below has to look at.  That code takes every call where the module cannot be used.
 _fast = None
+
+
+class _NoFast:
+    @staticmethod
+    def linear(*args):
+        return None
+
+    encode = linear
 
 
 def _fast_part():
@@ -236,10 +247,17 @@ def _fast_part():
     L = lib()
     try:
         from . import _fast as module
+        found = getattr(module, "built_for", "an unknown torch")
+        why = None if found == built_for() else f"compiled for {found}, this is {built_for()}"
     except ImportError as e:
-        raise FileNotFoundError(f"native part of the binding: {e}; build it with `python -m paper_2311_12023_b200.build`") from e
-    module.setup(*[ctypes.cast(f, ctypes.c_void_p).value for f in (L.lqlora_linear_fwd, L.lqlora_linear_bwd_input, L.lqlora_packed_sizes, L.lqlora_encode)],
-                 torch.nn.Parameter, QMatrix)
+        why = str(e)
+    if why:
+        warnings.warn(f"the native part of the binding is not used ({why}); calls take about twice the host time. Build it with "
+                      "`python -m paper_2311_12023_b200.build`", RuntimeWarning, stacklevel=3)
+        module = _NoFast
+    else:
+        module.setup(*[ctypes.cast(f, ctypes.c_void_p).value for f in (L.lqlora_linear_fwd, L.lqlora_linear_bwd_input, L.lqlora_packed_sizes, L.lqlora_encode)],
+                     torch.nn.Parameter, QMatrix)
     _fast = module
     return module
 

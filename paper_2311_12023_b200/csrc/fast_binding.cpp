@@ -1,6 +1,7 @@
 // Marshalling of the layer calls and of the encoder in native code.  binding.py tries these first; they answer None for everything out of the
 // ordinary (tensor subclasses, wrapped tensors, wrong shapes or types, fields that are not integers), and the Python code then takes the call
-// and raises what it always raised.  Nothing is kept between calls: every argument is looked at each time.
+// and raises what it always raised.  It takes every call where this module is missing or was compiled for another torch or Python (`built_for`,
+// see build.py).  Nothing is kept between calls: every argument is looked at each time.
 //
 // What bounded a small call was this work in Python: linear_fwd on one row of a 4096 x 4096 matrix, host time per call 11.9 us, now 6.7, of which 5.6 are the two launches; encoder 22.6 and 9.4.
 #include <ATen/PythonTorchFunctionTLS.h>
@@ -206,5 +207,7 @@ PyMODINIT_FUNC PyInit__fast(void) {
     s_N = PyUnicode_InternFromString("N"); s_K = PyUnicode_InternFromString("K"); s_cfg = PyUnicode_InternFromString("cfg");
     s_b0 = PyUnicode_InternFromString("b0"); s_B0 = PyUnicode_InternFromString("B0"); s_b1 = PyUnicode_InternFromString("b1");
     s_B1 = PyUnicode_InternFromString("B1"); s_b2 = PyUnicode_InternFromString("b2");
-    return PyModule_Create(&module);
+    PyObject* m = PyModule_Create(&module);
+    if (m && PyModule_AddStringConstant(m, "built_for", LQLORA_BUILT_FOR) != 0) { Py_DECREF(m); return nullptr; }
+    return m;
 }
