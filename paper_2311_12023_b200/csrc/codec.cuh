@@ -113,37 +113,68 @@ __device__ __forceinline__ void curve_encode(const float (&u)[32], float r_lo, f
         words[2] |= (word[3] & 0x44444444u) << 1;
     }
 }
-// Code j of a group's words becomes c.
+// Code c into place j (any lane's own) of a group's words, which hold nothing there yet; the words stay in registers.
 template <int B>
-__device__ __forceinline__ void replace_code(uint32_t (&words)[B], int j, uint32_t c) {
-    uint32_t field[B] = {}, code[B] = {};
-    deposit_code<B>(field, j, (1u << B) - 1u);
-    deposit_code<B>(code, j, c);
+__device__ __forceinline__ void add_code(uint32_t (&words)[B], int j, uint32_t c) {
+    uint32_t one[B] = {};
+    if constexpr (B == 8) {
 #pragma unroll
-    for (int w = 0; w < B; ++w) words[w] = (words[w] & ~field[w]) | code[w];
+        for (int w = 0; w < B; ++w) one[w] = (j >> 2) == w ? c << (8 * (j & 3)) : 0u;
+    } else {
+        deposit_code<B>(one, j, c);
+    }
+#pragma unroll
+    for (int w = 0; w < B; ++w) words[w] |= one[w];
 }
-// Elements close to a threshold, and rows whose reciprocal is not a normal number, are decided with the IEEE quotient and the full search: the
-// warp goes through its marked rows (`marked`: this lane's), a lane per element.  at(row, j) reads the warp's tile, close(x^) and
-// exact(quotient) are the search's.  With 3-bit codes 3 to 5 % of the warps have such a row, with 8-bit codes every third: one lane going through its 32
-// elements alone held the other 31 for up to 2500 instructions.  us per call in a graph, that / this: 8192 x 8192 3 bits 69.3 / 60.7, 4 bits in blocks
-// of 32 77.5 / 69.5, 8 bits 143.7 / 116.0; 11008 x 4096 4 bits 57.1 / 51.1; 1024 x 1024 3 bits 9.0 / 6.4.
+// Elements close to a threshold, and rows whose reciprocal is not a normal number, are decided with the IEEE quotient and the full search
+// (`marked`: this lane's row has some).  at(row, j) reads the warp's tile, look(x^, code) gives the fast search's code and whether x^ is close,
+// exact(quotient) is the full search.
+// Up to kRowsTogether marked rows: the warp takes them one after the other, a lane per element, and builds the row's words anew.  Ordinary matrices
+// have one in 3 to 5 % of the warps with 3-bit codes and in every third with 8-bit codes, where one lane going through its 32 elements alone
+// holds the other 31.  More rows: each lane goes through its own, all at once (8-bit codes four elements at a time); about a hundred
+// instructions per row on one side, 1200 and some 60 per place with a close element on the other.
+// us per call in a graph, always a lane per row / always a lane per element (the codes handed over one by one) / this: 8192 x 8192 3 bits 69.2 / 60.6 /
+// 60.5, 4 bits in blocks of 32 77.4 / 69.3 / 67.7, 8 bits 144 / 116 / 110, 11008 x 4096 4 bits 57.6 / 50.4 / 49.4.  4096 x 4096, 3 bits, a value on a
+// threshold in every 32: 45 / 101 / 46, all of them there 60 / 1040 / 61, maxima of 1e-36 94 / 1075 / 94; 8 bits 52 / 163 / 56, 125 / 2970 / 116, 108 / 3010 / 116.
+constexpr int kRowsTogether = 8;
 template <int B, typename F, typename G, typename H>
-__device__ __forceinline__ void encode_exact(F at, G close, H exact, bool marked, float s_lo, float s_hi, float r_lo, float r_hi, uint32_t (&words)[B]) {
+__device__ __forceinline__ void encode_exact(F at, G look, H exact, bool marked, float s_lo, float s_hi, float r_lo, float r_hi, uint32_t (&words)[B]) {
+    constexpr uint32_t zero_code = (1u << (B - 1)) - 1u;
+    constexpr int kAtOnce = B == 8 ? 4 : 1;
     const int lane = threadIdx.x & 31;
     uint32_t rows = __ballot_sync(0xffffffffu, marked);
-    while (rows) {
-        const int row = __ffs(rows) - 1;
-        rows &= rows - 1;
-        const float sl = __shfl_sync(0xffffffffu, s_lo, row), sh = __shfl_sync(0xffffffffu, s_hi, row);
-        const float rl = __shfl_sync(0xffffffffu, r_lo, row), rh = __shfl_sync(0xffffffffu, r_hi, row);
-        const float u = at(row, lane), s = lane < 16 ? sl : sh, r = lane < 16 ? rl : rh;
-        const bool again = !(rl == rl) || !(rh == rh) || close(__fmul_rn(u, r));
-        uint32_t c = (1u << (B - 1)) - 1u;                    // the code of zero
-        if (again && s != 0.0f) c = exact(__fdiv_rn(u, s));
-        for (uint32_t m = __ballot_sync(0xffffffffu, again); m; m &= m - 1) {
-            const int j = __ffs(m) - 1;
-            const uint32_t cj = __shfl_sync(0xffffffffu, c, j);
-            if (lane == row) replace_code<B>(words, j, cj);
+    if (__popc(rows) <= kRowsTogether) {
+        while (rows) {
+            const int row = __ffs(rows) - 1;
+            rows &= rows - 1;
+            const float sl = __shfl_sync(0xffffffffu, s_lo, row), sh = __shfl_sync(0xffffffffu, s_hi, row);
+            const float rl = __shfl_sync(0xffffffffu, r_lo, row), rh = __shfl_sync(0xffffffffu, r_hi, row);
+            const float u = at(row, lane), s = lane < 16 ? sl : sh, r = lane < 16 ? rl : rh;
+            uint32_t c;
+            if (look(__fmul_rn(u, r), c) || !(r == r)) c = s != 0.0f ? exact(__fdiv_rn(u, s)) : zero_code;
+            uint32_t anew[B] = {};
+            add_code<B>(anew, lane, c);
+#pragma unroll
+            for (int w = 0; w < B; ++w) {
+                const uint32_t all = __reduce_or_sync(0xffffffffu, anew[w]);
+                if (lane == row) words[w] = all;
+            }
+        }
+    } else if (marked) {
+#pragma unroll
+        for (int w = 0; w < B; ++w) words[w] = 0u;
+#pragma unroll 1
+        for (int j0 = 0; j0 < 32; j0 += kAtOnce) {
+            const float s = j0 < 16 ? s_lo : s_hi, r = j0 < 16 ? r_lo : r_hi;
+            uint32_t c[kAtOnce];
+            bool again[kAtOnce];
+#pragma unroll
+            for (int i = 0; i < kAtOnce; ++i) again[i] = look(__fmul_rn(at(lane, j0 + i), r), c[i]) || !(r == r);
+#pragma unroll
+            for (int i = 0; i < kAtOnce; ++i) {
+                if (again[i]) c[i] = s != 0.0f ? exact(__fdiv_rn(at(lane, j0 + i), s)) : zero_code;
+                add_code<B>(words, j0 + i, c[i]);
+            }
         }
     }
 }
@@ -159,8 +190,9 @@ __device__ __forceinline__ float search_reciprocal(float s) {
 // One CTA: 32 rows x 256 columns.  Thread (row = tid % 32, grp = tid / 32) owns 32 consecutive
 // columns of one row: it finds the block absmax (with its neighbours through shared memory when
 // B0 > 32), the 32 codes, and writes the b0 words of its group to the packed slab.
+// (2-bit codes: asked for four CTAs per SM the compiler takes 63 registers; left alone it takes 48, five fit, and 8192 x 8192 took 56.3 us, not 55.3.)
 template <int B>
-__global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restrict__ W, uint32_t* __restrict__ codes,
+__global__ void __launch_bounds__(256, B == 2 ? 4 : 0) encode_codes_kernel(const float* __restrict__ W, uint32_t* __restrict__ codes,
                                                            float* __restrict__ absmax, int N, int K, int B0, int logB0) {
     __shared__ float red[8][33];
     __shared__ __align__(16) float4 tile[8][32 * 8];   // per warp: 32 rows x 32 columns
@@ -260,9 +292,10 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
     if constexpr (B <= 4) {
         uint32_t closest = (r_lo == r_lo && r_hi == r_hi) ? Curve<B>::kMask : 0u;
         curve_encode<B>(u, r_lo, r_hi, words, closest);
-        encode_exact<B>(in_tile, [&](float x) {
+        encode_exact<B>(in_tile, [&](float x, uint32_t& c) {
             uint32_t b0, b1;
             curve_bits<B>(pack2(x, 0.0f), b0, b1);
+            c = (b0 >> (23 - B)) & ((1u << B) - 1u);
             return (b0 & Curve<B>::kMask) < Curve<B>::kLim;
         }, [&](float x) { return nearest_code<B>(x, nullptr); }, closest < Curve<B>::kLim, s_lo, s_hi, r_lo, r_hi, words);
     } else {
@@ -281,9 +314,11 @@ __global__ void __launch_bounds__(256) encode_codes_kernel(const float* __restri
                 margin = fminf(margin, fabsf(xh - e.x));
             }
         }
-        encode_exact<B>(in_tile, [&](float x) {
+        encode_exact<B>(in_tile, [&](float x, uint32_t& c) {
             const uint32_t k = min(__float2uint_rd(fmaf(x, bin_scale, bin_scale)), static_cast<uint32_t>(nb));
-            return !(fabsf(x - bins[k].x) > 1e-6f);
+            const float2 e = bins[k];
+            c = static_cast<uint32_t>(__float_as_int(e.y)) + ((x > e.x) ? 1u : 0u);
+            return !(fabsf(x - e.x) > 1e-6f);
         }, [&](float x) { return nearest_code<B>(x, th8); }, !(margin > 1e-6f), s_lo, s_hi, r_lo, r_hi, words);
     }
     dev::pdl_launch_dependents();                // the scale kernel may take its place (it waits for this one)
