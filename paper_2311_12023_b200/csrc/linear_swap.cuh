@@ -6,26 +6,29 @@
 // Roles: warps 0 and 1 load this CTA's half of the (one or two) token boxes by TMA, warp 2 the packed codes (bulk
 // copies, a ring of their own), warp 3 of the leader issues the MMAs, sixteen warps dequantize.  Four of those share a
 // step of 64 contraction elements (one thread = one row of 64 weights, so a block of 64 or more costs one table), four
-// steps are in work at a time.  A ring stage holds a step's token rows and weight tile.  The slices of the contraction are further
+// steps are in work at a time.  The slices of the contraction are further
 // pairs of the same cluster: each CTA lays its fp32 accumulators down in its own (idle) shared memory and adds up and stores its share of the
 // tokens (rank order: the same bits on every run).
 // Forward reads the weight tile as a K-major operand, the input gradient the same bytes as an MN-major operand.
-// Forward with one token box (at most 256 tokens per pair): the weights go from the registers into tensor memory instead (32 columns
-// per stage), which a row operand may be read from.  Accumulators take at most 256 of the 512 columns there, eight stages the rest; with two
-// boxes the accumulators need them all.  The row operand in tensor memory is K-major only, so the input gradient stays in shared memory.
+// A ring stage is one step: its token rows and its weight tile in shared memory.
+// Forward with one token box (at most 256 tokens per pair): the weights go from the registers into tensor memory instead (32 columns per step), which a
+// row operand may be read from, and a stage is two steps, with one wait and one commit for both.  Accumulators take at most 256 of the 512
+// columns there, four stages the rest; with two boxes the accumulators need them all.  The row operand in tensor memory is K-major only, so the input
+// gradient stays in shared memory.
 // Every wait is bounded (see linear_tc.cuh).
 //
-// With one token box a stage is two steps, with one wait and one commit for both: without loads and dequantization a step still took 370 clocks, of which
-// the issuing warp spent 140 in a wait that was satisfied and 170 to 210 issuing.  What every step needs is requested before tensor memory, the
-// code book and the cluster barrier are set up, and arrivals on that barrier are relaxed (the initialisation of the mbarriers has a fence of its own): a
-// releasing arrival waited for the scale loads in front of it.  us as a graph, one step per stage and a set-up in front of the loads / this: 8192 x 8192 NF3,
-// 128 rows 27.6 / 24.6, without a rank-r term (a memset in front of the kernel before) 30.9 / 23.2, 28672 x 8192 83.5 / 73.4, input gradient 30.9 / 29.2.
-// What bounds it: the loop of the issuing warp (32-bit descriptors, no divisions), then dequantization (about 450 clocks per step of an SM, of which
-// the pipe of byte permutes and logic is busy 275; warps started out of step, 24 of them with 72 registers, changed nothing or cost time): about 500 clocks per 64
-// weights of a row and warp).  A weight tile in shared memory costs its bandwidth twice, when written and when read by the tensor
-// core, and with wide codes or many tokens it takes the room of ring stages.  us as a graph, in shared / in tensor memory: 8192 x 8192
-// NF3 128 rows 28.0 / 26.7 (1.05), 512 rows 52.9 / 50.2, 28672 x 8192 NF3 128 rows 95.2 / 90.8, 8-bit codes 256 rows 62.5 / 60.4; shapes
-// whose grid leaves many SMs idle are even (4096 x 4096 NF4 64 rows 16.6 / 16.7).
+// Two steps per stage: without loads and dequantization a step took 370 clocks, of which the issuing warp spent 140 in a wait that was satisfied and 170 to
+// 210 issuing.  The input gradient has no use for it: over 1900 plans of drawn calls one step per stage takes between 3 % less (blocks of 16, more than 128
+// tokens) and 2.5 % more (2-bit codes, few tokens) time, and 8 to 10 % less with 8-bit codes and more than 128 tokens, whose two-step stages are too few.
+// What every step needs is requested before tensor memory, the code book and the cluster barrier are set up, and arrivals on that barrier are relaxed
+// (the initialisation of the mbarriers has a fence of its own): a releasing arrival waited for the scale loads in front of it.
+// us as a graph, one step per stage and a set-up in front of the loads / this: 8192 x 8192 NF3, 128 rows 27.6 / 24.6, without a rank-r term (a
+// memset in front of the kernel before) 30.9 / 23.2, 28672 x 8192 83.5 / 73.4.
+// What bounds it: dequantization, about 450 clocks per step of an SM, of which the pipe of byte permutes and logic is busy 275 (warps started
+// out of step, 24 of them with 72 registers, changed nothing or cost time).  A weight tile in shared memory costs its bandwidth twice, when written and when
+// read by the tensor core, and with wide codes or many tokens it takes the room of ring stages: when the weights went to tensor memory, 8192 x 8192
+// NF3 took 28.0 / 26.7 us at 128 rows and 52.9 / 50.2 at 512, 28672 x 8192 NF3 95.2 / 90.8 at 128 rows (one step per stage; shapes whose grid leaves many
+// SMs idle were even).
 #pragma once
 
 #include <atomic>
@@ -42,8 +45,6 @@ constexpr int kSwWBytes = 128 * 128;                            // this CTA's bf
 constexpr int kSwMaxStages = 8;
 constexpr uint32_t kSwTmemA = 256;                              // first column of the weights in tensor memory (32 per stage)
 constexpr int kSwTail = 512;                                    // barriers, tensor-memory slot, abort flag
-// Steps of 64 contraction elements per stage, i.e. per round of waits and commits: two with one token box, one with two.
-constexpr int swap_stage_steps(int nbox) { return nbox == 1 ? 2 : 1; }
 
 struct SwapParams {
     QView q;
@@ -57,7 +58,7 @@ struct SwapParams {
     const __nv_bfloat16* L1; // forward with the weights in tensor memory: [N][r], read directly
     int r;
     int nbox, box;           // token boxes (1 or 2) and tokens per box (a multiple of 16, at most 256; half of them per CTA)
-    int ss, sp;              // stages (of swap_stage_steps steps) of the token + weight ring and of the packed-code ring
+    int ss, sp;              // stages (of one step; weights in tensor memory: two) of the token + weight ring and of the packed-code ring
     uint32_t tail_off;       // of the barriers, behind the rings
     uint32_t tmem_cols;
 };
@@ -256,16 +257,18 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int B, bool BWD, bool TA, int PS>
+template <int B, bool BWD, bool TA, int NBOX>
 __global__ void __launch_bounds__(kSwThreads, 1)
 tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT,
                       const __grid_constant__ CUtensorMap tmF, const SwapParams p) {
+    constexpr int PS = TA ? 2 : 1;                                       // steps of 64 contraction elements per stage, i.e. per round of waits and commits
+    static_assert(!TA || NBOX == 1, "two warps request the boxes of a stage");
     constexpr int P_BYTES = 1024 * B;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
     const int half_box = p.box >> 1, half_bytes = half_box * 128;
-    const int nbox = PS == 2 ? 1 : 2;
-    const int x_bytes = nbox * half_bytes;
+    constexpr int kBoxWarps = PS * NBOX;                                 // a warp per token box of a stage (one or two)
+    const int x_bytes = NBOX * half_bytes;
     constexpr int W_BYTES = TA ? 0 : kSwWBytes;
     const int step_bytes = W_BYTES + x_bytes;                            // [weight tile][token boxes] of a step; a stage is PS of them
     uint8_t* p_ring = base + p.ss * PS * step_bytes;
@@ -279,7 +282,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_rank() & 1u;                           // CTA of the pair; 0 = leader
     const int c0 = p.c_base + blockIdx.x * 128;                          // first output column of this CTA
-    const int m0 = blockIdx.y * (nbox * p.box);                          // first token
+    const int m0 = blockIdx.y * (NBOX * p.box);                          // first token
     const int nsplit = gridDim.z, split = blockIdx.z;
     const int q_lo = static_cast<int>(static_cast<long long>(p.steps_q) * split / nsplit);
     const int nq = static_cast<int>(static_cast<long long>(p.steps_q) * (split + 1) / nsplit) - q_lo;
@@ -349,9 +352,9 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     if (warp < 2) {
         if (warp == 0 && elect_one()) {
             for (int s = 0; s < kSwMaxStages; ++s) {
-                // two token boxes (of a step, or of two) and four dequantization warps per step; leader: also the word of the second
+                // the token boxes and four dequantization warps per step; leader: also the word of the second
                 // CTA that its stage is complete
-                mbar_init(full(s), 2 + 4 * PS + (rank == 0 ? 1 : 0));
+                mbar_init(full(s), kBoxWarps + 4 * PS + (rank == 0 ? 1 : 0));
                 mbar_init(empty(s), 1);
             }
             mbar_init(fbar(0), 1);
@@ -365,7 +368,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         __syncwarp();
         asm volatile("bar.sync 1, 64;" ::: "memory");
         if (lead) pdl_wait();
-        if (elect_one()) {
+        if (warp < kBoxWarps && elect_one()) {
             for (int i = 0; i < early_x; ++i) issue_box(warp, i, i);
         }
         __syncwarp();
@@ -405,7 +408,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
     bool acc_ok = false;
     int issued = early_p;         // stages whose codes have been requested (warp 2)
 
-    if (warp < 2) {
+    if (warp < kBoxWarps) {
         // ------------------------------------------------------------------ token boxes
         RingAt r(early_x, p.ss);
         int round = early_x;
@@ -477,7 +480,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
                             tc_mma2_lo(tmem, a + ka, b + 2, idesc, 1u);
                             tc_mma2_lo(tmem, a + 2 * ka, b + 4, idesc, 1u);
                             tc_mma2_lo(tmem, a + 3 * ka, b + 6, idesc, 1u);
-                            if (PS == 1) {
+                            if (NBOX == 2) {
                                 const uint32_t b2 = b + box16;
                                 tc_mma2_lo(tmem + 256, a, b2, idesc, keep);
                                 tc_mma2_lo(tmem + 256, a + ka, b2 + 2, idesc, 1u);
@@ -601,7 +604,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             tc_fence_after();
             const int quarter = warp & 3, chunks = (p.box + 31) >> 5;
             float* accbuf = reinterpret_cast<float*>(base);           // [token][128 columns], over the idle rings
-            for (int ch = dw >> 2; ch < nbox * chunks; ch += 4) {
+            for (int ch = dw >> 2; ch < NBOX * chunks; ch += 4) {
                 const int h = ch / chunks, t0 = (ch - h * chunks) * 32;
                 uint32_t v[32];
                 tmem_ld32(tmem + (static_cast<uint32_t>(quarter * 32) << 16) + h * 256 + t0, v);
@@ -633,7 +636,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         // every CTA adds up and stores its share of the tokens from the CTAs with the same columns; the barriers are executed
         // by all threads of all CTAs, whatever happened before
         const uint32_t acc_addr = ring;
-        const int tokens = nbox * p.box;
+        const int tokens = NBOX * p.box;
         const int t_lo = tokens * split / nsplit, t_hi = tokens * (split + 1) / nsplit;
         __syncthreads();
         cluster_barrier();
@@ -670,9 +673,9 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         // the phase then waits for the boxes alone.  A box of stage j is issued behind the end of stage j - ss, so the last ss stages
         // that any box was issued for are the ones that can be open, each in the phase j / ss of its place in the ring.
         if (warp == 0) {
-            const int top = max(reached[0], reached[1]);
+            const int top = kBoxWarps == 2 ? max(reached[0], reached[1]) : reached[0];
             for (int j = max(0, top - p.ss); j < top; ++j) {
-                int missing = (j >= reached[0] ? 1 : 0) + (j >= reached[1] ? 1 : 0) + (rank == 0 && j >= reached[3] ? 1 : 0);
+                int missing = (j >= reached[0] ? 1 : 0) + (kBoxWarps == 2 && j >= reached[1] ? 1 : 0) + (rank == 0 && j >= reached[3] ? 1 : 0);
                 for (int w = 0; w < 4 * PS; ++w) missing += (j >= reached[kSwFirstDeq + 4 * PS * (j & (4 / PS - 1)) + w] ? 1 : 0);
                 if (lane < missing) mbar_arrive(full(j % p.ss));
                 let_land(full(j % p.ss), (j / p.ss) & 1);
@@ -695,7 +698,7 @@ inline int tc_max_clusters(int n) {
     if (known >= 0) return known;
     const int fallback[4] = {74, 33, 22, 15};
     int got = 0;
-    auto kern = tc_swap_linear_kernel<3, false, false, 1>;
+    auto kern = tc_swap_linear_kernel<3, false, false, 2>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2, 1, n / 2);
     cfg.blockDim = dim3(kSwThreads);
@@ -722,25 +725,25 @@ struct SwapPlan {
     double us;                       // estimated time
 };
 
-// Ring depths in stages; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase
-// while the one before it can be incomplete.  A dequantization warp works on every fourth step, i.e. on every fourth (one step per
-// stage) or second stage; with g for that number:
-//   - it may wait for stage j % ss to be free (the tensor core is done with stage j - ss) once stage j - 2 ss is known to be
-//     done; its own stage j - g waited for j - g - ss, hence ss >= g;
-//   - it may wait for the codes of stage j once those of stage j - sp are known to have landed: they have where its own
-//     group used them (sp a multiple of g) or where the tensor core is done with that stage (sp >= ss).
+// Ring depths of a plan; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase while the
+// one before it can be incomplete.  A dequantization warp works on every fourth step:
+//   - it may wait for stage j % ss to be free (the tensor core is done with step j - ss) once step j - 2 ss is known to be
+//     done; its own step j - 4 waited for j - 4 - ss, hence ss >= 4;
+//   - it may wait for the codes of step j once those of step j - sp are known to have landed: they have where its own
+//     group used them (sp a multiple of four) or where the tensor core is done with that step (sp >= ss).
+// (With the weights in tensor memory the kernel takes depths of its own, see run_swap; what fits here fits there.)
+// As many stages of weights as fit beside four of codes, then codes.  Fewer stages of weights for as many of codes took more shared memory, which the
+// scales miss in L1: 10112 x 15616 input gradient, 8-bit codes in blocks of 16, 17 rows, 95 us with 8 and 4 stages, 113 with 7 and 8.
 inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
-    const int steps = swap_stage_steps(pl.nbox), g = 4 / steps;
-    const int stage = steps * (kSwWBytes + pl.nbox * pl.box * 64), pk = steps * 1024 * b0;
+    const int stage = kSwWBytes + pl.nbox * pl.box * 64, pk = 1024 * b0;
     const int fixed = 1024 + kSwTail + (b0 == 8 ? 32768 : 0);
     const int room = kSmemLimit - fixed;
-    pl.ss = (room - g * pk) / stage;
-    if (pl.ss > kSwMaxStages / steps) pl.ss = kSwMaxStages / steps;
-    if (pl.ss < g) return false;
-    while (pl.ss > g && (room - pl.ss * stage) / pk < pl.ss) --pl.ss;      // (wide codes: no fewer stages of codes than of weights)
+    pl.ss = (room - 4 * pk) / stage;
+    if (pl.ss > kSwMaxStages) pl.ss = kSwMaxStages;
+    if (pl.ss < 4) return false;
     pl.sp = (room - pl.ss * stage) / pk;
     if (pl.sp > kSwMaxStages) pl.sp = kSwMaxStages;
-    if (pl.sp < pl.ss) pl.sp = g;
+    if (pl.sp < pl.ss) pl.sp = 4;
     const int bytes = pl.ss * stage + pl.sp * pk;
     if (ks > 1 && pl.nbox * pl.box * 512 > bytes) return false;      // the accumulators are laid over the rings
     pl.smem = fixed + bytes;
@@ -850,10 +853,10 @@ inline const SwapPlan& swap_plan(int b0, int B0, bool backward, int64_t M, int64
     return e.plan;
 }
 
-template <int B, bool BWD, bool TA, int PS>
+template <int B, bool BWD, bool TA, int NBOX>
 inline int launch_swap(const CUtensorMap& tX, const CUtensorMap& tT, const CUtensorMap& tF, const SwapParams& p, const SwapPlan& pl,
                        int smem, int pairs, cudaStream_t st, bool first) {
-    auto kern = tc_swap_linear_kernel<B, BWD, TA, PS>;
+    auto kern = tc_swap_linear_kernel<B, BWD, TA, NBOX>;
     static bool attr_done = false;
     if (!attr_done) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
@@ -898,7 +901,7 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     p.L1 = static_cast<const __nv_bfloat16*>(L1); p.r = r;
     p.clear_status = first ? 1 : 0;
     int smem = pl.smem;
-    p.tail_off = swap_stage_steps(pl.nbox) * (pl.ss * (kSwWBytes + pl.nbox * pl.box * 64) + pl.sp * 1024 * q.b0);
+    p.tail_off = pl.ss * (kSwWBytes + pl.nbox * pl.box * 64) + pl.sp * 1024 * q.b0;
     const bool ta = !backward && pl.nbox == 1;      // (256 columns of accumulators and eight stages of 32 columns fill tensor memory)
     if (ta) {
         // Without weight tiles four stages of two steps of both rings always fit (256 tokens, 8-bit codes: 230,912 of 232,448 bytes, code
@@ -925,10 +928,10 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     const int pairs = (cols + 255) / 256;
     auto go = [&](auto bits) {
         constexpr int B = decltype(bits)::value;
-        if (ta) return launch_swap<B, false, true, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
-        if (!backward) return launch_swap<B, false, false, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
-        if (pl.nbox == 1) return launch_swap<B, true, false, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
-        return launch_swap<B, true, false, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (ta) return launch_swap<B, false, true, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (!backward) return launch_swap<B, false, false, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (pl.nbox == 1) return launch_swap<B, true, false, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        return launch_swap<B, true, false, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
     };
     switch (q.b0) {
         case 2: return go(std::integral_constant<int, 2>());
