@@ -774,24 +774,53 @@ inline int pre_splits(int mtiles, int steps, long long main_ctas) {
     }
     if (want < 1) want = 1;
     while (want & (want - 1)) want &= want - 1;
+    // Not two splits of more than 37 row tiles: a graph of calls with 65 of them (130 CTAs in clusters of two) before 40 clusters of four of the linear kernel
+    // ended in a launch failure, and neither reading nor checks of every address in both kernels showed why.
+    if (want == 2 && mtiles > 37) want = 1;
     return want;
 }
 
-// The split of a call that costs least by a simple model: waves of clusters, each with a fixed cost, its steps (the
-// slower of dequantization and tensor core, softened) and its reduction, or the pre-product that runs beside it where that takes longer.  Fitted to
-// the timings of all chunk counts and slices of 1400 drawn shapes (2 to 8 bits, 9 to 2000 rows, with and without a rank-r term): the plan that it
-// picks takes 1.8 % longer than the best one on average (3.4 % with the constants before, which did not count the clusters that the
-// pre-product displaces).  us as a
-// graph, plans and kernel before / now: 4096 x 4096 NF4, 64 rows 16.1 / 15.4; 28672 x 8192 NF3, 128 rows 83 / 73; 4008 x 15616 NF3, 517 rows 61.4 / 61.5;
-// 1024 x 1024 NF3, 512 rows 11.8 / 10.3.  Left slower: 1664 x 11776 NF3 input gradient, 778 rows 38 / 45; 2904 x 4288 NF3, 309 rows 18.6 / 21.3.
+// Clusters of a linear kernel (`ks` pairs each) that a rank-r pre-product beside it, `mtiles` row tiles of `w` CTAs, keeps out of their GPCs while
+// it runs.  Read off from the timings (the number of free clusters below which a call takes a second wave): single CTAs fill TPCs together, but an
+// odd number of up to 13 holds a TPC each; beside larger clusters a GPC has a few SMs to spare, which small ones take first.
+inline int clusters_kept_out(int ks, int mtiles, int w) {
+    const bool odd = mtiles & 1;
+    const int tpcs = w > 1 ? mtiles * w / 2 : odd ? mtiles : mtiles / 2;
+    if (ks == 1) return w == 1 && mtiles >= 15 ? mtiles / 2 + (odd ? 2 : 0) : tpcs;
+    if (ks == 2) return w >= 4 ? tpcs / 2 : w == 1 && odd && mtiles < 17 ? (mtiles < 11 ? 0 : 2) : tpcs > 8 ? (tpcs - 7) / 2 : 0;
+    if (ks == 3) return w == 8 ? 0 : w == 4 ? mtiles - 1 : w == 2 ? (mtiles > 4 ? mtiles - 4 : 0) : mtiles < 7 ? 0 : odd ? (mtiles - 5) / 2 : mtiles < 14 ? 0 : mtiles < 18 ? 3 : tpcs - 5;
+    return w == 4 ? mtiles : w == 8 ? 0 : tpcs > 10 ? 7 : 0;          // (a cluster of eight per GPC in place of two)
+}
+// Time until `n` clusters of `first` us have run in `slots` places, `late` of which are free only after `at` us; clusters that follow another one in
+// its place take `next` us.
+inline double makespan(long long n, double first, double next, long long slots, long long late, double at) {
+    long long rounds = n / slots - 2 - static_cast<long long>(at / next);      // that all places have behind them in any case
+    if (rounds < 0) rounds = 0;
+    double t_early = first + static_cast<double>(rounds) * next, t_late = t_early + at;
+    for (long long done = rounds * slots;;) {
+        const bool early = late == 0 || t_early <= t_late;
+        double& t = early ? t_early : t_late;
+        done += early ? slots - late : late;
+        if (done >= n) return t;
+        t += next;
+    }
+}
+
+// The split of a call that costs least by a simple model: places for clusters, each cluster with a fixed cost, its steps (the slower of
+// dequantization and tensor core, softened; slower with more SMs at work) and its reduction; the pre-product, which keeps places occupied at first and is
+// waited for at the end.  Fitted to the timings of all plausible chunk counts and slices of 2400 drawn calls (2 to 8 bits, 9 to 2000 rows, with and
+// without a rank-r term); on 1200 others the plan that it picks takes 0.4 % longer than the best one on average, and more than a tenth longer in 12 of
+// them.  (The model before counted whole waves and took one slice 15 % dearer than estimated: 1.5 %, and 62.  us as a graph, its plan / this one: 13848 x 4224
+// NF4, 601 rows 99.8 / 68; 4784 x 21120 NF8, 445 rows 182 / 142; 9216 x 16896 NF4 input gradient, 19 rows 84 / 63; 2688 x 2304 NF2, 283 rows 17.4 / 14.1.)
 inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
     SwapPlan best{};
     best.us = -1.0;
     double best_score = 0.0;
-    // us per step of 128 x 64 weights: through tensor memory, through shared memory; small blocks cost more tables
-    static const double dq_ta[4] = {0.22, 0.245, 0.355, 0.50}, dq_smem[4] = {0.245, 0.27, 0.355, 0.525};
-    const double dq_block = B0 == 16 ? 1.15 : B0 == 32 ? 1.06 : 1.0;
+    // us per step of 128 x 64 weights: through tensor memory; input gradient, one box; two boxes forward, input gradient.  Small blocks cost more tables.
+    static const double dq_us[4][4] = {{0.212, 0.23, 0.329, 0.478}, {0.242, 0.258, 0.338, 0.497}, {0.233, 0.256, 0.32, 0.511}, {0.25, 0.271, 0.317, 0.507}};
+    static const double red_us[3] = {0.021, 0.0235, 0.025};          // sum over two, three, four slices, per token
     const long long pairs = (out_cols + 255) / 256;
+    const int mtiles = static_cast<int>((M + 127) / 128);
     int first = static_cast<int>((M + 511) / 512);
     // The search covers eight numbers of chunks.  Where the chunks of all of them are too large for the rings (8-bit codes
     // above 11136 rows), it starts at the fewest that are not: a plan exists for every number of rows.
@@ -807,31 +836,33 @@ inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t
         pl.chunks = static_cast<int>((M + tokens - 1) / tokens);
         pl.tmem_cols = 32;
         while (static_cast<int>(pl.tmem_cols) < (pl.nbox == 2 ? 512 : pl.box)) pl.tmem_cols *= 2;
+        const bool ta = !backward && pl.nbox == 1;
+        const double block = B0 == 16 ? (ta ? 1.17 : 1.12) : B0 == 32 ? (ta ? 1.05 : 1.04) : 1.0;
+        const double dq = block * dq_us[2 * (pl.nbox - 1) + (backward ? 1 : 0)][bits_index(b0)], mma = (pl.nbox == 1 ? 0.00085 : 0.00097) * tokens;
         for (int ks = 1; ks <= 4 && ks <= steps_q; ++ks) {
             if (!swap_rings(b0, ks, pl)) continue;
             pl.ks = ks;
-            pl.ctas = 2 * pairs * pl.chunks * ks;
-            const double dq = dq_block * (!backward && pl.nbox == 1 ? dq_ta : dq_smem)[bits_index(b0)], mma = 0.001 * tokens;
-            const double step = std::pow(dq * dq * dq * dq + mma * mma * mma * mma, 0.25);
-            // a rank-r pre-product runs beside this kernel and takes SMs out of the GPCs, which costs large clusters most
-            long long at_once = tc_max_clusters(2 * ks);
-            double pre = 0.0;
+            const long long n = pairs * pl.chunks, slots = tc_max_clusters(2 * ks);
+            pl.ctas = 2 * n * ks;
+            const double busy = static_cast<double>(2 * ks * (n < slots ? n : slots)) / dec::sm_count_cached();
+            const double step = std::sqrt(std::sqrt(dq * dq * dq * dq + mma * mma * mma * mma)) * (1.0 + (steps_d > 0 ? 0.155 : 0.22) * busy);
+            const double sum = ks == 1 ? 0.013 * tokens : 0.6 + red_us[ks - 2] * tokens;
+            const double body = (steps_d > 0 ? 5.6 : 4.2) + ((steps_q + ks - 1) / ks + steps_d) * step + sum;
+            double pre = 0.0, tail = 0.0;
+            long long late = 0;
             if (steps_d > 0) {
-                const int mtiles = static_cast<int>((M + 127) / 128), w = pre_splits(mtiles, steps_q, pl.ctas);
-                // Single CTAs fill a TPC together; an odd number of one-split tiles is launched one by one and holds a TPC each.  Beside clusters of
-                // four and six a GPC has a TPC or two to spare, which small pre-product clusters take first.
-                const int tpcs = w == 1 ? (mtiles % 2 && ks == 1 ? mtiles : (mtiles + 1) / 2) : mtiles * w / 2;
-                at_once -= ks == 1 ? tpcs : ks == 2 ? (w >= 4 ? (tpcs > 2 ? mtiles * (w / 4) : 0) : tpcs > 5 ? (tpcs - 4) / 2 : 0) : ks == 3 ? (tpcs > 4 ? (tpcs - 2) / 3 : 0) : mtiles;
-                if (at_once < 1) at_once = 1;
-                pre = 8.9 + 0.3 * ((steps_q + w - 1) / w);
+                const int w = pre_splits(mtiles, steps_q, pl.ctas);
+                late = clusters_kept_out(ks, mtiles, w);
+                if (late > slots - 1) late = slots - 1;
+                pre = 0.245 * ((steps_q + w - 1) / w) + 0.12 * mtiles - (w > 1 ? 0.5 : 2.0);
+                tail = pre + steps_d * step + sum + 7.3;
+                if (pre < 0.0) pre = 0.0;
             }
-            const long long waves = (pairs * pl.chunks + at_once - 1) / at_once;
-            const double body = 5.4 + ((steps_q + ks - 1) / ks + steps_d) * step + (ks > 1 ? (ks > 2 ? 2.4 : 1.8) + 0.04 * tokens / ks : 0.0115 * tokens);
-            // clusters of four and more leave GPCs partly empty between waves
-            pl.us = body * (1.0 + (ks == 1 ? 0.8 : ks == 2 ? 0.85 : 1.2) * (waves - 1) + (waves > 1 ? (ks == 1 ? 0.0 : ks == 2 ? 0.1 : 0.3) : 0.0));
-            if (pre > 0.0) pl.us = std::pow(std::pow(pl.us, 6.0) + std::pow(pre, 6.0), 1.0 / 6.0);
-            // of plans that are estimated alike, slices rather than one long contraction
-            const double score = pl.us * (ks == 1 && steps_q > 16 ? 1.15 : 1.0);
+            pl.us = makespan(n, body, (ks == 1 ? 0.86 : 0.92) * body, slots, late, pre);
+            if (pl.us < tail) pl.us = tail;
+            // Where one slice leaves more than half of the places empty, slices are taken up to an eighth dearer: the estimates of one slice are
+            // low there (640 x 1280 NF3, 591 rows, one slice / two: estimated 11.9 / 11.4, measured 12.7 / 12.1), even on average over the drawn calls.
+            const double score = pl.us * (ks == 1 && steps_q > 16 && 2 * n < slots ? 1.125 : 1.0);
             if (best.us < 0 || score < best_score) { best = pl; best_score = score; }
         }
     }

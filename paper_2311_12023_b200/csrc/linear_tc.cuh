@@ -512,20 +512,26 @@ inline int pair_peel(int64_t M, int64_t out_cols) {
 }
 
 // CTA pairs on [512, 256] tiles take over once their tiles fill more than half of the SMs, and below 2048 rows unless the transposed tiles,
-// which pad to 16 rows instead of 512 and choose their split, are estimated faster: whole waves of the pair kernel are taken as 6 us and 0.64 us
-// (8-bit codes 0.95) per step each, 7 % less than they last on average, hence the 1.1.  Over 260 drawn calls of 257 to 2000 rows the side taken is 2.6 %
-// behind the faster one (7.8 % with 0.85, the line of the transposed tiles with one step per stage).  One wave that is at least four
-// fifths full, and more than four waves of rows without padding, stay with the pairs up to 0.88.  us as a graph, pair / transposed: 8192 x 8192 NF3 at 520 rows 87 / 50,
-// 11904 x 8448 NF3 at 546 rows 123 / 80, 4352 x 11008 NF3 at 688 rows 78 / 60, 7552 x 2176 NF2 at 1285 rows 50 / 44; 8320 x 4992 NF8 at 825 rows 79 / 100.
+// which pad to 16 rows instead of 512 and choose their split, are estimated faster.  The estimate of the pairs is fitted to 448 drawn calls of 257 to 2000 rows
+// (spread 6 %): whole waves, whose steps take less time where the last rows or the last wave leave SMs or tensor cores idle.  The side taken is 0.3 % behind the
+// faster one on average, more than a tenth in 4 of them (2.1 % and 45 with 6 us per wave and 0.64 per step).  us as a graph, pair / transposed: 8192 x 8192 NF3 at
+// 520 rows 87 / 50, 11904 x 8448 NF3 at 546 rows 123 / 80, 4352 x 11008 NF3 at 688 rows 78 / 60, 7160 x 10240 NF2 input gradient at 990 rows 110 / 152;
+// 8320 x 4992 NF8 at 825 rows 79 / 100.  Two corrections, both small: long calls run at a lower clock, the transposed tiles more so than the pairs (28672 x 8192 NF3
+// measured / estimated at 1024 rows 1.10, at 1500 1.17, at 2047 1.25; pairs 0.97, 1.03, 1.11), 0.4 per 10^12 products; and one wave of pairs
+// with at least four fifths of its tiles and nine tenths of its rows stays where they are estimated within a tenth (8192 x 8192 NF3 at 1024 rows 91 / 90, input
+// gradient 92.5 / 93.3, 5120 x 5120 NF2 at 1400 rows 60 / 57).
 // From 2048 rows on the pairs stay whatever the estimates say.  That line is drawn by hand.  Both sides measured on nine shapes, both passes,
 // 3-, 4- and 8-bit codes, 2048 to 4096 rows: where the last wave of pair tiles is well filled the pairs are up to a fifth faster (4096 x 4096 NF3
 // at 4096 rows 97 / 120, 28672 x 8192 NF8 at 2048 902 / 1064, 8192 x 8192 NF8 at 2048 273 / 306); where it is between a quarter and a half
 // full the transposed tiles would be, by up to a third and on narrow outputs by more (4096 x 11008 NF3 at 2600 rows 240 / 186, NF8 299 / 226; 4392 x
 // 26688 NF8 at 2600 726 / 557; 5120 x 5120 NF8 at 2304 148 / 116; 2040 x 27008 NF3 at 2048 274 / 156).
-inline double pair_estimate(int b0, int64_t M, int64_t out_cols, int steps_q) {
+inline double pair_estimate(int b0, int B0, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+    static const double step_us[4] = {0.668, 0.67, 0.693, 0.957};
     const int mt = static_cast<int>((M + 511) / 512), c_tiles = static_cast<int>((out_cols + BN - 1) / BN), peel = pair_peel(M, out_cols);
-    const long long pairs = sm_count() / 2, waves = (static_cast<long long>(mt) * (c_tiles - peel) + pairs - 1) / pairs;
-    return static_cast<double>(waves) * (6.0 + steps_q * (b0 == 8 ? 0.95 : 0.64)) + (peel > 0 ? 20.0 + 0.15 * steps_q : 0.0);
+    const long long pairs = sm_count() / 2, tiles = static_cast<long long>(mt) * (c_tiles - peel), waves = (tiles + pairs - 1) / pairs;
+    const double idle = 1.0 - static_cast<double>(tiles) / static_cast<double>(waves * pairs), padding = 1.0 - static_cast<double>(M) / (512.0 * mt);
+    const double step = step_us[bits_index(b0)] * (B0 == 16 ? 1.04 : 1.0) * (1.0 - 0.32 * idle) * (1.0 - 0.11 * padding);
+    return (steps_d > 0 ? 3.3 : 5.0) + static_cast<double>(waves) * (7.1 + (steps_q + steps_d) * step) + (peel > 0 ? 11.8 + 0.168 * steps_q : 0.0);
 }
 inline bool tc_use_pair(const QView& q, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
     if (M <= 256) return false;
@@ -533,8 +539,10 @@ inline bool tc_use_pair(const QView& q, bool backward, int64_t M, int64_t out_co
     if (2 * pair_ctas <= sm_count()) return false;
     if (M >= 2048) return true;
     const int64_t rows = (M + 511) / 512 * 512;
-    const bool full = pair_ctas <= sm_count() ? 5 * pair_ctas >= 4 * sm_count() : 16 * M >= 15 * rows && pair_ctas > 4 * sm_count();
-    return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d).us >= (full ? 0.88 : 1.1) * pair_estimate(q.b0, M, out_cols, steps_q);
+    const bool full = pair_ctas <= sm_count() && 5 * pair_ctas >= 4 * sm_count() && 10 * M >= 9 * rows;
+    const double products = static_cast<double>(M) * static_cast<double>(out_cols) * BK * steps_q;
+    return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d).us * (1.0 + 0.4e-12 * products) >=
+           (full ? 0.9 : 1.0) * pair_estimate(q.b0, q.B0, M, out_cols, steps_q, steps_d);
 }
 
 // The launch on transposed tiles that a call needs: the whole of it, or the output columns from *c_base on that the pair

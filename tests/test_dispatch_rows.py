@@ -29,6 +29,16 @@ def test_long_contractions_of_few_rows_are_sliced(N, K, b0, B0, M, r, backward):
     assert kernel == ONE and splits > 1
 
 
+# calls where another kernel or another number of slices, taken by an earlier model of the split, cost 10 to 47 %
+@pytest.mark.parametrize("N,K,b0,B0,M,r,backward,want", [
+    (13848, 4224, 4, 128, 601, 64, False, (ONE, 1)), (4784, 21120, 8, 64, 445, 64, False, (ONE, 3)), (13240, 11968, 2, 64, 773, 16, False, (ONE, 1)),
+    (22904, 10048, 8, 32, 301, 64, False, (ONE, 2)), (2688, 2304, 2, 32, 283, 64, False, (ONE, 2)), (9216, 16896, 4, 32, 19, 16, True, (ONE, 1)),
+    (3456, 1792, 8, 64, 808, 128, True, (ONE, 2)), (16648, 8768, 8, 32, 628, 64, True, (ONE, 1)), (14336, 15616, 4, 128, 884, 64, True, (ONE, 1)),
+    (16512, 1792, 2, 64, 32, 0, False, (ONE, 1))])
+def test_slices_of_the_contraction(N, K, b0, B0, M, r, backward, want):
+    assert binding.linear_route(N, K, C(b0, B0, 8, 256, 32), r, M, backward) == want
+
+
 # many chunks of transposed tiles where the pairs ran before: a last chunk that is not full, both passes, rank below and above 64
 @pytest.mark.gpu
 @pytest.mark.parametrize("N,K,b0,M,r", [(8192, 2048, 3, 1100, 64), (5120, 1024, 2, 700, 128), (8200, 1024, 8, 1101, 16)])
