@@ -32,7 +32,7 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
 }
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 
 // One lane of the (converged) warp.  A role that issues copies or tensor-core instructions runs its loop with the whole
 // warp and guards only the issue with this: operands stay in uniform registers.  Inside an `if (lane == 0)` loop every
@@ -55,6 +55,9 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 // start while its predecessor in the stream still runs; pdl_wait() blocks until that predecessor
 // has completed and its memory is visible, pdl_launch_dependents() lets the successor start early.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The same for a thread that goes on to request copies (TMA, bulk) of what that kernel wrote with ordinary stores: the copies read through the async
+// proxy, which the wait alone does not order behind those stores.
+__device__ __forceinline__ void pdl_wait_for_copies() { pdl_wait(); fence_proxy_async_global(); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 constexpr long long kWaitCycles = 4000000000LL;   // about two seconds

@@ -346,7 +346,8 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
 
     // Everything that a step needs is requested first; what follows (tensor memory, the code book, the barrier of the cluster) takes about
     // as long as those requests.  Only arrivals on the other CTA's barriers have to wait for the cluster.
-    // (Without a rank-r term this is the first kernel of its call, launched while the one in front ends: it waits for that one before it reads.)
+    // (Without a rank-r term this is the first kernel of its call, launched while the one in front ends: it waits for that one before it reads.  With one, the
+    // pre-product has waited, fence included, before it let this kernel start.)
     const bool lead = p.steps_d == 0;
     const int early_x = min(p.ss, nq / PS), early_p = min(p.sp, (nq + PS - 1) / PS);
     if (warp < 2) {
@@ -367,7 +368,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
         }
         __syncwarp();
         asm volatile("bar.sync 1, 64;" ::: "memory");
-        if (lead) pdl_wait();
+        if (lead) pdl_wait_for_copies();
         if (warp < kBoxWarps && elect_one()) {
             for (int i = 0; i < early_x; ++i) issue_box(warp, i, i);
         }
@@ -380,7 +381,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             }
             fence_barrier_init();
             fence_proxy_async();
-            if (lead) pdl_wait();
+            if (lead) pdl_wait_for_copies();
             for (int i = 0; i < early_p; ++i) issue_codes(i, i);
         }
         __syncwarp();
@@ -417,8 +418,7 @@ tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_cons
             const int step = PS == 1 ? round : 2 * round + warp;
             if (step >= nq && step < nq + PS && step < total) {
                 // the rank-r intermediate comes from the kernel in front (programmatic dependent launch)
-                pdl_wait();
-                fence_proxy_async_all();
+                pdl_wait_for_copies();
             }
             __syncwarp();
             if (elect_one()) issue_box(warp, round, r.s);

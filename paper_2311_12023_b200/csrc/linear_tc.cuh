@@ -227,7 +227,7 @@ __device__ __forceinline__ void lowrank_body(const CUtensorMap& tmA, const CUten
     // The CTAs of a cluster write into each other's shared memory at the end; that is allowed once every CTA of the
     // cluster runs, which the first phase of the cluster barrier establishes: arrive here, wait before the first store.
     if (CL && nsplit > 1) dec::cluster_arrive_relaxed();
-    pdl_wait();                   // started while the previous kernel of the stream ends; everything below comes after it
+    pdl_wait_for_copies();        // started while the previous kernel of the stream ends; everything below comes after it
     // cleared before this CTA lets the dependent kernel start: that kernel is launched once all CTAs have passed here
     if (p.clear_status && tile == 0 && split == 0 && threadIdx.x == 0) *p.status = 0;
     pdl_launch_dependents();      // the linear kernel behind this one needs T only in its last steps

@@ -164,8 +164,7 @@ tc_pair_linear_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             const uint32_t p_dst = smem_u32(p_ring) + s * P_BYTES;
             const int my_m = m0 + static_cast<int>(rank) * 128;
             if (step == p.steps_q) {
-                pdl_wait();                           // the rank-r intermediate comes from the kernel in front
-                fence_proxy_async_all();
+                pdl_wait_for_copies();                // the rank-r intermediate comes from the kernel in front
             }
             __syncwarp();
             if (elect_one()) {

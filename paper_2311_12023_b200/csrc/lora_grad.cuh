@@ -88,8 +88,7 @@ __device__ __forceinline__ void wgrad_body(const CUtensorMap& tmA, const CUtenso
             }
             __syncwarp();
         }
-        pdl_wait();
-        fence_proxy_async_all();
+        pdl_wait_for_copies();
         for (int i = 0; i < first; ++i) {
             const uint32_t b_dst = ring0 + i * stage_bytes + A_BYTES;
             const int m = (s_lo + i) * BK;
