@@ -1,5 +1,7 @@
 """Calls enqueued one behind the other without a synchronisation: the first kernel of a call starts while the last one of the call
 before it ends, so each has to wait before it reads what that one writes (the result, the workspace) or overwrites it."""
+import types
+
 import numpy as np
 import pytest
 import torch
@@ -177,8 +179,10 @@ class EncodeChain:
 def test_encodes_between_calls_give_the_bits_of_synchronised_ones(monkeypatch):
     chain = EncodeChain()
     with monkeypatch.context() as m:                  # a synchronisation behind every call of the library
-        check = binding._check
+        check, native = binding._check, binding._fast or binding._fast_part()
         m.setattr(binding, "_check", lambda status, where: (check(status, where), torch.cuda.synchronize()))
+        m.setattr(binding, "_fast", types.SimpleNamespace(**{name: lambda *a, f=getattr(native, name): (f(*a), torch.cuda.synchronize())[0]
+                                                             for name in ("linear", "encode")}))      # (these do not come by _check)
         want = chain.take(chain.run)
     for _ in range(20):
         assert [i for i, (a, b) in enumerate(zip(want, chain.take(chain.run))) if not torch.equal(a, b)] == []
@@ -187,3 +191,85 @@ def test_encodes_between_calls_give_the_bits_of_synchronised_ones(monkeypatch):
         chain.run()
     for _ in range(10):
         assert [i for i, (a, b) in enumerate(zip(want, chain.take(graph.replay))) if not torch.equal(a, b)] == []
+
+
+class PlainChain:
+    """Decode-sized calls without a rank-r term on one workspace: a kernel in front of each clears the arrival counters that the one before has
+    counted up, and is itself launched while that one ends.  Every result is the next call's input."""
+
+    def __init__(self, rows, b0):
+        cfg = C(b0, 64, 8, 64, 32)
+        square, wide, narrow = (Layer(9300 + i, N, K, cfg, r=0) for i, (N, K) in enumerate(((1024, 1024), (2048, 1024), (512, 1024))))
+        self.layers = [(square, False), (square, True), (wide, False), (wide, True), (narrow, False), (narrow, True), (square, False)] * 3
+        for layer, backward in self.layers:
+            q = layer.q
+            kernel, splits = binding.linear_route(q.N, q.K, cfg, 0, rows, backward)
+            if kernel == binding.PATH_STREAM:                    # (the wide matrix's input gradient takes transposed tiles from nine rows on)
+                assert splits > 1
+            else:
+                assert layer is wide and backward and rows > 8
+        self.ws = torch.empty(max(binding.linear_workspace_bytes(l.q.N, l.q.K, cfg, 0, rows) for l, _ in self.layers), dtype=torch.uint8, device="cuda")
+        self.x = binding.bf16_from_bits(inputs.activations(9310, rows, 1024))
+        self.y = [torch.empty(rows, l.q.K if b else l.q.N, dtype=torch.bfloat16, device="cuda") for l, b in self.layers]
+
+    def run(self, synchronize=False):
+        x = self.x
+        for (layer, backward), y in zip(self.layers, self.y):
+            x = (binding.linear_bwd_input if backward else binding.linear_fwd)(layer.q, None, None, x, out=y, workspace=self.ws)
+            if synchronize:
+                torch.cuda.synchronize()
+
+    def take(self, run, **kwargs):
+        for t in self.y:
+            t.fill_(float("nan"))
+        self.ws.fill_(0x5A)
+        run(**kwargs)
+        torch.cuda.synchronize()
+        assert binding.workspace_status(self.ws) == 0
+        return [t.clone() for t in self.y]
+
+
+@pytest.mark.parametrize("b0", [2, 3, 4, 8])
+@pytest.mark.parametrize("rows", [1, 3, 8, 16])
+def test_plain_decode_calls_give_the_bits_of_synchronised_ones(rows, b0):
+    chain = PlainChain(rows, b0)
+    want = chain.take(chain.run, synchronize=True)
+    assert all(bool(torch.isfinite(t.float()).all()) and bool((t != 0).any()) for t in want)
+    for _ in range(10):
+        assert [i for i, (a, b) in enumerate(zip(want, chain.take(chain.run))) if not same_bits(a, b)] == []
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        chain.run()
+    for _ in range(5):
+        assert [i for i, (a, b) in enumerate(zip(want, chain.take(graph.replay))) if not same_bits(a, b)] == []
+
+
+@pytest.mark.parametrize("b0,rows", [(3, 48), (8, 40), (2, 300)])
+def test_a_matrix_encoded_in_front_of_a_plain_call(b0, rows):
+    """Transposed tiles without a rank-r term are the first kernel of their call: copies of the codes, loads of the scales and copies of the
+    activations wait for the encoder, and for the call that wrote the activations."""
+    cfg, N, K = C(b0, 64, 8, 64, 32), 768, 768
+    W = [torch.from_numpy(inputs.gaussian(9400 + i, (N, K), 0.04)).cuda() for i in range(3)]
+    q = binding.alloc_qmatrix(N, K, cfg, torch.device("cuda"))
+    assert binding.linear_path(N, K, cfg, 0, rows, False) == binding.PATH_TC_ONE
+    ws = torch.empty(max(binding.linear_workspace_bytes(N, K, cfg, 0, rows), binding.packed_sizes(N, K, cfg)[3]), dtype=torch.uint8, device="cuda")
+    x = binding.bf16_from_bits(inputs.activations(9410, rows, K))
+    ys = [torch.empty(rows, N, dtype=torch.bfloat16, device="cuda") for _ in range(9)]
+
+    def run(synchronize=False):
+        sync = torch.cuda.synchronize if synchronize else lambda: None
+        a = x
+        for i, y in enumerate(ys):
+            binding.encode(W[i % 3], cfg, out=q, workspace=ws)
+            sync()
+            a = (binding.linear_bwd_input if i % 2 else binding.linear_fwd)(q, None, None, a, out=y, workspace=ws)
+            sync()
+        torch.cuda.synchronize()
+        return [y.clone() for y in ys]
+
+    want = run(synchronize=True)
+    assert all(bool(torch.isfinite(t.float()).all()) and bool((t != 0).any()) for t in want)
+    for _ in range(10):
+        for y in ys:
+            y.fill_(float("nan"))
+        assert [i for i, (a, b) in enumerate(zip(want, run())) if not same_bits(a, b)] == []
