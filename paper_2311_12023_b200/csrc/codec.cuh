@@ -40,9 +40,9 @@ __device__ __forceinline__ uint32_t nearest_code(float x, const float* __restric
 // Two elements per instruction (fma.f32x2).
 //
 // What bounds the kernel: loads in flight (a CTA loads, then computes, then stores) and instruction issue, 17 instructions per 3-bit weight
-// (25.6 before, with a saturating sum over the thresholds; 4-bit codes looked a bin table up in shared memory).  us per call in a graph with
-// the scale kernel, before / now: 8192 x 8192 2 bits 60 / 58, 3 bits 75 / 70, blocks of 16 80 / 74, 4 bits 89 / 80; 11008 x 4096 4 bits
-// 64.7 / 57.6.  The scalar form of the same polynomials: 4 bits 88 and 63.
+// (25.6 with a saturating sum over the thresholds; 4-bit codes looked a bin table up in shared memory).  us per call in a graph with
+// the scale kernel, those searches / the curve, both with a lane per marked row (times now: see encode_exact): 8192 x 8192 2 bits 60 / 58, 3 bits
+// 75 / 70, blocks of 16 80 / 74, 4 bits 89 / 80; 11008 x 4096 4 bits 64.7 / 57.6.  The scalar form of the same polynomials: 4 bits 88 and 63.
 template <int B> struct Curve {
     static constexpr int NE = curve_even(B), NO = curve_odd(B);
     static constexpr uint32_t kMask = (1u << (23 - B)) - 1u;               // fraction bits

@@ -58,7 +58,7 @@ struct SwapParams {
     const __nv_bfloat16* L1; // forward with the weights in tensor memory: [N][r], read directly
     int r;
     int nbox, box;           // token boxes (1 or 2) and tokens per box (a multiple of 16, at most 256; half of them per CTA)
-    int ss, sp;              // stages (of one step; weights in tensor memory: two) of the token + weight ring and of the packed-code ring
+    int ss, sp;              // stages (of one or two steps) of the token + weight ring and of the packed-code ring
     uint32_t tail_off;       // of the barriers, behind the rings
     uint32_t tmem_cols;
 };
@@ -257,12 +257,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-template <int B, bool BWD, bool TA, int NBOX>
+template <int B, bool BWD, bool TA, int NBOX, int PS>
 __global__ void __launch_bounds__(kSwThreads, 1)
 tc_swap_linear_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmT,
                       const __grid_constant__ CUtensorMap tmF, const SwapParams p) {
-    constexpr int PS = TA ? 2 : 1;                                       // steps of 64 contraction elements per stage, i.e. per round of waits and commits
-    static_assert(!TA || NBOX == 1, "two warps request the boxes of a stage");
+    // PS: steps of 64 contraction elements per stage, i.e. per round of waits and commits
+    static_assert(PS * NBOX <= 2, "two warps request the boxes of a stage");
     constexpr int P_BYTES = 1024 * B;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -698,7 +698,7 @@ inline int tc_max_clusters(int n) {
     if (known >= 0) return known;
     const int fallback[4] = {74, 33, 22, 15};
     int got = 0;
-    auto kern = tc_swap_linear_kernel<3, false, false, 2>;
+    auto kern = tc_swap_linear_kernel<3, false, false, 2, 1>;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2, 1, n / 2);
     cfg.blockDim = dim3(kSwThreads);
@@ -719,31 +719,36 @@ inline int tc_max_clusters(int n) {
 
 struct SwapPlan {
     int chunks, nbox, box, ks;       // token chunks, boxes and tokens per box, slices of the contraction
+    int ps;                          // steps per stage
     int ss, sp, smem;
     uint32_t tmem_cols;
     long long ctas;
     double us;                       // estimated time
 };
 
-// Ring depths of a plan; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase while the
-// one before it can be incomplete.  A dequantization warp works on every fourth step:
-//   - it may wait for stage j % ss to be free (the tensor core is done with step j - ss) once step j - 2 ss is known to be
-//     done; its own step j - 4 waited for j - 4 - ss, hence ss >= 4;
-//   - it may wait for the codes of step j once those of step j - sp are known to have landed: they have where its own
-//     group used them (sp a multiple of four) or where the tensor core is done with that step (sp >= ss).
-// (With the weights in tensor memory the kernel takes depths of its own, see run_swap; what fits here fits there.)
-// As many stages of weights as fit beside four of codes, then codes.  Fewer stages of weights for as many of codes took more shared memory, which the
+// Steps per stage: two where the weights go to tensor memory.
+inline int swap_stage_steps(int b0, bool backward, int nbox, int box) { (void)b0; (void)box; return nbox == 1 && !backward ? 2 : 1; }
+
+// Ring depths of a plan in stages; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase while the
+// one before it can be incomplete.  A dequantization warp works on every fourth step, i.e. on every g-th stage, g = 4 (one step per stage) or 2:
+//   - it may wait for stage j % ss to be free (the tensor core is done with stage j - ss) once stage j - 2 ss is known to be
+//     done; its own stage j - g waited for j - g - ss, hence ss >= g;
+//   - it may wait for the codes of stage j once those of stage j - sp are known to have landed: they have where its own
+//     group used them (sp a multiple of g) or where the tensor core is done with that stage (sp >= ss).
+// (With the weights in tensor memory the kernel takes depths of its own, see run_swap; what fits here with one step per stage fits there.)
+// As many stages of weights as fit beside g of codes, then codes.  Fewer stages of weights for as many of codes took more shared memory, which the
 // scales miss in L1: 10112 x 15616 input gradient, 8-bit codes in blocks of 16, 17 rows, 95 us with 8 and 4 stages, 113 with 7 and 8.
-inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
-    const int stage = kSwWBytes + pl.nbox * pl.box * 64, pk = 1024 * b0;
+inline bool swap_rings(int b0, bool backward, int ks, SwapPlan& pl) {
+    const int steps = backward ? pl.ps : 1, g = 4 / steps;
+    const int stage = steps * (kSwWBytes + pl.nbox * pl.box * 64), pk = steps * 1024 * b0;
     const int fixed = 1024 + kSwTail + (b0 == 8 ? 32768 : 0);
     const int room = kSmemLimit - fixed;
-    pl.ss = (room - 4 * pk) / stage;
-    if (pl.ss > kSwMaxStages) pl.ss = kSwMaxStages;
-    if (pl.ss < 4) return false;
+    pl.ss = (room - g * pk) / stage;
+    if (pl.ss > kSwMaxStages / steps) pl.ss = kSwMaxStages / steps;
+    if (pl.ss < g) return false;
     pl.sp = (room - pl.ss * stage) / pk;
     if (pl.sp > kSwMaxStages) pl.sp = kSwMaxStages;
-    if (pl.sp < pl.ss) pl.sp = 4;
+    if (pl.sp < pl.ss) pl.sp = g;
     const int bytes = pl.ss * stage + pl.sp * pk;
     if (ks > 1 && pl.nbox * pl.box * 512 > bytes) return false;      // the accumulators are laid over the rings
     pl.smem = fixed + bytes;
@@ -753,8 +758,8 @@ inline bool swap_rings(int b0, int ks, SwapPlan& pl) {
 // Tokens of the largest chunk whose rings fit: 512, and 384 for 8-bit codes (their code book takes 32 KB of shared memory).
 inline int swap_max_tokens(int b0) {
     SwapPlan pl{};
-    pl.nbox = 2;
-    for (pl.box = 256; pl.box > 16 && !swap_rings(b0, 1, pl); pl.box -= 16) {}
+    pl.nbox = 2; pl.ps = 1;
+    for (pl.box = 256; pl.box > 16 && !swap_rings(b0, true, 1, pl); pl.box -= 16) {}
     return 2 * pl.box;
 }
 
@@ -812,7 +817,7 @@ inline double makespan(long long n, double first, double next, long long slots, 
 // without a rank-r term); on 1200 others the plan that it picks takes 0.4 % longer than the best one on average, and more than a tenth longer in 12 of
 // them.  (The model before counted whole waves and took one slice 15 % dearer than estimated: 1.5 %, and 62.  us as a graph, its plan / this one: 13848 x 4224
 // NF4, 601 rows 99.8 / 68; 4784 x 21120 NF8, 445 rows 182 / 142; 9216 x 16896 NF4 input gradient, 19 rows 84 / 63; 2688 x 2304 NF2, 283 rows 17.4 / 14.1.)
-inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
+inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d, bool beside_pre) {
     SwapPlan best{};
     best.us = -1.0;
     double best_score = 0.0;
@@ -832,6 +837,7 @@ inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t
         if (ch > first && per < 32) break;
         pl.nbox = per > 256 ? 2 : 1;
         pl.box = ((per + pl.nbox - 1) / pl.nbox + 15) / 16 * 16;
+        pl.ps = swap_stage_steps(b0, backward, pl.nbox, pl.box);
         const int tokens = pl.nbox * pl.box;
         pl.chunks = static_cast<int>((M + tokens - 1) / tokens);
         pl.tmem_cols = 32;
@@ -840,17 +846,17 @@ inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t
         const double block = B0 == 16 ? (ta ? 1.17 : 1.12) : B0 == 32 ? (ta ? 1.05 : 1.04) : 1.0;
         const double dq = block * dq_us[2 * (pl.nbox - 1) + (backward ? 1 : 0)][bits_index(b0)], mma = (pl.nbox == 1 ? 0.00085 : 0.00097) * tokens;
         for (int ks = 1; ks <= 4 && ks <= steps_q; ++ks) {
-            if (!swap_rings(b0, ks, pl)) continue;
+            if (!swap_rings(b0, backward, ks, pl)) continue;
             pl.ks = ks;
             const long long n = pairs * pl.chunks, slots = tc_max_clusters(2 * ks);
             pl.ctas = 2 * n * ks;
             const double busy = static_cast<double>(2 * ks * (n < slots ? n : slots)) / dec::sm_count_cached();
-            const double step = std::sqrt(std::sqrt(dq * dq * dq * dq + mma * mma * mma * mma)) * (1.0 + (steps_d > 0 ? 0.155 : 0.22) * busy);
+            const double step = std::sqrt(std::sqrt(dq * dq * dq * dq + mma * mma * mma * mma)) * (1.0 + (beside_pre ? 0.155 : 0.22) * busy);
             const double sum = ks == 1 ? 0.013 * tokens : 0.6 + red_us[ks - 2] * tokens;
-            const double body = (steps_d > 0 ? 5.6 : 4.2) + ((steps_q + ks - 1) / ks + steps_d) * step + sum;
+            const double body = (beside_pre ? 5.6 : 4.2) + ((steps_q + ks - 1) / ks + steps_d) * step + sum;
             double pre = 0.0, tail = 0.0;
             long long late = 0;
-            if (steps_d > 0) {
+            if (beside_pre) {
                 const int w = pre_splits(mtiles, steps_q, pl.ctas);
                 late = clusters_kept_out(ks, mtiles, w);
                 if (late > slots - 1) late = slots - 1;
@@ -869,25 +875,26 @@ inline SwapPlan make_swap_plan(int b0, int B0, bool backward, int64_t M, int64_t
     return best;
 }
 
-// The same, with the plans of the last few shapes kept by the calling thread (pure arithmetic, about 3 us).
-inline const SwapPlan& swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d) {
-    struct Entry { int b0 = 0, B0 = 0, steps_q = 0, steps_d = 0; bool backward = false; int64_t M = 0, out_cols = 0; SwapPlan plan; };
+// The same, with the plans of the last few shapes kept by the calling thread (pure arithmetic, some microseconds).  beside_pre: the rank-r pre-product of the
+// call runs beside the launch (not where it covers the columns that the pair kernel leaves).
+inline const SwapPlan& swap_plan(int b0, int B0, bool backward, int64_t M, int64_t out_cols, int steps_q, int steps_d, bool beside_pre) {
+    struct Entry { int b0 = 0, B0 = 0, steps_q = 0, steps_d = 0; bool backward = false, beside_pre = false; int64_t M = 0, out_cols = 0; SwapPlan plan; };
     constexpr int kEntries = 32;
     thread_local Entry cache[kEntries];
     const uint64_t h = (static_cast<uint64_t>(M) * 0x9E3779B97F4A7C15ull) ^ (static_cast<uint64_t>(out_cols) * 0xC2B2AE3D27D4EB4Full) ^
-                       (static_cast<uint64_t>(steps_q * 8 + steps_d * 64 + b0 + B0 * 4096 + (backward ? 16 : 0)) * 0x165667B19E3779F9ull);
+                       (static_cast<uint64_t>(steps_q * 8 + steps_d * 64 + b0 + B0 * 4096 + (backward ? 16 : 0) + (beside_pre ? 32 : 0)) * 0x165667B19E3779F9ull);
     Entry& e = cache[(h >> 40) % kEntries];
-    if (e.b0 != b0 || e.B0 != B0 || e.backward != backward || e.M != M || e.out_cols != out_cols || e.steps_q != steps_q || e.steps_d != steps_d) {
-        e.plan = make_swap_plan(b0, B0, backward, M, out_cols, steps_q, steps_d);
-        e.b0 = b0; e.B0 = B0; e.backward = backward; e.M = M; e.out_cols = out_cols; e.steps_q = steps_q; e.steps_d = steps_d;
+    if (e.b0 != b0 || e.B0 != B0 || e.backward != backward || e.beside_pre != beside_pre || e.M != M || e.out_cols != out_cols || e.steps_q != steps_q || e.steps_d != steps_d) {
+        e.plan = make_swap_plan(b0, B0, backward, M, out_cols, steps_q, steps_d, beside_pre);
+        e.b0 = b0; e.B0 = B0; e.backward = backward; e.beside_pre = beside_pre; e.M = M; e.out_cols = out_cols; e.steps_q = steps_q; e.steps_d = steps_d;
     }
     return e.plan;
 }
 
-template <int B, bool BWD, bool TA, int NBOX>
+template <int B, bool BWD, bool TA, int NBOX, int PS>
 inline int launch_swap(const CUtensorMap& tX, const CUtensorMap& tT, const CUtensorMap& tF, const SwapParams& p, const SwapPlan& pl,
                        int smem, int pairs, cudaStream_t st, bool first) {
-    auto kern = tc_swap_linear_kernel<B, BWD, TA, NBOX>;
+    auto kern = tc_swap_linear_kernel<B, BWD, TA, NBOX, PS>;
     static bool attr_done = false;
     if (!attr_done) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
@@ -932,7 +939,7 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     p.L1 = static_cast<const __nv_bfloat16*>(L1); p.r = r;
     p.clear_status = first ? 1 : 0;
     int smem = pl.smem;
-    p.tail_off = pl.ss * (kSwWBytes + pl.nbox * pl.box * 64) + pl.sp * 1024 * q.b0;
+    p.tail_off = pl.ps * (pl.ss * (kSwWBytes + pl.nbox * pl.box * 64) + pl.sp * 1024 * q.b0);
     const bool ta = !backward && pl.nbox == 1;      // (256 columns of accumulators and eight stages of 32 columns fill tensor memory)
     if (ta) {
         // Without weight tiles four stages of two steps of both rings always fit (256 tokens, 8-bit codes: 230,912 of 232,448 bytes, code
@@ -959,10 +966,10 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
     const int pairs = (cols + 255) / 256;
     auto go = [&](auto bits) {
         constexpr int B = decltype(bits)::value;
-        if (ta) return launch_swap<B, false, true, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
-        if (!backward) return launch_swap<B, false, false, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
-        if (pl.nbox == 1) return launch_swap<B, true, false, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
-        return launch_swap<B, true, false, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (ta) return launch_swap<B, false, true, 1, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (!backward) return launch_swap<B, false, false, 2, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if (pl.nbox == 1) return launch_swap<B, true, false, 1, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        return launch_swap<B, true, false, 2, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
     };
     switch (q.b0) {
         case 2: return go(std::integral_constant<int, 2>());

@@ -541,7 +541,7 @@ inline bool tc_use_pair(const QView& q, bool backward, int64_t M, int64_t out_co
     const int64_t rows = (M + 511) / 512 * 512;
     const bool full = pair_ctas <= sm_count() && 5 * pair_ctas >= 4 * sm_count() && 10 * M >= 9 * rows;
     const double products = static_cast<double>(M) * static_cast<double>(out_cols) * BK * steps_q;
-    return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d).us * (1.0 + 0.4e-12 * products) >=
+    return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d, steps_d > 0).us * (1.0 + 0.4e-12 * products) >=
            (full ? 0.9 : 1.0) * pair_estimate(q.b0, q.B0, M, out_cols, steps_q, steps_d);
 }
 
@@ -549,10 +549,10 @@ inline bool tc_use_pair(const QView& q, bool backward, int64_t M, int64_t out_co
 // kernel leaves (none where *c_base is not below out_cols).
 inline SwapPlan call_swap_plan(const QView& q, bool backward, bool pair, int64_t M, int64_t out_cols, int steps_q, int steps_d, int* c_base) {
     *c_base = 0;
-    if (!pair) return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d);
+    if (!pair) return swap_plan(q.b0, q.B0, backward, M, out_cols, steps_q, steps_d, steps_d > 0);
     const int peel = pair_peel(M, out_cols);
     *c_base = (static_cast<int>((out_cols + BN - 1) / BN) - peel) * BN;
-    return peel > 0 ? swap_plan(q.b0, q.B0, backward, M, out_cols - *c_base, steps_q, steps_d) : SwapPlan{};
+    return peel > 0 ? swap_plan(q.b0, q.B0, backward, M, out_cols - *c_base, steps_q, steps_d, false) : SwapPlan{};
 }
 
 // C = contraction length, out_cols = width of the output of the linear kernel that follows.
@@ -562,7 +562,7 @@ inline PrePlan pre_plan(const QView& q, bool backward, int64_t C, int r, int64_t
     pl.steps = static_cast<int>((C + BK - 1) / BK);
     const int steps_d = (r + BK - 1) / BK;
     const long long main_ctas = tc_use_pair(q, backward, M, out_cols, pl.steps, steps_d) ? 2 * ((M + 511) / 512) * ((out_cols + BN - 1) / BN)
-                                                                                        : swap_plan(q.b0, q.B0, backward, M, out_cols, pl.steps, steps_d).ctas;
+                                                                                        : swap_plan(q.b0, q.B0, backward, M, out_cols, pl.steps, steps_d, steps_d > 0).ctas;
     pl.nsplit = pre_splits(pl.mtiles, pl.steps, main_ctas);
     pl.steps_per_split = (pl.steps + pl.nsplit - 1) / pl.nsplit;
     pl.rp = (r <= 64) ? 64 : 128;
@@ -619,15 +619,9 @@ constexpr int kTcMinRowsBwd = 9;  // input gradient of matrices with at least 20
 
 inline bool tc_supported(const QView& q, int r, int64_t M, bool backward) {
     (void)r;
-    // With two steps per stage of the transposed tiles, over some 75 drawn calls each (512 .. 28672 rows and columns, with and without a rank-r term), transposed /
-    // streaming: forward 1 row 1.34, 4 rows 1.24, 8 rows 1.12, 12 rows 1.05, 16 rows 0.98; input gradient 1 to 4 rows 1.05, 8 rows 0.95, 9 rows 0.76, 16 rows 0.66 (matrices
-    // of fewer than 2048 rows among them, which stay with the streaming kernels up to 16 rows all the same).  One step per stage:
-    // us as a graph, streaming / transposed, 2-, 3-, 4- and 8-bit codes of 8192 x 8192, rank 64: forward 1 row 17 / 24, 18 / 24, 25 / 30, 29 / 42; 8 rows
-    // 19 / 24, 20 / 24, 27 / 31, 32 / 42; 16 rows 24 / 24, 25 / 25, 31 / 31, 42 / 42 (other shapes: streaming at most 3 % behind at 16 rows, up to a
-    // quarter ahead on 28672 x 8192).  Input gradient 1 row 25 / 25, 26 / 26, 29 / 32, 36 / 44; 8 rows 27 / 25, 28 / 26, 31 / 32, 38 / 44; 9 rows (two
-    // token groups) 36 / 26, 40 / 26, 47 / 32, 58 / 44.  One line for all widths and shapes: 2- and 3-bit input gradients of 1 to 8 rows stay with the
-    // streaming kernels although the transposed tiles would be faster on few rows of weights (2048 x 8192 1 row 13 / 12, 8 rows 15 / 12; 4096 x
-    // 4096 8 rows 14.6 / 13; even on 11008 x 4096 and behind on 28672 x 8192, 70 / 72).
+    // Geometric means of transposed / streaming over some 75 drawn calls for each number of rows (512 .. 28672 rows and columns, 2 to 8 bits): forward 1 row 1.34,
+    // 8 rows 1.12, 16 rows 0.98 (8192 x 8192 even, 28672 x 8192 up to a quarter dearer); input gradient 1 to 4 rows 1.05, 8 rows 0.95, 9 rows (a second token
+    // group for the streaming kernels) 0.76.  One line for all shapes: around it the faster side depends on the shape, and the streaming kernels keep the even cases.
     const int min_rows = (backward && q.N >= 2048) ? kTcMinRowsBwd : kTcMinRows;
     if (M < min_rows) return false;
     if (q.N % 8 != 0 || q.K % 8 != 0) return false;
@@ -663,7 +657,7 @@ inline int tc_launch(const QView& q, const void* L1, const void* L2, int r, cons
         PreParams pp;
         pp.T = T; pp.status = reinterpret_cast<int*>(ws);
         pp.M = M; pp.r = r; pp.rp = pl.rp; pp.steps = pl.steps; pp.steps_per_split = pl.steps_per_split; pp.stages = 0;
-        pp.clear_status = 1;           // first kernel of the call (run_linear issues no memset when there is a rank-r term)
+        pp.clear_status = 1;           // first kernel of the call
         const int rc = backward ? launch_pre<true>(tPA, tPB, pp, pl.mtiles, pl.nsplit, st)
                                 : launch_pre<false>(tPA, tPB, pp, pl.mtiles, pl.nsplit, st);
         if (rc != LQLORA_OK) return rc;
