@@ -18,8 +18,9 @@
 // Every wait is bounded (see linear_tc.cuh).
 //
 // Two steps per stage: without loads and dequantization a step took 370 clocks, of which the issuing warp spent 140 in a wait that was satisfied and 170 to
-// 210 issuing.  The input gradient has no use for it: over 1900 plans of drawn calls one step per stage takes between 3 % less (blocks of 16, more than 128
-// tokens) and 2.5 % more (2-bit codes, few tokens) time, and 8 to 10 % less with 8-bit codes and more than 128 tokens, whose two-step stages are too few.
+// 210 issuing.  The input gradient has little use for it: over 1900 plans of drawn calls one step per stage takes up to 2 % less time (8 to 10 % with 8-bit codes
+// and more than 128 tokens, whose two-step stages are too few), but 2.5 % more with 2-bit codes and up to 64 tokens (4944 x 11968, 18 rows 27.3 / 25.7 us), which
+// therefore keep two.
 // What every step needs is requested before tensor memory, the code book and the cluster barrier are set up, and arrivals on that barrier are relaxed
 // (the initialisation of the mbarriers has a fence of its own): a releasing arrival waited for the scale loads in front of it.
 // us as a graph, one step per stage and a set-up in front of the loads / this: 8192 x 8192 NF3, 128 rows 27.6 / 24.6, without a rank-r term (a
@@ -726,8 +727,8 @@ struct SwapPlan {
     double us;                       // estimated time
 };
 
-// Steps per stage: two where the weights go to tensor memory.
-inline int swap_stage_steps(int b0, bool backward, int nbox, int box) { (void)b0; (void)box; return nbox == 1 && !backward ? 2 : 1; }
+// Steps per stage: two where the weights go to tensor memory, and in 2-bit input gradients of few tokens (see the top of the file).
+inline int swap_stage_steps(int b0, bool backward, int nbox, int box) { return nbox == 1 && (!backward || (b0 == 2 && box <= 64)) ? 2 : 1; }
 
 // Ring depths of a plan in stages; false when they do not fit.  A barrier tells only the parity of its phase, so nobody may wait for a phase while the
 // one before it can be incomplete.  A dequantization warp works on every fourth step, i.e. on every g-th stage, g = 4 (one step per stage) or 2:
@@ -968,6 +969,8 @@ inline int run_swap(const QView& q, const void* L1, const void* L2, int r, const
         constexpr int B = decltype(bits)::value;
         if (ta) return launch_swap<B, false, true, 1, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
         if (!backward) return launch_swap<B, false, false, 2, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
+        if constexpr (B == 2)
+            if (pl.ps == 2) return launch_swap<B, true, false, 1, 2>(tX, tT, tF, p, pl, smem, pairs, st, first);
         if (pl.nbox == 1) return launch_swap<B, true, false, 1, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
         return launch_swap<B, true, false, 2, 1>(tX, tT, tF, p, pl, smem, pairs, st, first);
     };
