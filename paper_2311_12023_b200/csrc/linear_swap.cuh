@@ -781,7 +781,7 @@ inline int pre_splits(int mtiles, int steps, long long main_ctas) {
     if (want < 1) want = 1;
     while (want & (want - 1)) want &= want - 1;
     // Not two splits of more than 37 row tiles: a graph of calls with 65 of them (130 CTAs in clusters of two) before 40 clusters of four of the linear kernel
-    // ended in a launch failure, and neither reading nor checks of every address in both kernels showed why.
+    // ended in a launch failure, and neither reading nor checks of ring positions, copies, loads and accumulator addresses in the kernels showed why.
     if (want == 2 && mtiles > 37) want = 1;
     return want;
 }

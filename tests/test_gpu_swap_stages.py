@@ -40,3 +40,24 @@ def test_calls_without_rank_term_follow_each_other():
     for _ in range(5):
         assert torch.equal(chain(False), want)
     assert all(binding.workspace_status(w) == 0 for w in ws)
+
+
+# input gradient: two steps per stage up to 64 tokens of 2-bit codes, one otherwise; one token box and two
+@pytest.mark.parametrize("b0,M", [(2, 17), (2, 64), (2, 65), (2, 257), (3, 64), (4, 129), (8, 24), (8, 200), (8, 256), (8, 300)])
+@pytest.mark.parametrize("N,K,B0", [(2056, 192, 16), (712, 576, 64)])
+def test_steps_per_stage_of_the_input_gradient(N, K, B0, b0, M):
+    cfg = C(b0, B0, 8, 64, 32)
+    assert binding.linear_path(N, K, cfg, 48, M, True) == binding.PATH_TC_ONE
+    A = inputs.gaussian(8300 + N + b0, (N, K), 0.02)
+    l1b, l2b = inputs.lowrank_factors(8301 + K, N, K, 48, 0.03)
+    run_case(A, l1b, l2b, cfg, M, seed=8400 + M)
+
+
+def test_more_than_37_row_tiles_of_the_pre_product():
+    """One split of the contraction per row tile, whatever the linear kernel leaves idle; the last tile is one row."""
+    N, K, M = 512, 512, 4865
+    cfg = C(3, 64, 8, 64, 32)
+    assert binding.linear_path(N, K, cfg, 64, M, False) == binding.PATH_TC_ONE
+    A = inputs.gaussian(8500, (N, K), 0.03)
+    l1b, l2b = inputs.lowrank_factors(8501, N, K, 64, 0.03)
+    run_case(A, l1b, l2b, cfg, M, seed=8502, rows=inputs.sample_rows(8503, M, count=24, tile=128))
